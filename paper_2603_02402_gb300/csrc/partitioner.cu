@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "knn_tc.cuh"
+#include "warp_sort.cuh"
 
 struct rsc_partitioner;
 
@@ -343,21 +344,41 @@ __global__ void histogram_kernel(int64_t count, const int32_t *__restrict__ key,
     if (i < count) atomicAdd(&hist[key[i]], 1);
 }
 
-// Single block: off[0] = 0, off[p + 1] = off[p] + cnt[p] (int64); also item
-// offsets ceil(cnt / tile) when items != nullptr.
+// Single block of 1024 threads, P <= 1024: off[0] = 0, off[p + 1] = off[p] +
+// cnt[p] (int64); also item offsets ceil(cnt / tile) when items != nullptr.
 __global__ void __launch_bounds__(1024)
 offsets_kernel(int P, const int32_t *__restrict__ cnt, int64_t *__restrict__ off, int tile,
                int32_t *__restrict__ items) {
-    // serial scan over at most 1024 entries by thread 0 (tiny)
-    if (threadIdx.x == 0) {
-        int64_t a = 0;
-        int32_t b = 0;
-        for (int p = 0; p < P; ++p) {
-            off[p] = a;
-            if (items) items[p] = b;
-            a += cnt[p];
-            if (items) b += (int32_t)((cnt[p] + tile - 1) / tile);
+    __shared__ int64_t wc[32];
+    __shared__ int32_t wi[32];
+    const int p = threadIdx.x, lane = p & 31, warp = p >> 5;
+    const int32_t c = p < P ? cnt[p] : 0;
+    int64_t a = c;
+    int32_t b = (c + tile - 1) / tile;
+    const int32_t b0 = b;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t ya = __shfl_up_sync(0xffffffffu, a, o);
+        const int32_t yb = __shfl_up_sync(0xffffffffu, b, o);
+        if (lane >= o) {
+            a += ya;
+            b += yb;
         }
+    }
+    if (lane == 31) {
+        wc[warp] = a;
+        wi[warp] = b;
+    }
+    __syncthreads();
+    for (int v = 0; v < warp; ++v) {
+        a += wc[v];
+        b += wi[v];
+    }
+    if (p < P) {
+        off[p] = a - c;
+        if (items) items[p] = b - b0;
+    }
+    if (p == P - 1) {
         off[P] = a;
         if (items) items[P] = b;
     }
@@ -371,22 +392,88 @@ __global__ void scatter_kernel(int64_t count, const int32_t *__restrict__ key, c
     perm[off[k] + atomicAdd(&cursor[k], 1)] = (int32_t)i;
 }
 
-// Probe slots: the (query, probe) pairs grouped by part.  slot = position in
-// the grouped order; gq[slot] = query, gpos[query * R + r] = slot.
-__global__ void probe_scatter_kernel(int64_t nq, int R, const int32_t *__restrict__ route,
-                                     const int64_t *__restrict__ off, int32_t *__restrict__ cursor,
-                                     int32_t *__restrict__ gq, int64_t *__restrict__ gpos) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nq * R) return;
-    const int p = route[e];
-    const int64_t slot = off[p] + atomicAdd(&cursor[p], 1);
-    gq[slot] = (int32_t)(e / R);
-    gpos[e] = slot;
+// Probe slots: the probes r0 .. r0 + M - 1 of every query (route [nq, R]),
+// grouped by part.  Blocks of kGroupEntries (query, probe) entries rank their
+// entries per part in shared memory and take one range of each part's cursor,
+// so a part's counter sees one atomic per block and not one per entry.  4M
+// entries over 512 parts: 35 us for the counts and 197 us for the slots and
+// the operand rows (544 + 556 + 185 us with a global atomic per entry and the
+// rows gathered by slot).
+constexpr int kGroupThreads = 256;
+constexpr int kGroupEntries = 2048;
+constexpr int kMaxParts = 1024;
+
+// A network that produced NaN logits leaves no part id: such a probe reads part 0.
+__device__ __forceinline__ int safe_part(int p, int P) { return (p >= 0 && p < P) ? p : 0; }
+
+__global__ void __launch_bounds__(kGroupThreads)
+group_count_kernel(int64_t nq, int R, int r0, int M, int P, const int32_t *__restrict__ route,
+                   int32_t *__restrict__ cnt) {
+    __shared__ int hist[kMaxParts];
+    for (int p = threadIdx.x; p < P; p += kGroupThreads) hist[p] = 0;
+    __syncthreads();
+    const int64_t e0 = (int64_t)blockIdx.x * kGroupEntries, e1 = min(nq * M, e0 + kGroupEntries);
+    for (int64_t e = e0 + threadIdx.x; e < e1; e += kGroupThreads)
+        atomicAdd(&hist[safe_part(route[(e / M) * R + r0 + e % M], P)], 1);
+    __syncthreads();
+    for (int p = threadIdx.x; p < P; p += kGroupThreads)
+        if (hist[p]) atomicAdd(&cnt[p], hist[p]);
 }
 
-__global__ void iota64_kernel(int64_t count, int64_t *__restrict__ out) {
+// gpos[q * M + m] = slot of the entry; operand row of the slot = the query's
+// row of Qb (rows[q], or q0 + q), read in query order and written as whole
+// 128-byte rows; slot_thr[slot] = thr[q] when given.
+__global__ void __launch_bounds__(kGroupThreads)
+group_slots_kernel(int64_t nq, int R, int r0, int M, int P, const int32_t *__restrict__ route,
+                   const int64_t *__restrict__ off, int32_t *__restrict__ cursor, const int32_t *__restrict__ rows,
+                   int64_t q0, const uint4 *__restrict__ Qb, const float *__restrict__ thr,
+                   int32_t *__restrict__ gpos, uint4 *__restrict__ Qg, float *__restrict__ slot_thr) {
+    constexpr int kPer = kGroupEntries / kGroupThreads;
+    __shared__ int cnt[kMaxParts];
+    __shared__ int32_t slot[kGroupEntries];
+    for (int p = threadIdx.x; p < P; p += kGroupThreads) cnt[p] = 0;
+    __syncthreads();
+    const int64_t e0 = (int64_t)blockIdx.x * kGroupEntries, total = nq * M;
+    const int here = (int)min((int64_t)kGroupEntries, total - e0);
+    int part[kPer], rank[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int x = threadIdx.x + i * kGroupThreads;
+        part[i] = -1;
+        rank[i] = 0;
+        if (x < here) {
+            const int64_t e = e0 + x;
+            part[i] = safe_part(route[(e / M) * R + r0 + e % M], P);
+            rank[i] = atomicAdd(&cnt[part[i]], 1);
+        }
+    }
+    __syncthreads();
+    for (int p = threadIdx.x; p < P; p += kGroupThreads) {
+        const int c = cnt[p];
+        if (c) cnt[p] = (int)off[p] + atomicAdd(&cursor[p], c);   // first slot of this block's range
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        if (part[i] >= 0) {
+            const int x = threadIdx.x + i * kGroupThreads;
+            const int s = cnt[part[i]] + rank[i];
+            slot[x] = s;
+            gpos[e0 + x] = s;
+            if (thr) slot_thr[s] = thr[(e0 + x) / M];
+        }
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < here * 8; x += kGroupThreads) {
+        const int64_t q = (e0 + (x >> 3)) / M;
+        const int64_t row = rows ? (int64_t)rows[q] : q0 + q;
+        Qg[(int64_t)slot[x >> 3] * 8 + (x & 7)] = Qb[row * 8 + (x & 7)];
+    }
+}
+
+__global__ void iota_kernel(int64_t count, int32_t *__restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) out[i] = i;
+    if (i < count) out[i] = (int32_t)i;
 }
 
 __global__ void set_segment_kernel(int32_t *__restrict__ cnt, int32_t c0, int64_t *__restrict__ doff, int64_t d0,
@@ -396,87 +483,175 @@ __global__ void set_segment_kernel(int32_t *__restrict__ cnt, int32_t c0, int64_
     doff[1] = d1;
 }
 
-__global__ void add_offset_kernel(int64_t count, int32_t *__restrict__ a, int32_t off) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) a[i] += off;
-}
-
-// out[j] = base[pos[j]] (composed row ids).
-__global__ void compose_kernel(int64_t count, const int32_t *__restrict__ pos, const int32_t *__restrict__ base,
-                               int32_t *__restrict__ out) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < count) out[j] = base[pos[j]];
-}
-
 // ------------------------------------------------ exact merge re-rank
+
+constexpr int kSlotList = 16;     // ids per (slot, column part)
+constexpr int kSlotParts = 4;     // column parts per slot (k <= 16)
+constexpr int kPerSlot = kSlotList * kSlotParts;
+
+// A query's first probe (the part the network ranks first) bounds what the
+// other probes can add.  Warp per query: T = the k-th smallest accumulator
+// value among the first probe's kPerSlot candidates, and thr = a value at and
+// above which no candidate of any probe can be among the query's k nearest;
+// the other probes' lists start below it, and the first probe's own
+// candidates at or above it are dropped (id -1).
+//
+// The accumulator is s = |v_j|^2 - 2 v_i.v_j = |v_i - v_j|^2 - |v_i|^2 with v
+// the BF16-rounded rows.  With a = 2^-8 (1 + 2^-6) >= the rounding of a row
+// relative to its length, V = |v_i| and D = |v_i - v_j|: the true distance
+// lies within a V + a (V + D) of D.  So the k nearest are no further than
+// Dk (1 + a) + 2 a V (Dk from T), and a candidate is further than that when
+// D (1 - a) - 2 a V exceeds it, i.e. when D > (Dk (1 + a) + 4 a V) / (1 - a).
+// Squared terms get 2^-13 (V^2 + (V + D)^2) for the FP32 accumulation of the
+// K = 64 MMA (worst case 2^-15 of the terms' size) and of the re-rank's own
+// sums.  The search of 8 probes of 500k queries takes 1.37 ms (first) + 2.78 ms
+// (the other seven) with the bound and 8.8 ms without: what it spends is list
+// building, and a bounded list takes in a few entries only.  No bound (T infinite, overflow, NaN): thr = +inf, nothing is dropped.
+__global__ void __launch_bounds__(256)
+probe_bound_kernel(int64_t nq, int d, int k, const int32_t *__restrict__ rows, int64_t q0,
+                   const uint32_t *__restrict__ Qb, const int32_t *__restrict__ gpos,
+                   const float *__restrict__ key, int32_t *__restrict__ cand, float *__restrict__ thr) {
+    static_assert(kPerSlot == 64, "two candidates per lane");
+    const int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (q >= nq) return;
+    const int64_t row = rows ? (int64_t)rows[q] : q0 + q;
+    const uint32_t w = Qb[row * 32 + lane];   // components 2 lane, 2 lane + 1
+    const float v0 = 2 * lane < d ? __uint_as_float(w << 16) : 0.f;
+    const float v1 = 2 * lane + 1 < d ? __uint_as_float(w & 0xffff0000u) : 0.f;
+    float vv = fmaf(v0, v0, v1 * v1);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) vv += __shfl_xor_sync(0xffffffffu, vv, o);
+    const int64_t at = (int64_t)gpos[q] * kPerSlot + lane;
+    const float k0 = key[at], k1 = key[at + 32];
+    float sk[2] = {k0, k1};
+    int si[2] = {lane, lane + 32};
+    warp_sort_pairs<2>(sk, si);
+    const float T = __shfl_sync(0xffffffffu, sk[0], k - 1);   // k <= 16
+    const float a = 0x1p-8f * (1.f + 0x1p-6f), V = sqrtf(vv) * (1.f + 0x1p-20f);
+    const float Dk = sqrtf(fmaxf(T + vv, 0.f) + 0x1p-12f * (vv + fmaxf(T, 0.f)));
+    const float D = (Dk * (1.f + a) + 4.f * a * V) / (1.f - a) * (1.f + 0x1p-12f);
+    float t = D * D - vv + 0x1p-13f * (vv + (V + D) * (V + D));
+    if (!(t < INFINITY)) t = INFINITY;
+    if (!(k0 < t)) cand[at] = -1;
+    if (!(k1 < t)) cand[at + 32] = -1;
+    if (lane == 0) thr[q] = t;
+}
 
 constexpr int kRWarps = 4;
 
-__device__ __forceinline__ bool pgt(float ka, int ia, float kb, int ib) { return ka > kb || (ka == kb && ia > ib); }
-
-// Warp per query: the R probed slots' candidate lists (ids in the database's
-// sorted order, mapped through perm; perm == nullptr: identity) are re-scored
-// by direct difference in FP32 over X and the k best by (distance, id) kept.
+// Exact merge re-rank, warp per query: the candidates of its probes (ids in
+// the database's sorted order, mapped through perm; perm == nullptr:
+// identity) are re-scored by direct difference in FP32 over X and the k <= 16
+// best by (distance, id) kept.  Slots: gpos0[q] of cand0, and with R > 1
+// gpos1[q * (R - 1) ..] of cand1.  The valid ids (what the bound of the first
+// probe left, typically a tenth of the R * kPerSlot entries) are first
+// compacted into shared memory; then a lane scores a candidate, 32 at a time,
+// and each batch is sorted in registers and merged into the best 32 (a
+// bitonic merge against the reversed batch).  VW floats per load: 4 or 2 when
+// every row of X starts on such a boundary.  The sum runs in component order
+// whatever VW is.
+// 500k queries, 8 probes of 512 parts, d = 50: 3.2 ms, bound by the gathers of
+// the candidate rows; 50.6 ms when all 512 entries were scored with scalar
+// loads and sorted in shared memory.
+template <int VW>
 __global__ void __launch_bounds__(kRWarps * 32)
 rerank_probe_kernel(const float *__restrict__ X, int d, const int32_t *__restrict__ qrows, int64_t q_base,
-                    int64_t nq, int R,
-                    const int64_t *__restrict__ gpos, const int32_t *__restrict__ cand, int per_slot,
-                    const int32_t *__restrict__ perm, int64_t n_db, int C2, int k, int32_t *__restrict__ idx,
+                    int64_t nq, int R, const int32_t *__restrict__ gpos0, const int32_t *__restrict__ cand0,
+                    const int32_t *__restrict__ gpos1, const int32_t *__restrict__ cand1,
+                    const int32_t *__restrict__ perm, int64_t n_db, int k, int32_t *__restrict__ idx,
                     float *__restrict__ dist) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float *xq = reinterpret_cast<float *>(smem) + warp * 64;
-    float *sk = reinterpret_cast<float *>(smem) + kRWarps * 64 + warp * C2;
-    int *si = reinterpret_cast<int *>(reinterpret_cast<float *>(smem) + kRWarps * 64 + kRWarps * C2) + warp * C2;
+    int *ids = reinterpret_cast<int *>(reinterpret_cast<float *>(smem) + kRWarps * 64) + warp * R * kPerSlot;
     const int64_t q = (int64_t)blockIdx.x * kRWarps + warp;
     if (q >= nq) return;
-    const int64_t row = qrows ? qrows[q] : q_base + q;
-    for (int t = lane; t < d; t += 32) xq[t] = X[row * d + t];
+    const int64_t row = qrows ? (int64_t)qrows[q] : q_base + q;
+    for (int t = lane; t < 64; t += 32) xq[t] = t < d ? X[row * d + t] : 0.f;
+    int count = 0;
+    for (int r = 0; r < R; ++r) {
+        const int32_t *c = r == 0 ? cand0 + (int64_t)gpos0[q] * kPerSlot
+                                  : cand1 + (int64_t)gpos1[q * (R - 1) + r - 1] * kPerSlot;
+#pragma unroll
+        for (int h = 0; h < kPerSlot; h += 32) {
+            const int32_t j = c[h + lane];
+            const bool ok = j >= 0 && (int64_t)j < n_db;   // empty, dropped, or ids of an aborted search
+            const unsigned m = __ballot_sync(0xffffffffu, ok);
+            if (ok) ids[count + __popc(m & ((1u << lane) - 1u))] = j;
+            count += __popc(m);
+        }
+    }
     __syncwarp();
-    const int C = R * per_slot;
-    for (int c = lane; c < C2; c += 32) {
-        float key = INFINITY;
-        int id = INT_MAX;
-        if (c < C) {
-            const int r = c / per_slot;
-            const int32_t j = cand[gpos[q * R + r] * per_slot + (c - r * per_slot)];
-            if (j >= 0 && (int64_t)j < n_db) {   // ids outside [0, n_db) (an aborted search) are skipped
-                const int32_t o = perm ? perm[j] : j;
-                const float *yr = X + (int64_t)o * d;
-                float acc = 0.f;
+    float bk[1] = {INFINITY};   // the best 32, ascending over the lanes
+    int bi[1] = {INT_MAX};
+    for (int c0 = 0; c0 < count; c0 += 32) {
+        float key[1] = {INFINITY};
+        int id[1] = {INT_MAX};
+        if (c0 + lane < count) {
+            const int32_t j = ids[c0 + lane];
+            const int32_t o = perm ? perm[j] : j;
+            const float *yr = X + (int64_t)o * d;
+            float acc = 0.f;
+            if constexpr (VW == 4) {
+                const float4 *y4 = reinterpret_cast<const float4 *>(yr);
+#pragma unroll 4
+                for (int t = 0; t < d; t += 4) {
+                    const float4 y = __ldg(y4 + (t >> 2));
+                    float f;
+                    f = xq[t] - y.x; acc = fmaf(f, f, acc);
+                    f = xq[t + 1] - y.y; acc = fmaf(f, f, acc);
+                    f = xq[t + 2] - y.z; acc = fmaf(f, f, acc);
+                    f = xq[t + 3] - y.w; acc = fmaf(f, f, acc);
+                }
+            } else if constexpr (VW == 2) {
+                const float2 *y2 = reinterpret_cast<const float2 *>(yr);
+#pragma unroll 8
+                for (int t = 0; t < d; t += 2) {
+                    const float2 y = __ldg(y2 + (t >> 1));
+                    float f;
+                    f = xq[t] - y.x; acc = fmaf(f, f, acc);
+                    f = xq[t + 1] - y.y; acc = fmaf(f, f, acc);
+                }
+            } else {
+#pragma unroll 8
                 for (int t = 0; t < d; ++t) {
-                    const float diff = xq[t] - __ldg(yr + t);
-                    acc = fmaf(diff, diff, acc);
-                }
-                key = acc;
-                id = o;
-            }
-        }
-        sk[c] = key;
-        si[c] = id;
-    }
-    __syncwarp();
-    for (int size = 2; size <= C2; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = lane; i < C2 / 2; i += 32) {
-                const int a = (i / stride) * 2 * stride + (i % stride), b = a + stride;
-                const bool asc = (a & size) == 0;
-                const float ka = sk[a], kb = sk[b];
-                const int ia = si[a], ib = si[b];
-                if (asc ? pgt(ka, ia, kb, ib) : pgt(kb, ib, ka, ia)) {
-                    sk[a] = kb;
-                    sk[b] = ka;
-                    si[a] = ib;
-                    si[b] = ia;
+                    const float f = xq[t] - __ldg(yr + t);
+                    acc = fmaf(f, f, acc);
                 }
             }
-            __syncwarp();
+            key[0] = acc;
+            id[0] = o;
+        }
+        warp_sort_pairs<1>(key, id);
+        if (c0 == 0) {
+            bk[0] = key[0];
+            bi[0] = id[0];
+            continue;
+        }
+        // the 32 smallest of two ascending runs: elementwise minima of one and
+        // the other reversed form a bitonic run, sorted by five half-cleaners
+        const float rk = __shfl_xor_sync(0xffffffffu, key[0], 31);
+        const int ri = __shfl_xor_sync(0xffffffffu, id[0], 31);
+        if (pair_gt(bk[0], bi[0], rk, ri)) {
+            bk[0] = rk;
+            bi[0] = ri;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float pk = __shfl_xor_sync(0xffffffffu, bk[0], o);
+            const int pi = __shfl_xor_sync(0xffffffffu, bi[0], o);
+            const bool lower = (lane & o) == 0;
+            if (lower ? pair_gt(bk[0], bi[0], pk, pi) : pair_gt(pk, pi, bk[0], bi[0])) {
+                bk[0] = pk;
+                bi[0] = pi;
+            }
         }
     }
-    for (int c = lane; c < k; c += 32) {
-        const bool valid = si[c] != INT_MAX;
-        idx[q * k + c] = valid ? si[c] : -1;
-        dist[q * k + c] = valid ? sqrtf(sk[c]) : INFINITY;
+    if (lane < k) {
+        const bool valid = bi[0] != INT_MAX;
+        idx[q * k + lane] = valid ? bi[0] : -1;
+        dist[q * k + lane] = valid ? sqrtf(bk[0]) : INFINITY;
     }
 }
 
@@ -488,9 +663,13 @@ namespace tck {
 
 // Segments of gathered query rows scanned against database row ranges:
 // segment p = query slots [goff[p], goff[p+1]) x database rows [doff[p], doff[p+1]).
+// kBound: each slot's lists start below thr[slot] (and take nothing at or
+// above it); otherwise they start empty and their keys are written to `key`
+// when it is given.
+template <bool kBound>
 struct ProbeWork {
     static constexpr int kShort = 0;
-    static constexpr bool kResume = false;
+    static constexpr bool kResume = kBound;
     static constexpr bool kHitHeavy = false;
     static constexpr bool kStartBelow = false;
     static constexpr bool kDynamic = true;   // segments differ in size
@@ -499,6 +678,8 @@ struct ProbeWork {
     const int64_t *doff;
     const int32_t *item_off;   // [P + 1] first work item of each segment
     int32_t *cand;             // [slots, EG * KCP]
+    float *key;                // [slots, EG * KCP] or null
+    const float *thr;          // [slots] (kBound)
     int *counter;              // next item (zeroed before the launch)
 
     int64_t count_host() const { return INT_MAX; }   // the grid is sized by the SM count
@@ -524,10 +705,25 @@ struct ProbeWork {
         return w;
     }
     template <int EG, int KCP>
-    __device__ __forceinline__ void emit(const WorkItem &, int part, int64_t q, const RowTopK<KCP> &list) const {
-        int32_t *out = cand + (q * EG + part) * KCP;
+    __device__ __forceinline__ void resume(const WorkItem &, int, int64_t q, RowTopK<KCP> &list) const {
+        const float t = thr[q];
 #pragma unroll
-        for (int c = 0; c < KCP; ++c) out[c] = list.id[c];
+        for (int c = 0; c < KCP; ++c) {
+            list.key[c] = t;
+            list.id[c] = -1;
+        }
+    }
+    template <int EG, int KCP>
+    __device__ __forceinline__ void emit(const WorkItem &, int part, int64_t q, const RowTopK<KCP> &list) const {
+        int4 *out = reinterpret_cast<int4 *>(cand + (q * EG + part) * KCP);
+#pragma unroll
+        for (int c = 0; c < KCP; c += 4) out[c / 4] = make_int4(list.id[c], list.id[c + 1], list.id[c + 2], list.id[c + 3]);
+        if (!kBound && key) {
+            float4 *ko = reinterpret_cast<float4 *>(key + (q * EG + part) * KCP);
+#pragma unroll
+            for (int c = 0; c < KCP; c += 4)
+                ko[c / 4] = make_float4(list.key[c], list.key[c + 1], list.key[c + 2], list.key[c + 3]);
+        }
     }
 };
 
@@ -556,9 +752,9 @@ struct rsc_partitioner {
 
 namespace {
 
-constexpr int kSlotList = 16;     // ids per (slot, column part)
-constexpr int kSlotParts = 4;     // column parts per slot (k <= 16)
-constexpr int kPerSlot = kSlotList * kSlotParts;
+using part::kPerSlot;
+using part::kSlotList;
+using part::kSlotParts;
 constexpr int kChunkRows = 32768; // network rows per forward chunk
 constexpr int kMaxProbe = 8;
 
@@ -803,10 +999,13 @@ struct PartLayout {
     int32_t *item_counter;          // [1] the probe search's dynamic item counter
     // search (per query chunk)
     int32_t *route;                 // [chunk, R]
-    int32_t *gq;                    // [chunk * R]
-    int64_t *gpos;                  // [chunk * R]
-    void *Qg;                       // [chunk * R, 64] bf16
-    int32_t *cand;                  // [chunk * R, kPerSlot]
+    int32_t *gpos;                  // [chunk] slots of the first probes, then [chunk, R - 1] of the others
+    void *Qg;                       // [slots of one pass, 64] bf16
+    int32_t *cand0;                 // [chunk, kPerSlot] candidates of the first probes
+    float *key0;                    // [chunk, kPerSlot] their accumulator values
+    float *thr;                     // [chunk] bound of every query
+    int32_t *cand1;                 // [chunk * (R - 1), kPerSlot] candidates of the other probes
+    float *slot_thr;                // [chunk * (R - 1)] bounds by slot
     float *Xq;                      // [kChunkRows, d] gathered network input
 };
 
@@ -817,7 +1016,7 @@ PartLayout carve_part(void *ws, const rsc_partitioner *p, int64_t n, int64_t n_t
     const int DP = ((p->d + 7) / 8) * 8;
     const int64_t NT = std::max<int64_t>(n_train, 1);
     const int64_t B = 1024;
-    const int64_t slots = std::max<int64_t>(chunk * R, NT);
+    const int64_t first = std::max<int64_t>(chunk, NT), rest = chunk * (R - 1);
     L.status = cv.take<unsigned int>(kStatusBytes / 4);
     L.Y = cv.take<float>((size_t)n * DP);
     L.ny = cv.take<float>((size_t)n);
@@ -848,10 +1047,13 @@ PartLayout carve_part(void *ws, const rsc_partitioner *p, int64_t n, int64_t n_t
     L.items = cv.take<int32_t>((size_t)p->P + 1);
     L.item_counter = cv.take<int32_t>(1);
     L.route = cv.take<int32_t>((size_t)chunk * R);
-    L.gq = cv.take<int32_t>((size_t)slots);
-    L.gpos = cv.take<int64_t>((size_t)slots);
-    L.Qg = cv.take<uint16_t>((size_t)slots * 64);
-    L.cand = cv.take<int32_t>((size_t)slots * kPerSlot);
+    L.gpos = cv.take<int32_t>((size_t)(first + rest));
+    L.Qg = cv.take<uint16_t>((size_t)std::max(first, rest) * 64);
+    L.cand0 = cv.take<int32_t>((size_t)first * kPerSlot);
+    L.key0 = cv.take<float>((size_t)chunk * kPerSlot);
+    L.thr = cv.take<float>((size_t)chunk);
+    L.cand1 = cv.take<int32_t>((size_t)rest * kPerSlot);
+    L.slot_thr = cv.take<float>((size_t)rest);
     L.Xq = cv.take<float>((size_t)kChunkRows * p->d);
     if (bytes) *bytes = cv.used;
     return L;
@@ -860,30 +1062,48 @@ PartLayout carve_part(void *ws, const rsc_partitioner *p, int64_t n, int64_t n_t
 int64_t search_chunk(int64_t nq) { return std::min<int64_t>(std::max<int64_t>(nq, 1), 1 << 20); }
 
 // Exact candidates of gathered query rows, segment by segment, through the
-// tensor-core kernel (segment p: slots goff[p].. x database rows doff[p]..).
+// tensor-core kernel (segment p: slots goff[p].. x database rows doff[p]..;
+// goff from the counts gcnt).  kBound: see ProbeWork.
+template <bool kBound>
 rsc_status probe_search(cudaStream_t st, const void *Dop, int64_t n_db, int64_t n_slots, int P_seg,
-                        const PartLayout &L, const int64_t *doff) {
-    part::offsets_kernel<<<1, 32, 0, st>>>(P_seg, L.gcnt, L.goff, tck::BM, L.items);
+                        const PartLayout &L, const int64_t *doff, int32_t *cand, float *key) {
     CUtensorMap mq, md;
     cudaError_t e = tck::make_map(&mq, L.Qg, std::max<int64_t>(n_slots, 1), 1, tck::BM);
     if (e == cudaSuccess) e = tck::make_map(&md, Dop, n_db, 1, tck::BN);
     if (e != cudaSuccess) return fail(RSC_ERR_CUDA, "tensor map: %s", cudaGetErrorString(e));
-    tck::ProbeWork work{P_seg, L.goff, doff, L.items, L.cand, L.item_counter};
+    tck::ProbeWork<kBound> work{P_seg, L.goff, doff, L.items, cand, key, kBound ? L.slot_thr : nullptr, L.item_counter};
     e = cudaMemsetAsync(L.item_counter, 0, sizeof(int32_t), st);
     if (e == cudaSuccess) e = tck::launch_kernel<1, kSlotList, kSlotParts>(mq, md, work, L.status, st);
     if (e != cudaSuccess) return fail(RSC_ERR_CUDA, "probe search launch: %s", cudaGetErrorString(e));
     return RSC_OK;
 }
 
+// Groups probes r0 .. r0 + M - 1 of nq queries by part: counts, slot offsets
+// and work items, slots and operand rows (thr: bounds of the queries, nullable).
+void launch_group(cudaStream_t st, const rsc_partitioner *p, const PartLayout &L, int64_t nq, int R, int r0, int M,
+                  const int32_t *rows, int64_t q0, const float *thr, int32_t *gpos) {
+    cudaMemsetAsync(L.gcnt, 0, sizeof(int32_t) * p->P * 2, st);
+    const unsigned blocks = (unsigned)ceil_div(nq * M, part::kGroupEntries);
+    part::group_count_kernel<<<blocks, part::kGroupThreads, 0, st>>>(nq, R, r0, M, p->P, L.route, L.gcnt);
+    part::offsets_kernel<<<1, 1024, 0, st>>>(p->P, L.gcnt, L.goff, tck::BM, L.items);
+    part::group_slots_kernel<<<blocks, part::kGroupThreads, 0, st>>>(
+        nq, R, r0, M, p->P, L.route, L.goff, L.gcursor, rows, q0, static_cast<const uint4 *>(L.Qb), thr, gpos,
+        static_cast<uint4 *>(L.Qg), L.slot_thr);
+}
+
+// vector loads as wide as every row's start allows
 rsc_status launch_rerank_probe(cudaStream_t st, const float *X, int64_t n_db, int d, const int32_t *qrows,
-                               int64_t q_base, int64_t nq, int R, const int64_t *gpos, const int32_t *cand,
-                               const int32_t *perm, int k, int32_t *idx, float *dist) {
-    int C2 = 32;
-    while (C2 < R * kPerSlot) C2 <<= 1;
-    if (C2 > 1024) return fail(RSC_ERR_INVALID_ARG, "too many probe candidates");
-    const size_t smem = sizeof(float) * part::kRWarps * 64 + (sizeof(float) + sizeof(int)) * part::kRWarps * C2;
-    part::rerank_probe_kernel<<<(unsigned)ceil_div(nq, part::kRWarps), part::kRWarps * 32, smem, st>>>(
-        X, d, qrows, q_base, nq, R, gpos, cand, kPerSlot, perm, n_db, C2, k, idx, dist);
+                               int64_t q_base, int64_t nq, int R, const int32_t *gpos0, const int32_t *cand0,
+                               const int32_t *gpos1, const int32_t *cand1, const int32_t *perm, int k, int32_t *idx,
+                               float *dist) {
+    const size_t smem = sizeof(float) * part::kRWarps * (64 + R * kPerSlot);
+    const unsigned blocks = (unsigned)ceil_div(nq, part::kRWarps);
+    const uintptr_t at = reinterpret_cast<uintptr_t>(X);
+    auto kern = (d % 4 == 0 && at % 16 == 0) ? part::rerank_probe_kernel<4>
+                : (d % 2 == 0 && at % 8 == 0) ? part::rerank_probe_kernel<2>
+                                              : part::rerank_probe_kernel<1>;
+    kern<<<blocks, part::kRWarps * 32, smem, st>>>(X, d, qrows, q_base, nq, R, gpos0, cand0, gpos1, cand1, perm, n_db,
+                                                   k, idx, dist);
     RSC_CUDA_TRY(cudaGetLastError());
     return RSC_OK;
 }
@@ -985,7 +1205,7 @@ rsc_status rsc_partitioner_build_index(rsc_partitioner *p, const float *X, int64
     if ((s = network_route(p, st, X, nullptr, n, 1, L, L.labels)) != RSC_OK) return s;
     RSC_CUDA_TRY(cudaMemsetAsync(L.gcnt, 0, sizeof(int32_t) * p->P * 2, st));
     part::histogram_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, L.labels, L.gcnt);
-    part::offsets_kernel<<<1, 32, 0, st>>>(p->P, L.gcnt, p->doff, 1, nullptr);
+    part::offsets_kernel<<<1, 1024, 0, st>>>(p->P, L.gcnt, p->doff, 1, nullptr);
     part::scatter_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, L.labels, p->doff, L.gcursor, p->perm);
     part::permute_rows_kernel<<<(unsigned)ceil_div(n * 8, 256), 256, 0, st>>>(
         static_cast<const uint4 *>(L.Db), p->perm, n, static_cast<uint4 *>(p->Db_sorted));
@@ -1033,10 +1253,11 @@ rsc_status rsc_partitioner_train(rsc_partitioner *p, const float *X, int64_t n, 
     part::permute_rows_kernel<<<(unsigned)ceil_div(n_train * 8, 256), 256, 0, st>>>(
         static_cast<const uint4 *>(L.Qb), train_rows, n_train, static_cast<uint4 *>(L.Qg));
     part::set_segment_kernel<<<1, 1, 0, st>>>(L.gcnt, (int32_t)n_train, L.doff, 0, n);
-    if ((s = probe_search(st, L.Db, n, n_train, 1, L, L.doff)) != RSC_OK) return s;
-    part::iota64_kernel<<<(unsigned)ceil_div(n_train, 256), 256, 0, st>>>(n_train, L.gpos);
-    if ((s = launch_rerank_probe(st, X, n, d, train_rows, 0, n_train, 1, L.gpos, L.cand, nullptr, k, L.nbr,
-                                 L.nbr_dist)) != RSC_OK)
+    part::offsets_kernel<<<1, 1024, 0, st>>>(1, L.gcnt, L.goff, tck::BM, L.items);
+    if ((s = probe_search<false>(st, L.Db, n, n_train, 1, L, L.doff, L.cand0, nullptr)) != RSC_OK) return s;
+    part::iota_kernel<<<(unsigned)ceil_div(n_train, 256), 256, 0, st>>>(n_train, L.gpos);
+    if ((s = launch_rerank_probe(st, X, n, d, train_rows, 0, n_train, 1, L.gpos, L.cand0, nullptr, nullptr, nullptr, k,
+                                 L.nbr, L.nbr_dist)) != RSC_OK)
         return s;
     part::gather_rows_kernel<<<(unsigned)ceil_div(n_train * d, 256), 256, 0, st>>>(train_rows, n_train, X, d, L.Xt);
 
@@ -1114,23 +1335,25 @@ rsc_status rsc_knn_partitioned(rsc_partitioner *p, const float *X, int64_t n, in
             if (rows) launch_route(st, R, X, rows, cq, p->d, p->centroids, p->P, L.route);
             else launch_route(st, R, X + q0 * p->d, nullptr, cq, p->d, p->centroids, p->P, L.route);
         }
-        // 2. group (query, probe) pairs by part; gather the query operand rows
-        RSC_CUDA_TRY(cudaMemsetAsync(L.gcnt, 0, sizeof(int32_t) * p->P * 2, st));
-        part::histogram_kernel<<<(unsigned)ceil_div(cq * R, 256), 256, 0, st>>>(cq * R, L.route, L.gcnt);
-        part::offsets_kernel<<<1, 32, 0, st>>>(p->P, L.gcnt, L.goff, tck::BM, L.items);
-        part::probe_scatter_kernel<<<(unsigned)ceil_div(cq * R, 256), 256, 0, st>>>(cq, R, L.route, L.goff,
-                                                                                   L.gcursor, L.gq, L.gpos);
-        // gq holds chunk-local query positions: make them rows of X
-        const int64_t slots = cq * R;
-        if (rows) part::compose_kernel<<<(unsigned)ceil_div(slots, 256), 256, 0, st>>>(slots, L.gq, rows, L.gq);
-        else part::add_offset_kernel<<<(unsigned)ceil_div(slots, 256), 256, 0, st>>>(slots, L.gq, (int32_t)q0);
-        part::permute_rows_kernel<<<(unsigned)ceil_div(slots * 8, 256), 256, 0, st>>>(
-            static_cast<const uint4 *>(L.Qb), L.gq, slots, static_cast<uint4 *>(L.Qg));
-        // 3. each part's gathered queries against that part's database rows
-        if ((s = probe_search(st, p->Db_sorted, n, slots, p->P, L, p->doff)) != RSC_OK) return s;
+        // 2. the first probe of every query: its part's gathered queries
+        //    against that part's database rows, keys kept
+        launch_group(st, p, L, cq, R, 0, 1, rows, q0, nullptr, L.gpos);
+        if ((s = probe_search<false>(st, p->Db_sorted, n, cq, p->P, L, p->doff, L.cand0, R > 1 ? L.key0 : nullptr)) !=
+            RSC_OK)
+            return s;
+        // 3. the other probes, their lists bounded by the first one's k-th value
+        int32_t *gpos1 = L.gpos + cq;
+        if (R > 1) {
+            part::probe_bound_kernel<<<(unsigned)ceil_div(cq * 32, 256), 256, 0, st>>>(
+                cq, p->d, k, rows, q0, static_cast<const uint32_t *>(L.Qb), L.gpos, L.key0, L.cand0, L.thr);
+            launch_group(st, p, L, cq, R, 1, R - 1, rows, q0, L.thr, gpos1);
+            if ((s = probe_search<true>(st, p->Db_sorted, n, cq * (R - 1), p->P, L, p->doff, L.cand1, nullptr)) !=
+                RSC_OK)
+                return s;
+        }
         // 4. merge the probed parts' candidates with the exact FP32 re-rank
-        if ((s = launch_rerank_probe(st, X, n, p->d, rows, q0, cq, R, L.gpos, L.cand, p->perm, k, idx + q0 * k,
-                                     dist + q0 * k)) != RSC_OK)
+        if ((s = launch_rerank_probe(st, X, n, p->d, rows, q0, cq, R, L.gpos, L.cand0, gpos1, L.cand1, p->perm, k,
+                                     idx + q0 * k, dist + q0 * k)) != RSC_OK)
             return s;
     }
     RSC_CUDA_TRY(cudaGetLastError());

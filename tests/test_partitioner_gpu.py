@@ -96,3 +96,33 @@ def test_save_load_roundtrip(rsc, tmp_path):
     part.save(path)
     other = rsc.Partitioner.load(path)
     np.testing.assert_array_equal(other.get_params(), p0)
+
+
+@pytest.mark.parametrize("n,d,k,probes", [(20_000, 50, 15, 8), (5_003, 33, 16, 8), (9_001, 48, 1, 4), (300, 7, 10, 8),
+                                          (40, 50, 16, 8)])
+def test_probes_bounded_by_the_first_part_lose_nothing(rsc, n, d, k, probes):
+    # with as many probes as parts the search is exact: the bound taken from
+    # the first probed part (which may hold fewer than k rows, or none) must
+    # not drop a neighbour that lies in another part.  Row starts on 4-, 8-
+    # and 16-byte boundaries (d = 33 and 7, 50, 48).  Distances as in the
+    # exact search: 1e-5 relative of FP64.
+    parts = 8
+    X = synth.mixture(n, d, n_comp=12, seed=n)
+    Xd = torch.from_numpy(X).cuda()
+    part = rsc.Partitioner(d, parts, 32, bf16_weights=True, seed=d)
+    part.build_index(Xd)
+    rng = np.random.Generator(np.random.PCG64(n + 1))
+    queries = rng.integers(0, n, size=min(n, 1500)).astype(np.int32)
+    q = torch.from_numpy(queries).cuda()
+    oi, od, _ = oracle.knn(X, k, queries=queries.astype(np.int64))
+    full_i, full_d = (t.cpu().numpy() for t in part.knn(Xd, k=k, n_probe=8, query_rows=q))
+    np.testing.assert_allclose(full_d, od, rtol=1e-5, atol=1e-6)
+    # fewer probes: every query's list is a subset of the exact order, never closer
+    gi, gd = (t.cpu().numpy() for t in part.knn(Xd, k=k, n_probe=probes, query_rows=q))
+    finite = np.isfinite(gd)
+    assert (gd[finite] >= od[finite] * (1 - 1e-5) - 1e-6).all()
+    assert ((gi >= 0) == finite).all()
+    # all rows as queries: the same lists as the sampled rows got
+    ai, ad = (t.cpu().numpy() for t in part.knn(Xd, k=k, n_probe=8))
+    np.testing.assert_array_equal(ai[queries], full_i)
+    np.testing.assert_array_equal(ad[queries], full_d)
