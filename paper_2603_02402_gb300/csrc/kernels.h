@@ -69,6 +69,17 @@ cudaError_t launch_tc_gemm(cudaStream_t st, int M, int N, int K, const float *A,
                            const float *B, int64_t sbk, int64_t sbn, float *C, int64_t ldc, const float *bias,
                            int flags, unsigned int *status);
 
+// The partitioner's network and the R in {1, 2, 4, 8} largest logits of
+// `count` rows of X [., d] (rows[i], or i) in one kernel: out [count, R], value
+// descending, id ascending (INT_MAX where fewer than R logits are numbers).
+// The weights come packed by launch_mlp_route_pack (mlp_route_weight_bytes).
+bool mlp_route_supported(int d, int H, int P);
+size_t mlp_route_weight_bytes(int H, int P);
+cudaError_t launch_mlp_route_pack(cudaStream_t st, int d, int H, int P, const float *W1, const float *b1,
+                                  const float *W2, const float *b2, const float *W3, const float *b3, void *packed);
+cudaError_t launch_mlp_route(cudaStream_t st, const float *X, const int32_t *rows, int64_t count, int d, int H, int P,
+                             int R, const void *packed, int32_t *out, unsigned int *status);
+
 // ---- order.cu -------------------------------------------------------------------
 // Locality ordering: two-level k-means (C1 coarse clusters, then C2 sub-
 // clusters inside each; Lloyd on strided samples), then a stable counting

@@ -339,9 +339,12 @@ __global__ void top_logits_kernel(int64_t rows, int P, const float *__restrict__
 
 // ----------------------------------------------- counting sort by part
 
-__global__ void histogram_kernel(int64_t count, const int32_t *__restrict__ key, int32_t *__restrict__ hist) {
+// A network that produced NaN logits leaves no part id: such a row counts to part 0.
+__device__ __forceinline__ int safe_part(int p, int P) { return (p >= 0 && p < P) ? p : 0; }
+
+__global__ void histogram_kernel(int64_t count, int P, const int32_t *__restrict__ key, int32_t *__restrict__ hist) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) atomicAdd(&hist[key[i]], 1);
+    if (i < count) atomicAdd(&hist[safe_part(key[i], P)], 1);
 }
 
 // Single block of 1024 threads, P <= 1024: off[0] = 0, off[p + 1] = off[p] +
@@ -384,11 +387,11 @@ offsets_kernel(int P, const int32_t *__restrict__ cnt, int64_t *__restrict__ off
     }
 }
 
-__global__ void scatter_kernel(int64_t count, const int32_t *__restrict__ key, const int64_t *__restrict__ off,
+__global__ void scatter_kernel(int64_t count, int P, const int32_t *__restrict__ key, const int64_t *__restrict__ off,
                                int32_t *__restrict__ cursor, int32_t *__restrict__ perm) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
-    const int k = key[i];
+    const int k = safe_part(key[i], P);
     perm[off[k] + atomicAdd(&cursor[k], 1)] = (int32_t)i;
 }
 
@@ -402,9 +405,6 @@ __global__ void scatter_kernel(int64_t count, const int32_t *__restrict__ key, c
 constexpr int kGroupThreads = 256;
 constexpr int kGroupEntries = 2048;
 constexpr int kMaxParts = 1024;
-
-// A network that produced NaN logits leaves no part id: such a probe reads part 0.
-__device__ __forceinline__ int safe_part(int p, int P) { return (p >= 0 && p < P) ? p : 0; }
 
 __global__ void __launch_bounds__(kGroupThreads)
 group_count_kernel(int64_t nq, int R, int r0, int M, int P, const int32_t *__restrict__ route,
@@ -1007,7 +1007,12 @@ struct PartLayout {
     int32_t *cand1;                 // [chunk * (R - 1), kPerSlot] candidates of the other probes
     float *slot_thr;                // [chunk * (R - 1)] bounds by slot
     float *Xq;                      // [kChunkRows, d] gathered network input
+    void *packed;                   // the network's weights as the routing kernel reads them
 };
+
+// BF16 networks with H <= 256 run in the fused routing kernel; wider ones and
+// FP32 networks go through the GEMMs, kChunkRows rows at a time.
+bool fused_route(const rsc_partitioner *p) { return p->bf16 && mlp_route_supported(p->d, p->H, p->P); }
 
 PartLayout carve_part(void *ws, const rsc_partitioner *p, int64_t n, int64_t n_train, int k, int64_t chunk, int R,
                       size_t *bytes) {
@@ -1016,6 +1021,8 @@ PartLayout carve_part(void *ws, const rsc_partitioner *p, int64_t n, int64_t n_t
     const int DP = ((p->d + 7) / 8) * 8;
     const int64_t NT = std::max<int64_t>(n_train, 1);
     const int64_t B = 1024;
+    const bool fused = fused_route(p);
+    const size_t net_rows = fused ? (size_t)B : (size_t)kChunkRows;
     const int64_t first = std::max<int64_t>(chunk, NT), rest = chunk * (R - 1);
     L.status = cv.take<unsigned int>(kStatusBytes / 4);
     L.Y = cv.take<float>((size_t)n * DP);
@@ -1032,9 +1039,9 @@ PartLayout carve_part(void *ws, const rsc_partitioner *p, int64_t n, int64_t n_t
     L.order = cv.take<int32_t>((size_t)NT);
     L.Xb = cv.take<float>((size_t)B * p->d);
     L.T = cv.take<float>((size_t)B * p->P);
-    L.Z1 = cv.take<float>((size_t)kChunkRows * p->H);
-    L.Z2 = cv.take<float>((size_t)kChunkRows * p->H);
-    L.Z3 = cv.take<float>((size_t)kChunkRows * p->P);
+    L.Z1 = cv.take<float>(net_rows * p->H);
+    L.Z2 = cv.take<float>(net_rows * p->H);
+    L.Z3 = cv.take<float>(net_rows * p->P);
     L.dZ3 = cv.take<float>((size_t)B * p->P);
     L.dA = cv.take<float>((size_t)B * p->H);
     L.dZ = cv.take<float>((size_t)B * p->H);
@@ -1054,7 +1061,8 @@ PartLayout carve_part(void *ws, const rsc_partitioner *p, int64_t n, int64_t n_t
     L.thr = cv.take<float>((size_t)chunk);
     L.cand1 = cv.take<int32_t>((size_t)rest * kPerSlot);
     L.slot_thr = cv.take<float>((size_t)rest);
-    L.Xq = cv.take<float>((size_t)kChunkRows * p->d);
+    L.Xq = cv.take<float>(fused ? 0 : (size_t)kChunkRows * p->d);
+    L.packed = cv.take<uint8_t>(fused ? mlp_route_weight_bytes(p->H, p->P) : 0);
     if (bytes) *bytes = cv.used;
     return L;
 }
@@ -1137,6 +1145,13 @@ void launch_top_logits(cudaStream_t st, int R, int64_t rows, int P, const float 
 // Network top-R parts of `count` rows of X (ids `rows`, or rows 0..count-1).
 rsc_status network_route(const rsc_partitioner *p, cudaStream_t st, const float *X, const int32_t *rows,
                          int64_t count, int R, const PartLayout &L, int32_t *out) {
+    if (fused_route(p)) {
+        const float *W = p->params;
+        RSC_CUDA_TRY(launch_mlp_route_pack(st, p->d, p->H, p->P, W + w1_off(p), W + b1_off(p), W + w2_off(p),
+                                           W + b2_off(p), W + w3_off(p), W + b3_off(p), L.packed));
+        RSC_CUDA_TRY(launch_mlp_route(st, X, rows, count, p->d, p->H, p->P, R, L.packed, out, L.status));
+        return RSC_OK;
+    }
     for (int64_t c0 = 0; c0 < count; c0 += kChunkRows) {
         const int B = (int)std::min<int64_t>(kChunkRows, count - c0);
         const float *xb = X + c0 * p->d;
@@ -1204,9 +1219,9 @@ rsc_status rsc_partitioner_build_index(rsc_partitioner *p, const float *X, int64
     // every database row goes to the part its network output ranks first
     if ((s = network_route(p, st, X, nullptr, n, 1, L, L.labels)) != RSC_OK) return s;
     RSC_CUDA_TRY(cudaMemsetAsync(L.gcnt, 0, sizeof(int32_t) * p->P * 2, st));
-    part::histogram_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, L.labels, L.gcnt);
+    part::histogram_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, p->P, L.labels, L.gcnt);
     part::offsets_kernel<<<1, 1024, 0, st>>>(p->P, L.gcnt, p->doff, 1, nullptr);
-    part::scatter_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, L.labels, p->doff, L.gcursor, p->perm);
+    part::scatter_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, p->P, L.labels, p->doff, L.gcursor, p->perm);
     part::permute_rows_kernel<<<(unsigned)ceil_div(n * 8, 256), 256, 0, st>>>(
         static_cast<const uint4 *>(L.Db), p->perm, n, static_cast<uint4 *>(p->Db_sorted));
     RSC_CUDA_TRY(cudaGetLastError());

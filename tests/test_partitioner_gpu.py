@@ -126,3 +126,45 @@ def test_probes_bounded_by_the_first_part_lose_nothing(rsc, n, d, k, probes):
     ai, ad = (t.cpu().numpy() for t in part.knn(Xd, k=k, n_probe=8))
     np.testing.assert_array_equal(ai[queries], full_i)
     np.testing.assert_array_equal(ad[queries], full_d)
+
+
+def _bf16(a):
+    u = np.ascontiguousarray(a, dtype=np.float32).view(np.uint32).astype(np.uint64)
+    u = (u + 0x7FFF + ((u >> 16) & 1)) & 0xFFFF0000
+    return u.astype(np.uint32).view(np.float32).astype(np.float64)
+
+
+def _logits(part, X, d, P, H):
+    """The network on BF16-rounded operands, sums in FP64."""
+    w = part.get_params()
+    sizes = [H * d, H, H * H, H, P * H, P]
+    W1, b1, W2, b2, W3, b3 = np.split(w, np.cumsum(sizes)[:-1])
+    h = np.maximum(_bf16(X) @ _bf16(W1).reshape(H, d).T + b1, 0)
+    h = np.maximum(_bf16(h) @ _bf16(W2).reshape(H, H).T + b2, 0)
+    return _bf16(h) @ _bf16(W3).reshape(P, H).T + b3
+
+
+@pytest.mark.parametrize("n,d,P,H", [(20_001, 50, 600, 256), (5_000, 33, 9, 130), (3_000, 61, 256, 8),
+                                     (4_000, 20, 1024, 64), (3_000, 50, 257, 300)])
+def test_routing_follows_the_network(rsc, n, d, P, H):
+    # part counts around the 256-wide accumulators, hidden sizes around the K
+    # blocks, H = 300 through the GEMMs.  Each query's list comes from the part
+    # its largest logit names (rows whose two largest logits are closer than
+    # the network's rounding, 2^-7 of their size, may go either way).
+    X = synth.mixture(n, d, n_comp=30, seed=P)
+    Xd = torch.from_numpy(X).cuda()
+    part = rsc.Partitioner(d, P, H, bf16_weights=True, seed=H)
+    part.build_index(Xd)
+    z = _logits(part, X, d, P, H)
+    order = np.sort(z, axis=1)
+    clear = order[:, -1] - order[:, -2] > 2.0 ** -7 * np.abs(z).max(axis=1)
+    label = z.argmax(axis=1)
+    k = 10
+    gi = part.knn(Xd, k=k, n_probe=1)[0].cpu().numpy()
+    found = gi >= 0
+    near = np.where(found, gi, 0)
+    same = (label[near] == label[:, None]) | ~clear[near] | ~clear[:, None] | ~found
+    assert clear.mean() > 0.5
+    assert same.all()
+    size = np.bincount(label[clear], minlength=P)
+    assert (found.sum(axis=1)[clear] >= np.minimum(size[label[clear]], k)).all()
