@@ -76,6 +76,8 @@ def launches_per_step(metric, precision, n):
     two queued-row sorts).
     """
     knn = (3 if metric == "euclidean" else 1) + 2
+    if precision == "fp32" and n >= ORDER_MIN_ROWS:   # ordering, gather, tile table, records, split, merge, ties
+        knn += 39 + 5
     if precision == "bf16":
         knn += 1 + (39 + 12 if n >= ORDER_MIN_ROWS else 0)
     return knn + 8

@@ -99,7 +99,13 @@ typedef struct {
                             far from the query tile's to improve any of its
                             lists (exact: the candidates equal the full scan's).
                             0 = automatic (on with the ordering, one database
-                            split, d + 3 <= 64), 1 = off, 2 = on               */
+                            split, d + 3 <= 64), 1 = off, 2 = on.
+                            RSC_FP32 with both left automatic, n >= 16384,
+                            k <= 32 and db_splits 0 or 1 orders its rows and
+                            skips tiles in the same exact way (the k nearest
+                            are those of the full scan, ties by index); off in
+                            either field keeps its full scan, on is ignored
+                            (locality) or refused (prune)                      */
     int32_t stages;      /* tensor-core path: shared-memory stages of the
                             database-tile pipeline, 2 .. 6 (clamped to what the
                             list shape's shared memory holds); 0 = automatic

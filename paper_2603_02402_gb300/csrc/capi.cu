@@ -69,6 +69,7 @@ struct KnnPlan {
     int64_t split_len = 0;
     bool order = false; // locality ordering before the tensor-core search
     bool prune = false; // window pass + tile bounds + list pass instead of one full scan
+    bool simt_prune = false;   // FP32: ordered rows, tiles pruned inside the search kernel
     int stages = 0;     // tensor-core pipeline stages (0: as many as fit)
 };
 
@@ -162,6 +163,18 @@ rsc_status plan_knn(int64_t n, int32_t d, int32_t k, int32_t metric, const rsc_k
         if (!knn_simt_supported(p->DP, p->KC))
             return fail(RSC_ERR_UNSUPPORTED, "no SIMT kernel for DP=%d KC=%d", p->DP, p->KC);
     }
+    // FP32 with one database split (asked for or automatic): rows in locality
+    // order, the tiles that spheres cannot rule out (the same neighbours).
+    // Below kSimtPruneMinRows rows the ordering costs what the full scan does.
+    p->simt_prune = !tc && o->locality != 1 && o->prune == 0 && o->db_splits <= 1 && n >= kSimtPruneMinRows &&
+                    simt_pruned_list(k) > 0;
+    if (p->simt_prune) {
+        p->order = true;
+        p->KC = simt_pruned_list(k);
+        p->splits = 1;
+        p->split_len = n;
+        return RSC_OK;
+    }
     // database splits: enough CTAs to fill the GPU when there are few queries
     const int64_t qrows = tc ? 128 : 256;             // query rows per CTA work unit
     const int64_t target = 152;                       // work units wanted (persistent CTAs)
@@ -222,12 +235,14 @@ KnnLayout carve_knn(void *ws, int64_t n, const KnnPlan &p, size_t *bytes) {
     L.Rp = nullptr;
     if (p.order) {
         L.perm = cv.take<int32_t>((size_t)n);
-        L.order_scratch = cv.take<uint8_t>(order_scratch_bytes(n, p.DP));
+        L.order_scratch = cv.take<uint8_t>(
+            order_scratch_bytes(n, p.DP, 0, p.simt_prune ? simt_pruned_target() : OrderTarget{}));
         L.Rp = cv.take<float>((size_t)n * (p.metric == RSC_EUCLIDEAN ? ceil_div(p.d, 4) * 4 : p.DP));
     }
     L.st_key = nullptr;
     L.st_id = nullptr;
     L.prune_scratch = nullptr;
+    if (p.simt_prune) L.prune_scratch = cv.take<uint8_t>(simt_pruned_scratch_bytes(n, p.DP));
     if (p.prune) {
         L.st_key = cv.take<float>((size_t)n * p.parts * p.KC);
         L.st_id = cv.take<int32_t>((size_t)n * p.parts * p.KC);
@@ -536,6 +551,13 @@ rsc_status rsc_knn(const float *X, int64_t n, int32_t d, int32_t k, int32_t metr
         if (ev) RSC_CUDA_TRY(cudaEventRecord(ev[1], st));
         RSC_CUDA_TRY(launch_knn_tc_fp8(L.Qb, L.Db, n, d, metric, TcShape{p.parts, p.KC, p.stages}, p.splits, p.split_len,
                                        p.order ? kOrderWindow : 0, L.cand, L.status, st));
+    } else if (p.simt_prune) {
+        const OrderTarget target = simt_pruned_target();
+        RSC_CUDA_TRY(launch_locality_order(L.Y, n, p.DP, kOrderIters, L.perm, L.order_scratch, st, nullptr, 0, target));
+        if (ev) RSC_CUDA_TRY(cudaEventRecord(ev[1], st));
+        RSC_CUDA_TRY(launch_knn_simt_pruned(L.Y, L.ny, n, p.DP, d + (metric == RSC_COSINE ? 1 : 0), k, metric, L.perm,
+                                            order_leaves(L.order_scratch, n, p.DP, target), L.prune_scratch, L.cand,
+                                            L.status, st));
     } else {
         if (ev) RSC_CUDA_TRY(cudaEventRecord(ev[1], st));
         RSC_CUDA_TRY(launch_knn_simt(L.Y, L.ny, n, p.DP, d + (metric == RSC_COSINE ? 1 : 0), p.KC, p.splits,
@@ -553,6 +575,9 @@ rsc_status rsc_knn(const float *X, int64_t n, int32_t d, int32_t k, int32_t metr
     }
     RSC_CUDA_TRY(launch_rerank(R, rsr, n, d, metric, L.cand, p.KC, p.splits * p.parts, k, L.perm, p.order, idx, dist,
                                st));
+    if (p.simt_prune)
+        RSC_CUDA_TRY(launch_simt_ties(n, d, p.DP, d + (metric == RSC_COSINE ? 1 : 0), k, metric, L.prune_scratch, R,
+                                      rsr, idx, dist, st));
     if (ev) RSC_CUDA_TRY(cudaEventRecord(ev[3], st));
     return RSC_OK;
 }
@@ -571,10 +596,19 @@ rsc_status rsc_knn_scan_stats(int64_t n, int32_t d, int32_t k, int32_t metric, c
     const int64_t qt = ceil_div(n, BM), dt = ceil_div(n, BN);
     *pairs_total = qt * dt;
     *pairs_scanned = *pairs_total;
+    cudaStream_t st = opts ? static_cast<cudaStream_t>(opts->stream) : nullptr;
+    if (p.simt_prune) {   // counted by 64-row tiles
+        const KnnLayout L = carve_knn(workspace, n, p, nullptr);
+        unsigned long long tiles = 0;
+        RSC_CUDA_TRY(cudaMemcpyAsync(&tiles, simt_pruned_scanned(L.prune_scratch, n, p.DP), sizeof(tiles),
+                                     cudaMemcpyDeviceToHost, st));
+        RSC_CUDA_TRY(cudaStreamSynchronize(st));
+        *pairs_scanned = std::min<int64_t>(*pairs_total, (int64_t)((tiles + 1) / 2));
+        return RSC_OK;
+    }
     if (!p.prune) return RSC_OK;
     KnnLayout L = carve_knn(workspace, n, p, nullptr);
     const PruneOut po = prune_outputs(L.prune_scratch, n, BM, BN);
-    cudaStream_t st = opts ? static_cast<cudaStream_t>(opts->stream) : nullptr;
     int64_t kept = 0;
     int32_t overflow = 0;
     RSC_CUDA_TRY(cudaMemcpyAsync(&kept, po.tile_off + qt, sizeof(kept), cudaMemcpyDeviceToHost, st));

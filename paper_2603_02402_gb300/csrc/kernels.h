@@ -24,6 +24,26 @@ bool knn_simt_supported(int DP, int KC);
 cudaError_t launch_knn_simt(const float *Y, const float *ny, int64_t n, int DP, int width, int KC,
                             int splits, int64_t split_len, int32_t *cand, cudaStream_t st);
 
+// ---- knn_simt_prune.cu ------------------------------------------------------
+// The FP32 search on rows in locality order (perm) with exact tile pruning,
+// k <= 32: cand[q * L + c], L = simt_pruned_list(k) (0: k not supported), the
+// positions of the rows that can be among the k nearest of position q (-1
+// pads).  After the exact re-rank launch_simt_ties finishes the rows with more
+// such rows than L (R: the re-rank's rows by position).
+constexpr int64_t kSimtPruneMinRows = 16384;
+struct OrderTarget;
+struct OrderLeaves;
+OrderTarget simt_pruned_target();   // the ordering this search wants
+int simt_pruned_list(int k);
+size_t simt_pruned_scratch_bytes(int64_t n, int DP);
+// (tile of 64 rows, 128 query rows) pairs scanned by the last search, on the device
+const unsigned long long *simt_pruned_scanned(void *scratch, int64_t n, int DP);
+cudaError_t launch_knn_simt_pruned(const float *Y, const float *ny, int64_t n, int DP, int width, int k, int metric,
+                                   const int32_t *perm, const OrderLeaves &leaves, void *scratch, int32_t *cand,
+                                   unsigned int *status, cudaStream_t st);
+cudaError_t launch_simt_ties(int64_t n, int d, int DP, int width, int k, int metric, void *scratch, const float *R,
+                             int64_t rs, int32_t *idx, float *dist, cudaStream_t st);
+
 // ---- knn_tc.cu ------------------------------------------------------------
 // BF16 tensor-core candidate search.  Qb/Db: [n, 64 * tc_kb(d, metric)] bf16
 // operand rows built by launch_prep_bf16 from the FP32 prep rows Y.  Each
@@ -96,13 +116,37 @@ struct OrderShape {
     int64_t m1, step1, m2, step2;
     int nchunk;
 };
-OrderShape order_shape(int64_t n);
-size_t order_scratch_bytes(int64_t n, int DP, int groups = 0);
+// leaf_rows: rows aimed at per sub-cluster.  spread: as many coarse clusters as
+// there can be (sub-clusters make up the rest, at least three each: coarse
+// clusters often hold more than one true cluster), centroids that start far apart
+// (spread_centroids_kernel), and rows that may go to a leaf of their second
+// nearest coarse cluster: leaves that hold one true cluster each, for searches
+// whose tiles follow the leaves.
+struct OrderTarget {
+    int leaf_rows = kOrderLeafRows;
+    bool spread = false;
+};
+OrderShape order_shape(int64_t n, OrderTarget target = {});
+size_t order_scratch_bytes(int64_t n, int DP, int groups = 0, OrderTarget target = {});
 // perm[sorted position] = original row, for the FP32 prep rows Y [n, DP].
 // goff (device, [G + 1], nullable): row groups (samples) whose position
 // ranges must be kept; each group's rows come out in cluster order.
 cudaError_t launch_locality_order(const float *Y, int64_t n, int DP, int iters, int32_t *perm, void *scratch,
-                                  cudaStream_t st, const int64_t *goff = nullptr, int G = 0);
+                                  cudaStream_t st, const int64_t *goff = nullptr, int G = 0,
+                                  OrderTarget target = {});
+// The sub-clusters ("leaves") of the last ordering on this scratch, in order:
+// leaf l holds the sorted positions [off[l * stride], off[(l + 1) * stride]).
+// Its centroid is row c of cent with l = rank1[c / per] * per + rank2[c], and
+// var[c] the mean squared distance of its sampled rows from it (var: spread
+// targets only).
+struct OrderLeaves {
+    const int32_t *off;
+    int64_t stride;
+    int count, per;
+    const float *cent, *var;
+    const int32_t *rank1, *rank2;
+};
+OrderLeaves order_leaves(void *scratch, int64_t n, int DP, OrderTarget target = {});
 
 // ---- knn_tc_prune.cu / prune.cu ---------------------------------------------------
 // Pruned search on rows in locality order (one database split, KB = 1):

@@ -45,11 +45,12 @@ constexpr int kSub = 1024;           // keys per warp slice
 constexpr int kChunk = kSortWarps * kSub;   // keys per block (one count column per chunk)
 
 // Nearest centroid (squared distance |c|^2 - 2 x.c, ties to the lower index)
-// of rows i * step, i < m.  Thread per row; DP = padded row length.
-template <int DP>
+// of rows i * step, i < m.  Thread per row; DP = padded row length.  kTwo: the
+// second nearest as well (lab2; the nearest again when there is only one).
+template <int DP, bool kTwo>
 __global__ void __launch_bounds__(kAssignThreads)
 assign_kernel(const float *__restrict__ Y, int64_t m, int64_t step, const float *__restrict__ cent,
-              const float *__restrict__ cnorm, int C, int32_t *__restrict__ lab) {
+              const float *__restrict__ cnorm, int C, int32_t *__restrict__ lab, int32_t *__restrict__ lab2) {
     __shared__ __align__(16) float cs[kCentTile][DP];
     __shared__ float cn[kCentTile];
     // two keys per thread (keys i and i + half of the block's span), so every
@@ -73,8 +74,8 @@ assign_kernel(const float *__restrict__ Y, int64_t m, int64_t step, const float 
         z[4 * t4 + 2] = w.z;
         z[4 * t4 + 3] = w.w;
     }
-    float best0 = INFINITY, best1 = INFINITY;
-    int bi0 = 0, bi1 = 0;
+    float best0 = INFINITY, best1 = INFINITY, next0 = INFINITY, next1 = INFINITY;
+    int bi0 = 0, bi1 = 0, ni0 = -1, ni1 = -1;
     for (int c0 = 0; c0 < C; c0 += kCentTile) {
         const int nc = min(kCentTile, C - c0);
         __syncthreads();
@@ -107,18 +108,37 @@ assign_kernel(const float *__restrict__ Y, int64_t m, int64_t step, const float 
             }
             const float s0 = fmaf(-2.f, p0 + p1, cn[c]), s1 = fmaf(-2.f, q0 + q1, cn[c]);
             if (s0 < best0) {   // strict: the lower index wins ties
+                if (kTwo && best0 < INFINITY) {
+                    next0 = best0;
+                    ni0 = bi0;
+                }
                 best0 = s0;
                 bi0 = c0 + c;
+            } else if (kTwo && s0 < next0) {
+                next0 = s0;
+                ni0 = c0 + c;
             }
             if (s1 < best1) {
+                if (kTwo && best1 < INFINITY) {
+                    next1 = best1;
+                    ni1 = bi1;
+                }
                 best1 = s1;
                 bi1 = c0 + c;
+            } else if (kTwo && s1 < next1) {
+                next1 = s1;
+                ni1 = c0 + c;
             }
         }
     }
     if (a0) lab[i0] = bi0;
     if (a1) lab[i1] = bi1;
+    if (kTwo) {
+        if (a0) lab2[i0] = ni0 >= 0 ? ni0 : bi0;
+        if (a1) lab2[i1] = ni1 >= 0 ? ni1 : bi1;
+    }
 }
+
 // Centroid c <- row (c * n) / C; its squared norm alongside.
 __global__ void init_centroids_kernel(const float *__restrict__ Y, int64_t n, int DP, int C, float *__restrict__ cent,
                                       float *__restrict__ cnorm) {
@@ -194,16 +214,21 @@ chunk_scatter_kernel(const int32_t *__restrict__ lab, int64_t m, int64_t step, c
 
 // Centroid c <- mean of its rows (sorted positions [off[c * nchunk],
 // off[(c + 1) * nchunk])), summed in row order; an empty cluster keeps its
-// centroid.  Warp per centroid.
+// centroid.  Warp per centroid.  kVar: cvar, the rows' mean squared distance
+// from it.
+template <bool kVar>
 __global__ void centroid_mean_kernel(const float *__restrict__ Y, int DP, const int32_t *__restrict__ sorted_rows,
                                      const int32_t *__restrict__ off, int nchunk, int C, float *__restrict__ cent,
-                                     float *__restrict__ cnorm) {
+                                     float *__restrict__ cnorm, float *__restrict__ cvar) {
     const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (c >= C) return;
     const int32_t b = off[(int64_t)c * nchunk], e = off[(int64_t)(c + 1) * nchunk];
-    if (e == b) return;
-    float s0 = 0.f, s1 = 0.f;
+    if (e == b) {
+        if (kVar && lane == 0) cvar[c] = 0.f;
+        return;
+    }
+    float s0 = 0.f, s1 = 0.f, sq = 0.f;
     // rows fetched kMeanAhead at a time (independent loads), added in order
     constexpr int kMeanAhead = 8;
     for (int32_t p0 = b; p0 < e; p0 += kMeanAhead) {
@@ -222,6 +247,7 @@ __global__ void centroid_mean_kernel(const float *__restrict__ Y, int DP, const 
             if (p0 + u < e) {
                 s0 += v0[u];
                 s1 += v1[u];
+                if (kVar) sq = fmaf(v0[u], v0[u], fmaf(v1[u], v1[u], sq));
             }
         }
     }
@@ -231,20 +257,28 @@ __global__ void centroid_mean_kernel(const float *__restrict__ Y, int DP, const 
     if (lane < DP) cent[(int64_t)c * DP + lane] = s0;
     if (lane + 32 < DP) cent[(int64_t)c * DP + lane + 32] = s1;
     float q = (lane < DP ? s0 * s0 : 0.f) + (lane + 32 < DP ? s1 * s1 : 0.f);
-    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-    if (lane == 0) cnorm[c] = q;
+    for (int o = 16; o > 0; o >>= 1) {
+        q += __shfl_xor_sync(0xffffffffu, q, o);
+        if (kVar) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    }
+    if (lane == 0) {
+        cnorm[c] = q;
+        if (kVar) cvar[c] = sq * inv - q;
+    }
 }
 
 // Sub-cluster assignment: key i is row rows[i * step] (rows given) or
 // i * step; its coarse cluster c1 = lab1[row]; label = c1 * C2 + the nearest
 // of c1's C2 sub-centroids (|c|^2 - 2 x.c, ties to the lower index), written
-// at out[row] (by_row) or out[i].  Thread per key; the C2 sub-centroids of a
-// coarse cluster are read through L1 (neighbouring keys share them).
+// at out[row] (by_row) or out[i].  lab1b (nullable): a second coarse cluster of
+// every row, whose sub-centroids count too.  Thread per key; the C2
+// sub-centroids of a coarse cluster are read through L1 (neighbouring keys
+// share them).
 template <int DP>
 __global__ void __launch_bounds__(kAssignThreads)
 assign_sub_kernel(const float *__restrict__ Y, int64_t m, int64_t step, const int32_t *__restrict__ rows,
-                  const int32_t *__restrict__ lab1, const float *__restrict__ cent2, const float *__restrict__ cnorm2,
-                  int C2, bool by_row, const int32_t *__restrict__ rank1, const int32_t *__restrict__ rank2,
+                  const int32_t *__restrict__ lab1, const int32_t *__restrict__ lab1b,
+                  const float *__restrict__ cent2, const float *__restrict__ cnorm2, int C2, bool by_row, const int32_t *__restrict__ rank1, const int32_t *__restrict__ rank2,
                   int32_t *__restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
@@ -259,11 +293,13 @@ assign_sub_kernel(const float *__restrict__ Y, int64_t m, int64_t step, const in
         x[4 * t4 + 2] = v.z;
         x[4 * t4 + 3] = v.w;
     }
-    const int base = lab1[row] * C2;
+    const int base = lab1[row] * C2, base2 = lab1b ? lab1b[row] * C2 - C2 : 0;
     float best = INFINITY;
-    int bi = 0;
-    for (int c = 0; c < C2; ++c) {
-        const float4 *cr = reinterpret_cast<const float4 *>(cent2 + (int64_t)(base + c) * DP);
+    int bi = base;
+    const int count = lab1b ? 2 * C2 : C2;
+    for (int z = 0; z < count; ++z) {
+        const int c = z < C2 ? base + z : base2 + z;
+        const float4 *cr = reinterpret_cast<const float4 *>(cent2 + (int64_t)c * DP);
         float a0 = 0.f, a1 = 0.f;
 #pragma unroll
         for (int t4 = 0; t4 < DP / 4; t4 += 2) {
@@ -277,7 +313,7 @@ assign_sub_kernel(const float *__restrict__ Y, int64_t m, int64_t step, const in
             a1 = fmaf(x[4 * t4 + 6], w.z, a1);
             a1 = fmaf(x[4 * t4 + 7], w.w, a1);
         }
-        const float sv = fmaf(-2.f, a0 + a1, cnorm2[base + c]);
+        const float sv = fmaf(-2.f, a0 + a1, cnorm2[c]);
         if (sv < best) {
             best = sv;
             bi = c;
@@ -285,7 +321,7 @@ assign_sub_kernel(const float *__restrict__ Y, int64_t m, int64_t step, const in
     }
     // ranked key (position of the coarse cluster, then of the sub-cluster,
     // along their chains) for the final order; the plain label otherwise
-    out[by_row ? row : i] = rank1 ? rank1[base / C2] * C2 + rank2[base + bi] : base + bi;
+    out[by_row ? row : i] = rank1 ? rank1[bi / C2] * C2 + rank2[bi] : bi;
 }
 
 // Sub-centroid s of coarse cluster c <- the row at position b + (s * size) /
@@ -306,6 +342,84 @@ __global__ void init_sub_centroids_kernel(const float *__restrict__ Y, int DP, c
     }
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
     if (threadIdx.x == 0) cnorm2[g] = q;
+}
+
+// C starting centroids that lie far apart, out of kSpread rows evenly spaced in
+// a segment: the first, then C - 1 times the row farthest from those taken
+// (ties to the lower index).  Evenly spaced starts miss clusters (128 starts,
+// 100 clusters: 28 of them); their rows then share leaves with other clusters,
+// and every tile of such a leaf spans both.  Block per group of C centroids (cent [groups * C,
+// DP]): group g draws from positions [off[g * nchunk], off[(g + 1) * nchunk])
+// of `perm` (its coarse centroid `cent1` when that is empty), or, perm null,
+// from all n rows.  Thread per sampled row.
+constexpr int kSpread = 512;
+__global__ void __launch_bounds__(kSpread)
+spread_centroids_kernel(const float *__restrict__ Y, int64_t n, int DP, const int32_t *__restrict__ perm,
+                        const int32_t *__restrict__ off, int nchunk, int C, const float *__restrict__ cent1,
+                        float *__restrict__ cent, float *__restrict__ cnorm) {
+    extern __shared__ float rows[];   // [kSpread][DP + 1]
+    __shared__ float wv[kSpread / 32];
+    __shared__ int wi[kSpread / 32];
+    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = DP + 1;
+    const int64_t b = perm ? off[(int64_t)c * nchunk] : 0, size = (perm ? off[(int64_t)(c + 1) * nchunk] : n) - b;
+    const int m = (int)max((int64_t)1, min((int64_t)kSpread, size));
+    for (int x = tid; x < m * (DP / 4); x += kSpread) {
+        const int r = x / (DP / 4), q = x % (DP / 4);
+        const int64_t at = b + ((int64_t)r * size) / m;
+        const float *src = size > 0 ? Y + (perm ? (int64_t)perm[at] : at) * DP : cent1 + (int64_t)c * DP;
+        const float4 v = reinterpret_cast<const float4 *>(src)[q];
+        float *o = rows + r * W + 4 * q;
+        o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+    }
+    __syncthreads();
+    float far = INFINITY;   // squared distance to the nearest row taken so far
+    int pick = 0;
+    for (int s = 0; s < C; ++s) {
+        const int64_t g = (int64_t)c * C + s;
+        if (warp == 0) {
+            float q = 0.f;
+            for (int t = lane; t < DP; t += 32) {
+                const float v = rows[pick * W + t];
+                cent[g * DP + t] = v;
+                q = fmaf(v, v, q);
+            }
+            for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+            if (lane == 0) cnorm[g] = q;
+        }
+        float bv = -1.f;
+        int bi = tid;
+        if (tid < m) {
+            float d = 0.f;
+            for (int t = 0; t < DP; ++t) {
+                const float df = rows[tid * W + t] - rows[pick * W + t];
+                d = fmaf(df, df, d);
+            }
+            far = fminf(far, d);
+            bv = far < INFINITY ? far : -1.f;   // rows that are not numbers are not taken
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (ov > bv || (ov == bv && oi < bi)) {
+                bv = ov;
+                bi = oi;
+            }
+        }
+        if (lane == 0) {
+            wv[warp] = bv;
+            wi[warp] = bi;
+        }
+        __syncthreads();
+        bv = wv[0];
+        bi = wi[0];
+        for (int w = 1; w < kSpread / 32; ++w)
+            if (wv[w] > bv) {
+                bv = wv[w];
+                bi = wi[w];
+            }
+        pick = bi < m ? bi : 0;
+        __syncthreads();
+    }
 }
 
 // Greedy nearest-neighbour chain through each group of gsize consecutive
@@ -353,8 +467,10 @@ __global__ void __launch_bounds__(kChainThreads) chain_kernel(const float *__res
         const float *dl = D + last * gsize;
         for (int c = lane; c < gsize; c += 32) {
             if (seen[c]) continue;
-            const float s = dl[c];
-            if (s < best) {
+            // a distance that is not finite (rows with NaN or overflow) counts
+            // as infinite, so every step finds one of the unseen centroids
+            const float s = dl[c] < INFINITY ? dl[c] : INFINITY;
+            if (s < best || bi == INT_MAX) {
                 best = s;
                 bi = c;
             }
@@ -377,12 +493,12 @@ __global__ void __launch_bounds__(kChainThreads) chain_kernel(const float *__res
 }
 
 cudaError_t launch_assign_sub(const float *Y, int DP, int64_t m, int64_t step, const int32_t *rows,
-                              const int32_t *lab1, const float *cent2, const float *cnorm2, int C2, bool by_row,
-                              const int32_t *rank1, const int32_t *rank2, int32_t *out, cudaStream_t st) {
+                              const int32_t *lab1, const int32_t *lab1b, const float *cent2, const float *cnorm2,
+                              int C2, bool by_row, const int32_t *rank1, const int32_t *rank2, int32_t *out, cudaStream_t st) {
     const unsigned blocks = (unsigned)ceil_div(m, kAssignThreads);
 #define RSC_ASSIGN(dp)                                                                                       \
     case dp:                                                                                                 \
-        assign_sub_kernel<dp><<<blocks, kAssignThreads, 0, st>>>(Y, m, step, rows, lab1, cent2, cnorm2, C2, \
+        assign_sub_kernel<dp><<<blocks, kAssignThreads, 0, st>>>(Y, m, step, rows, lab1, lab1b, cent2, cnorm2, C2, \
                                                                  by_row, rank1, rank2, out);                 \
         break
     switch (DP) {
@@ -401,10 +517,15 @@ cudaError_t launch_assign_sub(const float *Y, int DP, int64_t m, int64_t step, c
 }
 
 cudaError_t launch_assign(const float *Y, int DP, int64_t m, int64_t step, const float *cent, const float *cnorm,
-                          int C, int32_t *lab, cudaStream_t st) {
+                          int C, int32_t *lab, int32_t *lab2, cudaStream_t st) {
     const unsigned blocks = (unsigned)ceil_div(m, 2 * kAssignThreads);   // two keys per thread
-#define RSC_ASSIGN(dp) \
-    case dp: assign_kernel<dp><<<blocks, kAssignThreads, 0, st>>>(Y, m, step, cent, cnorm, C, lab); break
+#define RSC_ASSIGN(dp)                                                                                            \
+    case dp:                                                                                                      \
+        if (lab2)                                                                                                 \
+            assign_kernel<dp, true><<<blocks, kAssignThreads, 0, st>>>(Y, m, step, cent, cnorm, C, lab, lab2);    \
+        else                                                                                                      \
+            assign_kernel<dp, false><<<blocks, kAssignThreads, 0, st>>>(Y, m, step, cent, cnorm, C, lab, nullptr); \
+        break
     switch (DP) {
         RSC_ASSIGN(8);
         RSC_ASSIGN(16);
@@ -437,10 +558,15 @@ cudaError_t counting_sort(const int32_t *lab, int64_t m, int64_t step, const int
 
 }  // namespace
 
-OrderShape order_shape(int64_t n) {
+OrderShape order_shape(int64_t n, OrderTarget target) {
     OrderShape s;
-    s.C2 = kOrderSub;
-    s.C1 = (int)std::min<int64_t>(kOrderMaxCoarse, std::max<int64_t>(1, ceil_div(n, (int64_t)kOrderSub * kOrderLeafRows)));
+    if (target.spread) {
+        s.C1 = (int)std::min<int64_t>(kOrderMaxCoarse, ceil_div(n, (int64_t)128));
+        s.C2 = (int)std::min<int64_t>(kOrderSub, 2 + ceil_div(n, (int64_t)s.C1 * target.leaf_rows));
+    } else {
+        s.C2 = kOrderSub;
+        s.C1 = (int)std::min<int64_t>(kOrderMaxCoarse, std::max<int64_t>(1, ceil_div(n, (int64_t)kOrderSub * target.leaf_rows)));
+    }
     s.m1 = std::min<int64_t>(n, (int64_t)s.C1 * 64);
     s.step1 = n / s.m1;
     s.m1 = n / s.step1;                    // keys i * step1, i < m1, all inside [0, n)
@@ -454,12 +580,13 @@ OrderShape order_shape(int64_t n) {
 namespace {
 
 struct OrderLayout {
-    float *cent1, *cnorm1, *cent2, *cnorm2;
-    int32_t *lab1, *lab, *perm1, *cnt, *off, *srows, *rank1, *rank2;
+    float *cent1, *cnorm1, *cent2, *cnorm2, *cvar2;
+    // cvar2: mean squared radius of the leaves; lab1b: second nearest coarse cluster (spread targets only)
+    int32_t *lab1, *lab1b, *lab, *perm1, *cnt, *off, *srows, *rank1, *rank2;
     int64_t *ssum;
 };
 
-OrderLayout order_layout(void *scratch, int64_t n, int DP, const OrderShape &s, int groups, size_t *bytes) {
+OrderLayout order_layout(void *scratch, int64_t n, int DP, const OrderShape &s, int groups, bool two, size_t *bytes) {
     Carve cv(scratch);
     OrderLayout L;
     const int C = std::max(s.C1 * s.C2, groups);   // widest counting sort
@@ -467,7 +594,9 @@ OrderLayout order_layout(void *scratch, int64_t n, int DP, const OrderShape &s, 
     L.cnorm1 = cv.take<float>((size_t)s.C1);
     L.cent2 = cv.take<float>((size_t)s.C1 * s.C2 * DP);
     L.cnorm2 = cv.take<float>((size_t)s.C1 * s.C2);
+    L.cvar2 = two ? cv.take<float>((size_t)s.C1 * s.C2) : nullptr;
     L.lab1 = cv.take<int32_t>((size_t)n);
+    L.lab1b = two ? cv.take<int32_t>((size_t)n) : nullptr;
     L.lab = cv.take<int32_t>((size_t)n);
     L.perm1 = cv.take<int32_t>((size_t)n);
     const size_t ncnt = (size_t)C * s.nchunk;
@@ -483,10 +612,16 @@ OrderLayout order_layout(void *scratch, int64_t n, int DP, const OrderShape &s, 
 
 }  // namespace
 
-size_t order_scratch_bytes(int64_t n, int DP, int groups) {
+size_t order_scratch_bytes(int64_t n, int DP, int groups, OrderTarget target) {
     size_t bytes = 0;
-    order_layout(nullptr, n, DP, order_shape(n), groups, &bytes);
+    order_layout(nullptr, n, DP, order_shape(n, target), groups, target.spread, &bytes);
     return bytes;
+}
+
+OrderLeaves order_leaves(void *scratch, int64_t n, int DP, OrderTarget target) {
+    const OrderShape s = order_shape(n, target);
+    const OrderLayout L = order_layout(scratch, n, DP, s, 0, target.spread, nullptr);
+    return {L.off, s.nchunk, s.C1 * s.C2, s.C2, L.cent2, L.cvar2, L.rank1, L.rank2};
 }
 
 namespace {
@@ -509,40 +644,54 @@ __global__ void group_key_kernel(const int32_t *__restrict__ rows, int64_t n, co
 }  // namespace
 
 cudaError_t launch_locality_order(const float *Y, int64_t n, int DP, int iters, int32_t *perm, void *scratch,
-                                  cudaStream_t st, const int64_t *goff, int G) {
-    const OrderShape s = order_shape(n);
+                                  cudaStream_t st, const int64_t *goff, int G, OrderTarget target) {
+    const OrderShape s = order_shape(n, target);
     if (DP % 8 != 0 || DP > 64) return cudaErrorInvalidValue;
     if (goff && (G < 1 || G > kOrderMaxLeaves)) return cudaErrorInvalidValue;
-    const OrderLayout L = order_layout(scratch, n, DP, s, goff ? G : 0, nullptr);
+    const OrderLayout L = order_layout(scratch, n, DP, s, goff ? G : 0, target.spread, nullptr);
     const int C = s.C1 * s.C2;
     const int mean_warps = 4;
     cudaError_t e;
+    const int spread_smem = (int)sizeof(float) * kSpread * (DP + 1);
+    if (target.spread && (e = cudaFuncSetAttribute(spread_centroids_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   spread_smem)) != cudaSuccess)
+        return e;
     // level 1: coarse k-means (Lloyd on a strided sample), then every row
-    init_centroids_kernel<<<s.C1, 32, 0, st>>>(Y, n, DP, s.C1, L.cent1, L.cnorm1);
+    if (target.spread)
+        spread_centroids_kernel<<<1, kSpread, spread_smem, st>>>(Y, n, DP, nullptr, nullptr, 0, s.C1, nullptr, L.cent1,
+                                                                 L.cnorm1);
+    else
+        init_centroids_kernel<<<s.C1, 32, 0, st>>>(Y, n, DP, s.C1, L.cent1, L.cnorm1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int nch1 = (int)ceil_div(s.m1, kChunk);
     for (int it = 0; it < iters; ++it) {
-        if ((e = launch_assign(Y, DP, s.m1, s.step1, L.cent1, L.cnorm1, s.C1, L.lab1, st)) != cudaSuccess) return e;
+        if ((e = launch_assign(Y, DP, s.m1, s.step1, L.cent1, L.cnorm1, s.C1, L.lab1, nullptr, st)) != cudaSuccess) return e;
         if ((e = counting_sort(L.lab1, s.m1, s.step1, nullptr, s.C1, L.cnt, L.off, L.ssum, L.srows, st)) != cudaSuccess)
             return e;
-        centroid_mean_kernel<<<(unsigned)ceil_div(s.C1, mean_warps), mean_warps * 32, 0, st>>>(
-            Y, DP, L.srows, L.off, nch1, s.C1, L.cent1, L.cnorm1);
+        centroid_mean_kernel<false><<<(unsigned)ceil_div(s.C1, mean_warps), mean_warps * 32, 0, st>>>(
+            Y, DP, L.srows, L.off, nch1, s.C1, L.cent1, L.cnorm1, nullptr);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if ((e = launch_assign(Y, DP, n, 1, L.cent1, L.cnorm1, s.C1, L.lab1, st)) != cudaSuccess) return e;
+    if ((e = launch_assign(Y, DP, n, 1, L.cent1, L.cnorm1, s.C1, L.lab1, L.lab1b, st)) != cudaSuccess)
+        return e;
     if ((e = counting_sort(L.lab1, n, 1, nullptr, s.C1, L.cnt, L.off, L.ssum, L.perm1, st)) != cudaSuccess) return e;
     // level 2: C2 sub-clusters inside each coarse cluster (sample in coarse order)
-    init_sub_centroids_kernel<<<C, 32, 0, st>>>(Y, DP, L.perm1, L.off, s.nchunk, s.C2, L.cent1, L.cent2, L.cnorm2);
+    if (target.spread) {
+        spread_centroids_kernel<<<s.C1, kSpread, spread_smem, st>>>(Y, n, DP, L.perm1, L.off, s.nchunk, s.C2, L.cent1,
+                                                                    L.cent2, L.cnorm2);
+    } else {
+        init_sub_centroids_kernel<<<C, 32, 0, st>>>(Y, DP, L.perm1, L.off, s.nchunk, s.C2, L.cent1, L.cent2, L.cnorm2);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int nch2 = (int)ceil_div(s.m2, kChunk);
     for (int it = 0; it < iters; ++it) {
-        if ((e = launch_assign_sub(Y, DP, s.m2, s.step2, L.perm1, L.lab1, L.cent2, L.cnorm2, s.C2, false, nullptr,
+        if ((e = launch_assign_sub(Y, DP, s.m2, s.step2, L.perm1, L.lab1, L.lab1b, L.cent2, L.cnorm2, s.C2, false, nullptr,
                                    nullptr, L.lab, st)) != cudaSuccess)
             return e;
         if ((e = counting_sort(L.lab, s.m2, s.step2, L.perm1, C, L.cnt, L.off, L.ssum, L.srows, st)) != cudaSuccess) return e;
-        centroid_mean_kernel<<<(unsigned)ceil_div(C, mean_warps), mean_warps * 32, 0, st>>>(Y, DP, L.srows, L.off,
-                                                                                            nch2, C, L.cent2,
-                                                                                            L.cnorm2);
+        auto mean = L.cvar2 ? centroid_mean_kernel<true> : centroid_mean_kernel<false>;
+        mean<<<(unsigned)ceil_div(C, mean_warps), mean_warps * 32, 0, st>>>(Y, DP, L.srows, L.off, nch2, C, L.cent2,
+                                                                            L.cnorm2, L.cvar2);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     // chains through the coarse centroids and through each cluster's sub-centroids
@@ -554,8 +703,8 @@ cudaError_t launch_locality_order(const float *Y, int64_t n, int DP, int iters, 
     chain_kernel<<<s.C1, kChainThreads, sm2, st>>>(L.cent2, DP, s.C2, L.rank2);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // every row (walked in coarse order, so a block shares its sub-centroids), keyed by its ranks; the final sort
-    if ((e = launch_assign_sub(Y, DP, n, 1, L.perm1, L.lab1, L.cent2, L.cnorm2, s.C2, true, L.rank1, L.rank2, L.lab,
-                               st)) != cudaSuccess)
+    if ((e = launch_assign_sub(Y, DP, n, 1, L.perm1, L.lab1, L.lab1b, L.cent2, L.cnorm2, s.C2, true, L.rank1, L.rank2,
+                               L.lab, st)) != cudaSuccess)
         return e;
     if (!goff) return counting_sort(L.lab, n, 1, nullptr, C, L.cnt, L.off, L.ssum, perm, st);
     // groups (samples) keep their row ranges: the cluster order, then a stable

@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "rerank.cuh"
 #include "warp_sort.cuh"
 
 namespace rsc {
@@ -21,11 +22,9 @@ namespace {
 constexpr int kWarps = 16;   // queries per block: neighbouring queries share candidate rows in L1
 
 // Warp per query, 8 lanes per candidate row.  In step g, lanes 8 r + s
-// (r < 4, s < 8) score candidate 4 g + r of the current 32: lane s takes
-// components 4 s .. 4 s + 3 and 32 + 4 s .. 32 + 4 s + 3 (two 16-byte loads
-// when rows start on 16-byte boundaries, else scalar loads; the same sums
-// either way), an FMA chain over its eight, and three xor shuffles add the
-// eight partial sums; candidate c's sum then goes to lane c % 32.  One load
+// (r < 4, s < 8) score candidate 4 g + r of the current 32 (rerank.cuh: eight
+// components per lane, an FMA chain over them, three xor shuffles);
+// candidate c's sum then goes to lane c % 32.  One load
 // instruction of the warp touches 4 candidate rows instead of 32 (a lane per
 // row): the gathers are bound by the L1's line lookups, not by bytes.
 // E = (candidate slots rounded up to a power of two) / 32 (key, id) pairs per
@@ -47,32 +46,8 @@ rerank_kernel(const float *__restrict__ R, int64_t rs, int64_t n, int d, int met
     const int64_t qr = r_by_pos ? q : qo;                      // its row in R
     const bool cosine = metric == RSC_COSINE;
 
-    // this lane's components of a row.  Loads stop at the last 4-aligned piece
-    // holding a component below d; the rest of that piece is zero padding
-    // except the cosine rows' flag at column d, which is cleared.
-    auto load8 = [&](const float *row, float (&v)[8]) {
-        if (vec) {
-            const float4 *r4 = reinterpret_cast<const float4 *>(row);
-            const float4 a = (4 * s < d) ? __ldg(r4 + s) : make_float4(0.f, 0.f, 0.f, 0.f);
-            const float4 b = (32 + 4 * s < d) ? __ldg(r4 + 8 + s) : make_float4(0.f, 0.f, 0.f, 0.f);
-            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-            v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-        } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                v[i] = (4 * s + i < d) ? __ldg(row + 4 * s + i) : 0.f;
-                v[4 + i] = (32 + 4 * s + i < d) ? __ldg(row + 32 + 4 * s + i) : 0.f;
-            }
-        }
-        if (cosine) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if ((i < 4 ? 4 * s + i : 28 + 4 * s + i) == d) v[i] = 0.f;
-        }
-    };
-
     float xv[8];
-    load8(R + qr * rs, xv);
+    rr::load8(R + qr * rs, s, d, cosine, vec, xv);
     const bool fq = cosine && R[qr * rs + d] != 0.f;
 
     float key[E];
@@ -97,16 +72,8 @@ rerank_kernel(const float *__restrict__ R, int64_t rs, int64_t n, int d, int met
             // an empty slot scores row 0 and is dropped below (no branch)
             const int yr = max(__shfl_sync(0xffffffffu, row, 4 * g + r), 0);
             float yv[8];
-            load8(R + (int64_t)yr * rs, yv);
-            float part = 0.f;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float diff = xv[i] - yv[i];
-                part = fmaf(diff, diff, part);
-            }
-            part += __shfl_xor_sync(0xffffffffu, part, 1);
-            part += __shfl_xor_sync(0xffffffffu, part, 2);
-            part += __shfl_xor_sync(0xffffffffu, part, 4);
+            rr::load8(R + (int64_t)yr * rs, s, d, cosine, vec, yv);
+            const float part = rr::dist2(xv, yv);
             const float got = __shfl_sync(0xffffffffu, part, 8 * (lane & 3));
             if ((lane >> 2) == g && row >= 0) key[e] = got;
         }

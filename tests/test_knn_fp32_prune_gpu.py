@@ -1,0 +1,87 @@
+"""The pruned FP32 search (rows in locality order, from 16,384 rows on)
+against the full scan and the FP64 oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2603_02402_gb300 import synth
+from test_knn_gpu import rsc, run_knn  # noqa: F401
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _both(rsc, X, k, metric="euclidean"):
+    p = run_knn(rsc, X, k, metric=metric, precision="fp32")
+    f = run_knn(rsc, X, k, metric=metric, precision="fp32", prune="off")
+    return p, f
+
+
+@pytest.mark.parametrize("n,d,k,comp,metric", [
+    (16_384, 50, 15, 30, "euclidean"), (16_385, 50, 15, 30, "cosine"), (16_447, 3, 16, 5, "euclidean"),
+    (20_001, 8, 1, 12, "euclidean"), (33_333, 50, 17, 60, "euclidean"), (20_000, 64, 32, 20, "euclidean"),
+    (18_000, 63, 30, 20, "cosine"), (40_011, 17, 5, 9, "euclidean"), (30_000, 1, 15, 4, "euclidean"),
+    (70_000, 50, 15, 40, "euclidean"),
+])
+def test_pruned_equals_full_scan(rsc, n, d, k, comp, metric):  # noqa: F811
+    # tiles of 64 and 128 rows with ragged ends, both list lengths (k <= 16,
+    # k <= 32), component counts around the four-component step; more than one
+    # chunk of 512 tiles at 40,011 and 70,000 rows
+    X = synth.mixture(n, d, n_comp=comp, seed=n + k)
+    (pi, pd), (fi, fd) = _both(rsc, X, k, metric)
+    np.testing.assert_array_equal(pd, fd)
+    np.testing.assert_array_equal(pi, fi)
+
+
+def test_unclustered_and_far_from_the_origin(rsc):  # noqa: F811
+    # rows that no sphere separates, then a cluster pair with a large offset
+    rng = np.random.Generator(np.random.PCG64(5))
+    U = rng.uniform(-1, 1, (20_000, 12)).astype(np.float32)
+    M = synth.mixture(20_000, 50, n_comp=2, seed=6) + np.float32(1e3)
+    for X in (U, M):
+        (pi, pd), (fi, fd) = _both(rsc, X, 15)
+        np.testing.assert_array_equal(pi, fi)
+        np.testing.assert_array_equal(pd, fd)
+
+
+@pytest.mark.parametrize("case", ["grid", "duplicates", "one point"])
+def test_more_ties_than_a_list_holds(rsc, case):  # noqa: F811
+    # equal distances beyond the list's length: the lowest ids win, as in the
+    # oracle.  Integer coordinates: the squared distances are exact in FP32
+    # and in FP64, so ids must agree exactly.
+    rng = np.random.Generator(np.random.PCG64(7))
+    if case == "grid":      # 24 and 32 neighbours at equal distance
+        X = np.stack(np.meshgrid(*[np.arange(12)] * 4), -1).reshape(-1, 4).astype(np.float32)
+    elif case == "duplicates":
+        X = np.repeat(rng.integers(0, 9, (410, 6)), 50, axis=0).astype(np.float32)
+    else:
+        X = np.full((17_000, 5), 3, dtype=np.float32)
+    X = X[rng.permutation(len(X))]
+    gi, gd = run_knn(rsc, X, 15, precision="fp32")
+    q = synth.query_sample(len(X), 300, seed=3)
+    oi, od, _ = oracle.knn(X, 15, queries=q)
+    np.testing.assert_array_equal(gi[q], oi)
+    np.testing.assert_allclose(gd[q], od, rtol=1e-6)
+
+
+def test_cosine_rows_that_are_zero_or_not_numbers(rsc):  # noqa: F811
+    X = synth.mixture(18_000, 20, n_comp=10, seed=8)
+    X[[5, 9_000, 17_999]] = 0.0
+    X[100, 3] = np.nan
+    X[200, 4] = np.inf
+    (pi, pd), (fi, fd) = _both(rsc, X, 15, "cosine")
+    np.testing.assert_array_equal(pi, fi)
+    np.testing.assert_array_equal(pd, fd)
+    assert pi[5].tolist()[:3] == [5, 9_000, 17_999]
+
+
+def test_scan_stats_of_the_pruned_search(rsc):  # noqa: F811
+    n = 30_000
+    X = torch.from_numpy(synth.mixture(n, 50, n_comp=40, seed=1)).cuda()
+    for prune in ("auto", "off"):
+        ws = torch.empty(rsc.rsc_knn_workspace_size(n, 50, 15, prune=prune), dtype=torch.uint8, device="cuda")
+        rsc.rsc_knn(X, 15, workspace=ws, prune=prune)
+        scanned, total = rsc.rsc_knn_scan_stats(n, 50, 15, ws, precision="fp32", prune=prune)
+        tiles = -(-n // 128)
+        assert total == tiles * tiles
+        assert scanned == total if prune == "off" else 0 < scanned < 0.3 * total

@@ -350,3 +350,18 @@ def test_bounded_wait_times_out_and_the_next_call_recovers(rsc):
     check_knn(X, gi.cpu().numpy(), gd.cpu().numpy(), oi, od, on, allow_miss=MISS["bf16"])
     with pytest.raises(rsc.RscError):
         rsc.rsc_set_wait_budget(-1)
+
+
+@pytest.mark.parametrize("metric", ["euclidean", "cosine"])
+def test_ordered_search_of_rows_that_are_not_numbers(rsc, metric):
+    # a NaN row makes the Euclidean column means NaN and with them every row
+    # (no neighbours: ids -1); a cosine row stays alone and is nobody's
+    # neighbour.  The ordering's centroid chains have no finite distance then.
+    X = synth.mixture(17_000, 20, n_comp=10, seed=3)
+    X[0] = np.nan
+    gi, gd = run_knn(rsc, X, 15, metric=metric, precision="bf16")
+    assert (gi[0] == -1).all() and np.isinf(gd[0]).all()
+    if metric == "euclidean":
+        assert (gi == -1).all()
+    else:
+        assert (gi[1:] > 0).all()
