@@ -155,7 +155,7 @@ OrderLeaves order_leaves(void *scratch, int64_t n, int DP, OrderTarget target = 
 // improve one of its lists, and the list pass resumes the lists over them.
 constexpr int64_t kPruneListCap = int64_t(1) << 28;   // kept (query tile, tile) pairs stored at most
 struct PruneShape {
-    int qtiles, dtiles, nchunk;
+    int qtiles, dtiles, nchunk, chunk_tiles;
     int64_t cap;
 };
 struct PruneOut {

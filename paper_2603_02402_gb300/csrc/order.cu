@@ -41,8 +41,16 @@ namespace {
 constexpr int kCentTile = 64;        // centroids staged in shared memory per pass
 constexpr int kAssignThreads = 128;
 constexpr int kSortWarps = 8;        // warps per block in the counting sort
-constexpr int kSub = 1024;           // keys per warp slice
-constexpr int kChunk = kSortWarps * kSub;   // keys per block (one count column per chunk)
+constexpr int kMaxSub = 1024;        // keys per warp slice at most
+
+// Keys per warp slice of a sort of m keys (a block, one chunk, sorts kSortWarps
+// slices one after the other in 32-key steps): enough chunks for every SM
+// before the slices get longer.  68,579 keys: 5 us a scatter with slices of
+// 128, 16 us with slices of 1,024 on nine blocks.
+int sub_len(int64_t m) {
+    return (int)std::min<int64_t>(kMaxSub, std::max<int64_t>(128, ceil_div(m, (int64_t)kSortWarps * 152 * 32) * 32));
+}
+int64_t chunk_len(int64_t m) { return (int64_t)kSortWarps * sub_len(m); }
 
 // Nearest centroid (squared distance |c|^2 - 2 x.c, ties to the lower index)
 // of rows i * step, i < m.  Thread per row; DP = padded row length.  kTwo: the
@@ -154,21 +162,21 @@ __global__ void init_centroids_kernel(const float *__restrict__ Y, int64_t n, in
     if (threadIdx.x == 0) cnorm[c] = s;
 }
 
-// Per-chunk label counts: block b counts keys [b * kChunk, (b + 1) * kChunk)
+// Per-chunk label counts: block b counts keys [b * chunk, (b + 1) * chunk)
 // into cnt[label * nchunk + b] (kSortWarps warps, shared-memory atomics).
 __global__ void __launch_bounds__(kSortWarps * 32)
-chunk_hist_kernel(const int32_t *__restrict__ lab, int64_t m, int C, int nchunk, int32_t *__restrict__ cnt) {
+chunk_hist_kernel(const int32_t *__restrict__ lab, int64_t m, int C, int sub, int nchunk, int32_t *__restrict__ cnt) {
     extern __shared__ int32_t hs[];   // [C]
     const int ch = blockIdx.x;
     for (int c = threadIdx.x; c < C; c += blockDim.x) hs[c] = 0;
     __syncthreads();
-    const int64_t b = (int64_t)ch * kChunk, e = min(m, b + kChunk);
+    const int64_t chunk = (int64_t)kSortWarps * sub, b = ch * chunk, e = min(m, b + chunk);
     for (int64_t r = b + threadIdx.x; r < e; r += blockDim.x) atomicAdd(&hs[lab[r]], 1);
     __syncthreads();
     for (int c = threadIdx.x; c < C; c += blockDim.x) cnt[(int64_t)c * nchunk + ch] = hs[c];
 }
 
-// Stable scatter, block per chunk: warp w walks its kSub-key slice of the
+// Stable scatter, block per chunk: warp w walks its sub-key slice of the
 // chunk in key order, 32 keys a step; keys with equal labels within a step
 // are ranked by lane (match_any) and a per-(warp, label) cursor carries the
 // count across steps.  The cursors start at the chunk's offset plus the
@@ -176,14 +184,14 @@ chunk_hist_kernel(const int32_t *__restrict__ lab, int64_t m, int C, int nchunk,
 // rows[r * step] (rows given) or r * step.
 __global__ void __launch_bounds__(kSortWarps * 32)
 chunk_scatter_kernel(const int32_t *__restrict__ lab, int64_t m, int64_t step, const int32_t *__restrict__ rows,
-                     int C, int nchunk, const int32_t *__restrict__ off, int32_t *__restrict__ out) {
+                     int C, int sub, int nchunk, const int32_t *__restrict__ off, int32_t *__restrict__ out) {
     extern __shared__ int32_t cur_s[];   // [kSortWarps][C]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ch = blockIdx.x;
     int32_t *cur = cur_s + warp * C;
     for (int c = lane; c < C; c += 32) cur[c] = 0;
     __syncwarp();
-    const int64_t b = (int64_t)ch * kChunk + (int64_t)warp * kSub, e = min(m, b + kSub);
+    const int64_t b = ((int64_t)ch * kSortWarps + warp) * sub, e = min(m, b + sub);
     for (int64_t r = b + lane; r < e; r += 32) atomicAdd(&cur[lab[r]], 1);
     __syncthreads();
     // exclusive prefix over the warps, per label, plus the chunk offset
@@ -229,25 +237,32 @@ __global__ void centroid_mean_kernel(const float *__restrict__ Y, int DP, const 
         return;
     }
     float s0 = 0.f, s1 = 0.f, sq = 0.f;
-    // rows fetched kMeanAhead at a time (independent loads), added in order
-    constexpr int kMeanAhead = 8;
-    for (int32_t p0 = b; p0 < e; p0 += kMeanAhead) {
-        float v0[kMeanAhead], v1[kMeanAhead];
+    // the additions keep the row order; a lane fetches the row ids 32 at a time
+    // and the rows come kMeanAhead at a time, so a cluster costs a load latency
+    // per 16 rows (two per 8 when each row's id was read just before it: 54 us
+    // a launch at 68,579 rows, 144 clusters)
+    constexpr int kMeanAhead = 16;
+    const int l0 = min(lane, DP - 1), l1 = min(lane + 32, DP - 1);
+    for (int32_t q0 = b; q0 < e; q0 += 32) {
+        const int32_t mine = q0 + lane < e ? sorted_rows[q0 + lane] : 0;
+        const int m = min(32, e - q0);
+        for (int p0 = 0; p0 < m; p0 += kMeanAhead) {
+            float v0[kMeanAhead], v1[kMeanAhead];
 #pragma unroll
-        for (int u = 0; u < kMeanAhead; ++u) {
-            v0[u] = v1[u] = 0.f;
-            if (p0 + u < e) {
-                const float *y = Y + (int64_t)sorted_rows[p0 + u] * DP;
-                if (lane < DP) v0[u] = y[lane];
-                if (lane + 32 < DP) v1[u] = y[lane + 32];
+            for (int u = 0; u < kMeanAhead; ++u) {
+                // rows past m are row 0 and are not added; components past DP
+                // repeat the last and are not stored
+                const float *y = Y + (int64_t)__shfl_sync(0xffffffffu, mine, p0 + u) * DP;
+                v0[u] = y[l0];
+                v1[u] = y[l1];
             }
-        }
 #pragma unroll
-        for (int u = 0; u < kMeanAhead; ++u) {
-            if (p0 + u < e) {
-                s0 += v0[u];
-                s1 += v1[u];
-                if (kVar) sq = fmaf(v0[u], v0[u], fmaf(v1[u], v1[u], sq));
+            for (int u = 0; u < kMeanAhead; ++u) {
+                if (p0 + u < m) {
+                    s0 += v0[u];
+                    s1 += v1[u];
+                    if (kVar) sq += (lane < DP ? v0[u] * v0[u] : 0.f) + (lane + 32 < DP ? v1[u] * v1[u] : 0.f);
+                }
             }
         }
     }
@@ -270,11 +285,11 @@ __global__ void centroid_mean_kernel(const float *__restrict__ Y, int DP, const 
 // Sub-cluster assignment: key i is row rows[i * step] (rows given) or
 // i * step; its coarse cluster c1 = lab1[row]; label = c1 * C2 + the nearest
 // of c1's C2 sub-centroids (|c|^2 - 2 x.c, ties to the lower index), written
-// at out[row] (by_row) or out[i].  lab1b (nullable): a second coarse cluster of
-// every row, whose sub-centroids count too.  Thread per key; the C2
+// at out[row] (by_row) or out[i].  kTwo: lab1b, a second coarse cluster of every row,
+// whose sub-centroids count too.  Thread per key; the C2
 // sub-centroids of a coarse cluster are read through L1 (neighbouring keys
 // share them).
-template <int DP>
+template <int DP, bool kTwo>
 __global__ void __launch_bounds__(kAssignThreads)
 assign_sub_kernel(const float *__restrict__ Y, int64_t m, int64_t step, const int32_t *__restrict__ rows,
                   const int32_t *__restrict__ lab1, const int32_t *__restrict__ lab1b,
@@ -293,12 +308,12 @@ assign_sub_kernel(const float *__restrict__ Y, int64_t m, int64_t step, const in
         x[4 * t4 + 2] = v.z;
         x[4 * t4 + 3] = v.w;
     }
-    const int base = lab1[row] * C2, base2 = lab1b ? lab1b[row] * C2 - C2 : 0;
+    const int base = lab1[row] * C2, base2 = kTwo ? lab1b[row] * C2 - C2 : 0;
     float best = INFINITY;
     int bi = base;
-    const int count = lab1b ? 2 * C2 : C2;
+    const int count = kTwo ? 2 * C2 : C2;
     for (int z = 0; z < count; ++z) {
-        const int c = z < C2 ? base + z : base2 + z;
+        const int c = kTwo && z >= C2 ? base2 + z : base + z;
         const float4 *cr = reinterpret_cast<const float4 *>(cent2 + (int64_t)c * DP);
         float a0 = 0.f, a1 = 0.f;
 #pragma unroll
@@ -321,7 +336,7 @@ assign_sub_kernel(const float *__restrict__ Y, int64_t m, int64_t step, const in
     }
     // ranked key (position of the coarse cluster, then of the sub-cluster,
     // along their chains) for the final order; the plain label otherwise
-    out[by_row ? row : i] = rank1 ? rank1[bi / C2] * C2 + rank2[bi] : bi;
+    out[by_row ? row : i] = rank1 ? rank1[(kTwo ? bi : base) / C2] * C2 + rank2[bi] : bi;
 }
 
 // Sub-centroid s of coarse cluster c <- the row at position b + (s * size) /
@@ -357,10 +372,10 @@ __global__ void __launch_bounds__(kSpread)
 spread_centroids_kernel(const float *__restrict__ Y, int64_t n, int DP, const int32_t *__restrict__ perm,
                         const int32_t *__restrict__ off, int nchunk, int C, const float *__restrict__ cent1,
                         float *__restrict__ cent, float *__restrict__ cnorm) {
-    extern __shared__ float rows[];   // [kSpread][DP + 1]
-    __shared__ float wv[kSpread / 32];
-    __shared__ int wi[kSpread / 32];
-    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = DP + 1;
+    extern __shared__ __align__(16) float rows[];   // [kSpread][DP]
+    __shared__ unsigned wv[2][kSpread / 32];
+    __shared__ int wi[2][kSpread / 32];
+    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t b = perm ? off[(int64_t)c * nchunk] : 0, size = (perm ? off[(int64_t)(c + 1) * nchunk] : n) - b;
     const int m = (int)max((int64_t)1, min((int64_t)kSpread, size));
     for (int x = tid; x < m * (DP / 4); x += kSpread) {
@@ -368,10 +383,15 @@ spread_centroids_kernel(const float *__restrict__ Y, int64_t n, int DP, const in
         const int64_t at = b + ((int64_t)r * size) / m;
         const float *src = size > 0 ? Y + (perm ? (int64_t)perm[at] : at) * DP : cent1 + (int64_t)c * DP;
         const float4 v = reinterpret_cast<const float4 *>(src)[q];
-        float *o = rows + r * W + 4 * q;
-        o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+        reinterpret_cast<float4 *>(rows)[r * (DP / 4) + q] = v;
     }
     __syncthreads();
+    // the thread's own row in registers, the taken one from shared memory (one
+    // 16-byte read for the whole warp)
+    float4 own[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+        own[q] = 4 * q < DP && tid < m ? reinterpret_cast<const float4 *>(rows)[tid * (DP / 4) + q] : make_float4(0.f, 0.f, 0.f, 0.f);
     float far = INFINITY;   // squared distance to the nearest row taken so far
     int pick = 0;
     for (int s = 0; s < C; ++s) {
@@ -379,46 +399,44 @@ spread_centroids_kernel(const float *__restrict__ Y, int64_t n, int DP, const in
         if (warp == 0) {
             float q = 0.f;
             for (int t = lane; t < DP; t += 32) {
-                const float v = rows[pick * W + t];
+                const float v = rows[pick * DP + t];
                 cent[g * DP + t] = v;
                 q = fmaf(v, v, q);
             }
             for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
             if (lane == 0) cnorm[g] = q;
         }
-        float bv = -1.f;
-        int bi = tid;
+        // bits of the distance + 1 (non-negative floats order as their bits);
+        // 0: no row, or one that is no number, which is not taken
+        unsigned key = 0;
         if (tid < m) {
-            float d = 0.f;
-            for (int t = 0; t < DP; ++t) {
-                const float df = rows[tid * W + t] - rows[pick * W + t];
-                d = fmaf(df, df, d);
+            const float4 *taken = reinterpret_cast<const float4 *>(rows + pick * DP);
+            float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                if (4 * q >= DP) break;   // uniform
+                const float4 v = taken[q];
+                const float e0 = own[q].x - v.x, e1 = own[q].y - v.y, e2 = own[q].z - v.z, e3 = own[q].w - v.w;
+                d0 = fmaf(e0, e0, d0);
+                d1 = fmaf(e1, e1, d1);
+                d0 = fmaf(e2, e2, d0);
+                d1 = fmaf(e3, e3, d1);
             }
-            far = fminf(far, d);
-            bv = far < INFINITY ? far : -1.f;   // rows that are not numbers are not taken
+            far = fminf(far, d0 + d1);
+            key = far < INFINITY ? __float_as_uint(far) + 1u : 0u;
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (ov > bv || (ov == bv && oi < bi)) {
-                bv = ov;
-                bi = oi;
-            }
-        }
+        const unsigned best = __reduce_max_sync(0xffffffffu, key);
+        const int who = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
         if (lane == 0) {
-            wv[warp] = bv;
-            wi[warp] = bi;
+            wv[s & 1][warp] = best;
+            wi[s & 1][warp] = warp * 32 + who;
         }
-        __syncthreads();
-        bv = wv[0];
-        bi = wi[0];
-        for (int w = 1; w < kSpread / 32; ++w)
-            if (wv[w] > bv) {
-                bv = wv[w];
-                bi = wi[w];
-            }
-        pick = bi < m ? bi : 0;
-        __syncthreads();
+        __syncthreads();   // the other half of wv / wi is written in the next round
+        const unsigned v = lane < kSpread / 32 ? wv[s & 1][lane] : 0u;
+        const unsigned top = __reduce_max_sync(0xffffffffu, v);
+        const int w = __ffs(__ballot_sync(0xffffffffu, lane < kSpread / 32 && v == top)) - 1;
+        pick = wi[s & 1][w];
+        if (pick >= m) pick = 0;
     }
 }
 
@@ -430,7 +448,7 @@ spread_centroids_kernel(const float *__restrict__ Y, int64_t n, int DP, const in
 // gsize <= kChainMax: the block first fills the group's squared-distance
 // matrix (every entry summed over t in order), then one warp walks it.
 constexpr int kChainMax = 128;
-constexpr int kChainThreads = 256;
+constexpr int kChainThreads = 1024;
 static_assert(kOrderMaxCoarse <= kChainMax && kOrderSub <= kChainMax, "chain groups fit the seen flags");
 __global__ void __launch_bounds__(kChainThreads) chain_kernel(const float *__restrict__ cent, int DP, int gsize,
                                                               int32_t *__restrict__ rank) {
@@ -443,15 +461,39 @@ __global__ void __launch_bounds__(kChainThreads) chain_kernel(const float *__res
     for (int e = tid; e < gsize * DP; e += kChainThreads) cs[(e / DP) * W + e % DP] = C[e];
     for (int c = tid; c < gsize; c += kChainThreads) seen[c] = false;
     __syncthreads();
-    for (int e = tid; e < gsize * gsize; e += kChainThreads) {
-        const int a = e / gsize, c = e - a * gsize;   // D[a][c] = |cent_c - cent_a|^2
-        const float *ca = cs + a * W, *cc = cs + c * W;
-        float s = 0.f;
-        for (int t = 0; t < DP; ++t) {
-            const float df = cc[t] - ca[t];
-            s = fmaf(df, df, s);
+    // D[a][c] = |cent_c - cent_a|^2, 4 x 4 entries per thread (half a shared
+    // load per entry and component instead of two)
+    const int side = (gsize + 3) / 4;
+    for (int e = tid; e < side * side; e += kChainThreads) {
+        const int a0 = e / side * 4, c0 = e % side * 4;
+        const float *ca[4], *cc[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            ca[i] = cs + min(a0 + i, gsize - 1) * W;
+            cc[i] = cs + min(c0 + i, gsize - 1) * W;
         }
-        D[e] = s;
+        float s[4][4] = {};
+#pragma unroll 2
+        for (int t = 0; t < DP; ++t) {
+            float x[4], y[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                x[i] = ca[i][t];
+                y[i] = cc[i][t];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float df = y[j] - x[i];
+                    s[i][j] = fmaf(df, df, s[i][j]);
+                }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (a0 + i < gsize && c0 + j < gsize) D[(a0 + i) * gsize + c0 + j] = s[i][j];
     }
     __syncthreads();
     if (tid >= 32) return;
@@ -462,27 +504,23 @@ __global__ void __launch_bounds__(kChainThreads) chain_kernel(const float *__res
     }
     __syncwarp();
     for (int pos = 1; pos < gsize; ++pos) {
-        float best = INFINITY;
+        // smallest distance of an unseen centroid, then the lowest index among
+        // equals; a distance that is not finite (rows with NaN or overflow)
+        // counts as infinite, so every step finds one.  Distances are not
+        // negative: their bits order as they do.
+        unsigned best = 0xffffffffu;
         int bi = INT_MAX;
         const float *dl = D + last * gsize;
         for (int c = lane; c < gsize; c += 32) {
             if (seen[c]) continue;
-            // a distance that is not finite (rows with NaN or overflow) counts
-            // as infinite, so every step finds one of the unseen centroids
-            const float s = dl[c] < INFINITY ? dl[c] : INFINITY;
-            if (s < best || bi == INT_MAX) {
+            const unsigned s = __float_as_uint(dl[c] < INFINITY ? dl[c] : INFINITY);
+            if (s < best) {
                 best = s;
                 bi = c;
             }
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (ob < best || (ob == best && oi < bi)) {
-                best = ob;
-                bi = oi;
-            }
-        }
+        const unsigned least = __reduce_min_sync(0xffffffffu, best);
+        bi = __reduce_min_sync(0xffffffffu, best == least ? bi : INT_MAX);
         last = bi;
         if (lane == 0) {
             seen[bi] = true;
@@ -496,11 +534,13 @@ cudaError_t launch_assign_sub(const float *Y, int DP, int64_t m, int64_t step, c
                               const int32_t *lab1, const int32_t *lab1b, const float *cent2, const float *cnorm2,
                               int C2, bool by_row, const int32_t *rank1, const int32_t *rank2, int32_t *out, cudaStream_t st) {
     const unsigned blocks = (unsigned)ceil_div(m, kAssignThreads);
-#define RSC_ASSIGN(dp)                                                                                       \
-    case dp:                                                                                                 \
-        assign_sub_kernel<dp><<<blocks, kAssignThreads, 0, st>>>(Y, m, step, rows, lab1, lab1b, cent2, cnorm2, C2, \
-                                                                 by_row, rank1, rank2, out);                 \
-        break
+#define RSC_ASSIGN(dp)                                                                                            \
+    case dp: {                                                                                                    \
+        auto kern = lab1b ? assign_sub_kernel<dp, true> : assign_sub_kernel<dp, false>;                           \
+        kern<<<blocks, kAssignThreads, 0, st>>>(Y, m, step, rows, lab1, lab1b, cent2, cnorm2, C2, by_row, rank1,  \
+                                                rank2, out);                                                      \
+        break;                                                                                                    \
+    }
     switch (DP) {
         RSC_ASSIGN(8);
         RSC_ASSIGN(16);
@@ -545,14 +585,14 @@ cudaError_t launch_assign(const float *Y, int DP, int64_t m, int64_t step, const
 // of each key: rows[r * step] when rows is given, else r * step).
 cudaError_t counting_sort(const int32_t *lab, int64_t m, int64_t step, const int32_t *rows, int C, int32_t *cnt,
                           int32_t *off, int64_t *ssum, int32_t *out, cudaStream_t st) {
-    const int nchunk = (int)ceil_div(m, kChunk);
+    const int sub = sub_len(m), nchunk = (int)ceil_div(m, chunk_len(m));
     const size_t sm = sizeof(int32_t) * kSortWarps * C;
     cudaError_t e = cudaFuncSetAttribute(chunk_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(sizeof(int32_t) * kSortWarps * kOrderMaxLeaves));
     if (e != cudaSuccess) return e;
-    chunk_hist_kernel<<<nchunk, kSortWarps * 32, sizeof(int32_t) * C, st>>>(lab, m, C, nchunk, cnt);
+    chunk_hist_kernel<<<nchunk, kSortWarps * 32, sizeof(int32_t) * C, st>>>(lab, m, C, sub, nchunk, cnt);
     if ((e = seg_scan::launch(cnt, (int64_t)C * nchunk, off, ssum, st)) != cudaSuccess) return e;
-    chunk_scatter_kernel<<<nchunk, kSortWarps * 32, sm, st>>>(lab, m, step, rows, C, nchunk, off, out);
+    chunk_scatter_kernel<<<nchunk, kSortWarps * 32, sm, st>>>(lab, m, step, rows, C, sub, nchunk, off, out);
     return cudaGetLastError();
 }
 
@@ -573,7 +613,7 @@ OrderShape order_shape(int64_t n, OrderTarget target) {
     s.m2 = std::min<int64_t>(n, (int64_t)s.C1 * s.C2 * 32);
     s.step2 = n / s.m2;
     s.m2 = n / s.step2;
-    s.nchunk = (int)ceil_div(n, kChunk);   // the full sorts have the most chunks
+    s.nchunk = (int)ceil_div(n, chunk_len(n));
     return s;
 }
 
@@ -599,7 +639,9 @@ OrderLayout order_layout(void *scratch, int64_t n, int DP, const OrderShape &s, 
     L.lab1b = two ? cv.take<int32_t>((size_t)n) : nullptr;
     L.lab = cv.take<int32_t>((size_t)n);
     L.perm1 = cv.take<int32_t>((size_t)n);
-    const size_t ncnt = (size_t)C * s.nchunk;
+    // the samples' sorts may have more chunks than the full one
+    const int64_t most = std::max<int64_t>(s.nchunk, std::max(ceil_div(s.m1, chunk_len(s.m1)), ceil_div(s.m2, chunk_len(s.m2))));
+    const size_t ncnt = (size_t)C * most;
     L.cnt = cv.take<int32_t>(ncnt);
     L.off = cv.take<int32_t>(ncnt + 1);
     L.ssum = cv.take<int64_t>(seg_scan::kMaxSegs);
@@ -652,7 +694,7 @@ cudaError_t launch_locality_order(const float *Y, int64_t n, int DP, int iters, 
     const int C = s.C1 * s.C2;
     const int mean_warps = 4;
     cudaError_t e;
-    const int spread_smem = (int)sizeof(float) * kSpread * (DP + 1);
+    const int spread_smem = (int)sizeof(float) * kSpread * DP;
     if (target.spread && (e = cudaFuncSetAttribute(spread_centroids_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    spread_smem)) != cudaSuccess)
         return e;
@@ -663,7 +705,7 @@ cudaError_t launch_locality_order(const float *Y, int64_t n, int DP, int iters, 
     else
         init_centroids_kernel<<<s.C1, 32, 0, st>>>(Y, n, DP, s.C1, L.cent1, L.cnorm1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int nch1 = (int)ceil_div(s.m1, kChunk);
+    const int nch1 = (int)ceil_div(s.m1, chunk_len(s.m1));
     for (int it = 0; it < iters; ++it) {
         if ((e = launch_assign(Y, DP, s.m1, s.step1, L.cent1, L.cnorm1, s.C1, L.lab1, nullptr, st)) != cudaSuccess) return e;
         if ((e = counting_sort(L.lab1, s.m1, s.step1, nullptr, s.C1, L.cnt, L.off, L.ssum, L.srows, st)) != cudaSuccess)
@@ -683,7 +725,7 @@ cudaError_t launch_locality_order(const float *Y, int64_t n, int DP, int iters, 
         init_sub_centroids_kernel<<<C, 32, 0, st>>>(Y, DP, L.perm1, L.off, s.nchunk, s.C2, L.cent1, L.cent2, L.cnorm2);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int nch2 = (int)ceil_div(s.m2, kChunk);
+    const int nch2 = (int)ceil_div(s.m2, chunk_len(s.m2));
     for (int it = 0; it < iters; ++it) {
         if ((e = launch_assign_sub(Y, DP, s.m2, s.step2, L.perm1, L.lab1, L.lab1b, L.cent2, L.cnorm2, s.C2, false, nullptr,
                                    nullptr, L.lab, st)) != cudaSuccess)

@@ -30,7 +30,7 @@ namespace rsc {
 namespace {
 
 constexpr int kCen = 64;           // centre stride (floats); v has at most 64 components
-constexpr int kChunkTiles = 256;   // database tiles per block in the bound passes
+constexpr int kMaxChunkTiles = 256;   // database tiles per block in the bound passes at most
 constexpr int kBoundThreads = 128; // query tiles per block in the bound passes
 constexpr int kStage = 32;         // database tiles staged in shared memory at once
 constexpr int kGroupTiles = 16;    // database tiles per group sphere (tested before its tiles)
@@ -122,6 +122,123 @@ __global__ void tile_sphere_kernel(const uint16_t *__restrict__ Qb, int64_t n, i
     }
 }
 
+// Spheres of the 256-row database tiles and of the two 128-row query tiles in
+// each, block per database tile, in one read: a thread keeps its eight 16-byte
+// pieces (component block lane & 7 of rows 4 i + (lane >> 3) of its warp's 32)
+// between the mean and the radius pass.  Warps 0-3 hold the first query tile.
+// (1M rows: 133 us as two launches of tile_sphere_kernel, which read the rows
+// four times and hold a warp per tile; 68,579 rows: 66 us.)
+constexpr int kPairBM = 128, kPairBN = 256;
+__global__ void __launch_bounds__(256)
+tile_pair_sphere_kernel(const uint16_t *__restrict__ Qb, int64_t n, int W, int dv, int qtiles,
+                        float *__restrict__ qcen, float *__restrict__ qrad, float *__restrict__ qn,
+                        float *__restrict__ dcen, float *__restrict__ drad, float *__restrict__ dn,
+                        float *__restrict__ row_norm) {
+    __shared__ float sum[8][kCen];   // per warp
+    __shared__ float cen[3][kCen];   // query tiles, database tile
+    __shared__ float red[3][8];
+    const int g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, half = warp >> 2;
+    const int ch = lane & 7, rs = lane >> 3;
+    const int64_t r0 = (int64_t)g * kPairBN + warp * 32 + rs;
+    int nv = dv - 8 * ch;   // valid components of this lane's 8
+    nv = nv < 0 ? 0 : (nv > 8 ? 8 : nv);
+    uint4 piece[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        piece[i] = r0 + 4 * i < n ? *reinterpret_cast<const uint4 *>(Qb + (r0 + 4 * i) * W + 8 * ch) : make_uint4(0u, 0u, 0u, 0u);
+    auto unpack = [&](const uint4 &u, float (&v)[8]) {
+        const uint32_t w4[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            v[2 * i] = 2 * i < nv ? __uint_as_float(w4[i] << 16) : 0.f;
+            v[2 * i + 1] = 2 * i + 1 < nv ? __uint_as_float(w4[i] & 0xffff0000u) : 0.f;
+        }
+    };
+    float c[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) c[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        float v[8];
+        unpack(piece[i], v);
+#pragma unroll
+        for (int x = 0; x < 8; ++x) c[x] += v[x];
+    }
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        c[x] += __shfl_xor_sync(0xffffffffu, c[x], 8);
+        c[x] += __shfl_xor_sync(0xffffffffu, c[x], 16);
+        if (rs == 0) sum[warp][8 * ch + x] = c[x];
+    }
+    __syncthreads();
+    const int rows = (int)min((int64_t)kPairBN, n - (int64_t)g * kPairBN), rows0 = min(rows, kPairBM), rows1 = rows - rows0;
+    if (tid < kCen) {
+        const float a = (sum[0][tid] + sum[1][tid]) + (sum[2][tid] + sum[3][tid]);
+        const float b = (sum[4][tid] + sum[5][tid]) + (sum[6][tid] + sum[7][tid]);
+        cen[0][tid] = a / (float)rows0;
+        cen[1][tid] = rows1 > 0 ? b / (float)rows1 : 0.f;
+        cen[2][tid] = (a + b) / (float)rows;
+    }
+    __syncthreads();
+    float cq[8], cd[8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        cq[x] = cen[half][8 * ch + x];
+        cd[x] = cen[2][8 * ch + x];
+    }
+    float mq = 0.f, md = 0.f, mn = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const bool ok = r0 + 4 * i < n;
+        float v[8];
+        unpack(piece[i], v);
+        float dq = 0.f, dd = 0.f, nn = 0.f;
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            const float eq = v[x] - cq[x], ed = v[x] - cd[x];
+            dq = fmaf(eq, eq, dq);
+            dd = fmaf(ed, ed, dd);
+            nn = fmaf(v[x], v[x], nn);
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            dq += __shfl_xor_sync(0xffffffffu, dq, o);
+            dd += __shfl_xor_sync(0xffffffffu, dd, o);
+            nn += __shfl_xor_sync(0xffffffffu, nn, o);
+        }
+        if (ok) {
+            mq = fmaxf(mq, dq);
+            md = fmaxf(md, dd);
+            mn = fmaxf(mn, nn);
+            if (ch == 0) row_norm[r0 + 4 * i] = nn;
+        }
+    }
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) {
+        mq = fmaxf(mq, __shfl_xor_sync(0xffffffffu, mq, o));
+        md = fmaxf(md, __shfl_xor_sync(0xffffffffu, md, o));
+        mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    }
+    if (lane == 0) {
+        red[0][warp] = mq;
+        red[1][warp] = md;
+        red[2][warp] = mn;
+    }
+    __syncthreads();
+    auto max4 = [&](int k, int w) { return fmaxf(fmaxf(red[k][w], red[k][w + 1]), fmaxf(red[k][w + 2], red[k][w + 3])); };
+    auto radius = [](float d2) { return sqrtf(d2) * (1.f + 0x1p-10f) + 1e-6f; };
+    if (tid < kCen) dcen[(int64_t)g * kCen + tid] = cen[2][tid];
+    if (tid < 2 * kCen && 2 * g + (tid >> 6) < qtiles) qcen[(int64_t)(2 * g) * kCen + tid] = cen[tid >> 6][tid & 63];
+    if (tid == 0) {
+        drad[g] = radius(fmaxf(max4(1, 0), max4(1, 4)));
+        dn[g] = fmaxf(max4(2, 0), max4(2, 4));
+    }
+    if (tid < 2 && 2 * g + tid < qtiles) {
+        qrad[2 * g + tid] = radius(max4(0, 4 * tid));
+        qn[2 * g + tid] = max4(2, 4 * tid);
+    }
+}
+
 // tau_Q = max over the query tile's rows and parts of (saved threshold +
 // |v_i|^2); infinite while some list is not full.  Warp per query tile.
 __global__ void tile_tau_kernel(const float *__restrict__ st_key, int64_t n, int EG, int KCP,
@@ -199,21 +316,20 @@ __device__ __forceinline__ bool sphere_drop(const float (&c)[kCen], const float 
     return gap > 0.f && gap * gap - beta * nt - margin > tq;
 }
 
-// Thread per query tile Q, block column = a chunk of kChunkTiles database
-// tiles: count the kept tiles of (Q, chunk) and record them as bits, one
-// 32-bit word per stage of kStage tiles (bits[(Q * nchunk + chunk) * kWords
-// + stage]).  Each group of kGroupTiles tiles is tested first: a query tile
+// Thread per query tile Q, block column = a chunk of `chunk_tiles` database
+// tiles (a multiple of kStage): count the kept tiles of (Q, chunk) and record
+// them as bits, one 32-bit word per stage of kStage tiles (bits[(Q * nchunk +
+// chunk) * words + stage], words = chunk_tiles / kStage).  Each group of kGroupTiles tiles is tested first: a query tile
 // that drops the group skips its tiles (each of them would be dropped too).
-constexpr int kWords = kChunkTiles / kStage;
 static_assert(kStage == 32, "one bit word per stage");
 
 __global__ void __launch_bounds__(kBoundThreads)
-prune_tiles_kernel(int qtiles, int dtiles, int nchunk, int qpt, int window, float beta,
+prune_tiles_kernel(int qtiles, int dtiles, int nchunk, int chunk_tiles, int qpt, int window, float beta,
                    const float *__restrict__ qcen, const float *__restrict__ qrad, const float *__restrict__ qn,
                    const float *__restrict__ tau, const float *__restrict__ dcen, const float *__restrict__ drad,
                    const float *__restrict__ dn, const float *__restrict__ gcen, const float *__restrict__ grad,
                    const float *__restrict__ gn, int32_t *__restrict__ cnt, uint32_t *__restrict__ bits) {
-    static_assert(kStage % kGroupTiles == 0 && kChunkTiles % kStage == 0, "stages hold whole groups");
+    static_assert(kStage % kGroupTiles == 0 && kMaxChunkTiles % kStage == 0, "stages hold whole groups");
     constexpr int kStageGroups = kStage / kGroupTiles;
     __shared__ __align__(16) float sc[kStage][kCen];
     __shared__ __align__(16) float sgc[kStageGroups][kCen];
@@ -235,8 +351,8 @@ prune_tiles_kernel(int qtiles, int dtiles, int nchunk, int qpt, int window, floa
     // the query tile's window (already scanned by the first pass)
     const int tw = active ? Q / qpt : 0;
     const int wlo = max(0, tw - window), whi = min(dtiles, tw + window + 1);
-    const int t0 = chunk * kChunkTiles, t1 = min(dtiles, t0 + kChunkTiles);
-    uint32_t *wout = bits + ((int64_t)(active ? Q : 0) * nchunk + chunk) * kWords;
+    const int t0 = chunk * chunk_tiles, t1 = min(dtiles, t0 + chunk_tiles);
+    uint32_t *wout = bits + ((int64_t)(active ? Q : 0) * nchunk + chunk) * (chunk_tiles / kStage);
     int kept = 0;
     for (int s0 = t0, w = 0; s0 < t1; s0 += kStage, ++w) {
         const int ns = min(kStage, t1 - s0);
@@ -277,15 +393,15 @@ prune_tiles_kernel(int qtiles, int dtiles, int nchunk, int qpt, int window, floa
 // tiles[off[Q * nchunk + chunk] ..] (entries past cap are dropped: the list
 // pass then falls back to the full scan outside the window).
 __global__ void __launch_bounds__(256)
-fill_tiles_kernel(int qtiles, int dtiles, int nchunk, const uint32_t *__restrict__ bits,
+fill_tiles_kernel(int qtiles, int dtiles, int nchunk, int chunk_tiles, const uint32_t *__restrict__ bits,
                   const int64_t *__restrict__ off, int32_t *__restrict__ tiles, int64_t cap) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // Q * nchunk + chunk
     if (e >= (int64_t)qtiles * nchunk) return;
     const int chunk = (int)(e % nchunk);
-    const uint32_t *win = bits + e * kWords;
+    const uint32_t *win = bits + e * (chunk_tiles / kStage);
     int64_t pos = off[e];
-    const int t0 = chunk * kChunkTiles;
-    const int nw = (int)ceil_div(min(dtiles - t0, kChunkTiles), kStage);
+    const int t0 = chunk * chunk_tiles;
+    const int nw = (int)ceil_div(min(dtiles - t0, chunk_tiles), kStage);
     for (int w = 0; w < nw; ++w) {
         uint32_t word = win[w];
         while (word) {
@@ -493,7 +609,13 @@ PruneShape prune_shape(int64_t n, int BM, int BN) {
     PruneShape s;
     s.qtiles = (int)ceil_div(n, BM);
     s.dtiles = (int)ceil_div(n, BN);
-    s.nchunk = (int)ceil_div(s.dtiles, kChunkTiles);
+    // short chunks while there are few query tiles, so the bound pass has blocks
+    // for every SM (68,579 rows: 160 us on ten blocks of 256 tiles a thread,
+    // against 45 blocks of 32)
+    s.chunk_tiles = kStage;
+    while (s.chunk_tiles < kMaxChunkTiles && ceil_div(s.qtiles, kBoundThreads) * ceil_div(s.dtiles, s.chunk_tiles) > 1024)
+        s.chunk_tiles *= 2;
+    s.nchunk = (int)ceil_div(s.dtiles, s.chunk_tiles);
     const int64_t all = (int64_t)s.qtiles * s.dtiles;
     s.cap = std::min<int64_t>(all, kPruneListCap);
     return s;
@@ -525,7 +647,7 @@ PruneLayout prune_layout(void *scratch, int64_t n, const PruneShape &s, size_t *
     L.tau = cv.take<float>((size_t)s.qtiles);
     const size_t ncnt = (size_t)s.qtiles * s.nchunk;
     L.cnt = cv.take<int32_t>(ncnt);
-    L.bits = cv.take<uint32_t>(ncnt * kWords);
+    L.bits = cv.take<uint32_t>(ncnt * (s.chunk_tiles / kStage));
     L.off = cv.take<int64_t>(ncnt + 1);
     L.ssum = cv.take<int64_t>(seg_scan::kMaxSegs);
     L.out.tile_off = cv.take<int64_t>((size_t)s.qtiles + 1);
@@ -563,10 +685,9 @@ cudaError_t launch_prune_bounds(const void *Qb, int64_t n, int d, int metric, in
     const int dv = metric == RSC_COSINE ? d + 1 : d;
     const float beta = metric == RSC_COSINE ? 1.f : 0.f;
     const uint16_t *q16 = static_cast<const uint16_t *>(Qb);
-    tile_sphere_kernel<<<(unsigned)ceil_div((int64_t)s.qtiles * 32, 256), 256, 0, st>>>(
-        q16, n, W, dv, BM, s.qtiles, nullptr, nullptr, qcen, qrad, qn, row_norm);
-    tile_sphere_kernel<<<(unsigned)ceil_div((int64_t)s.dtiles * 32, 256), 256, 0, st>>>(
-        q16, n, W, dv, BN, s.dtiles, nullptr, nullptr, dcen, drad, dn, nullptr);
+    if (BM != kPairBM || BN != kPairBN) return cudaErrorInvalidValue;
+    tile_pair_sphere_kernel<<<(unsigned)s.dtiles, 256, 0, st>>>(q16, n, W, dv, s.qtiles, qcen, qrad, qn, dcen, drad, dn,
+                                                               row_norm);
     tile_tau_kernel<<<(unsigned)ceil_div((int64_t)s.qtiles * 32, 256), 256, 0, st>>>(st_key, n, EG, KCP, row_norm,
                                                                                      s.qtiles, BM, tau);
     const int ngroups = (int)ceil_div(s.dtiles, kGroupTiles);
@@ -574,11 +695,11 @@ cudaError_t launch_prune_bounds(const void *Qb, int64_t n, int d, int metric, in
         dcen, drad, dn, s.dtiles, ngroups, PL.gcen, PL.grad, PL.gn);
     const dim3 grid((unsigned)ceil_div(s.qtiles, kBoundThreads), (unsigned)s.nchunk);
     const int qpt = BN / BM;
-    prune_tiles_kernel<<<grid, kBoundThreads, 0, st>>>(s.qtiles, s.dtiles, s.nchunk, qpt, window, beta, qcen, qrad,
+    prune_tiles_kernel<<<grid, kBoundThreads, 0, st>>>(s.qtiles, s.dtiles, s.nchunk, s.chunk_tiles, qpt, window, beta, qcen, qrad,
                                                        qn, tau, dcen, drad, dn, PL.gcen, PL.grad, PL.gn, cnt, PL.bits);
     cudaError_t e = seg_scan::launch(cnt, (int64_t)ncnt, off, PL.ssum, st, s.cap, out->overflow);
     if (e != cudaSuccess) return e;
-    fill_tiles_kernel<<<(unsigned)ceil_div((int64_t)ncnt, 256), 256, 0, st>>>(s.qtiles, s.dtiles, s.nchunk, PL.bits,
+    fill_tiles_kernel<<<(unsigned)ceil_div((int64_t)ncnt, 256), 256, 0, st>>>(s.qtiles, s.dtiles, s.nchunk, s.chunk_tiles, PL.bits,
                                                                              off, out->tiles, s.cap);
     tile_offsets_kernel<<<(unsigned)ceil_div(s.qtiles + 1, 256), 256, 0, st>>>(s.qtiles, s.nchunk, off,
                                                                                out->tile_off);
