@@ -89,6 +89,17 @@ std::vector<rsc_knn_opts> knn_candidates(const rsc_knn_opts &base, int64_t n, in
     std::vector<rsc_knn_opts> out;
     std::vector<int> parts_opts = {0};
     if (base.precision != RSC_FP32) parts_opts = {4, 2};
+    if (base.precision == RSC_FP32 && n < kSimtPruneMinRows) {
+        // the default of small FP32 inputs, spelled out (its default candidate
+        // count is explicit, so the planner does not consult the table)
+        rsc_knn_opts o = base;
+        o.db_splits = 0;
+        o.candidates = k + 8;
+        o.tc_parts = 0;
+        o.stages = 0;
+        size_t bytes = 0;
+        if (rsc_knn_workspace_size(n, d, k, metric, &o, &bytes) == RSC_OK) out.push_back(o);
+    }
     for (int parts : parts_opts) {
         for (int sp : {1, 2, 4, 8}) {
             rsc_knn_opts o = base;

@@ -61,7 +61,7 @@ constexpr int kSupportedKC[] = {16, 32, 64};
 
 struct KnnPlan {
     int precision = RSC_FP32;
-    int d = 0, metric = 0;
+    int d = 0, metric = 0, k = 0;
     int DP = 0;         // padded FP32 row length
     int KC = 0;         // ids per candidate list
     int parts = 1;      // candidate lists per query per split
@@ -70,6 +70,7 @@ struct KnnPlan {
     bool order = false; // locality ordering before the tensor-core search
     bool prune = false; // window pass + tile bounds + list pass instead of one full scan
     bool simt_prune = false;   // FP32: ordered rows, tiles pruned inside the search kernel
+    bool simt_flat = false;    // FP32, fewer rows: parts of the database, lists merged in the re-rank
     int stages = 0;     // tensor-core pipeline stages (0: as many as fit)
 };
 
@@ -122,6 +123,7 @@ rsc_status plan_knn(int64_t n, int32_t d, int32_t k, int32_t metric, const rsc_k
     p->stages = o->stages;
     p->precision = o->precision;
     p->d = d;
+    p->k = k;
     p->metric = metric;
     const bool tc = o->precision == RSC_BF16 || o->precision == RSC_FP8;   // tensor-core candidate search
     p->order = tc && (o->locality == 2 || (o->locality == 0 && n >= kOrderMinRows));
@@ -173,6 +175,17 @@ rsc_status plan_knn(int64_t n, int32_t d, int32_t k, int32_t metric, const rsc_k
         p->KC = simt_pruned_list(k);
         p->splits = 1;
         p->split_len = n;
+        return RSC_OK;
+    }
+    // fewer rows, the split left automatic: the same kernel over parts of the
+    // database (the full scan's kernel is left for explicit splits, k > 32 and
+    // the plain full scan of larger inputs)
+    p->simt_flat = !tc && o->db_splits == 0 && n < kSimtPruneMinRows && simt_pruned_list(k) > 0;
+    if (p->simt_flat) {
+        p->KC = simt_pruned_list(k);
+        p->splits = 1;
+        p->split_len = n;
+        if (o->prune == 2) return fail(RSC_ERR_UNSUPPORTED, "prune needs BF16, the locality ordering, one database split and d + 3 <= 64");
         return RSC_OK;
     }
     // database splits: enough CTAs to fill the GPU when there are few queries
@@ -229,7 +242,7 @@ KnnLayout carve_knn(void *ws, int64_t n, const KnnPlan &p, size_t *bytes) {
         L.Db = cv.take<uint8_t>((size_t)n * 64);
         L.amax = cv.take<unsigned int>(1);
     }
-    L.cand = cv.take<int32_t>((size_t)p.splits * p.parts * n * p.KC);
+    L.cand = p.simt_flat ? nullptr : cv.take<int32_t>((size_t)p.splits * p.parts * n * p.KC);
     L.perm = nullptr;
     L.order_scratch = nullptr;
     L.Rp = nullptr;
@@ -242,6 +255,7 @@ KnnLayout carve_knn(void *ws, int64_t n, const KnnPlan &p, size_t *bytes) {
     L.st_key = nullptr;
     L.st_id = nullptr;
     L.prune_scratch = nullptr;
+    if (p.simt_flat) L.prune_scratch = cv.take<uint8_t>(simt_flat_scratch_bytes(n, p.DP, p.k));
     if (p.simt_prune) L.prune_scratch = cv.take<uint8_t>(simt_pruned_scratch_bytes(n, p.DP));
     if (p.prune) {
         L.st_key = cv.take<float>((size_t)n * p.parts * p.KC);
@@ -558,6 +572,10 @@ rsc_status rsc_knn(const float *X, int64_t n, int32_t d, int32_t k, int32_t metr
         RSC_CUDA_TRY(launch_knn_simt_pruned(L.Y, L.ny, n, p.DP, d + (metric == RSC_COSINE ? 1 : 0), k, metric, L.perm,
                                             order_leaves(L.order_scratch, n, p.DP, target), L.prune_scratch, L.cand,
                                             L.status, st));
+    } else if (p.simt_flat) {
+        if (ev) RSC_CUDA_TRY(cudaEventRecord(ev[1], st));
+        RSC_CUDA_TRY(launch_knn_simt_flat(L.Y, L.ny, n, p.DP, d + (metric == RSC_COSINE ? 1 : 0), k, L.prune_scratch,
+                                          L.status, st));
     } else {
         if (ev) RSC_CUDA_TRY(cudaEventRecord(ev[1], st));
         RSC_CUDA_TRY(launch_knn_simt(L.Y, L.ny, n, p.DP, d + (metric == RSC_COSINE ? 1 : 0), p.KC, p.splits,
@@ -572,6 +590,14 @@ rsc_status rsc_knn(const float *X, int64_t n, int32_t d, int32_t k, int32_t metr
         rsr = (metric == RSC_EUCLIDEAN) ? ceil_div(d, 4) * 4 : p.DP;
         RSC_CUDA_TRY(launch_gather_rows(R, rs, n, (int)rs, L.perm, L.Rp, rsr, st));
         R = L.Rp;
+    }
+    if (p.simt_flat) {
+        const int width = d + (metric == RSC_COSINE ? 1 : 0);
+        RSC_CUDA_TRY(launch_rerank_parts(R, rsr, n, d, metric, simt_flat_parts(L.prune_scratch, n, p.DP, k), width, k,
+                                         idx, dist, st));
+        RSC_CUDA_TRY(launch_simt_flat_ties(n, d, p.DP, width, k, metric, L.prune_scratch, R, rsr, idx, dist, st));
+        if (ev) RSC_CUDA_TRY(cudaEventRecord(ev[3], st));
+        return RSC_OK;
     }
     RSC_CUDA_TRY(launch_rerank(R, rsr, n, d, metric, L.cand, p.KC, p.splits * p.parts, k, L.perm, p.order, idx, dist,
                                st));

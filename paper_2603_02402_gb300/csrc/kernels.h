@@ -44,6 +44,27 @@ cudaError_t launch_knn_simt_pruned(const float *Y, const float *ny, int64_t n, i
 cudaError_t launch_simt_ties(int64_t n, int d, int DP, int width, int k, int metric, void *scratch, const float *R,
                              int64_t rs, int32_t *idx, float *dist, cudaStream_t st);
 
+// The FP32 search of rows in their own order, k <= 32 (fewer than
+// kSimtPruneMinRows): every query's lists of simt_flat_segs parts of the
+// database, merged and re-ranked by launch_rerank_parts, ties as above.
+constexpr int kSimtFlatSegs = 16;
+struct SimtParts {
+    const float *key;     // [n rounded up to 128][segs][list], each list ascending
+    const int32_t *id;    // row ids, -1 pads
+    const float *vv;      // |y|^2 of every row
+    int segs, list;
+    int *tie_count;       // rows for the ties pass
+    int32_t *tie_rows;    // (row, place in the records)
+    float *tie_bound;
+};
+int simt_flat_segs(int64_t n, int DP);
+size_t simt_flat_scratch_bytes(int64_t n, int DP, int k);
+SimtParts simt_flat_parts(void *scratch, int64_t n, int DP, int k);
+cudaError_t launch_knn_simt_flat(const float *Y, const float *ny, int64_t n, int DP, int width, int k, void *scratch,
+                                 unsigned int *status, cudaStream_t st);
+cudaError_t launch_simt_flat_ties(int64_t n, int d, int DP, int width, int k, int metric, void *scratch, const float *R,
+                                  int64_t rs, int32_t *idx, float *dist, cudaStream_t st);
+
 // ---- knn_tc.cu ------------------------------------------------------------
 // BF16 tensor-core candidate search.  Qb/Db: [n, 64 * tc_kb(d, metric)] bf16
 // operand rows built by launch_prep_bf16 from the FP32 prep rows Y.  Each
@@ -266,6 +287,11 @@ void tuned_store(int kind, int precision, int metric, int d, int k, int kx, int6
 cudaError_t launch_rerank(const float *R, int64_t rs, int64_t n, int d, int metric,
                           const int32_t *cand, int KC, int splits, int k, const int32_t *perm, bool r_by_pos,
                           int32_t *idx, float *dist, cudaStream_t st);
+// The same re-rank of the candidates that the lists of an FP32 search's parts
+// name (rows in their own order, k <= 32): only those within reach of the k-th
+// smallest key are scored.  width: components of the searched rows.
+cudaError_t launch_rerank_parts(const float *R, int64_t rs, int64_t n, int d, int metric, const SimtParts &parts,
+                                int width, int k, int32_t *idx, float *dist, cudaStream_t st);
 // dst row i <- src row perm[i] (width floats per row).
 cudaError_t launch_gather_rows(const float *src, int64_t src_stride, int64_t n, int width, const int32_t *perm,
                                float *dst, int64_t dst_stride, cudaStream_t st);

@@ -284,12 +284,7 @@ struct List {
         k = k_;
         w = w_;
     }
-    // largest s that may still belong to one of the k nearest
-    __device__ __forceinline__ float reach_of(float t) const {
-        const float far = v2 + sqrtf(fmaxf(t + vv, 0.f));   // V + D
-        const float e = 1.25f * 0x1p-24f * (float)(w + 20) * (2.f * v2 * far + far * far);
-        return t + 2.f * e + 0x1p-22f * fabsf(t);
-    }
+    __device__ __forceinline__ float reach_of(float t) const { return rr::reach(t, vv, v2, w); }
     __device__ __forceinline__ float reach() const {
         float t = top.key[0];
 #pragma unroll
@@ -378,8 +373,10 @@ struct Args {
     uint32_t *bits;         // [CTAs][stride / 32] tiles an item keeps
     int32_t *big;           // [kBigItems][1 + kSeeds] items to be split, their seeds (-1 pads)
     int *big_count, *unit;  // their number (may exceed kBigItems), next part
-    float *part_key;        // [kBigItems][kSegs][KC][kQ] lists of the parts
-    int32_t *part_id;
+    float *part_key;        // [query slots][part_segs][KC] lists of the parts; a slot is a query
+    int32_t *part_id;       // tile pair's (split: position in `big`; flat: item) kQ rows
+    int part_segs;
+    float *vv;              // [query slots] |y|^2 (flat)
     unsigned long long *scanned;   // tiles scanned (a statistic)
     unsigned int *status;
 };
@@ -415,8 +412,12 @@ __device__ __forceinline__ void emit(const Args &g, const List<KC> &tk, int64_t 
 // items are put on a list instead, as long as it has room, and kSplit = true
 // runs them in up to kSegs parts, each over a segment of the database from
 // the item's own surroundings on, whose lists merge_kernel joins.
-template <int KC, bool kSplit>
+// kFlat: rows in their own order, part_segs parts per item and no tests: the
+// search of fewer rows than an ordering pays for (see launch_knn_simt_flat).
+enum { kWhole, kSplitItems, kFlat };
+template <int KC, int kMode>
 __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
+    constexpr bool kSplit = kMode == kSplitItems, kIsFlat = kMode == kFlat;
     extern __shared__ __align__(128) uint8_t sm[];
     const int DP = g.DP;
     const Smem m = smem_layout(DP);
@@ -452,9 +453,10 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
         return true;
     };
     const int64_t tiles = *g.T;   // an odd count is followed by an empty tile
-    const int64_t seg_len = seg_tiles(tiles);
-    const int segs = (int)ceil_div(tiles, seg_len);
-    const int64_t units = kSplit ? (int64_t)min(*g.big_count, kBigItems) * segs : ceil_div(tiles, (int64_t)2);
+    const int64_t seg_len = kIsFlat ? ceil_div(tiles, (int64_t)g.part_segs) : seg_tiles(tiles);
+    const int segs = kIsFlat ? g.part_segs : (int)ceil_div(tiles, seg_len);
+    const int64_t pairs = ceil_div(tiles, (int64_t)2);
+    const int64_t units = kIsFlat ? pairs * segs : kSplit ? (int64_t)min(*g.big_count, kBigItems) * segs : pairs;
     uint32_t tile_no = 0;     // tiles consumed by this CTA so far (stage tile_no % kStages)
     uint32_t items = 0;
     unsigned long long scanned = 0;
@@ -547,14 +549,14 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
         const int64_t unit = *item_s;
         if (unit >= units) break;
         const int32_t *big = g.big + unit / segs * (1 + kSeeds);   // kSplit
-        const int64_t item = kSplit ? (int64_t)big[0] : unit;
+        const int64_t item = kSplit ? (int64_t)big[0] : kIsFlat ? unit / segs : unit;
         if (tid == 0) {
             tc::mbar_arrive_expect_tx(xfull, 2 * x_bytes);
             tc::bulk_load(xs, g.rec + (2 * item) * rf, x_bytes, xfull);
             tc::bulk_load(xs + DP * kR, g.rec + (2 * item + 1) * rf, x_bytes, xfull);
         }
         // centres of the two query tiles
-        {
+        if (!kIsFlat) {
             const int h = tid >> 6, u = tid & 63;
             cen[tid] = u < DP ? g.cenT[(int64_t)u * g.stride + 2 * item + h] : 0.f;
         }
@@ -568,10 +570,17 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
         const float *xr = xs + (tid >> 6) * DP * kR + (tid & 63);
         for (int t = 0; t < g.width; ++t) nn = fmaf(xr[t * kR], xr[t * kR], nn);
         tk.start(nn, g.k, g.width);
-        const float rq[2] = {g.rad[2 * item], g.rad[2 * item + 1]}, nq[2] = {g.nmax[2 * item], g.nmax[2 * item + 1]};
+        float rq[2] = {0.f, 0.f}, nq[2] = {0.f, 0.f};
+        if (!kIsFlat) {
+            rq[0] = g.rad[2 * item];
+            rq[1] = g.rad[2 * item + 1];
+            nq[0] = g.nmax[2 * item];
+            nq[1] = g.nmax[2 * item + 1];
+        }
         const int wlo = (int)max((int64_t)0, 2 * item - kWin), whi = (int)min(tiles, 2 * item + 2 + kWin);
         // the range of tiles in chunks, from the chunk of the query tiles on
-        const int64_t lo = kSplit ? (unit % segs) * seg_len : 0, hi = kSplit ? min(tiles, lo + seg_len) : tiles;
+        const int64_t lo = kMode != kWhole ? min(tiles, (unit % segs) * seg_len) : 0;
+        const int64_t hi = kMode != kWhole ? min(tiles, lo + seg_len) : tiles;
         const int chunks = (int)ceil_div(hi - lo, (int64_t)kChunk), c0 = kSplit ? 0 : (int)((2 * item) / kChunk);
         const int64_t most = max((int64_t)64, tiles / 16);
         uint32_t *bits = g.bits + (int64_t)blockIdx.x * ceil_div(tiles, (int64_t)kChunk) * kWords;
@@ -596,9 +605,20 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
             if (tid < kSeeds) seeds[tid] = big[1 + tid];
             while (n_seeds < kSeeds && big[1 + n_seeds] >= 0) ++n_seeds;
         }
+        int64_t done = 0;   // flat: tiles of the part scanned so far
+        bool first = true;
         while (true) {
             int nl = 0;
-            if (step == kWindow) {
+            if (kIsFlat) {   // the part's tiles, from the query's own on when they are among them
+                const int64_t len = hi - lo, from = 2 * item >= lo && 2 * item < hi ? 2 * item - lo : 0;
+                nl = (int)min((int64_t)kChunk, len - done);
+                if (nl <= 0) break;
+                for (int x = tid; x < nl; x += kQ) {
+                    const int64_t at = from + done + x;
+                    list[x] = (int)(lo + (at < len ? at : at - len));
+                }
+                done += nl;
+            } else if (step == kWindow) {
                 nl = whi - wlo;
                 const int own = (int)(2 * item) - wlo;   // the query tiles themselves first
                 if (tid < nl) list[tid] = wlo + (tid == 0 ? own : tid <= own ? tid - 1 : tid);
@@ -726,21 +746,30 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
             }
             __syncthreads();
             if (nl > 0) {
-                if (!scan(nl, step == kWindow)) return;
+                if (!scan(nl, first)) return;
                 fresh = true;
+                first = false;
             }
+            if (kIsFlat) continue;
             if (step == kWindow) step = kSplit ? (n_seeds > 0 ? kNearest : kChunks) : kMark;
             else if (step == kNearest) {
                 step = kSplit ? kChunks : kAgain;
                 kept = 0;
             }
         }
-        if (kSplit) {
-            const int64_t at = ((unit / segs) * kSegs + unit % segs) * KC;
+        if (kMode != kWhole) {
+            const int64_t slot = (kIsFlat ? item : unit / segs) * kQ + tid;
+            if (live) {
+                float *pk = g.part_key + (slot * g.part_segs + unit % segs) * KC;
+                int32_t *pi = g.part_id + (slot * g.part_segs + unit % segs) * KC;
 #pragma unroll
-            for (int c = 0; c < KC; ++c) {
-                g.part_key[(at + c) * kQ + tid] = tk.top.key[c];
-                g.part_id[(at + c) * kQ + tid] = tk.top.id[c];
+                for (int c = 0; c < KC; c += 4) {
+                    *reinterpret_cast<float4 *>(pk + c) =
+                        make_float4(tk.top.key[c], tk.top.key[c + 1], tk.top.key[c + 2], tk.top.key[c + 3]);
+                    *reinterpret_cast<int4 *>(pi + c) =
+                        make_int4(tk.top.id[c], tk.top.id[c + 1], tk.top.id[c + 2], tk.top.id[c + 3]);
+                }
+                if (kIsFlat && unit % segs == 0) g.vv[slot] = nn;
             }
         } else if (live && !deferred) {
             emit(g, tk, item, tid);
@@ -765,11 +794,11 @@ __global__ void __launch_bounds__(kQ) merge_kernel(const Args g) {
     List<KC> tk;
     tk.start(nn, g.k, g.width);
     for (int s = 0; s < segs; ++s) {
-        const int64_t at = ((int64_t)b * kSegs + s) * KC;
+        const int64_t at = (((int64_t)b * kQ + tid) * g.part_segs + s) * KC;
 #pragma unroll 1
         for (int c = 0; c < KC; ++c) {
-            const float v = g.part_key[(at + c) * kQ + tid];
-            const int j = g.part_id[(at + c) * kQ + tid];
+            const float v = g.part_key[at + c];
+            const int j = g.part_id[at + c];
             if (j < 0 || !(v < tk.top.thr())) break;   // ascending
             bool have = false;
 #pragma unroll
@@ -907,6 +936,8 @@ Args make_args(const Layout &L, int64_t n, int DP, int width, int k, int metric,
     g.unit = L.counters + 6;
     g.part_key = L.part_key;
     g.part_id = L.part_id;
+    g.part_segs = kSegs;
+    g.vv = nullptr;
     g.status = status;
     return g;
 }
@@ -928,8 +959,8 @@ namespace simtp {
 template <int KC>
 cudaError_t launch_list(const Args &g, int64_t tiles, cudaStream_t st) {
     const int smem = smem_layout(g.DP).total;
-    auto whole = simt_pruned_kernel<KC, false>;
-    auto split = simt_pruned_kernel<KC, true>;
+    auto whole = simt_pruned_kernel<KC, kWhole>;
+    auto split = simt_pruned_kernel<KC, kSplitItems>;
     cudaError_t e = cudaFuncSetAttribute(whole, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(split, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -963,6 +994,148 @@ cudaError_t launch_simt_ties(int64_t n, int d, int DP, int width, int k, int met
     using namespace simtp;
     const Layout L = layout(scratch, n, DP);
     const Args g = make_args(L, n, DP, width, k, metric, nullptr, nullptr);
+    const bool vec = rs % 4 == 0 && reinterpret_cast<uintptr_t>(R) % 16 == 0;
+    ties_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n, (int64_t)4), 8 * sm_count()), 128, 0, st>>>(
+        g, R, rs, d, metric == RSC_COSINE, vec, idx, dist);
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------------- rows as they are
+
+namespace simtp {
+
+// Block per tile of 64 rows in their own order: record, ids, tile tables (the
+// tile that completes an odd count is empty).
+__global__ void __launch_bounds__(256)
+pack_flat_kernel(const float *__restrict__ Y, const float *__restrict__ ny, int64_t n, int DP, float *__restrict__ rec,
+                 int32_t *__restrict__ ids, int32_t *__restrict__ tile_pos, int32_t *__restrict__ tile_rows,
+                 int32_t *__restrict__ T) {
+    __shared__ float ys[64][kR + 1];
+    const int64_t t = blockIdx.x, r0 = t * kR;
+    const int tid = threadIdx.x, rows = (int)max((int64_t)0, min((int64_t)kR, n - r0));
+    const int r = tid >> 2, l = tid & 3;
+    for (int c = l; c < DP / 4; c += 4) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < rows) v = reinterpret_cast<const float4 *>(Y + (r0 + r) * DP)[c];
+        ys[4 * c][r] = v.x;
+        ys[4 * c + 1][r] = v.y;
+        ys[4 * c + 2][r] = v.z;
+        ys[4 * c + 3][r] = v.w;
+    }
+    if (l == 0) ids[r0 + r] = r < rows ? (int32_t)(r0 + r) : INT_MAX;
+    __syncthreads();
+    float *out = rec + t * record_floats(DP);
+    for (int e = tid; e < DP * kR; e += 256) out[e] = ys[e >> 6][e & 63];
+    if (tid < kR) out[DP * kR + tid] = tid < rows ? ny[r0 + tid] : NAN;
+    if (tid == 0) {
+        tile_pos[t] = (int32_t)r0;
+        tile_rows[t] = rows;
+        if (t == 0) *T = (int32_t)ceil_div(n, (int64_t)kR);
+    }
+}
+
+struct FlatLayout {
+    float *rec, *part_key, *vv, *tie_bound;
+    int32_t *ids, *tile_pos, *tile_rows, *part_id, *tie_rows;
+    int *counters;   // tie_count, counter, scanned (64 bits), tiles
+    size_t bytes;
+};
+FlatLayout flat_layout(void *scratch, int64_t n, int DP, int k) {
+    Carve cv(scratch);
+    FlatLayout L;
+    const int64_t items = ceil_div(n, (int64_t)kQ);
+    const size_t parts = (size_t)items * kQ * simt_flat_segs(n, DP) * simt_pruned_list(k);
+    L.rec = cv.take<float>((size_t)items * 2 * record_floats(DP));
+    L.ids = cv.take<int32_t>((size_t)items * kQ);
+    L.tile_pos = cv.take<int32_t>((size_t)items * 2);
+    L.tile_rows = cv.take<int32_t>((size_t)items * 2);
+    L.part_key = cv.take<float>(parts);
+    L.part_id = cv.take<int32_t>(parts);
+    L.vv = cv.take<float>((size_t)items * kQ);
+    L.tie_rows = cv.take<int32_t>((size_t)2 * n);
+    L.tie_bound = cv.take<float>((size_t)n);
+    L.counters = cv.take<int>(5);
+    L.bytes = cv.used;
+    return L;
+}
+
+Args flat_args(const FlatLayout &L, int64_t n, int DP, int width, int k, unsigned int *status) {
+    Args g = {};
+    g.rec = L.rec;
+    g.ids = L.ids;
+    g.tile_pos = L.tile_pos;
+    g.tile_rows = L.tile_rows;
+    g.tie_count = L.counters;
+    g.counter = L.counters + 1;
+    g.scanned = reinterpret_cast<unsigned long long *>(L.counters + 2);
+    g.T = L.counters + 4;
+    g.n = n;
+    g.DP = DP;
+    g.width = width;
+    g.k = k;
+    g.part_key = L.part_key;
+    g.part_id = L.part_id;
+    g.part_segs = simt_flat_segs(n, DP);
+    g.vv = L.vv;
+    g.tie_rows = L.tie_rows;
+    g.tie_bound = L.tie_bound;
+    g.status = status;
+    return g;
+}
+
+}  // namespace simtp
+
+// Why parts and this kernel below kSimtPruneMinRows: the full scan's kernel
+// keeps 32 values per row and split and its re-rank scores them all (10,000
+// rows: 491 + 267 us, 2,700 rows: 105 + 120 us); here a list takes in only what
+// can be among the k nearest and the re-rank scores what the merged lists leave
+// (409 + 22 us and 61 + 12 us).
+// Parts per query tile pair: the count whose waves of persistent CTAs cost
+// least, a part costing its tiles plus about three (lists built anew, the
+// query tiles fetched).
+int simt_flat_segs(int64_t n, int DP) {
+    const int64_t items = ceil_div(n, (int64_t)simtp::kQ), tiles = ceil_div(n, (int64_t)simtp::kR);
+    const int64_t slots = 152 * (DP <= 56 ? 2 : 1);   // CTAs an SM holds
+    int best = 1;
+    int64_t cost = INT64_MAX;
+    for (int s = 1; s <= kSimtFlatSegs && s <= tiles; ++s) {
+        const int64_t c = ceil_div(items * s, slots) * (ceil_div(tiles, (int64_t)s) + 3);
+        if (c < cost) {
+            cost = c;
+            best = s;
+        }
+    }
+    return best;
+}
+
+size_t simt_flat_scratch_bytes(int64_t n, int DP, int k) { return simtp::flat_layout(nullptr, n, DP, k).bytes; }
+
+SimtParts simt_flat_parts(void *scratch, int64_t n, int DP, int k) {
+    const simtp::FlatLayout L = simtp::flat_layout(scratch, n, DP, k);
+    return {L.part_key, L.part_id, L.vv, simt_flat_segs(n, DP), simt_pruned_list(k), L.counters, L.tie_rows, L.tie_bound};
+}
+
+cudaError_t launch_knn_simt_flat(const float *Y, const float *ny, int64_t n, int DP, int width, int k, void *scratch,
+                                 unsigned int *status, cudaStream_t st) {
+    using namespace simtp;
+    const FlatLayout L = flat_layout(scratch, n, DP, k);
+    const Args g = flat_args(L, n, DP, width, k, status);
+    cudaError_t e = cudaMemsetAsync(L.counters, 0, 5 * sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    const int64_t items = ceil_div(n, (int64_t)kQ);
+    pack_flat_kernel<<<(unsigned)(2 * items), 256, 0, st>>>(Y, ny, n, DP, L.rec, L.ids, L.tile_pos, L.tile_rows,
+                                                           L.counters + 4);
+    const int smem = smem_layout(DP).total;
+    auto kern = simt_pruned_list(k) == 24 ? simt_pruned_kernel<24, kFlat> : simt_pruned_kernel<kMaxList, kFlat>;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+    kern<<<(unsigned)std::min<int64_t>(items * g.part_segs, 2 * sm_count()), kQ, smem, st>>>(g);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_simt_flat_ties(int64_t n, int d, int DP, int width, int k, int metric, void *scratch, const float *R,
+                                  int64_t rs, int32_t *idx, float *dist, cudaStream_t st) {
+    using namespace simtp;
+    const Args g = flat_args(flat_layout(scratch, n, DP, k), n, DP, width, k, nullptr);
     const bool vec = rs % 4 == 0 && reinterpret_cast<uintptr_t>(R) % 16 == 0;
     ties_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n, (int64_t)4), 8 * sm_count()), 128, 0, st>>>(
         g, R, rs, d, metric == RSC_COSINE, vec, idx, dist);

@@ -629,24 +629,7 @@ rerank_probe_kernel(const float *__restrict__ X, int d, const int32_t *__restric
             bi[0] = id[0];
             continue;
         }
-        // the 32 smallest of two ascending runs: elementwise minima of one and
-        // the other reversed form a bitonic run, sorted by five half-cleaners
-        const float rk = __shfl_xor_sync(0xffffffffu, key[0], 31);
-        const int ri = __shfl_xor_sync(0xffffffffu, id[0], 31);
-        if (pair_gt(bk[0], bi[0], rk, ri)) {
-            bk[0] = rk;
-            bi[0] = ri;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float pk = __shfl_xor_sync(0xffffffffu, bk[0], o);
-            const int pi = __shfl_xor_sync(0xffffffffu, bi[0], o);
-            const bool lower = (lane & o) == 0;
-            if (lower ? pair_gt(bk[0], bi[0], pk, pi) : pair_gt(pk, pi, bk[0], bi[0])) {
-                bk[0] = pk;
-                bi[0] = pi;
-            }
-        }
+        warp_merge_best(bk[0], bi[0], key[0], id[0]);
     }
     if (lane < k) {
         const bool valid = bi[0] != INT_MAX;

@@ -33,6 +33,16 @@ __device__ __forceinline__ void load8(const float *row, int s, int d, bool cosin
     }
 }
 
+// A bound for the FP32 search: whatever has s = |y_j|^2 - 2 y_i.y_j above
+// reach(t) is further by the re-rank than k rows at or below t, when k rows lie
+// at or below t.  vv, v: |y_i|^2 and |y_i|, w: components (knn_simt_prune.cu
+// derives it).
+__device__ __forceinline__ float reach(float t, float vv, float v, int w) {
+    const float far = v + sqrtf(fmaxf(t + vv, 0.f));   // |y_i| + distance
+    const float e = 1.25f * 0x1p-24f * (float)(w + 20) * (2.f * v * far + far * far);
+    return t + 2.f * e + 0x1p-22f * fabsf(t);
+}
+
 // Sum of squared differences of the two rows (every lane of the eight gets it).
 __device__ __forceinline__ float dist2(const float (&x)[8], const float (&y)[8]) {
     float part = 0.f;

@@ -59,6 +59,29 @@ __device__ __forceinline__ void warp_sort_pairs(float (&key)[E], int (&id)[E]) {
     }
 }
 
+// The 32 smallest of two ascending runs, one pair per lane each, into (bk, bi):
+// elementwise minima of one and the other reversed form a bitonic run, sorted
+// by five half-cleaners.
+__device__ __forceinline__ void warp_merge_best(float &bk, int &bi, float key, int id) {
+    const int lane = threadIdx.x & 31;
+    const float rk = __shfl_xor_sync(0xffffffffu, key, 31);
+    const int ri = __shfl_xor_sync(0xffffffffu, id, 31);
+    if (pair_gt(bk, bi, rk, ri)) {
+        bk = rk;
+        bi = ri;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float pk = __shfl_xor_sync(0xffffffffu, bk, o);
+        const int pi = __shfl_xor_sync(0xffffffffu, bi, o);
+        const bool lower = (lane & o) == 0;
+        if (lower ? pair_gt(bk, bi, pk, pi) : pair_gt(pk, pi, bk, bi)) {
+            bk = pk;
+            bi = pi;
+        }
+    }
+}
+
 // Squared distance sum_t (xq_t - y_t)^2 for t < d, accumulated in t order
 // (the same rounding whichever loader runs).  w4 > 0: the row is 16-byte
 // aligned and its first 4 * w4 floats (w4 <= 16) are read as independent

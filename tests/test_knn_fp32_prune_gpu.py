@@ -85,3 +85,35 @@ def test_scan_stats_of_the_pruned_search(rsc):  # noqa: F811
         tiles = -(-n // 128)
         assert total == tiles * tiles
         assert scanned == total if prune == "off" else 0 < scanned < 0.3 * total
+
+
+@pytest.mark.parametrize("n,d,k,metric", [
+    (1, 50, 1, "euclidean"), (20, 3, 20, "euclidean"), (64, 50, 15, "euclidean"), (65, 8, 16, "cosine"),
+    (129, 64, 17, "euclidean"), (2_700, 50, 15, "euclidean"), (2_701, 50, 32, "cosine"), (5_000, 7, 32, "euclidean"),
+    (10_001, 33, 5, "euclidean"), (16_383, 50, 16, "euclidean"),
+])
+def test_parts_of_small_inputs_equal_one_scan(rsc, n, d, k, metric):  # noqa: F811
+    # fewer rows than the ordering pays for: the database in parts, the lists
+    # merged within reach of the k-th; explicit splits keep the plain scan
+    X = synth.mixture(n, d, n_comp=7, seed=n)
+    pi, pd = run_knn(rsc, X, k, metric=metric, precision="fp32")
+    fi, fd = run_knn(rsc, X, k, metric=metric, precision="fp32", db_splits=1)
+    np.testing.assert_array_equal(pd, fd)
+    np.testing.assert_array_equal(pi, fi)
+
+
+@pytest.mark.parametrize("case", ["grid", "duplicates", "one point"])
+def test_ties_of_small_inputs(rsc, case):  # noqa: F811
+    rng = np.random.Generator(np.random.PCG64(17))
+    if case == "grid":      # 24 and 32 neighbours at equal distance
+        X = np.stack(np.meshgrid(*[np.arange(8)] * 4), -1).reshape(-1, 4).astype(np.float32)
+    elif case == "duplicates":   # 80 rows at distance zero: more than are scored at once
+        X = np.repeat(rng.integers(0, 9, (40, 6)), 80, axis=0).astype(np.float32)
+    else:
+        X = np.full((3_000, 5), 3, dtype=np.float32)
+    X = X[rng.permutation(len(X))]
+    for k in (15, 32):
+        gi, gd = run_knn(rsc, X, k, precision="fp32")
+        oi, od, _ = oracle.knn(X, k)
+        np.testing.assert_array_equal(gi, oi)
+        np.testing.assert_allclose(gd, od, rtol=1e-6)
