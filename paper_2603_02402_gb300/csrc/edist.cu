@@ -64,32 +64,40 @@ constexpr int kSmem = kBarOff + 256 + 1024;
 constexpr uint32_t kTmemCols = 256;   // two accumulators of BN columns
 constexpr int kSample = 4096;         // rows averaged for the centre c
 
-// c = mean of up to kSample rows spread over the gathered order (one block;
-// thread t sums column t % d over its share of the rows, then the block
-// reduces in shared memory).
+// c = mean of up to kSample rows spread over the gathered order.  Block per 8
+// columns, thread (slice, column) sums its column over rows slice, slice + 32,
+// ... in order, then the slices are added in order.  Row ids and values are
+// fetched 16 rows ahead of the additions (602 us as one block that walked all
+// columns with a dependent pair of loads per row, 100k cells; 27 us so).
 __global__ void __launch_bounds__(256) centre_kernel(const float *__restrict__ X, const int32_t *__restrict__ cell,
                                                      int64_t n, int64_t n_rows, int d, float *__restrict__ centre) {
     __shared__ float part[256];
     const int m = (int)std::min<int64_t>(n, kSample);
-    const int t = threadIdx.x;
-    for (int c0 = 0; c0 < d; c0 += 8) {   // 8 columns at a time, 32 threads per column
-        const int col = c0 + (t & 7), sl = t >> 3;
-        float s = 0.f;
-        if (col < d)
-            for (int r = sl; r < m; r += 32) {
-                const int64_t p = (int64_t)r * n / m;
-                int64_t row = cell ? cell[p] : p;
-                if (row < 0 || row >= n_rows) row = 0;   // recorded by the prep kernel
-                s += X[row * d + col];
+    const int t = threadIdx.x, c0 = 8 * blockIdx.x, col = c0 + (t & 7), sl = t >> 3;
+    constexpr int kAhead = 16;
+    float s = 0.f;
+    if (col < d)
+        for (int r0 = sl; r0 < m; r0 += 32 * kAhead) {
+            int64_t row[kAhead];
+            float v[kAhead];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const int64_t p = (int64_t)min(r0 + 32 * u, m - 1) * n / m;
+                row[u] = cell ? cell[p] : p;
+                if (row[u] < 0 || row[u] >= n_rows) row[u] = 0;   // recorded by the prep kernel
             }
-        part[t] = s;
-        __syncthreads();
-        if (t < 8 && c0 + t < d) {
-            float a = 0.f;
-            for (int k = 0; k < 32; ++k) a += part[k * 8 + t];
-            centre[c0 + t] = a / (float)m;
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) v[u] = X[row[u] * d + col];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u)
+                if (r0 + 32 * u < m) s += v[u];
         }
-        __syncthreads();
+    part[t] = s;
+    __syncthreads();
+    if (t < 8 && c0 + t < d) {
+        float a = 0.f;
+        for (int k = 0; k < 32; ++k) a += part[k * 8 + t];
+        centre[c0 + t] = a / (float)m;
     }
 }
 
@@ -100,61 +108,95 @@ __device__ __forceinline__ void split3(float v, __nv_bfloat16 &a, __nv_bfloat16 
     c = __float2bfloat16_rn(r1 - __bfloat162float(b));
 }
 
-// Thread per gathered position p: the A and B operand rows (3 x 128 bytes
-// each) of cell cell[p] (or p), and its group.
-__global__ void __launch_bounds__(256) prep_kernel(const float *__restrict__ X, const int32_t *__restrict__ cell,
-                                                   int64_t n, int64_t n_rows, int d, unsigned int *status,
-                                                   const float *__restrict__ centre,
-                                                   const int64_t *__restrict__ offsets, int G,
-                                                   __nv_bfloat16 *__restrict__ A, __nv_bfloat16 *__restrict__ B,
-                                                   int32_t *__restrict__ group) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    int64_t row = cell ? cell[p] : p;
-    if (row < 0 || row >= n_rows) {   // bad cell index: recorded, row 0 read instead
-        record_status(status, RSC_ERR_INVALID_ARG);
-        row = 0;
-    }
-    const float *x = X + row * d;
-    __nv_bfloat16 *a = A + p * (64 * KB), *b = B + p * (64 * KB);
-    const __nv_bfloat16 z = __float2bfloat16_rn(0.f), one = __float2bfloat16_rn(1.f);
-    float nrm = 0.f;
-    for (int t = 0; t < 64; ++t) {
-        if (t < d) {
-            const float y = x[t] - centre[t];
-            nrm = fmaf(y, y, nrm);
-            const __nv_bfloat16 h = __float2bfloat16_rn(y);
-            const __nv_bfloat16 l = __float2bfloat16_rn(y - __bfloat162float(h));
-            const __nv_bfloat16 h2 = __float2bfloat16_rn(-2.f * __bfloat162float(h));   // exact
-            const __nv_bfloat16 l2 = __float2bfloat16_rn(-2.f * __bfloat162float(l));   // exact
-            a[t] = h;
-            a[64 + t] = l;
-            a[128 + t] = h;
-            b[t] = h2;
-            b[64 + t] = h2;
-            b[128 + t] = l2;
-        } else {
-            a[t] = a[64 + t] = a[128 + t] = z;
-            b[t] = b[64 + t] = b[128 + t] = z;
+// The A and B operand rows (3 x 128 bytes each) of gathered positions, and
+// their groups.  A warp takes 32 cells: it reads their rows of X one after the
+// other (coalesced, eight in flight) into shared memory, a lane then centres
+// its own cell and sums its norm in component order, and the operand rows go
+// out as 16-byte pieces in address order.  (390 us for 100k cells with a thread
+// per cell, whose 2-byte stores touched 32 rows each; 43 us so.)
+constexpr int kPrepWarps = 4;
+__global__ void __launch_bounds__(kPrepWarps * 32)
+prep_kernel(const float *__restrict__ X, const int32_t *__restrict__ cell, int64_t n, int64_t n_rows, int d,
+            unsigned int *status, const float *__restrict__ centre, const int64_t *__restrict__ offsets, int G,
+            __nv_bfloat16 *__restrict__ A, __nv_bfloat16 *__restrict__ B, int32_t *__restrict__ group) {
+    __shared__ float ys[kPrepWarps][32][65];          // odd stride: lane-per-cell access is conflict free
+    __shared__ __nv_bfloat16 digit[kPrepWarps][32][4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t p0 = ((int64_t)blockIdx.x * kPrepWarps + warp) * 32, p = p0 + lane;
+    if (p0 >= n) return;
+    const int here = (int)std::min<int64_t>(32, n - p0);
+    int64_t row = 0;
+    if (lane < here) {
+        row = cell ? cell[p] : p;
+        if (row < 0 || row >= n_rows) {   // bad cell index: recorded, row 0 read instead
+            record_status(status, RSC_ERR_INVALID_ARG);
+            row = 0;
         }
     }
-    __nv_bfloat16 nh, nm, nl;
-    split3(nrm, nh, nm, nl);
-    a[d] = a[d + 1] = a[d + 2] = one;
-    a[d + 3] = nh;
-    a[d + 4] = nm;
-    a[d + 5] = nl;
-    b[d] = nh;
-    b[d + 1] = nm;
-    b[d + 2] = nl;
-    b[d + 3] = b[d + 4] = b[d + 5] = one;
-    int lo = 0, hi = G - 1;   // group of position p: last g with offsets[g] <= p
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (offsets[mid] <= p) lo = mid;
-        else hi = mid - 1;
+    float (*y)[65] = ys[warp];
+    const int t0 = min(lane, d - 1), t1 = min(lane + 32, d - 1);   // components past d repeat the last and are dropped
+    for (int c0 = 0; c0 < 32; c0 += 8) {
+        float v0[8], v1[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float *x = X + __shfl_sync(0xffffffffu, row, c0 + u) * d;
+            v0[u] = x[t0];
+            v1[u] = x[t1];
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            y[c0 + u][lane] = v0[u];
+            y[c0 + u][lane + 32] = v1[u];
+        }
     }
-    group[p] = lo;
+    __syncwarp();
+    float nrm = 0.f;
+    for (int t = 0; t < d; ++t) {
+        const float v = y[lane][t] - centre[t];
+        y[lane][t] = v;
+        nrm = fmaf(v, v, nrm);
+    }
+    for (int t = d; t < 64; ++t) y[lane][t] = 0.f;
+    split3(nrm, digit[warp][lane][0], digit[warp][lane][1], digit[warp][lane][2]);
+    if (lane < here) {
+        int lo = 0, hi = G - 1;   // group of position p: last g with offsets[g] <= p
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (offsets[mid] <= p) lo = mid;
+            else hi = mid - 1;
+        }
+        group[p] = lo;
+    }
+    __syncwarp();
+    // A = [h, 1, 1, 1, n^h, n^m, n^l | l | h], B = [-2h, n^h, n^m, n^l, 1, 1, 1 | -2h | -2l]
+    const __nv_bfloat16 one = __float2bfloat16_rn(1.f);
+    for (int e = lane; e < here * 24; e += 32) {
+        const int c = e / 24, ch = e - 24 * c, kb = ch >> 3;
+        __align__(16) __nv_bfloat16 a[8], b[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int t = 8 * (ch & 7) + i;
+            const float v = y[c][t];
+            const __nv_bfloat16 h = __float2bfloat16_rn(v);
+            const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
+            const __nv_bfloat16 h2 = __float2bfloat16_rn(-2.f * __bfloat162float(h));   // exact
+            const __nv_bfloat16 l2 = __float2bfloat16_rn(-2.f * __bfloat162float(l));   // exact
+            a[i] = kb == 1 ? l : h;
+            b[i] = kb == 2 ? l2 : h2;
+            if (t >= d) {   // zeros (-2 * 0 would be -0) but for the norm's columns
+                a[i] = b[i] = __float2bfloat16_rn(0.f);
+                if (kb == 0 && t < d + 3) {
+                    a[i] = one;
+                    b[i] = digit[warp][c][t - d];
+                } else if (kb == 0 && t < d + 6) {
+                    a[i] = digit[warp][c][t - d - 3];
+                    b[i] = one;
+                }
+            }
+        }
+        reinterpret_cast<uint4 *>(A + (p0 + c) * (64 * KB))[ch] = *reinterpret_cast<const uint4 *>(a);
+        reinterpret_cast<uint4 *>(B + (p0 + c) * (64 * KB))[ch] = *reinterpret_cast<const uint4 *>(b);
+    }
 }
 
 // Per 32-column chunk of the gathered order: the group of its first column and
@@ -628,9 +670,9 @@ rsc_status run_edistance_sums(const float *X, int64_t n_rows, int32_t d, const i
     if (L.bits)
         RSC_CUDA_TRY(cudaMemcpyAsync(L.bits, p.bits.data(), sizeof(uint32_t) * p.bits.size(), cudaMemcpyHostToDevice,
                                      st));
-    ed::centre_kernel<<<1, 256, 0, st>>>(X, cell, p.n, n_rows, d, L.centre);
-    ed::prep_kernel<<<(unsigned)ceil_div(p.n, 256), 256, 0, st>>>(X, cell, p.n, n_rows, d, L.status, L.centre,
-                                                                   L.offsets, p.G, L.A, L.B, L.group);
+    ed::centre_kernel<<<(unsigned)ceil_div(d, 8), 256, 0, st>>>(X, cell, p.n, n_rows, d, L.centre);
+    ed::prep_kernel<<<(unsigned)ceil_div(p.n, 32 * ed::kPrepWarps), 32 * ed::kPrepWarps, 0, st>>>(
+        X, cell, p.n, n_rows, d, L.status, L.centre, L.offsets, p.G, L.A, L.B, L.group);
     const int64_t chunks = ceil_div(p.n, 32);
     ed::chunk_kernel<<<(unsigned)ceil_div(chunks, 256), 256, 0, st>>>(L.group, L.offsets, p.n, L.chunk);
     RSC_CUDA_TRY(cudaGetLastError());
