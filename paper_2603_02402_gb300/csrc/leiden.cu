@@ -7,9 +7,9 @@
 // round is one launch over all vertices:
 //   move     warp per vertex: the weights to each neighbouring community are
 //            summed exactly and in no particular order: for rows of up to 32
-//            entries in registers (lanes with equal labels found by
-//            match.any, their weights added by redux.sync in 16-bit pieces),
-//            for longer rows in an open-addressing table (64-bit atomic adds;
+//            entries by every lane for its own label (labels and weights read
+//            back from shared memory), for longer rows in an open-addressing
+//            table (64-bit atomic adds;
 //            the warp's own table in shared memory up to 128 entries, the
 //            vertex's table in global memory beyond; read back and cleared);
 //            the warp picks
@@ -84,39 +84,55 @@ __device__ __forceinline__ int64_t warp_sum(int64_t v) {
     return v;
 }
 
-__device__ __forceinline__ i128 shfl_xor_i128(i128 v, int o) {
-    const uint64_t lo = (uint64_t)v, hi = (uint64_t)(v >> 64);
-    const uint64_t l2 = __shfl_xor_sync(0xffffffffu, lo, o), h2 = __shfl_xor_sync(0xffffffffu, hi, o);
-    return (i128)(((unsigned __int128)h2 << 64) | l2);
-}
-
-// Warp-wide best (largest gain, then smallest label); c == kNone: no candidate.
+// Warp-wide best (largest gain, then smallest label); c == kNone: no
+// candidate.  The gains are compared 32 bits at a time from the top: lanes
+// below the maximum of a piece drop out (redux), five steps where exchanging
+// 128-bit values pairwise takes five rounds of five shuffles.
 __device__ __forceinline__ void warp_best(i128 &g, int32_t &c) {
+    bool in = c != kNone;
+    unsigned piece[4];
+    const unsigned __int128 u = (unsigned __int128)g ^ ((unsigned __int128)1 << 127);   // orders as unsigned
+    unsigned top[4];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const i128 og = shfl_xor_i128(g, o);
-        const int32_t oc = __shfl_xor_sync(0xffffffffu, c, o);
-        if (oc != kNone && (c == kNone || og > g || (og == g && oc < c))) {
-            g = og;
-            c = oc;
-        }
+    for (int i = 0; i < 4; ++i) {
+        piece[i] = (unsigned)(u >> (96 - 32 * i));
+        top[i] = __reduce_max_sync(0xffffffffu, in ? piece[i] : 0u);
+        in = in && piece[i] == top[i];
     }
+    c = (int32_t)__reduce_min_sync(0xffffffffu, in ? (unsigned)c : (unsigned)kNone);
+    const unsigned __int128 r = ((unsigned __int128)top[0] << 96) | ((unsigned __int128)top[1] << 64) |
+                                ((unsigned __int128)top[2] << 32) | top[3];
+    g = (i128)(r ^ ((unsigned __int128)1 << 127));
 }
 
 // Rows of at most 32 entries, without tables: lane l holds entry l's label c
-// (kNone when the entry is skipped) and weight w.  Lanes with equal labels
-// find each other (match.any) and add their weights exactly in four 16-bit
-// pieces (redux.sync.add over the lanes of the label); the label's first lane
-// is its leader.  Returns the label's total weight.
-__device__ __forceinline__ int64_t label_sum(int32_t c, int64_t w, bool &leader) {
-    const unsigned peers = __match_any_sync(0xffffffffu, c);
-    const uint64_t u = (uint64_t)w;
-    const uint64_t p0 = __reduce_add_sync(peers, (unsigned)(u & 0xFFFF));
-    const uint64_t p1 = __reduce_add_sync(peers, (unsigned)((u >> 16) & 0xFFFF));
-    const uint64_t p2 = __reduce_add_sync(peers, (unsigned)((u >> 32) & 0xFFFF));
-    const uint64_t p3 = __reduce_add_sync(peers, (unsigned)(u >> 48));
-    leader = c != kNone && (int)(__ffs(peers) - 1) == (int)(threadIdx.x & 31);
-    return (int64_t)(p0 + (p1 << 16) + (p2 << 32) + (p3 << 48));
+// (kNone when the entry is skipped) and weight w.  The warp's labels and
+// weights go through shared memory and every lane adds up the weights of its
+// own label (broadcast reads, four entries a step, up to the row's length).
+// Returns the label's total weight; its first lane is its leader.
+// (Finding equal labels by match.any and adding by redux.sync over each
+// label's lanes runs once per distinct label: 331 us a round on average at
+// 200k vertices, 4.5M entries, 407 us where every label is another; so 239 us.)
+__device__ __forceinline__ int64_t label_sum(int32_t c, int64_t w, int deg, int32_t *lab_s, int64_t *wt_s, bool &leader) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    lab_s[lane] = c;
+    wt_s[lane] = w;
+    __syncwarp();
+    int64_t s = 0;
+    bool first = true;
+    const int4 *l4 = reinterpret_cast<const int4 *>(lab_s);
+    const longlong2 *w2 = reinterpret_cast<const longlong2 *>(wt_s);
+#pragma unroll 2
+    for (int j = 0; j < deg; j += 4) {   // entries past deg hold kNone and are never this lane's label
+        const int4 l = l4[j >> 2];
+        const longlong2 x = w2[j >> 1], y = w2[(j >> 1) + 1];
+        s += (l.x == c ? x.x : 0) + (l.y == c ? x.y : 0) + (l.z == c ? y.x : 0) + (l.w == c ? y.y : 0);
+        first = first && !(l.x == c && j < lane) && !(l.y == c && j + 1 < lane) && !(l.z == c && j + 2 < lane) &&
+                !(l.w == c && j + 3 < lane);
+    }
+    leader = c != kNone && first;
+    return s;
 }
 
 __global__ void weights_kernel(const float *__restrict__ data, int64_t nnz, int64_t *__restrict__ wt) {
@@ -213,7 +229,11 @@ move_kernel(int64_t nv, const int64_t *__restrict__ ip, const int32_t *__restric
     int64_t sa = 0;
     i128 gb = 0;
     int32_t best = kNone;
-    if (e1 - e0 <= 32) {   // warp-uniform: sums in registers
+    // tables in shared memory (33 to 128 entries), labels and weights of
+    // shorter rows
+    __shared__ __align__(16) int32_t s_key[kWarps][kSmemSlots];
+    __shared__ __align__(16) u64 s_sum[kWarps][kSmemSlots];
+    if (e1 - e0 <= 32) {   // warp-uniform
         int32_t c = kNone;
         int64_t w = 0;
         if (e0 + lane < e1) {
@@ -222,7 +242,8 @@ move_kernel(int64_t nv, const int64_t *__restrict__ ip, const int32_t *__restric
             if (u != v && w != 0) c = comm[u];
         }
         bool leader;
-        const int64_t sc = label_sum(c, w, leader);
+        const int64_t sc = label_sum(c, w, (int)(e1 - e0), s_key[threadIdx.x >> 5],
+                                     reinterpret_cast<int64_t *>(s_sum[threadIdx.x >> 5]), leader);
         if (leader) {
             if (c == a) {
                 sa = sc;
@@ -234,8 +255,6 @@ move_kernel(int64_t nv, const int64_t *__restrict__ ip, const int32_t *__restric
     }
     // longer rows: a table in shared memory (up to 128 entries) or the
     // vertex's own table in global memory
-    __shared__ int32_t s_key[kWarps][kSmemSlots];
-    __shared__ u64 s_sum[kWarps][kSmemSlots];
     const int64_t deg = e1 - e0;
     const bool in_smem = deg > 32 && deg <= kSmemSlots / 2;
     int64_t len = 0;
@@ -339,7 +358,9 @@ pick_kernel(int64_t nv, const int64_t *__restrict__ ip, const int32_t *__restric
     const int64_t e0 = ip[v], e1 = ip[v + 1];
     i128 gb = 0;
     int32_t best = kNone;
-    if (e1 - e0 <= 32) {   // warp-uniform: sums in registers
+    __shared__ __align__(16) int32_t s_key[kWarps][kSmemSlots];
+    __shared__ __align__(16) u64 s_sum[kWarps][kSmemSlots];
+    if (e1 - e0 <= 32) {   // warp-uniform
         int32_t S = kNone;
         int64_t w = 0;
         if (e0 + lane < e1) {
@@ -348,7 +369,8 @@ pick_kernel(int64_t nv, const int64_t *__restrict__ ip, const int32_t *__restric
             if (u != v && w != 0 && comm[u] == C) S = ref[u];
         }
         bool leader;
-        const int64_t sS = label_sum(S, w, leader);
+        const int64_t sS = label_sum(S, w, (int)(e1 - e0), s_key[threadIdx.x >> 5],
+                                     reinterpret_cast<int64_t *>(s_sum[threadIdx.x >> 5]), leader);
         if (leader && S != own) {
             const int64_t rS = (int64_t)rtot[S];
             if ((i128)(int64_t)ext[S] * m2 * 65536 >= (i128)G * rS * (totC - rS)) {
@@ -360,8 +382,6 @@ pick_kernel(int64_t nv, const int64_t *__restrict__ ip, const int32_t *__restric
             }
         }
     }
-    __shared__ int32_t s_key[kWarps][kSmemSlots];
-    __shared__ u64 s_sum[kWarps][kSmemSlots];
     const int64_t deg = e1 - e0;
     const bool in_smem = deg > 32 && deg <= kSmemSlots / 2;
     int64_t len = 0;
@@ -471,31 +491,48 @@ agg_insert_kernel(int64_t nv, const int64_t *__restrict__ ip, const int32_t *__r
     }
 }
 
-// Warp per node: mode 0 counts the used slots, mode 1 writes them (in slot
-// order) to the aggregate's row and clears the table.
+// Warp per node: mode 0 counts the used slots, mode 1 writes them to the
+// aggregate's row (in any order: no decision depends on it) and clears the
+// table.  A long table is shared out over the block: one warp alone walks the
+// table of a node that a community has grown into for 120 us.
+constexpr int64_t kLongTable = 512;
 __global__ void __launch_bounds__(kBlock)
 agg_row_kernel(int64_t K, const int64_t *__restrict__ toff, int32_t *__restrict__ hkey, u64 *__restrict__ hsum,
                int mode, int64_t *__restrict__ cnt, const int64_t *__restrict__ nip, int32_t *__restrict__ ncol,
                int64_t *__restrict__ nwt) {
-    const int lane = threadIdx.x & 31;
-    const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (c >= K) return;
-    const int64_t T = toff[c], len = toff[c + 1] - T;
-    int64_t run = mode ? nip[c] : 0;
-    for (int64_t s0 = 0; s0 < len; s0 += 32) {
-        const int64_t s = s0 + lane;
-        const int32_t t = s < len ? __ldcg(hkey + T + s) : -1;
-        const unsigned b = __ballot_sync(0xffffffffu, t >= 0);
-        if (mode && t >= 0) {
-            const int64_t p = run + __popc(b & ((1u << lane) - 1u));
-            ncol[p] = t;
-            nwt[p] = (int64_t)__ldcg(hsum + T + s);
-            hkey[T + s] = -1;
-            hsum[T + s] = 0;
+    __shared__ int fill[kWarps];   // entries of a warp's node taken so far
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t c0 = (int64_t)blockIdx.x * kWarps;
+    // slots [s, s + 32 step) of node c's table, 32 a step; the warp takes its share of the row
+    auto walk = [&](int64_t c, int x, int64_t first, int64_t step) {
+        const int64_t T = toff[c], len = toff[c + 1] - T, row = mode ? nip[c] : 0;
+#pragma unroll 2
+        for (int64_t s0 = first; s0 < len; s0 += step) {
+            const int64_t s = s0 + lane;
+            const int32_t t = s < len ? __ldcg(hkey + T + s) : -1;
+            const unsigned b = __ballot_sync(0xffffffffu, t >= 0);
+            if (b == 0) continue;
+            int run = 0;
+            if (lane == 0) run = atomicAdd(&fill[x], __popc(b));
+            run = __shfl_sync(0xffffffffu, run, 0);
+            if (mode && t >= 0) {
+                const int64_t p = row + run + __popc(b & ((1u << lane) - 1u));
+                ncol[p] = t;
+                nwt[p] = (int64_t)__ldcg(hsum + T + s);
+                hkey[T + s] = -1;
+                hsum[T + s] = 0;
+            }
         }
-        run += __popc(b);
-    }
-    if (!mode && lane == 0) cnt[c] = run;
+    };
+    if (threadIdx.x < kWarps) fill[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t c = c0 + warp;
+    if (c < K && toff[c + 1] - toff[c] <= kLongTable) walk(c, warp, 0, 32);
+    for (int x = 0; x < kWarps && c0 + x < K; ++x)
+        if (toff[c0 + x + 1] - toff[c0 + x] > kLongTable) walk(c0 + x, x, 32 * warp, 32 * kWarps);
+    if (mode) return;
+    __syncthreads();
+    if (threadIdx.x < kWarps && c0 + threadIdx.x < K) cnt[c0 + threadIdx.x] = fill[threadIdx.x];
 }
 
 // ------------------------------------------------------------- output
