@@ -426,24 +426,40 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                 const int j0 = jb + sq.m * BN + cbeg;
                 const int valid = rag ? tail - cbeg : C::kCols;
                 if (Work::kStartBelow && first && !rag) {
-                    // first tile of empty lists: the largest of the kCols / 8
-                    // minima of 8 columns bounds the KCP-th smallest value from
-                    // above (kCols / 8 >= KCP distinct values lie at or below
-                    // it), so the lists start from that bound instead of +inf
-                    // and never take the larger values in
-                    float gmax = -INFINITY;
+                    // first tile of empty lists: the largest of G minima of groups
+                    // of columns bounds the G-th smallest value from above, so the
+                    // lists start from that bound instead of +inf and never take
+                    // the larger values in.  Groups as wide as leave G >= the
+                    // entries wanted: 8 columns (16 of 128), 4 (16 of 64) or 2 (64
+                    // of 128); short lists of kShort entries use minima of 8 (8 of
+                    // 64 or 16 of 128).
+                    constexpr int kWide = C::kCols / 8 >= KCP ? 8 : C::kCols / 4 >= KCP ? 4 : 2;
+                    static_assert(C::kCols / kWide >= KCP && C::kCols / 8 >= (Work::kShort > 0 ? Work::kShort : 1),
+                                  "enough groups");
+                    constexpr int kLoad = KCP >= 64 ? 16 : 32;   // long lists leave little register room
+                    // (a group of nothing but NaN counts as unbounded)
+                    float gmax = -INFINITY, gmax8 = -INFINITY;
+                    auto up = [](float g, float m) { return fmaxf(g, m == m ? m : INFINITY); };
 #pragma unroll 1
-                    for (int c0 = 0; c0 < C::kCols; c0 += 32) {
-                        float vv[32];
+                    for (int c0 = 0; c0 < C::kCols; c0 += kLoad) {
+                        float vv[kLoad];
                         __syncwarp();
-                        tc::tmem_ld32(tb + c0, vv);
+                        if constexpr (kLoad == 32) tc::tmem_ld32(tb + c0, vv);
+                        else tc::tmem_ld16(tb + c0, vv);
                         tc::tmem_wait_ld();
-                        float g[4];
 #pragma unroll
-                        for (int h = 0; h < 4; ++h) g[h] = min8(vv + 8 * h);
-                        gmax = fmaxf(gmax, fmaxf(fmaxf(g[0], g[1]), fmaxf(g[2], g[3])));
+                        for (int h = 0; h < kLoad / 8; ++h) {
+                            const float *x = vv + 8 * h;
+                            const float p0 = fminf(x[0], x[1]), p1 = fminf(x[2], x[3]), p2 = fminf(x[4], x[5]), p3 = fminf(x[6], x[7]);
+                            const float q0 = fminf(p0, p1), q1 = fminf(p2, p3), m = fminf(q0, q1);
+                            if constexpr (kWide == 2) gmax = up(up(up(up(gmax, p0), p1), p2), p3);
+                            if constexpr (kWide == 4) gmax = up(up(gmax, q0), q1);
+                            if constexpr (kWide == 8) gmax = up(gmax, m);
+                            if constexpr (Work::kShort > 0 && kWide < 8) gmax8 = up(gmax8, m);
+                        }
                     }
-                    if constexpr (C::kCols / 8 >= KCP) tk.start_below(gmax);
+                    if constexpr (Work::kShort > 0 && kWide < 8) gmax = wi.short_list ? gmax8 : gmax;
+                    tk.start_below(gmax);
                 }
                 if constexpr (C::kResident && Work::kHitHeavy) {
                     // 64 columns at a time held in registers: minima of 8, one
@@ -560,6 +576,31 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
     }
 }
 
+// The first N entries of a list to or from memory, 16 bytes at a time (lists
+// start on 16-byte boundaries): a thread's list is a run of its own, so every
+// store instruction of a warp touches 32 of them.
+template <int N>
+__device__ __forceinline__ void put_ids(int32_t *out, const int *id) {
+#pragma unroll
+    for (int c = 0; c < N; c += 4) *reinterpret_cast<int4 *>(out + c) = make_int4(id[c], id[c + 1], id[c + 2], id[c + 3]);
+}
+template <int N>
+__device__ __forceinline__ void put_keys(float *out, const float *key) {
+#pragma unroll
+    for (int c = 0; c < N; c += 4)
+        *reinterpret_cast<float4 *>(out + c) = make_float4(key[c], key[c + 1], key[c + 2], key[c + 3]);
+}
+template <int N>
+__device__ __forceinline__ void get_list(const float *keys, const int32_t *ids, float *key, int *id) {
+#pragma unroll
+    for (int c = 0; c < N; c += 4) {
+        const float4 k = *reinterpret_cast<const float4 *>(keys + c);
+        const int4 i = *reinterpret_cast<const int4 *>(ids + c);
+        key[c] = k.x; key[c + 1] = k.y; key[c + 2] = k.z; key[c + 3] = k.w;
+        id[c] = i.x; id[c + 1] = i.y; id[c + 2] = i.z; id[c + 3] = i.w;
+    }
+}
+
 // Whole-matrix work: query tile qt (BM rows) x database split sp.
 struct PlainWork {
     static constexpr int kShort = 0;   // never used (short_list is false)
@@ -600,9 +641,7 @@ struct PlainWork {
     }
     template <int EG, int KCP>
     __device__ __forceinline__ void emit(const WorkItem &w, int part, int64_t q, const RowTopK<KCP> &list) const {
-        int32_t *out = cand + ((int64_t)(w.tag * EG + part) * n + q) * KCP;
-#pragma unroll
-        for (int c = 0; c < KCP; ++c) out[c] = list.id[c];
+        put_ids<KCP>(cand + ((int64_t)(w.tag * EG + part) * n + q) * KCP, list.id);
     }
 };
 

@@ -64,13 +64,9 @@ struct BatchedWork {
     template <int EG, int KCP>
     __device__ __forceinline__ void emit(const WorkItem &w, int part, int64_t q, const RowTopK<KCP> &list) const {
         if (!w.short_list) {
-            int32_t *out = cand_w + ((int64_t)part * N + q) * KCP;
-#pragma unroll
-            for (int c = 0; c < KCP; ++c) out[c] = list.id[c];
+            put_ids<KCP>(cand_w + ((int64_t)part * N + q) * KCP, list.id);
         } else {
-            int32_t *out = cand_x + (((int64_t)q * S + w.tag) * EG + part) * kShort;
-#pragma unroll
-            for (int c = 0; c < kShort; ++c) out[c] = list.id[c];
+            put_ids<kShort>(cand_x + (((int64_t)q * S + w.tag) * EG + part) * kShort, list.id);
         }
     }
 };
@@ -128,18 +124,12 @@ struct BatchedWindowWork {
     __device__ __forceinline__ void emit(const WorkItem &w, int part, int64_t q, const RowTopK<KCP> &list) const {
         if (!w.short_list) {
             const int64_t base = ((int64_t)part * N + q) * KCP;
-#pragma unroll
-            for (int c = 0; c < KCP; ++c) {
-                st_w[base + c] = list.key[c];
-                cand_w[base + c] = list.id[c];
-            }
+            put_keys<KCP>(st_w + base, list.key);
+            put_ids<KCP>(cand_w + base, list.id);
         } else {
             const int64_t base = (((int64_t)q * S + w.tag) * EG + part) * kShort;
-#pragma unroll
-            for (int c = 0; c < kShort; ++c) {
-                st_x[base + c] = list.key[c];
-                cand_x[base + c] = list.id[c];
-            }
+            put_keys<kShort>(st_x + base, list.key);
+            put_ids<kShort>(cand_x + base, list.id);
         }
     }
 };
@@ -204,30 +194,18 @@ struct BatchedListWork {
     __device__ __forceinline__ void resume(const WorkItem &w, int part, int64_t q, RowTopK<KCP> &list) const {
         if (!w.short_list) {
             const int64_t base = ((int64_t)part * N + q) * KCP;
-#pragma unroll
-            for (int c = 0; c < KCP; ++c) {
-                list.key[c] = st_w[base + c];
-                list.id[c] = cand_w[base + c];
-            }
+            get_list<KCP>(st_w + base, cand_w + base, list.key, list.id);
         } else {
             const int64_t base = (((int64_t)q * S + w.tag) * EG + part) * kShort;
-#pragma unroll
-            for (int c = 0; c < kShort; ++c) {
-                list.key[c] = st_x[base + c];
-                list.id[c] = cand_x[base + c];
-            }
+            get_list<kShort>(st_x + base, cand_x + base, list.key, list.id);
         }
     }
     template <int EG, int KCP>
     __device__ __forceinline__ void emit(const WorkItem &w, int part, int64_t q, const RowTopK<KCP> &list) const {
         if (!w.short_list) {
-            int32_t *out = cand_w + ((int64_t)part * N + q) * KCP;
-#pragma unroll
-            for (int c = 0; c < KCP; ++c) out[c] = list.id[c];
+            put_ids<KCP>(cand_w + ((int64_t)part * N + q) * KCP, list.id);
         } else {
-            int32_t *out = cand_x + (((int64_t)q * S + w.tag) * EG + part) * kShort;
-#pragma unroll
-            for (int c = 0; c < kShort; ++c) out[c] = list.id[c];
+            put_ids<kShort>(cand_x + (((int64_t)q * S + w.tag) * EG + part) * kShort, list.id);
         }
     }
 };

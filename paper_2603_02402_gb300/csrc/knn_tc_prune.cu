@@ -56,11 +56,8 @@ struct WindowWork {
     template <int EG, int KCP>
     __device__ __forceinline__ void emit(const WorkItem &, int part, int64_t q, const RowTopK<KCP> &list) const {
         const int64_t base = (q * EG + part) * KCP;
-#pragma unroll
-        for (int c = 0; c < KCP; ++c) {
-            st_key[base + c] = list.key[c];
-            st_id[base + c] = list.id[c];
-        }
+        put_keys<KCP>(st_key + base, list.key);
+        put_ids<KCP>(st_id + base, list.id);
     }
 };
 
@@ -116,17 +113,11 @@ struct ListWork {
     template <int EG, int KCP>
     __device__ __forceinline__ void resume(const WorkItem &, int part, int64_t q, RowTopK<KCP> &list) const {
         const int64_t base = (q * EG + part) * KCP;
-#pragma unroll
-        for (int c = 0; c < KCP; ++c) {
-            list.key[c] = st_key[base + c];
-            list.id[c] = st_id[base + c];
-        }
+        get_list<KCP>(st_key + base, st_id + base, list.key, list.id);
     }
     template <int EG, int KCP>
     __device__ __forceinline__ void emit(const WorkItem &, int part, int64_t q, const RowTopK<KCP> &list) const {
-        int32_t *out = cand + ((int64_t)part * n + q) * KCP;
-#pragma unroll
-        for (int c = 0; c < KCP; ++c) out[c] = list.id[c];
+        put_ids<KCP>(cand + ((int64_t)part * n + q) * KCP, list.id);
     }
 };
 
