@@ -365,3 +365,14 @@ def test_ordered_search_of_rows_that_are_not_numbers(rsc, metric):
         assert (gi == -1).all()
     else:
         assert (gi[1:] > 0).all()
+
+
+@pytest.mark.parametrize("metric", ["euclidean", "cosine"])
+@pytest.mark.parametrize("n,d,k,cands", [(70, 50, 32, 96), (97, 5, 9, 128), (300, 50, 17, 70), (2049, 33, 31, 128)])
+def test_many_candidates_re_ranked(rsc, metric, n, d, k, cands):
+    # more than 64 candidates a row, merged 32 at a time; lists that are not
+    # full when there are fewer rows than candidates
+    X = synth.mixture(n, d, n_comp=4, seed=n)
+    oi, od, on = oracle.knn(X, k, metric=oracle.EUCLIDEAN if metric == "euclidean" else oracle.COSINE)
+    gi, gd = run_knn(rsc, X, k, metric=metric, precision="bf16", candidates=cands)
+    check_knn(X, gi, gd, oi, od, on, metric=metric, allow_miss=MISS["bf16"])
