@@ -215,6 +215,21 @@ struct BatchedListWork {
 namespace {
 
 constexpr int kXWarps = 4;
+constexpr int kXGroup = 256;   // candidates whose distances a warp holds: 16 samples of four parts, 32 of two
+
+// Floats of a staged row: an odd number of 16 bytes, so that the lanes' 16-byte
+// reads of their own rows share no bank.
+__host__ __device__ __forceinline__ int cross_step(int w4) { return 4 * (w4 | 1); }
+
+template <int E>
+size_t cross_smem(int w4) {
+    return kXWarps * sizeof(float) * (68 + (w4 > 0 ? 32 * cross_step(w4) : 0) + 2 * 32 * E + 2 * (kXGroup + 32));
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t to, const float *from) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(to), "l"(from) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // One warp per query position q (original row qo = perm[q], or q without a
 // permutation): for every sample, re-score its cross candidates exactly
@@ -223,6 +238,12 @@ constexpr int kXWarps = 4;
 // S * k_cross entries by (distance, id) with a register bitonic network
 // (E = L2 / 32 entries per lane).  Candidate ids are positions, mapped to
 // original rows through perm; R holds the rows by position when r_by_pos.
+//
+// 32 candidates at a time, which lie in a row: eight lanes copy a candidate's
+// row to shared memory (a lane that reads a row of its own touches 32 lines an
+// instruction, and those lookups were what the kernel waited for), then a lane
+// sums a row in order.  The distances of 32 samples are kept, and a lane picks
+// its sample's best.  600k rows, 32 samples, d = 50: 11.66 -> 9.55 ms.
 template <int E>
 __global__ void __launch_bounds__(kXWarps * 32)
 rerank_cross_kernel(const float *__restrict__ R, int64_t rs, int64_t N, int d, int metric, int w4,
@@ -230,15 +251,20 @@ rerank_cross_kernel(const float *__restrict__ R, int64_t rs, int64_t N, int d, i
                     const int32_t *__restrict__ perm, bool r_by_pos, const int32_t *__restrict__ idx_w,
                     const float *__restrict__ dist_w, int k_within, int k_cross, int parts,
                     int32_t *__restrict__ idx_x, float *__restrict__ dist_x) {
-    constexpr int L2 = 32 * E;
-    const int n_cand = parts * tck::BatchedWork::kShort;   // candidates per (query, sample)
-    __shared__ __align__(16) float xq_s[kXWarps][68];
-    __shared__ float rkey_s[kXWarps][L2];
-    __shared__ int rid_s[kXWarps][L2];
+    constexpr int L2 = 32 * E, kShort = tck::BatchedWork::kShort;
+    using u64 = unsigned long long;
+    constexpr u64 kNone = 0x7f8000007fffffffull;   // (+inf, INT_MAX)
+    const int sh = parts == 4 ? 4 : 3, n_cand = 1 << sh;   // candidates per (query, sample)
+    extern __shared__ __align__(16) uint8_t sm[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float *xq = xq_s[warp];
-    float *rkey = rkey_s[warp];
-    int *rid = rid_s[warp];
+    const int staged = w4 > 0 ? 32 * cross_step(w4) : 0;
+    float *xq = reinterpret_cast<float *>(sm) + warp * (68 + staged + 2 * L2 + 2 * (kXGroup + 32));
+    float *stage = xq + 68, *rkey = stage + staged;
+    int *rid = reinterpret_cast<int *>(rkey + L2);
+    u64 *pair = reinterpret_cast<u64 *>(rid + L2);   // sample s of the group, candidate c: s (n_cand + 1) + c
+    const uint32_t step = 4 * cross_step(w4);
+    const uint32_t put0 = (uint32_t)__cvta_generic_to_shared(stage) + (lane >> 3) * step + 16 * (lane & 7);
+    const bool lo8 = (lane & 7) < w4, hi8 = (lane & 7) + 8 < w4;
     const int64_t q = (int64_t)blockIdx.x * kXWarps + warp;
     if (q >= N) return;
     const int64_t qo = perm ? (int64_t)perm[q] : q;
@@ -260,48 +286,84 @@ rerank_cross_kernel(const float *__restrict__ R, int64_t rs, int64_t N, int d, i
     }
     __syncwarp();
     const bool fq = cosine && xq[d] != 0.f;
-    // two samples per pass: lanes 0-15 sample t, lanes 16-31 sample t + 1
-    // (lanes past n_cand hold +inf)
-    const int half = lane >> 4, hl = lane & 15;
-    for (int t0 = 0; t0 < S; t0 += 2) {
-        const int t = t0 + half;
-        float key = INFINITY;
-        int id = INT_MAX;
-        if (t < S && t != own && hl < n_cand) {
-            const int32_t jp = cand_x[((int64_t)q * S + t) * n_cand + hl];
-            if (jp >= 0 && (int64_t)jp < N) {   // ids outside [0, N) (an aborted search) are skipped
-                const int32_t j = perm ? perm[jp] : jp;
-                const float *yr = R + (int64_t)(r_by_pos ? jp : j) * rs;
-                float acc = row_dist2(xq, yr, d, w4);
-                if (cosine) {
-                    const bool fy = __ldg(yr + d) != 0.f;
-                    if (fq || fy) acc = (fq && fy) ? 0.f : 2.f;
-                }
-                key = cosine ? 0.5f * acc : sqrtf(acc);
-                id = j;
-            }
-        }
-        // sort each 16-lane half ascending by (key, id): bitonic over lanes
+    const int32_t *cand = cand_x + ((int64_t)q * S << sh);
+    for (int s0 = 0; s0 < S; s0 += kXGroup >> sh) {
+        const int group = min(kXGroup >> sh, S - s0), count = group << sh;
+        int32_t jp = cand[(s0 << sh) + min(lane, count - 1)];
+        for (int x0 = 0; x0 < count; x0 += 32) {
+            const int x = x0 + lane, t = s0 + (x >> sh);
+            // ids outside [0, N) (an aborted search) are skipped
+            const bool take = x < count && t != own && jp >= 0 && (int64_t)jp < N;
+            const int32_t p = take ? jp : (int32_t)q, j = perm ? perm[p] : p, row = r_by_pos ? p : j;
+            if (x0 + 32 < count) jp = cand[(s0 << sh) + min(x + 32, count - 1)];
+            float acc = 0.f;
+            if (w4 > 0) {
 #pragma unroll
-        for (int size = 2; size <= 16; size <<= 1) {
+                for (int r = 0; r < 8; ++r) {
+                    const float *y = R + (int64_t)__shfl_sync(0xffffffffu, row, r * 4 + (lane >> 3)) * rs + 4 * (lane & 7);
+                    if (lo8) cp_async16(put0 + r * 4 * step, y);
+                    if (hi8) cp_async16(put0 + r * 4 * step + 128, y + 32);
+                }
+                cp_async_wait();
+                __syncwarp();
+                const float4 *v4 = reinterpret_cast<const float4 *>(stage + lane * (step >> 2));
+                const float4 *q4 = reinterpret_cast<const float4 *>(xq);
+                int c = 0;
+#pragma unroll 4
+                for (; c < d >> 2; ++c) {
+                    const float4 v = v4[c], w = q4[c];
+                    float u = w.x - v.x;
+                    acc = fmaf(u, u, acc);
+                    u = w.y - v.y;
+                    acc = fmaf(u, u, acc);
+                    u = w.z - v.z;
+                    acc = fmaf(u, u, acc);
+                    u = w.w - v.w;
+                    acc = fmaf(u, u, acc);
+                }
+                for (c *= 4; c < d; ++c) {
+                    const float u = xq[c] - stage[lane * (step >> 2) + c];
+                    acc = fmaf(u, u, acc);
+                }
+                __syncwarp();
+            } else {
+                acc = row_dist2(xq, R + (int64_t)row * rs, d, 0);
+            }
+            if (cosine) {
+                const bool fy = __ldg(R + (int64_t)row * rs + d) != 0.f;
+                if (fq || fy) acc = (fq && fy) ? 0.f : 2.f;
+            }
+            // distances are not negative, so that their bits order as they do
+            // (NaN last, after the empty places)
+            if (x < count)
+                pair[x + (x >> sh)] =
+                    take ? (u64)__float_as_uint(cosine ? 0.5f * acc : sqrtf(acc)) << 32 | (uint32_t)j : kNone;
+        }
+        __syncwarp();
+        const int t = s0 + lane;
+        if (lane < group && t != own) {
+            u64 best[kShort];
 #pragma unroll
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                const float ok = __shfl_xor_sync(0xffffffffu, key, stride);
-                const int oi = __shfl_xor_sync(0xffffffffu, id, stride);
-                const bool up = (hl & size) == 0;          // this block sorts ascending
-                const bool lower = (hl & stride) == 0;     // this lane is the lower of the pair
-                const bool keep_min = (lower == up);
-                const bool take = keep_min ? pair_gt(key, id, ok, oi) : pair_gt(ok, oi, key, id);
-                if (take) {
-                    key = ok;
-                    id = oi;
+            for (int c = 0; c < kShort; ++c) best[c] = kNone;
+#pragma unroll 4
+            for (int c = 0; c < n_cand; ++c) {
+                u64 v = pair[lane * (n_cand + 1) + c];
+#pragma unroll
+                for (int i = 0; i < kShort; ++i) {
+                    const bool less = v < best[i];
+                    const u64 o = best[i];
+                    best[i] = less ? v : o;
+                    v = less ? o : v;
                 }
             }
+#pragma unroll
+            for (int c = 0; c < kShort; ++c)
+                if (c < k_cross) {
+                    rkey[t * k_cross + c] = __uint_as_float((uint32_t)(best[c] >> 32));
+                    rid[t * k_cross + c] = (int)(uint32_t)best[c];
+                }
         }
-        if (t < S && t != own && hl < k_cross) {
-            rkey[t * k_cross + hl] = key;
-            rid[t * k_cross + hl] = id;
-        }
+        __syncwarp();
     }
     // own sample: the first k_cross of the exact within list
     for (int c = lane; c < k_cross; c += 32) {
@@ -427,9 +489,12 @@ cudaError_t launch_rerank_cross(const float *R, int64_t rs, int64_t N, int d, in
     const unsigned blocks = (unsigned)ceil_div(N, kXWarps);
 #define RSC_RX(e)                                                                                                 \
     case 32 * e:                                                                                                  \
-        rerank_cross_kernel<e><<<blocks, kXWarps * 32, 0, st>>>(R, rs, N, d, metric, w4, b.samp_off, S, cand_x, \
-                                                                perm, r_by_pos, idx_w, dist_w, k_within, k_cross, \
-                                                                parts, idx_x, dist_x);                            \
+        if (cudaFuncSetAttribute(rerank_cross_kernel<e>, cudaFuncAttributeMaxDynamicSharedMemorySize,             \
+                                 (int)cross_smem<e>(w4)) != cudaSuccess)                                          \
+            return cudaGetLastError();                                                                            \
+        rerank_cross_kernel<e><<<blocks, kXWarps * 32, cross_smem<e>(w4), st>>>(                                  \
+            R, rs, N, d, metric, w4, b.samp_off, S, cand_x, perm, r_by_pos, idx_w, dist_w, k_within, k_cross,     \
+            parts, idx_x, dist_x);                                                                                \
         break
     switch (L2) {
         RSC_RX(1); RSC_RX(2); RSC_RX(4); RSC_RX(8); RSC_RX(16); RSC_RX(32);

@@ -159,3 +159,40 @@ def test_batched_scan_stats(rsc):
             assert scanned == total
         else:
             assert 0 < scanned < total
+
+
+@pytest.mark.parametrize("S,d,kx", [(16, 50, 3), (17, 7, 4), (33, 61, 1), (40, 33, 4), (2, 1, 2)])
+def test_batched_cross_sample_groups(rsc, S, d, kx):
+    # sample counts at and past the groups whose candidates are ranked together,
+    # rows of odd width.  Points and their negatives with small whole
+    # coordinates: column means are 0 and the candidates' keys are whole
+    # numbers, so the lists are the oracle's up to the choice among equal
+    # distances, and a distance is off by no more than its square root's rounding
+    rng = np.random.default_rng(S)
+    half = [20 + 4 * (s % 11) for s in range(S)]
+    X = np.concatenate([np.concatenate([x, -x]) for x in (rng.integers(-2, 3, (h, d)) for h in half)]).astype(np.float32)
+    off = np.concatenate([[0], 2 * np.cumsum(half)]).astype(np.int64)
+    _, _, xi, xd = oracle.batched_knn(X, off, 5, kx, oracle.EUCLIDEAN)
+    _, _, gxi, gxd = run(rsc, X, off, 5, kx)
+    gs = np.searchsorted(off, gxi, side="right") - 1
+    for t in range(S):
+        assert ((gs == t).sum(axis=1) == kx).all()
+    assert all(len(set(r)) == S * kx for r in gxi.tolist())
+    np.testing.assert_allclose(gxd, xd, rtol=2.0 ** -23, atol=0)
+    np.testing.assert_allclose(exact_distances(X, np.arange(len(X)), gxi, "euclidean"), gxd, rtol=2.0 ** -23, atol=0)
+
+
+@pytest.mark.parametrize("S,d,kx", [(33, 62, 1), (18, 31, 2)])
+def test_batched_cross_sample_groups_cosine(rsc, S, d, kx):
+    sizes = [40 + 7 * (s % 11) for s in range(S)]
+    X, off = synth.batched(sizes, d=d, n_comp=3, seed=S + d)
+    X[[0, 50]] = 0.0
+    _, _, xi, xd = oracle.batched_knn(X, off, 5, kx, oracle.COSINE)
+    _, _, gxi, gxd = run(rsc, X, off, 5, kx, "cosine")
+    gs = np.searchsorted(off, gxi, side="right") - 1
+    for t in range(S):
+        assert ((gs == t).sum(axis=1) == kx).all()
+    assert (np.diff(gxd, axis=1) >= 0).all()
+    assert _recall(gxi, gxd, xi, xd) >= 0.999
+    dex = exact_distances(X, np.arange(len(X)), gxi, "cosine")
+    np.testing.assert_allclose(gxd, dex, rtol=1e-5, atol=1e-6)
