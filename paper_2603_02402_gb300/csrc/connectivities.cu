@@ -133,6 +133,19 @@ __device__ __forceinline__ int count_below(const int *s, int x) {
     return p + (s[p] < x ? 1 : 0);
 }
 
+// Number of entries below x among s[0 .. N), in any order (16-byte aligned, N a
+// multiple of four; INT_MAX pads count for no x).
+template <int N>
+__device__ __forceinline__ int count_less(const int *s, int x) {
+    int c = 0;
+#pragma unroll
+    for (int t = 0; t < N / 4; ++t) {
+        const int4 v = reinterpret_cast<const int4 *>(s)[t];
+        c += (v.x < x) + (v.y < x) + (v.z < x) + (v.w < x);
+    }
+    return c;
+}
+
 // ---------------------------------------------------------------- smooth
 
 // 2^x by the ex2.approx.ftz.f32 instruction (PTX ISA; relative error about
@@ -230,14 +243,19 @@ smooth_row_kernel(const float *__restrict__ dist, int64_t n, int k, float2 *__re
 // every valid edge takes a bucket slot of its target (entries with weight 0
 // fill their slot and are dropped by the match pass); pushes past B with a
 // non-zero weight set bit c of ovf[i]; the non-zero own entries sorted by
-// column across the group into ocol / og.  Few registers per lane, so many
-// rows' atomics are in flight at once.
+// column across the group into ocol / og, by counting the smaller columns
+// through shared memory (eight 16-byte reads and 64 compares for 32 lanes; the
+// 15 exchange steps of a sort were a third of the kernel's instructions).  Few
+// registers per lane, so many rows' atomics are in flight at once.  300k rows,
+// k = 30: 158 -> 131 us, now the latency of the scattered pushes; 1M rows,
+// k = 15: 302 -> 298 us.
 template <int G>
 __global__ void __launch_bounds__(kThreads)
 push_group_kernel(const int32_t *__restrict__ idx, const float *__restrict__ dist, int64_t n, int k, int KP, int B,
                   const float2 *__restrict__ rs, int32_t *__restrict__ in_cnt, int2 *__restrict__ bucket,
                   uint32_t *__restrict__ ovf, int32_t *__restrict__ ocol, float *__restrict__ og,
                   int32_t *__restrict__ own_cnt) {
+    __shared__ __align__(16) int s_key[kThreads];
     const int lane = threadIdx.x & 31, l = lane & (G - 1), base = lane & ~(G - 1);
     const unsigned gbits = (G == 32) ? 0xffffffffu : ((1u << G) - 1);
     const int64_t i = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32 / G) + lane / G;
@@ -245,17 +263,15 @@ push_group_kernel(const int32_t *__restrict__ idx, const float *__restrict__ dis
     const int me = (int)i;
     int j = -1;
     float d = 0.f;
+    float2 ri = make_float2(0.f, 0.f);
     if (row_ok && l < k) {
         const int32_t jj = idx[i * k + l];
         d = dist[i * k + l];
+        ri = rs[i];
         if (jj >= 0 && (int64_t)jj < n && jj != me) j = jj;
     }
     const int slot = (j >= 0) ? atomicAdd(in_cnt + j, 1) : 0;
-    float a = 0.f;
-    if (j >= 0) {
-        const float2 ri = rs[i];
-        a = directed_weight(d, ri.x, ri.y);
-    }
+    const float a = (j >= 0) ? directed_weight(d, ri.x, ri.y) : 0.f;
     bool spill = false;
     if (j >= 0) {
         if (slot < B) bucket[(int64_t)j * B + slot] = make_int2(me, __float_as_int(a));
@@ -265,11 +281,22 @@ push_group_kernel(const int32_t *__restrict__ idx, const float *__restrict__ dis
     float val[1] = {a};
     const unsigned own = (__ballot_sync(0xffffffffu, key[0] != INT_MAX) >> base) & gbits;
     const unsigned sp = (__ballot_sync(0xffffffffu, spill) >> base) & gbits;
-    group_bitonic<G, 1>(key, val, l);
+    // an entry's place is the number of smaller columns; the places of distinct
+    // columns sum to c (c - 1) / 2, and rows with a column twice are sorted
+    s_key[threadIdx.x] = key[0];
+    __syncwarp();
+    const int c = __popc(own);
+    int at = count_less<G>(s_key + (threadIdx.x & ~(G - 1)), key[0]);
+    if (key[0] == INT_MAX) at = c + __popc(~own & ((1u << l) - 1u));
+    const int off = __reduce_add_sync(0xffffffffu, key[0] != INT_MAX ? 2 * at - (c - 1) : 0);
+    if (off != 0) {   // uniform
+        group_bitonic<G, 1>(key, val, l);
+        at = l;
+    }
     if (row_ok) {
-        if (l < KP) {
-            ocol[i * KP + l] = key[0];
-            og[i * KP + l] = val[0];
+        if (at < KP) {   // pads too: whole sectors
+            ocol[i * KP + at] = key[0];
+            og[i * KP + at] = val[0];
         }
         if (l == 0) {
             own_cnt[i] = __popc(own);
@@ -426,20 +453,28 @@ match_kernel(const int32_t *__restrict__ idx, const float *__restrict__ dist, in
     const unsigned gmask = gbits << base;
     const int64_t i = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * GPW + grp;
     const bool row_ok = i < n;
+    const int32_t *orow = ocol + (size_t)(row_ok ? i : 0) * KP;
+    float *grow = og + (size_t)(row_ok ? i : 0) * KP;
+    int2 *brow = bucket + (size_t)(row_ok ? i : 0) * B;
+    // the first places are read before the counts are known
     int oc = 0, ic = 0;
     if (row_ok) {
         oc = own_cnt[i];
         ic = min(in_cnt[i], B);
     }
-    const int32_t *orow = ocol + (size_t)(row_ok ? i : 0) * KP;
-    float *grow = og + (size_t)(row_ok ? i : 0) * KP;
-    int2 *brow = bucket + (size_t)(row_ok ? i : 0) * B;
+    int col[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int x = e * G + l;
+        col[e] = (x < KP) ? orow[x] : INT_MAX;
+    }
+    const int2 first = brow[l];
     int *so = s_own[warp][grp];
     float *sh = s_hit[warp][grp];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int x = e * G + l;
-        so[x] = (x < oc) ? orow[x] : INT_MAX;
+        so[x] = (x < oc) ? col[e] : INT_MAX;
         sh[x] = 0.f;
     }
     int src[NB];
@@ -450,7 +485,7 @@ match_kernel(const int32_t *__restrict__ idx, const float *__restrict__ dist, in
         src[e] = INT_MAX;
         wa[e] = 0.f;
         if (q < ic) {
-            const int2 t = brow[q];
+            const int2 t = e == 0 ? first : brow[q];
             src[e] = t.x;
             wa[e] = __int_as_float(t.y);
         }
@@ -630,9 +665,9 @@ __device__ __forceinline__ void put(int32_t *indices, float *data, int64_t p, in
 }
 
 // G lanes per row.  A row without flagged entries: its kept bucket entries
-// (at most B = NB G, NB per lane) are ranked by counting (rank = entries with
-// a smaller source), written to shared memory in order, and each own and
-// bucket entry is placed at its rank in the union.  A row with flagged
+// (at most B = NB G, NB per lane) go to shared memory, and each own and bucket
+// entry is placed at its rank in the union: the bucket entries below it, by
+// counting, plus the own ones (its position, or a binary search).  A row with flagged
 // entries gets its own and bucket entries written unsorted and is queued for
 // a whole-row sort; its flagged entries are placed by their source rows,
 // after its bucket entries.
@@ -649,11 +684,14 @@ emit_kernel(int64_t n, int k, int KP, int B, int MW, const int32_t *__restrict__
     constexpr int GPW = 32 / G;   // rows per warp
     static_assert(NB >= 2, "the bucket holds at least the 2G entries a row merges in registers");
     __shared__ int s_own[kThreads / 32][GPW][G * E];
-    __shared__ int s_in[kThreads / 32][GPW][2 * G];
+    __shared__ __align__(16) int s_in[kThreads / 32][GPW][2 * G];
     const int lane = threadIdx.x & 31, l = lane & (G - 1), grp = lane / G, warp = threadIdx.x >> 5;
     const int base = grp * G;
     const int64_t i = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * GPW + grp;
     const bool row_ok = i < n;
+    const int32_t *orow = ocol + (size_t)(row_ok ? i : 0) * KP;
+    const float *grow = og + (size_t)(row_ok ? i : 0) * KP;
+    const int2 *brow = bucket + (size_t)(row_ok ? i : 0) * B;
     int64_t start = 0;
     int oc = 0, ic = 0, ex = 0;
     if (row_ok) {
@@ -663,17 +701,19 @@ emit_kernel(int64_t n, int k, int KP, int B, int MW, const int32_t *__restrict__
         ex = extra[i];
         if (l == 0) indptr[i] = start;
     }
-    const int32_t *orow = ocol + (size_t)(row_ok ? i : 0) * KP;
-    const float *grow = og + (size_t)(row_ok ? i : 0) * KP;
-    const int2 *brow = bucket + (size_t)(row_ok ? i : 0) * B;
+    // the first places are read before the counts are known
     int col[E];
     float gv[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int x = e * G + l;
-        col[e] = (x < oc) ? orow[x] : INT_MAX;
-        gv[e] = (x < oc) ? grow[x] : 0.f;
+        col[e] = (x < KP) ? orow[x] : INT_MAX;
+        gv[e] = (x < KP) ? grow[x] : 0.f;
     }
+    const int2 first = brow[l];
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (e * G + l >= oc) col[e] = INT_MAX;
     int src[NB];
     float wa[NB];
 #pragma unroll
@@ -682,7 +722,7 @@ emit_kernel(int64_t n, int k, int KP, int B, int MW, const int32_t *__restrict__
         src[e] = INT_MAX;
         wa[e] = 0.f;
         if (q < ic) {
-            const int2 t = brow[q];
+            const int2 t = e == 0 ? first : brow[q];
             src[e] = t.x;
             wa[e] = __int_as_float(t.y);
         }
@@ -707,34 +747,32 @@ emit_kernel(int64_t n, int k, int KP, int B, int MW, const int32_t *__restrict__
             else long_rows[atomicAdd(long_count, 1)] = (int32_t)i;
         }
     }
-    // ranks of the bucket entries (pads are INT_MAX and never below a key);
-    // merged rows hold at most 2G of them, in src[0 .. 2)
-    const int icmax = __reduce_max_sync(0xffffffffu, hub ? 0 : ic);
-    int rk[NB];
-#pragma unroll
-    for (int e = 0; e < NB; ++e) rk[e] = 0;
-    for (int t = 0; t < icmax; ++t) {
-        const int v = __shfl_sync(0xffffffffu, t < G ? src[0] : src[1], base + (t & (G - 1)));
-        rk[0] += v < src[0];
-        rk[1] += v < src[1];
-    }
+    // places of the own and bucket entries among the bucket entries, by counting
+    // (merged rows hold at most 2G of these, in src[0 .. 2); pads are INT_MAX
+    // and never below a key; sources are distinct)
     int *so = s_own[warp][grp];
     int *si = s_in[warp][grp];
 #pragma unroll
     for (int e = 0; e < E; ++e) so[e * G + l] = col[e];
-    // position p < ic holds the entry of rank p, p >= ic a pad (ranks are a
-    // permutation of [0, ic): sources are distinct)
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        const int q = e * G + l;
-        si[(!hub && q < ic) ? rk[e] : q] = src[e];
-    }
+    for (int e = 0; e < 2; ++e) si[e * G + l] = src[e];
+    const int icmax = __reduce_max_sync(0xffffffffu, hub ? 0 : ic);
     __syncwarp();
+    int ro[E], rk[2] = {0, 0};
+#pragma unroll
+    for (int e = 0; e < E; ++e) ro[e] = 0;
+    for (int t = 0; t < icmax; t += 4) {
+        const int4 v = *reinterpret_cast<const int4 *>(si + t);
+#pragma unroll
+        for (int e = 0; e < E; ++e) ro[e] += (v.x < col[e]) + (v.y < col[e]) + (v.z < col[e]) + (v.w < col[e]);
+        rk[0] += (v.x < src[0]) + (v.y < src[0]) + (v.z < src[0]) + (v.w < src[0]);
+        if (icmax > G) rk[1] += (v.x < src[1]) + (v.y < src[1]) + (v.z < src[1]) + (v.w < src[1]);
+    }
     if (row_ok && !hub) {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int x = e * G + l;
-            if (x < oc) put(indices, data, start + x + count_below<2 * G>(si, col[e]), col[e], gv[e]);
+            if (x < oc) put(indices, data, start + x + ro[e], col[e], gv[e]);
         }
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
@@ -806,34 +844,82 @@ __device__ __forceinline__ int ceil_log2(int L) {
     return lp;
 }
 
-// Warp per queued row of up to kWarpSortMax entries, in shared memory.
+// Number of entries below x in the ascending run s[0 .. len).
+__device__ __forceinline__ int run_below(const int *s, int len, int x) {
+    int lo = 0;
+    while (len > 0) {
+        const int half = len >> 1;
+        if (s[lo + half] < x) {
+            lo += half + 1;
+            len -= half + 1;
+        } else {
+            len = half;
+        }
+    }
+    return lo;
+}
+
+// Warp per queued row of up to kWarpSortMax entries, in shared memory: the own
+// entries are an ascending run, the pushed ones in any order.  Up to kMergeMax
+// of these, an entry's place is the own entries below it (its position, or a
+// binary search) plus the pushed entries below it, by counting; the places of
+// distinct columns sum to L (L - 1) / 2, and a row where they do not, or with
+// more pushed entries, is sorted whole (the network's 28 to 45 steps through
+// shared memory cost a row of 100 to 200 entries about twice as much).
+// 300k rows, k = 30: 111 us sorting every row whole, 81 us so.
+constexpr int kMergeMax = 256;
+
 __global__ void __launch_bounds__(kSortWarps * 32)
 sort_mid_rows_kernel(const int64_t *__restrict__ indptr, int32_t *__restrict__ indices, float *__restrict__ data,
-                     int64_t cap, const int32_t *__restrict__ mid_rows, const int32_t *__restrict__ mid_count) {
+                     int64_t cap, const int32_t *__restrict__ own_cnt,
+                     const int32_t *__restrict__ mid_rows, const int32_t *__restrict__ mid_count) {
     __shared__ int s_col[kSortWarps][kWarpSortMax];
     __shared__ float s_w[kSortWarps][kWarpSortMax];
+    __shared__ __align__(16) int s_ex[kSortWarps][kMergeMax];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cnt = *mid_count;
-    int *sc = s_col[warp];
+    int *sc = s_col[warp], *se = s_ex[warp];
     float *sv = s_w[warp];
     for (int r = blockIdx.x * kSortWarps + warp; r < cnt; r += gridDim.x * kSortWarps) {
         const int64_t i = mid_rows[r];
         const int64_t b = indptr[i];
         const int L = (int)(indptr[i + 1] - b);
         if (b + L > cap) continue;   // capacity error already recorded
+        const int oc = own_cnt[i], x = L - oc;
         for (int t = lane; t < L; t += 32) {
             sc[t] = indices[b + t];
             sv[t] = data[b + t];
         }
         __syncwarp();
-        mirrored_bitonic(
-            L, ceil_log2(L), lane, 32,
-            [&](int x, int &c, float &w) { c = sc[x]; w = sv[x]; },
-            [&](int x, int c, float w) { sc[x] = c; sv[x] = w; },
-            [] { __syncwarp(); });
-        for (int t = lane; t < L; t += 32) {
-            indices[b + t] = sc[t];
-            data[b + t] = sv[t];
+        bool sorted = false;
+        if (x <= kMergeMax) {   // uniform
+            for (int t = lane; t < (x + 3 & ~3); t += 32) se[t] = t < x ? sc[oc + t] : INT_MAX;
+            __syncwarp();
+            int off = 0;
+            for (int t = lane; t < L; t += 32) {
+                const int v = sc[t];
+                int at = 0;
+                for (int u = 0; u < x; u += 4) {
+                    const int4 w = *reinterpret_cast<const int4 *>(se + u);
+                    at += (w.x < v) + (w.y < v) + (w.z < v) + (w.w < v);
+                }
+                at += t < oc ? t : run_below(sc, oc, v);
+                off += 2 * at - (L - 1);
+                indices[b + at] = v;
+                data[b + at] = sv[t];
+            }
+            sorted = __reduce_add_sync(0xffffffffu, off) == 0;
+        }
+        if (!sorted) {
+            mirrored_bitonic(
+                L, ceil_log2(L), lane, 32,
+                [&](int x, int &c, float &w) { c = sc[x]; w = sv[x]; },
+                [&](int x, int c, float w) { sc[x] = c; sv[x] = w; },
+                [] { __syncwarp(); });
+            for (int t = lane; t < L; t += 32) {
+                indices[b + t] = sc[t];
+                data[b + t] = sv[t];
+            }
         }
         __syncwarp();
     }
@@ -968,8 +1054,8 @@ cudaError_t launch_conn_fill(const int32_t *idx, const float *dist, int64_t n, i
     else if (k <= 64) launch_emit<32, 2>(idx, dist, n, k, s, indptr, indices, data, cap, w, st);
     else if (k <= 128) launch_emit<32, 4>(idx, dist, n, k, s, indptr, indices, data, cap, w, st);
     else launch_emit<32, 8>(idx, dist, n, k, s, indptr, indices, data, cap, w, st);
-    sort_mid_rows_kernel<<<sm_count() * 4, kSortWarps * 32, 0, st>>>(indptr, indices, data, cap, w.mid_rows,
-                                                                    w.mid_count);
+    sort_mid_rows_kernel<<<sm_count() * 4, kSortWarps * 32, 0, st>>>(indptr, indices, data, cap, w.own_cnt,
+                                                                    w.mid_rows, w.mid_count);
     sort_long_rows_kernel<<<sm_count() * 2, 1024, 0, st>>>(indptr, indices, data, cap, w.long_rows, w.long_count);
     return cudaGetLastError();
 }

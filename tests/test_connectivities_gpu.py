@@ -183,3 +183,26 @@ def test_full_size_graph_1m(rsc):
     st = assert_parity(rsc, i.astype(np.int32), d.astype(np.float32))
     print("1M graph", st)
     assert st["near_branch"] < 0.2 * len(X)
+
+
+@pytest.mark.parametrize("k", [5, 15, 16, 17, 30, 32])
+@pytest.mark.parametrize("degrees", [(3, 31, 32, 33, 60), (63, 64, 65, 66, 90), (200, 256, 271, 300), (400, 480, 512, 530)])
+def test_rows_with_many_sources(rsc, k, degrees):
+    # row h is listed by degrees[h] other rows, at the edges of the bucket, of
+    # the counted merge and of the row sort; half of the hubs' own neighbours
+    # list them back.  Same bounds as for random lists.
+    rng = np.random.default_rng(k + degrees[0])
+    n, hubs = 2000, len(degrees)
+    idx = np.empty((n, k), dtype=np.int32)
+    idx[:, 0] = np.arange(n)
+    for i in range(n):
+        idx[i, 1:] = hubs + rng.choice(n - hubs - 1, k - 1, replace=False)
+        idx[i, 1:] += (idx[i, 1:] >= i) if i >= hubs else 0
+    for h, m in enumerate(degrees):
+        back = idx[h, 1:1 + (k - 1) // 2]
+        others = np.setdiff1d(np.arange(hubs, n), idx[h, 1:])
+        rows = np.concatenate([back, rng.choice(others, m - len(back), replace=False)]) if m > len(back) else back[:m]
+        idx[rows, 1 + h % (k - 1)] = h
+    dist = np.sort(rng.uniform(0.5, 3.0, (n, k)).astype(np.float32), axis=1)
+    dist[:, 0] = 0.0
+    graph_parity(gpu_conn(rsc, idx, dist), idx, dist)
