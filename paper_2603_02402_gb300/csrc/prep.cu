@@ -56,35 +56,51 @@ colsum_partials_kernel(const float *__restrict__ X, int64_t n, int d, float *__r
     if (g == 0 && c < d) part[(int64_t)blockIdx.x * 64 + c] = (red[0][c] + red[1][c]) + (red[2][c] + red[3][c]);
 }
 
-// Thread (g, c) adds column c of partials g, g + 4, ... with Kahan
-// compensation; the four sums are added in a fixed order.  The chain of
-// additions is short next to the loads' latency, so 38 partials are fetched
-// ahead of it (1,216 partials: 22.7 us with a load per step, 14.5 us so).
-__global__ void __launch_bounds__(256) colmean_final_kernel(const float *__restrict__ part, int nb, int64_t n,
-                                                            int d, float *__restrict__ mu) {
-    __shared__ float red[4][64];
-    const int g = threadIdx.x >> 6, c = threadIdx.x & 63;
-    float s = 0.f, comp = 0.f;
-    if (c < d) {
-        constexpr int kAhead = 38;
-        for (int b0 = g; b0 < nb; b0 += 4 * kAhead) {
-            float v[kAhead];
+// Column means from the partials of nb blocks, of which the first nb_rows had
+// rows (the others hold 0): four columns per block, whose partials are fetched
+// at once; thread (g, c) adds partials g, g + 4, ... of a column with Kahan
+// compensation, and the four sums are added in a fixed order.  What is left is
+// the chain of 304 compensated additions (16 cycles each, 2.5 us): 1,216
+// partials x 50 columns 14.5 us with one block that fetched 38 of a thread's
+// partials at a time, 6.0 us so.
+constexpr int kMeanCols = 4;
+
+__global__ void __launch_bounds__(256) colmean_final_kernel(const float *__restrict__ part, int nb, int nb_rows,
+                                                            int64_t n, int d, float *__restrict__ mu) {
+    __shared__ float4 p[kColBlocks];
+    __shared__ float red[4][kMeanCols];
+    const int c0 = blockIdx.x * kMeanCols;
 #pragma unroll
-            for (int u = 0; u < kAhead; ++u) v[u] = b0 + 4 * u < nb ? part[(b0 + 4 * u) * 64 + c] : 0.f;
-#pragma unroll
-            for (int u = 0; u < kAhead; ++u) {
-                if (b0 + 4 * u < nb) {
-                    const float y = v[u] - comp;
-                    const float t = s + y;
-                    comp = (t - s) - y;
-                    s = t;
-                }
-            }
-        }
+    for (int u = 0; u < (kColBlocks + 255) / 256; ++u) {
+        const int b = u * 256 + threadIdx.x;
+        if (b < nb_rows) p[b] = *reinterpret_cast<const float4 *>(part + (int64_t)b * 64 + c0);
     }
-    red[g][c] = s - comp;
     __syncthreads();
-    if (g == 0 && c < d) mu[c] = (float)((double)((red[0][c] + red[1][c]) + (red[2][c] + red[3][c])) / (double)n);
+    const int g = threadIdx.x >> 2, c = threadIdx.x & 3;
+    if (g < 4) {
+        const float *col = reinterpret_cast<const float *>(p) + c;
+        float s = 0.f, comp = 0.f;
+        int b = g;
+#pragma unroll 8
+        for (; b < nb_rows; b += 4) {
+            const float y = col[4 * b] - comp;
+            const float t = s + y;
+            comp = (t - s) - y;
+            s = t;
+        }
+        for (; b < nb; b += 4) {   // a partial of 0; until one changes nothing
+            const float y = 0.f - comp;
+            const float t = s + y;
+            const float next = (t - s) - y;
+            if (t == s && next == comp) break;
+            comp = next;
+            s = t;
+        }
+        red[g][c] = s - comp;
+    }
+    __syncthreads();
+    if (g == 0 && c0 + c < d)
+        mu[c0 + c] = (float)((double)((red[0][c] + red[1][c]) + (red[2][c] + red[3][c])) / (double)n);
 }
 
 // A warp stages 32 consecutive rows (contiguous in X) through shared memory so
@@ -175,7 +191,9 @@ cudaError_t launch_prep_fp32(const float *X, int64_t n, int d, int DP, int metri
     float *mu = scratch + (size_t)kColBlocks * 64;
     if (metric == RSC_EUCLIDEAN) {
         colsum_partials_kernel<<<kColBlocks, 256, 0, st>>>(X, n, d, scratch);
-        colmean_final_kernel<<<1, 256, 0, st>>>(scratch, kColBlocks, n, d, mu);
+        const int64_t chunk = ceil_div(ceil_div(n, kColBlocks), 4) * 4;   // rows per block (colsum_partials_kernel)
+        colmean_final_kernel<<<(unsigned)ceil_div(d, kMeanCols), 256, 0, st>>>(
+            scratch, kColBlocks, (int)ceil_div(n, chunk), n, d, mu);
     }
     const int64_t rows_per_block = (int64_t)kWarps * kRowsPerWarp;
     const int64_t blocks = ceil_div(n, rows_per_block);
