@@ -184,6 +184,7 @@ strength_kernel(int64_t nv, const int64_t *__restrict__ ip, const int64_t *__res
         k[v] = s;
         tlen[v] = table_len(ip[v + 1] - ip[v]);
         if (s) atomicAdd(m2 + (blockIdx.x & (kCounters - 1)), (u64)s);
+        if (v == nv - 1) m2[kCounters] = (u64)ip[nv];   // the second set: entries of the level
     }
 }
 
@@ -588,7 +589,7 @@ using ldn::u64;
 
 struct LdLayout {
     unsigned int *status;
-    u64 *cnt;                        // kCounters spread counters
+    u64 *cnt;                        // kBanks sets of kCounters spread counters
     int64_t *ssum;                   // scan scratch
     int64_t *ip0, *wt0;              // level-0 graph (weights in fixed point)
     int32_t *col0;
@@ -603,12 +604,14 @@ struct LdLayout {
     int64_t hcap;
 };
 
+constexpr int kBanks = 2;   // sets of spread counters
+
 LdLayout carve_leiden(void *ws, int64_t n, int64_t nnz, size_t *bytes) {
     Carve cv(ws);
     LdLayout L;
     const size_t N = (size_t)n, E = (size_t)std::max<int64_t>(nnz, 1);
     L.status = cv.take<unsigned int>(kStatusBytes / sizeof(unsigned int));
-    L.cnt = cv.take<u64>(ldn::kCounters);
+    L.cnt = cv.take<u64>(kBanks * ldn::kCounters);
     L.ssum = cv.take<int64_t>(seg_scan::kMaxSegs);
     L.ip0 = cv.take<int64_t>(N + 1);
     L.col0 = cv.take<int32_t>(E);
@@ -646,15 +649,18 @@ LdLayout carve_leiden(void *ws, int64_t n, int64_t nnz, size_t *bytes) {
     return L;
 }
 
-// Sum of the spread counters (synchronises the stream), then clears them.
-rsc_status read_counter(const LdLayout &L, cudaStream_t st, u64 *out) {
-    u64 h[ldn::kCounters];
-    RSC_CUDA_TRY(cudaMemcpyAsync(h, L.cnt, sizeof h, cudaMemcpyDeviceToHost, st));
+// Sums of `banks` sets of spread counters (synchronises the stream), which are
+// then cleared.
+rsc_status read_counter(const LdLayout &L, cudaStream_t st, u64 *out, int banks = 1) {
+    u64 h[kBanks * ldn::kCounters];
+    const size_t bytes = sizeof(u64) * ldn::kCounters * (size_t)banks;
+    RSC_CUDA_TRY(cudaMemcpyAsync(h, L.cnt, bytes, cudaMemcpyDeviceToHost, st));
     RSC_CUDA_TRY(cudaStreamSynchronize(st));
-    u64 s = 0;
-    for (int i = 0; i < ldn::kCounters; ++i) s += h[i];
-    *out = s;
-    RSC_CUDA_TRY(cudaMemsetAsync(L.cnt, 0, sizeof h, st));
+    for (int b = 0; b < banks; ++b) {
+        out[b] = 0;
+        for (int i = 0; i < ldn::kCounters; ++i) out[b] += h[b * ldn::kCounters + i];
+    }
+    RSC_CUDA_TRY(cudaMemsetAsync(L.cnt, 0, bytes, st));
     return RSC_OK;
 }
 
@@ -757,7 +763,7 @@ rsc_status rsc_leiden(const int64_t *indptr, const int32_t *indices, const float
     LdLayout L = carve_leiden(workspace, n, nnz, nullptr);
     cudaStream_t st = static_cast<cudaStream_t>(opts ? opts->stream : nullptr);
     RSC_CUDA_TRY(cudaMemsetAsync(L.status, 0, kStatusBytes, st));
-    RSC_CUDA_TRY(cudaMemsetAsync(L.cnt, 0, sizeof(u64) * ldn::kCounters, st));
+    RSC_CUDA_TRY(cudaMemsetAsync(L.cnt, 0, sizeof(u64) * kBanks * ldn::kCounters, st));
     // level-0 graph: the caller's structure, fixed-point weights; checked
     RSC_CUDA_TRY(cudaMemcpyAsync(L.ip0, indptr, sizeof(int64_t) * (size_t)(n + 1), cudaMemcpyDeviceToDevice, st));
     if (nnz > 0) {
@@ -790,34 +796,39 @@ rsc_status rsc_leiden(const int64_t *indptr, const int32_t *indices, const float
         stats.launches += 4 + 1;   // ids, relabelling; the membership at the end of the run
         for (int level = 0; level < p.max_levels; ++level) {
             ++stats.levels;
-            int64_t level_nnz = 0;
-            RSC_CUDA_TRY(cudaMemcpyAsync(&level_nnz, ip + nv, sizeof level_nnz, cudaMemcpyDeviceToHost, st));
-            // strengths, 2m, vertex tables
+            // strengths, 2m and the number of entries, vertex tables
             const unsigned vb = blocks(nv * 32, ldn::kBlock);
             ldn::strength_kernel<<<vb, ldn::kBlock, 0, st>>>(nv, ip, wt, L.k, L.cnt, L.tlen);
             RSC_CUDA_TRY(cudaGetLastError());
-            u64 m2u = 0;
-            if ((s = read_counter(L, st, &m2u)) != RSC_OK) return s;
-            const int64_t m2 = (int64_t)m2u;
+            u64 sums[kBanks];
+            if ((s = read_counter(L, st, sums, 2)) != RSC_OK) return s;
+            const int64_t m2 = (int64_t)sums[0], level_nnz = (int64_t)sums[1];
             stats.launches += 1;
             if (m2 == 0) break;
             stats.launches += 2 + 5;   // table offsets; relabelling, totals and count after moving
             if ((s = table_offsets(L, nv, st)) != RSC_OK) return s;
-            // 1. local moving
+            // 1. local moving.  It ends after two rounds without a move: after
+            // a round with moves two more are sure to run, and their counts
+            // are read together (a read is a round trip of the host, about as
+            // long as a round on a small level).
             int quiet = 0;
-            for (int r = 0; r < p.max_rounds && quiet < 2; ++r) {
-                if ((s = compute_tot(L, nv, L.comm, L.tot, st)) != RSC_OK) return s;
-                ldn::move_kernel<<<vb, ldn::kBlock, 0, st>>>(nv, ip, col, wt, L.k, L.tot, L.comm, L.next, m2, p.G,
-                                                             r % 2, L.toff, L.hkey, L.hsum, L.cnt);
-                RSC_CUDA_TRY(cudaGetLastError());
-                u64 moves = 0;
-                if ((s = read_counter(L, st, &moves)) != RSC_OK) return s;
-                ++stats.move_rounds;
-                stats.launches += 2;
-                stats.entries += level_nnz;
-                stats.vertices += nv;
-                std::swap(L.comm, L.next);
-                quiet = moves ? 0 : quiet + 1;
+            for (int r = 0; r < p.max_rounds && quiet < 2;) {
+                const int ahead = std::min(2 - quiet, p.max_rounds - r);
+                for (int a = 0; a < ahead; ++a) {
+                    if ((s = compute_tot(L, nv, L.comm, L.tot, st)) != RSC_OK) return s;
+                    ldn::move_kernel<<<vb, ldn::kBlock, 0, st>>>(nv, ip, col, wt, L.k, L.tot, L.comm, L.next, m2, p.G,
+                                                                 (r + a) % 2, L.toff, L.hkey, L.hsum,
+                                                                 L.cnt + a * ldn::kCounters);
+                    RSC_CUDA_TRY(cudaGetLastError());
+                    std::swap(L.comm, L.next);
+                }
+                if ((s = read_counter(L, st, sums, ahead)) != RSC_OK) return s;
+                for (int a = 0; a < ahead; ++a) quiet = sums[a] ? 0 : quiet + 1;
+                r += ahead;
+                stats.move_rounds += ahead;
+                stats.launches += 2 * ahead;
+                stats.entries += ahead * level_nnz;
+                stats.vertices += ahead * nv;
             }
             if ((s = canon(L, nv, L.comm, st)) != RSC_OK) return s;
             if ((s = compute_tot(L, nv, L.comm, L.tot, st)) != RSC_OK) return s;
