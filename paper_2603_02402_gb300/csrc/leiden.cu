@@ -805,7 +805,7 @@ rsc_status rsc_leiden(const int64_t *indptr, const int32_t *indices, const float
             const int64_t m2 = (int64_t)sums[0], level_nnz = (int64_t)sums[1];
             stats.launches += 1;
             if (m2 == 0) break;
-            stats.launches += 2 + 5;   // table offsets; relabelling, totals and count after moving
+            stats.launches += seg_scan::launches(nv) + 5;   // table offsets; relabelling, totals and count after moving
             if ((s = table_offsets(L, nv, st)) != RSC_OK) return s;
             // 1. local moving.  It ends after two rounds without a move: after
             // a round with moves two more are sure to run, and their counts
@@ -836,7 +836,7 @@ rsc_status rsc_leiden(const int64_t *indptr, const int32_t *indices, const float
             u64 ncomm = 0;
             if ((s = read_counter(L, st, &ncomm)) != RSC_OK) return s;
             if ((int64_t)ncomm == nv) break;
-            stats.launches += 2 + 3 + 3;   // refinement set-up; relabelling; head flags and their scan
+            stats.launches += 2 + 3 + 1 + seg_scan::launches(nv);   // refinement set-up; relabelling; head flags and their scan
             // 2. refinement
             ldn::inner_kernel<<<vb, ldn::kBlock, 0, st>>>(nv, ip, col, wt, L.k, L.comm, 0, L.wC, nullptr, nullptr,
                                                           nullptr);
@@ -869,7 +869,7 @@ rsc_status rsc_leiden(const int64_t *indptr, const int32_t *indices, const float
             RSC_CUDA_TRY(cudaMemcpyAsync(&K, L.pos + nv, sizeof K, cudaMemcpyDeviceToHost, st));
             RSC_CUDA_TRY(cudaStreamSynchronize(st));
             if (K == nv) break;   // the refinement merged nothing
-            stats.launches += 10;
+            stats.launches += 6 + 2 * seg_scan::launches(K);
             RSC_CUDA_TRY(cudaMemsetAsync(L.ndeg, 0, sizeof(u64) * (size_t)K, st));
             ldn::node_kernel<<<blocks(nv), 256, 0, st>>>(nv, L.ref, L.pos, L.comm, ip, L.node, L.next, L.ndeg);
             ldn::top_kernel<<<blocks(n), 256, 0, st>>>(n, L.node, L.top);
@@ -909,7 +909,7 @@ rsc_status rsc_leiden(const int64_t *indptr, const int32_t *indices, const float
     RSC_CUDA_TRY(cudaMemcpyAsync(&K, L.pos + n, sizeof K, cudaMemcpyDeviceToHost, st));
     RSC_CUDA_TRY(cudaStreamSynchronize(st));
     if (n_communities) *n_communities = K;
-    stats.launches += 6 + (modularity ? 1 : 0);
+    stats.launches += 4 + seg_scan::launches(n) + (modularity ? 1 : 0);
     g_last_stats = stats;
     if (modularity) {
         // per community inside weight and strength; summed on the host in

@@ -212,3 +212,14 @@ def test_full_size_graph_properties(rsc):
     A = sp.csr_matrix((np.ones(keep.sum()), (rows[keep], ind[keep])), shape=(n, n))
     ncomp, lab = sp.csgraph.connected_components(A, directed=False)
     assert ncomp == K
+
+
+@pytest.mark.parametrize("n", [4095, 4096, 4097, 65535, 65536, 65537])
+def test_chains_at_the_scans_segments(rsc, n):
+    # vertex counts at the edges of the scans' segments and of the one-launch
+    # scan: a ring of chains, whose partition has to be the oracle's
+    i = np.arange(n)
+    w = np.where(i % 7 == 0, 1.0, 5.0)      # weight of i -> i + 1: chains of seven
+    j = (i + 1) % n
+    graph = csr(np.concatenate([i, j]), np.concatenate([j, i]), np.concatenate([w, w]), n)
+    assert_same(*run_both(rsc, graph))
