@@ -62,6 +62,17 @@ __device__ __forceinline__ void record_status(unsigned int *status, unsigned int
     if (status) atomicCAS(status, 0u, code);
 }
 
+// Asynchronous copies of 16 bytes from global to shared memory (both on a
+// 16-byte boundary), committed in groups; wait<N> leaves N groups in flight.
+__device__ __forceinline__ void cp_async16(uint32_t to, const float *from) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(to), "l"(from) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // Three-input minimum (one instruction on sm_100 and later).
 __device__ __forceinline__ float fmin3(float a, float b, float c) {
     float r;

@@ -226,11 +226,6 @@ size_t cross_smem(int w4) {
     return kXWarps * sizeof(float) * (68 + (w4 > 0 ? 32 * cross_step(w4) : 0) + 2 * 32 * E + 2 * (kXGroup + 32));
 }
 
-__device__ __forceinline__ void cp_async16(uint32_t to, const float *from) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(to), "l"(from) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // One warp per query position q (original row qo = perm[q], or q without a
 // permutation): for every sample, re-score its cross candidates exactly
 // (direct difference in FP32), keep the k_cross best by (distance, id), take
@@ -304,7 +299,8 @@ rerank_cross_kernel(const float *__restrict__ R, int64_t rs, int64_t N, int d, i
                     if (lo8) cp_async16(put0 + r * 4 * step, y);
                     if (hi8) cp_async16(put0 + r * 4 * step + 128, y + 32);
                 }
-                cp_async_wait();
+                cp_async_commit();
+                cp_async_wait<0>();
                 __syncwarp();
                 const float4 *v4 = reinterpret_cast<const float4 *>(stage + lane * (step >> 2));
                 const float4 *q4 = reinterpret_cast<const float4 *>(xq);

@@ -222,50 +222,71 @@ chunk_scatter_kernel(const int32_t *__restrict__ lab, int64_t m, int64_t step, c
 
 // Centroid c <- mean of its rows (sorted positions [off[c * nchunk],
 // off[(c + 1) * nchunk])), summed in row order; an empty cluster keeps its
-// centroid.  Warp per centroid.  kVar: cvar, the rows' mean squared distance
+// centroid.  Block per centroid.  kVar: cvar, the rows' mean squared distance
 // from it.
+//
+// A cluster's time is its rows' latencies (there are few clusters and the
+// largest holds several times the mean), so the block copies 64 rows at a time
+// into shared memory, two such stages in flight, and one warp adds them up.
+// 68,579 rows, 144 clusters: 35 us a launch with a warp per cluster that had 16
+// rows in flight, 11 us so.
+constexpr int kMeanThreads = 128;
+constexpr int kMeanRows = 64;
+constexpr int kMeanPasses = kMeanRows * 16 / kMeanThreads;   // 16 threads copy a row of up to 64 floats
+
 template <bool kVar>
-__global__ void centroid_mean_kernel(const float *__restrict__ Y, int DP, const int32_t *__restrict__ sorted_rows,
-                                     const int32_t *__restrict__ off, int nchunk, int C, float *__restrict__ cent,
-                                     float *__restrict__ cnorm, float *__restrict__ cvar) {
-    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (c >= C) return;
+__global__ void __launch_bounds__(kMeanThreads)
+centroid_mean_kernel(const float *__restrict__ Y, int DP, const int32_t *__restrict__ sorted_rows,
+                     const int32_t *__restrict__ off, int nchunk, int C, float *__restrict__ cent,
+                     float *__restrict__ cnorm, float *__restrict__ cvar) {
+    __shared__ __align__(16) float stage[2][kMeanRows][64];
+    const int c = blockIdx.x, lane = threadIdx.x & 31;
+    const int r16 = threadIdx.x >> 4, t16 = threadIdx.x & 15;
     const int32_t b = off[(int64_t)c * nchunk], e = off[(int64_t)(c + 1) * nchunk];
     if (e == b) {
-        if (kVar && lane == 0) cvar[c] = 0.f;
+        if (kVar && threadIdx.x == 0) cvar[c] = 0.f;
         return;
     }
     float s0 = 0.f, s1 = 0.f, sq = 0.f;
-    // the additions keep the row order; a lane fetches the row ids 32 at a time
-    // and the rows come kMeanAhead at a time, so a cluster costs a load latency
-    // per 16 rows (two per 8 when each row's id was read just before it: 54 us
-    // a launch at 68,579 rows, 144 clusters)
-    constexpr int kMeanAhead = 16;
-    const int l0 = min(lane, DP - 1), l1 = min(lane + 32, DP - 1);
-    for (int32_t q0 = b; q0 < e; q0 += 32) {
-        const int32_t mine = q0 + lane < e ? sorted_rows[q0 + lane] : 0;
-        const int m = min(32, e - q0);
-        for (int p0 = 0; p0 < m; p0 += kMeanAhead) {
-            float v0[kMeanAhead], v1[kMeanAhead];
+    int32_t ids[kMeanPasses];
+    auto fetch = [&](int32_t q0) {   // this thread's row ids of a stage
 #pragma unroll
-            for (int u = 0; u < kMeanAhead; ++u) {
-                // rows past m are row 0 and are not added; components past DP
-                // repeat the last and are not stored
-                const float *y = Y + (int64_t)__shfl_sync(0xffffffffu, mine, p0 + u) * DP;
-                v0[u] = y[l0];
-                v1[u] = y[l1];
-            }
+        for (int u = 0; u < kMeanPasses; ++u) ids[u] = sorted_rows[min(q0 + u * (kMeanThreads / 16) + r16, e - 1)];
+    };
+    auto copy = [&](int buf, int32_t q0) {
 #pragma unroll
-            for (int u = 0; u < kMeanAhead; ++u) {
-                if (p0 + u < m) {
-                    s0 += v0[u];
-                    s1 += v1[u];
-                    if (kVar) sq += (lane < DP ? v0[u] * v0[u] : 0.f) + (lane + 32 < DP ? v1[u] * v1[u] : 0.f);
-                }
+        for (int u = 0; u < kMeanPasses; ++u) {
+            const int r = u * (kMeanThreads / 16) + r16;
+            if (q0 + r < e && 4 * t16 < DP)
+                cp_async16((uint32_t)__cvta_generic_to_shared(&stage[buf][r][4 * t16]),
+                           Y + (int64_t)ids[u] * DP + 4 * t16);
+        }
+        cp_async_commit();
+    };
+    fetch(b);
+    copy(0, b);
+    fetch(min(b + kMeanRows, e - 1));
+    copy(1, b + kMeanRows);
+    int buf = 0;
+    for (int32_t q0 = b; q0 < e; q0 += kMeanRows, buf ^= 1) {
+        fetch(min(q0 + 2 * kMeanRows, e - 1));
+        cp_async_wait<1>();
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const float *v = &stage[buf][0][lane];
+            const int m = min(kMeanRows, e - q0);
+#pragma unroll 16
+            for (int r = 0; r < m; ++r) {   // components past DP are not stored
+                const float v0 = v[64 * r], v1 = v[64 * r + 32];
+                s0 += v0;
+                s1 += v1;
+                if (kVar) sq += (lane < DP ? v0 * v0 : 0.f) + (lane + 32 < DP ? v1 * v1 : 0.f);
             }
         }
+        __syncthreads();
+        copy(buf, q0 + 2 * kMeanRows);
     }
+    if (threadIdx.x >= 32) return;
     const float inv = 1.f / (float)(e - b);
     s0 *= inv;
     s1 *= inv;
@@ -692,7 +713,6 @@ cudaError_t launch_locality_order(const float *Y, int64_t n, int DP, int iters, 
     if (goff && (G < 1 || G > kOrderMaxLeaves)) return cudaErrorInvalidValue;
     const OrderLayout L = order_layout(scratch, n, DP, s, goff ? G : 0, target.spread, nullptr);
     const int C = s.C1 * s.C2;
-    const int mean_warps = 4;
     cudaError_t e;
     const int spread_smem = (int)sizeof(float) * kSpread * DP;
     if (target.spread && (e = cudaFuncSetAttribute(spread_centroids_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -710,7 +730,7 @@ cudaError_t launch_locality_order(const float *Y, int64_t n, int DP, int iters, 
         if ((e = launch_assign(Y, DP, s.m1, s.step1, L.cent1, L.cnorm1, s.C1, L.lab1, nullptr, st)) != cudaSuccess) return e;
         if ((e = counting_sort(L.lab1, s.m1, s.step1, nullptr, s.C1, L.cnt, L.off, L.ssum, L.srows, st)) != cudaSuccess)
             return e;
-        centroid_mean_kernel<false><<<(unsigned)ceil_div(s.C1, mean_warps), mean_warps * 32, 0, st>>>(
+        centroid_mean_kernel<false><<<(unsigned)s.C1, kMeanThreads, 0, st>>>(
             Y, DP, L.srows, L.off, nch1, s.C1, L.cent1, L.cnorm1, nullptr);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -732,8 +752,7 @@ cudaError_t launch_locality_order(const float *Y, int64_t n, int DP, int iters, 
             return e;
         if ((e = counting_sort(L.lab, s.m2, s.step2, L.perm1, C, L.cnt, L.off, L.ssum, L.srows, st)) != cudaSuccess) return e;
         auto mean = L.cvar2 ? centroid_mean_kernel<true> : centroid_mean_kernel<false>;
-        mean<<<(unsigned)ceil_div(C, mean_warps), mean_warps * 32, 0, st>>>(Y, DP, L.srows, L.off, nch2, C, L.cent2,
-                                                                            L.cnorm2, L.cvar2);
+        mean<<<(unsigned)C, kMeanThreads, 0, st>>>(Y, DP, L.srows, L.off, nch2, C, L.cent2, L.cnorm2, L.cvar2);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     // chains through the coarse centroids and through each cluster's sub-centroids
