@@ -44,8 +44,8 @@
 //
 // What bounds it: the FMA pipe and, next to it, the insertions (a row takes in
 // about 70 values).  50 components, k = 15, one GB300, whole call (in brackets
-// the full scan): 100,003 rows, 60 clusters 1.9 ms (25.9), of which this kernel
-// 0.87 and the ordering 0.8; 1M rows, 100 clusters 33.7 ms (2054); rows without
+// the full scan): 100,003 rows, 60 clusters 1.6 ms (25.9), of which this kernel
+// 0.8 and the ordering 0.5; 1M rows, 100 clusters 31 ms (2054); rows without
 // any clusters, of which no tile is dropped, 1.9 ms (1.5) at 16,384 rows, 9.1
 // (7.3) at 50,000, 25.0 (25.9) at 100,003.
 #include <float.h>

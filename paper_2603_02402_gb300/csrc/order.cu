@@ -388,6 +388,8 @@ __global__ void init_sub_centroids_kernel(const float *__restrict__ Y, int DP, c
 // DP]): group g draws from positions [off[g * nchunk], off[(g + 1) * nchunk])
 // of `perm` (its coarse centroid `cent1` when that is empty), or, perm null,
 // from all n rows.  Thread per sampled row.
+// 128 starts in one block: 135 us with two instructions a component, each start
+// written in its round and the rows read one after the other, 91 us so.
 constexpr int kSpread = 512;
 __global__ void __launch_bounds__(kSpread)
 spread_centroids_kernel(const float *__restrict__ Y, int64_t n, int DP, const int32_t *__restrict__ perm,
@@ -396,55 +398,62 @@ spread_centroids_kernel(const float *__restrict__ Y, int64_t n, int DP, const in
     extern __shared__ __align__(16) float rows[];   // [kSpread][DP]
     __shared__ unsigned wv[2][kSpread / 32];
     __shared__ int wi[2][kSpread / 32];
+    __shared__ float norms[kSpread];
+    __shared__ int32_t ids[kSpread];
+    __shared__ int taken[kOrderMaxCoarse];
     const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t b = perm ? off[(int64_t)c * nchunk] : 0, size = (perm ? off[(int64_t)(c + 1) * nchunk] : n) - b;
     const int m = (int)max((int64_t)1, min((int64_t)kSpread, size));
-    for (int x = tid; x < m * (DP / 4); x += kSpread) {
-        const int r = x / (DP / 4), q = x % (DP / 4);
-        const int64_t at = b + ((int64_t)r * size) / m;
-        const float *src = size > 0 ? Y + (perm ? (int64_t)perm[at] : at) * DP : cent1 + (int64_t)c * DP;
-        const float4 v = reinterpret_cast<const float4 *>(src)[q];
-        reinterpret_cast<float4 *>(rows)[r * (DP / 4) + q] = v;
+    // the rows' ids, then all rows at once
+    if (tid < m) {
+        const int64_t at = b + ((int64_t)tid * size) / m;
+        ids[tid] = size > 0 ? (perm ? perm[at] : (int32_t)at) : 0;
     }
     __syncthreads();
+    const float *from = size > 0 ? Y : cent1 + (int64_t)c * DP;
+    for (int x = tid; x < m * (DP / 4); x += kSpread) {
+        const int r = x / (DP / 4), q = x % (DP / 4);
+        cp_async16((uint32_t)__cvta_generic_to_shared(rows + r * DP + 4 * q), from + (int64_t)ids[r] * DP + 4 * q);
+    }
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
     // the thread's own row in registers, the taken one from shared memory (one
-    // 16-byte read for the whole warp)
-    float4 own[16];
+    // 16-byte read for the whole warp); |x - y|^2 = |x|^2 + |y|^2 - 2 x.y, two
+    // components an instruction (a start need not be the exact farthest)
+    unsigned long long own[32];
 #pragma unroll
-    for (int q = 0; q < 16; ++q)
-        own[q] = 4 * q < DP && tid < m ? reinterpret_cast<const float4 *>(rows)[tid * (DP / 4) + q] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int q = 0; q < 16; ++q) {
+        ulonglong2 v = make_ulonglong2(0, 0);
+        if (4 * q < DP && tid < m) v = reinterpret_cast<const ulonglong2 *>(rows)[tid * (DP / 4) + q];
+        own[2 * q] = v.x;
+        own[2 * q + 1] = v.y;
+    }
+    auto dot = [&](const float *row) {
+        unsigned long long a0 = 0, a1 = 0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            if (4 * q >= DP) break;   // uniform
+            const ulonglong2 v = reinterpret_cast<const ulonglong2 *>(row)[q];
+            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a0) : "l"(own[2 * q]), "l"(v.x));
+            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a1) : "l"(own[2 * q + 1]), "l"(v.y));
+        }
+        return (__uint_as_float((unsigned)a0) + __uint_as_float((unsigned)(a0 >> 32))) +
+               (__uint_as_float((unsigned)a1) + __uint_as_float((unsigned)(a1 >> 32)));
+    };
+    const float norm = tid < m ? dot(rows + tid * DP) : 0.f;
+    norms[tid] = norm;
+    __syncthreads();
     float far = INFINITY;   // squared distance to the nearest row taken so far
     int pick = 0;
     for (int s = 0; s < C; ++s) {
-        const int64_t g = (int64_t)c * C + s;
-        if (warp == 0) {
-            float q = 0.f;
-            for (int t = lane; t < DP; t += 32) {
-                const float v = rows[pick * DP + t];
-                cent[g * DP + t] = v;
-                q = fmaf(v, v, q);
-            }
-            for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-            if (lane == 0) cnorm[g] = q;
-        }
+        if (tid == 0) taken[s] = pick;
         // bits of the distance + 1 (non-negative floats order as their bits);
         // 0: no row, or one that is no number, which is not taken
         unsigned key = 0;
         if (tid < m) {
-            const float4 *taken = reinterpret_cast<const float4 *>(rows + pick * DP);
-            float d0 = 0.f, d1 = 0.f;
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                if (4 * q >= DP) break;   // uniform
-                const float4 v = taken[q];
-                const float e0 = own[q].x - v.x, e1 = own[q].y - v.y, e2 = own[q].z - v.z, e3 = own[q].w - v.w;
-                d0 = fmaf(e0, e0, d0);
-                d1 = fmaf(e1, e1, d1);
-                d0 = fmaf(e2, e2, d0);
-                d1 = fmaf(e3, e3, d1);
-            }
-            far = fminf(far, d0 + d1);
-            key = far < INFINITY ? __float_as_uint(far) + 1u : 0u;
+            far = fminf(far, (norm + norms[pick]) - 2.f * dot(rows + pick * DP));
+            key = far < INFINITY ? __float_as_uint(fmaxf(far, 0.f)) + 1u : 0u;
         }
         const unsigned best = __reduce_max_sync(0xffffffffu, key);
         const int who = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
@@ -458,6 +467,18 @@ spread_centroids_kernel(const float *__restrict__ Y, int64_t n, int DP, const in
         const int w = __ffs(__ballot_sync(0xffffffffu, lane < kSpread / 32 && v == top)) - 1;
         pick = wi[s & 1][w];
         if (pick >= m) pick = 0;
+    }
+    __syncthreads();
+    for (int s = warp; s < C; s += kSpread / 32) {
+        const int64_t g = (int64_t)c * C + s;
+        float q = 0.f;
+        for (int t = lane; t < DP; t += 32) {
+            const float v = rows[taken[s] * DP + t];
+            cent[g * DP + t] = v;
+            q = fmaf(v, v, q);
+        }
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if (lane == 0) cnorm[g] = q;
     }
 }
 
