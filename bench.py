@@ -58,28 +58,32 @@ TRAFFIC = {
 ED_SOURCES = ("edist.cu", "knn_tc.cuh", "tc_ptx.cuh")
 NND_SOURCES = ("nndescent.cu",)
 
-ORDER_MIN_ROWS = 16384   # automatic locality ordering from this many rows (BF16 path)
+ORDER_MIN_ROWS = 16384   # automatic locality ordering from this many rows
 
 
 def launches_per_step(metric, precision, n):
     """Kernels this library launches per graph step.
 
     rsc_knn: FP32 prep (column sums + column means + prep for Euclidean, prep
-    alone for cosine), the BF16 operand prep (tensor-core path), the locality
-    ordering (two k-means levels of 1 init + 2 Lloyd rounds x 6 + 5 for the
-    full assignment and sort, a sort being 4 launches, 2 chain passes, + 1
-    gather of the re-rank rows), the candidate
-    search (one launch, or 12 when pruned: window pass, 2 sphere passes, group
-    spheres, tau, count, scan (2), fill, offsets, item order, list pass) and
-    the re-rank;
+    alone for cosine), the re-rank, and
+      BF16 from ORDER_MIN_ROWS rows on: operand prep, the locality ordering with
+        the gather of the re-rank rows (33), the pruned search (10: window pass,
+        tile and group spheres, tau, kept tiles, scan, fill, offsets, item order,
+        list pass); below: operand prep and one scan;
+      FP32 from ORDER_MIN_ROWS rows on: the ordering (33), tile table, records,
+        search, its split items, their merge, ties; below: records, search, ties.
+    Scans of more than 65,536 counts take a second launch, which is not counted.
     rsc_connectivities: 8 (smooth, push, match, two scan launches, emit and the
-    two queued-row sorts).
+    two queued-row passes).
     """
-    knn = (3 if metric == "euclidean" else 1) + 2
-    if precision == "fp32" and n >= ORDER_MIN_ROWS:   # ordering, gather, tile table, records, split, merge, ties
-        knn += 39 + 5
-    if precision == "bf16":
-        knn += 1 + (39 + 12 if n >= ORDER_MIN_ROWS else 0)
+    ordered = n >= ORDER_MIN_ROWS
+    knn = (3 if metric == "euclidean" else 1) + 1
+    if precision == "fp32":
+        knn += 33 + 6 if ordered else 3
+    elif precision == "bf16":
+        knn += 1 + (33 + 10 if ordered else 1)
+    else:
+        knn += 1
     return knn + 8
 
 
@@ -613,11 +617,10 @@ def run_batched(args):
                          "kernel": "knn_tc_kernel (batched)",
                          "note": "whole call (prep + pruned search + both re-ranks) timed; 2*d flops per "
                                  "(query, row) pair computed: 128*256 per scanned tile pair"},
-            # prep 3, ordering 36 + 2 chains + 5 (sample-preserving partition), BF16 operands 1,
-            # pruned search 10 (2 sphere passes, nearest tiles, window pass, tau, count, scan (2),
-            # fill, list pass), gather + within re-rank + cross re-rank 3; 7 without the ordering
-            # (fewer than ORDER_MIN_ROWS rows)
-            "gpu_launches": (60 if n >= ORDER_MIN_ROWS else 7) * args.steps, "clocks": sampler.summary(),
+            # prep, ordering, sample-preserving partition, operands, pruned search, gather, the two
+            # re-ranks; scans of more than 65,536 counts take a second launch, which is not counted;
+            # 7 without the ordering (fewer than ORDER_MIN_ROWS rows)
+            "gpu_launches": (52 if n >= ORDER_MIN_ROWS else 7) * args.steps, "clocks": sampler.summary(),
             "autotune": {"choice": tuned, "best_ms": tune_ms}}
     if rank == 0 and not args.no_cpu_baseline:
         line["cpu_baseline"] = batched_baseline(X, off, kw, kx, out)
