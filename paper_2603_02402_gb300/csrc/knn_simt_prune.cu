@@ -77,7 +77,8 @@ constexpr int kMaxCtas = 320;             // persistent CTAs at most
 constexpr int kBigItems = 192;            // items that may be split
 constexpr int kSegs = 8;                  // parts of a split item at most
 constexpr int kSegTiles = 128;            // tiles per part at least
-constexpr long long kWaitBudget = 2000000000LL;   // ~1 s of SM clocks
+constexpr uint32_t kSleepNs = 2000;                // suspend of a wait per try
+constexpr long long kDrainBudget = 2000000000LL;   // ~1 s of SM clocks, for copies in flight when a CTA leaves
 
 // tiles at most: every leaf may end in a partial one; an even number
 __host__ __device__ inline int64_t tiles_max(int64_t n) { return (ceil_div(n, (int64_t)kR) + kOrderMaxLeaves + 2) / 2 * 2; }
@@ -379,6 +380,7 @@ struct Args {
     float *vv;              // [query slots] |y|^2 (flat)
     unsigned long long *scanned;   // tiles scanned (a statistic)
     unsigned int *status;
+    long long wait_budget;         // SM clocks a wait for a copy may take (tc_wait_budget)
 };
 
 // parts of a split item: segments of seg_tiles tiles
@@ -442,11 +444,16 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
     __syncthreads();
     List<KC> tk;
     tk.sbase = (uint32_t)__cvta_generic_to_shared(reinterpret_cast<float *>(sm + m.buf) + tid);
-    auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {   // bounded
-        if (tc::mbar_try_wait(bar, parity)) return true;
+    // bounded; a budget shorter than a few sleeps (which may outlast it) is polled
+    const bool poll = g.wait_budget < 8 * (long long)kSleepNs;
+    auto arrived = [&](uint64_t *bar, uint32_t parity) {
+        return poll ? tc::mbar_test_wait(bar, parity) : tc::mbar_try_wait_sleep(bar, parity, kSleepNs);
+    };
+    auto wait = [&](uint64_t *bar, uint32_t parity, long long budget) -> bool {
+        if (arrived(bar, parity)) return true;
         const long long t0 = clock64();
-        while (!tc::mbar_try_wait_sleep(bar, parity, 2000))
-            if (clock64() - t0 > kWaitBudget) {
+        while (!arrived(bar, parity))
+            if (clock64() - t0 > budget) {
                 record_status(g.status, RSC_ERR_TIMEOUT);
                 return false;
             }
@@ -474,7 +481,7 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
         }
         for (int i = 0; i < nl; ++i, ++tile_no) {
             const int s = tile_no % kStages;
-            const bool ok = wait(&full[s], (tile_no / kStages) & 1);
+            const bool ok = wait(&full[s], (tile_no / kStages) & 1, g.wait_budget);
             uint64_t acc[8][4];
 #pragma unroll
             for (int a = 0; a < 8; ++a)
@@ -508,8 +515,8 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
             // every read of the previous s tile is done
             if (__syncthreads_or(!ok)) {
                 if (tid == 0) {   // the copies in flight get their time again
-                    wait(&full[s], (tile_no / kStages) & 1);
-                    if (i + 1 < nl) wait(&full[(tile_no + 1) % kStages], ((tile_no + 1) / kStages) & 1);
+                    wait(&full[s], (tile_no / kStages) & 1, kDrainBudget);
+                    if (i + 1 < nl) wait(&full[(tile_no + 1) % kStages], ((tile_no + 1) / kStages) & 1, kDrainBudget);
                 }
                 return false;
             }
@@ -560,9 +567,9 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
             const int h = tid >> 6, u = tid & 63;
             cen[tid] = u < DP ? g.cenT[(int64_t)u * g.stride + 2 * item + h] : 0.f;
         }
-        const bool got = wait(xfull, items & 1);
+        const bool got = wait(xfull, items & 1, g.wait_budget);
         if (__syncthreads_or(!got)) {
-            if (tid == 0) wait(xfull, items & 1);
+            if (tid == 0) wait(xfull, items & 1, kDrainBudget);
             return;
         }
         const bool live = (tid & 63) < g.tile_rows[2 * item + (tid >> 6)];
@@ -939,6 +946,7 @@ Args make_args(const Layout &L, int64_t n, int DP, int width, int k, int metric,
     g.part_segs = kSegs;
     g.vv = nullptr;
     g.status = status;
+    g.wait_budget = tc_wait_budget();
     return g;
 }
 
@@ -1080,6 +1088,7 @@ Args flat_args(const FlatLayout &L, int64_t n, int DP, int width, int k, unsigne
     g.tie_rows = L.tie_rows;
     g.tie_bound = L.tie_bound;
     g.status = status;
+    g.wait_budget = tc_wait_budget();
     return g;
 }
 

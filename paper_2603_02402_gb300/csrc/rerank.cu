@@ -21,6 +21,16 @@ namespace {
 
 constexpr int kWarps = 16;   // queries per block: neighbouring queries share candidate rows in L1
 
+// Every candidate of the kernels below comes through here: list entry jp names
+// a position (its row in R, or perm's) when it lies in [0, n).  Empty entries
+// and what a search that gave up left in the lists do not: -1, id INT_MAX.
+__device__ __forceinline__ int candidate_row(int32_t jp, int64_t n, const int32_t *perm, bool r_by_pos, int &id) {
+    id = INT_MAX;
+    if (jp < 0 || (int64_t)jp >= n) return -1;
+    id = perm ? perm[jp] : jp;   // original id
+    return r_by_pos ? jp : id;
+}
+
 // Warp per query, 8 lanes per candidate row.  In step g, lanes 8 r + s
 // (r < 4, s < 8) score candidate 4 g + r of the current 32 (rerank.cuh: eight
 // components per lane, an FMA chain over them, three xor shuffles);
@@ -59,12 +69,7 @@ rerank_kernel(const float *__restrict__ R, int64_t rs, int64_t n, int d, int met
         id[e] = INT_MAX;
         if (c < C) {
             const int sp = c / KC, slot = c - sp * KC;
-            const int32_t jp = cand[((int64_t)sp * n + q) * KC + slot];
-            if (jp >= 0 && (int64_t)jp < n) {   // ids outside [0, n) (an aborted search) are skipped
-                const int32_t j = perm ? perm[jp] : jp;   // original id
-                row = r_by_pos ? jp : j;
-                id[e] = j;
-            }
+            row = candidate_row(cand[((int64_t)sp * n + q) * KC + slot], n, perm, r_by_pos, id[e]);
         }
         key[e] = INFINITY;
 #pragma unroll
@@ -125,12 +130,7 @@ rerank_stream_kernel(const float *__restrict__ R, int64_t rs, int64_t n, int d, 
         int id[1] = {INT_MAX};
         if (c < C) {
             const int sp = c / KC, slot = c - sp * KC;
-            const int32_t jp = cand[((int64_t)sp * n + q) * KC + slot];
-            if (jp >= 0 && (int64_t)jp < n) {   // ids outside [0, n) (an aborted search) are skipped
-                const int32_t j = perm ? perm[jp] : jp;   // original id
-                row = r_by_pos ? jp : j;
-                id[0] = j;
-            }
+            row = candidate_row(cand[((int64_t)sp * n + q) * KC + slot], n, perm, r_by_pos, id[0]);
         }
 #pragma unroll
         for (int g = 0; g < 8; ++g) {
@@ -194,7 +194,8 @@ rerank_parts_kernel(const float *__restrict__ R, int64_t rs, int64_t n, int d, i
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int c = e * 32 + lane;
-        id[e] = c < M ? pi[c] : -1;
+        int unused;
+        id[e] = c < M ? candidate_row(pi[c], n, nullptr, false, unused) : -1;
         key[e] = id[e] >= 0 ? order(pk[c]) : 0xffffffffu;
         lo = min(lo, key[e]);
     }

@@ -117,3 +117,31 @@ def test_ties_of_small_inputs(rsc, case):  # noqa: F811
         oi, od, _ = oracle.knn(X, k)
         np.testing.assert_array_equal(gi, oi)
         np.testing.assert_allclose(gd, od, rtol=1e-6)
+
+
+@pytest.mark.parametrize("n", [100, 5_000, 20_000])
+def test_search_that_gave_up_leaves_no_id_outside_the_rows(rsc, n):  # noqa: F811
+    # A wait budget of a few hundred SM clocks makes the search's first wait
+    # give up, so its lists keep what the workspace held: here every other
+    # entry is an id far past the rows (1.26e9, the bits of 8388608.0f) and
+    # the rest, the lists' last ones among them, are empty (-1).  The status
+    # word tells, no such id is followed or returned (what else that call
+    # returns is unspecified), and the next call is correct.
+    X = synth.mixture(n, 50, n_comp=7, seed=n)
+    fi, fd = run_knn(rsc, X, 15, precision="fp32", prune="off")
+    Xd = torch.from_numpy(X).cuda()
+    ws = torch.empty(rsc.rsc_knn_workspace_size(n, 50, 15, precision="fp32") // 4 * 4, dtype=torch.uint8, device="cuda")
+    ws.view(torch.int32).fill_(-1)
+    ws.view(torch.int32)[::2] = 0x4B000000
+    rsc.rsc_set_wait_budget(300)
+    try:
+        gi, _ = rsc.rsc_knn(Xd, 15, precision="fp32", workspace=ws)
+        assert rsc.rsc_workspace_status(ws) == rsc.RSC_ERR_TIMEOUT
+    finally:
+        rsc.rsc_set_wait_budget(0)
+    gi = gi.cpu().numpy()
+    assert ((gi >= -1) & (gi < n)).all()
+    gi, gd = rsc.rsc_knn(Xd, 15, precision="fp32", workspace=ws)
+    assert rsc.rsc_workspace_status(ws) == rsc.RSC_OK
+    np.testing.assert_array_equal(gi.cpu().numpy(), fi)
+    np.testing.assert_array_equal(gd.cpu().numpy(), fd)
