@@ -120,8 +120,10 @@ const char *rsc_last_error(void);
 
 /*
  * Budget, in SM clock cycles, of every bounded wait inside the tensor-core
- * kernels (the barrier waits of the TMA producer, the MMA issuer and the
- * epilogue) and of the FP32 search that copies its tiles; 0 restores the default of about 1 s.  A diagnostic for
+ * searches (the barrier waits of the TMA producer, the MMA issuer and the
+ * epilogue), of the FP32 search that copies its tiles and of the
+ * partitioner's routing kernel (its training GEMMs keep the default); 0
+ * restores the default of about 1 s.  A diagnostic for
  * exercising the timeout path (the paper has no counterpart): with a budget
  * of a few hundred cycles the first wait of a search gives up, the kernel
  * records RSC_ERR_TIMEOUT in the workspace status word, lets its in-flight

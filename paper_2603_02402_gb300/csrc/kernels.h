@@ -199,8 +199,8 @@ cudaError_t launch_knn_tc_list(const void *Qb, const void *Db, int64_t n, int d,
                                const int64_t *tile_off, const int32_t *order, const int32_t *overflow,
                                int32_t *cand, int *counter,
                                unsigned int *status, cudaStream_t st);
-// SM clock cycles each bounded wait of the tensor-core kernels and of the
-// pruned FP32 search may take before the kernel records RSC_ERR_TIMEOUT (process-wide, see
+// SM clock cycles each bounded wait of the tensor-core searches, of the pruned
+// FP32 search and of the partitioner's routing may take before the kernel records RSC_ERR_TIMEOUT (process-wide, see
 // rsc_set_wait_budget).
 long long tc_wait_budget();
 int knn_tc_bm();   // query rows per tensor-core work item

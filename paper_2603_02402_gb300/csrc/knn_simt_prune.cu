@@ -444,15 +444,12 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
     __syncthreads();
     List<KC> tk;
     tk.sbase = (uint32_t)__cvta_generic_to_shared(reinterpret_cast<float *>(sm + m.buf) + tid);
-    // bounded; a budget shorter than a few sleeps (which may outlast it) is polled
-    const bool poll = g.wait_budget < 8 * (long long)kSleepNs;
-    auto arrived = [&](uint64_t *bar, uint32_t parity) {
-        return poll ? tc::mbar_test_wait(bar, parity) : tc::mbar_try_wait_sleep(bar, parity, kSleepNs);
-    };
+    // bounded; a budget shorter than a few sleeps is polled
+    const uint32_t sleep_ns = g.wait_budget < 8 * (long long)kSleepNs ? 0 : kSleepNs;
     auto wait = [&](uint64_t *bar, uint32_t parity, long long budget) -> bool {
-        if (arrived(bar, parity)) return true;
+        if (tc::mbar_arrived(bar, parity, sleep_ns)) return true;
         const long long t0 = clock64();
-        while (!arrived(bar, parity))
+        while (!tc::mbar_arrived(bar, parity, sleep_ns))
             if (clock64() - t0 > budget) {
                 record_status(g.status, RSC_ERR_TIMEOUT);
                 return false;

@@ -200,6 +200,7 @@ constexpr int kThreads = kEpi + 64 + kStagers;
 constexpr int kMaxP = 1024;
 constexpr int kBias = 2 * kN + kMaxP;    // floats of the padded biases
 constexpr int kMaxR = 8;
+constexpr uint32_t kSleepNs = 20000;     // suspend of a wait per try
 constexpr int kOffX = 0;
 constexpr int kOffH = kOffX + kABlock;
 constexpr int kOffW = kOffH + 4 * kABlock;
@@ -257,7 +258,7 @@ template <int R>
 __global__ void __launch_bounds__(kThreads, 1)
 route_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, int64_t count, int d, int H, int P,
              const uint8_t *__restrict__ packed, const float *__restrict__ bias_g, int32_t *__restrict__ out,
-             unsigned int *status) {
+             unsigned int *status, long long wait_budget) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = align1024(smem_raw);
     uint8_t *sX = smem + kOffX, *sH = smem + kOffH, *sW = smem + kOffW;
@@ -304,12 +305,14 @@ route_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, int6
     const int kb = k_blocks(H), nc = chunks(P), nb = weight_blocks(H, P);
     const int64_t tiles = ceil_div(count, (int64_t)kTM);
 
+    // bounded; after the first try a budget shorter than a few sleeps is polled
+    const uint32_t sleep_ns = wait_budget < 8 * (long long)kSleepNs ? 0 : kSleepNs;
     auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {
         if (tc::mbar_try_wait(bar, parity)) return true;
         const long long t0 = clock64();
-        while (!tc::mbar_try_wait_sleep(bar, parity, 20000)) {
+        while (!tc::mbar_arrived(bar, parity, sleep_ns)) {
             if (*abort_flag) return false;
-            if (clock64() - t0 > kWaitBudget) {
+            if (clock64() - t0 > wait_budget) {
                 *abort_flag = 1;
                 record_status(status, RSC_ERR_TIMEOUT);
                 return false;
@@ -317,7 +320,7 @@ route_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, int6
         }
         return true;
     };
-    auto drain = [&](uint64_t *bar, uint32_t parity) {
+    auto drain = [&](uint64_t *bar, uint32_t parity) {   // the default budget, whatever is set
         const long long t0 = clock64();
         while (!tc::mbar_try_wait(bar, parity))
             if (clock64() - t0 > kWaitBudget) {
@@ -459,9 +462,8 @@ route_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, int6
                     tc::mbar_arrive_expect_tx(&full[s], kBlock);
                     tc::bulk_load(sW + s * kBlock, packed + (size_t)b * kBlock, kBlock, &full[s]);
                 }
-            if (!ok) {   // let every copy this thread started land before the CTA exits
-                for (uint32_t t = g > kStages ? g - kStages : 0; t < g; ++t) drain(&full[t % kStages], (t / kStages) & 1);
-            }
+            // every copy this thread started lands before the CTA exits, whichever role gave up
+            for (uint32_t t = g > kStages ? g - kStages : 0; t < g; ++t) drain(&full[t % kStages], (t / kStages) & 1);
         }
     } else if (warp == 9) {
         if (lane == 0) {
@@ -567,7 +569,7 @@ cudaError_t launch_mlp_route(cudaStream_t st, const float *X, const int32_t *row
     const uint8_t *w = static_cast<const uint8_t *>(packed);
     const float *bias = reinterpret_cast<const float *>(w + (size_t)weight_blocks(H, P) * kBlock);
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(count, (int64_t)mlp::kTM), sm_count());
-    kern<<<grid, kThreads, kSmem, st>>>(X, rows, count, d, H, P, w, bias, out, status);
+    kern<<<grid, kThreads, kSmem, st>>>(X, rows, count, d, H, P, w, bias, out, status, tc_wait_budget());
     return cudaGetLastError();
 }
 

@@ -73,6 +73,12 @@ __device__ __forceinline__ bool mbar_try_wait_sleep(uint64_t *bar, uint32_t pari
     return ok != 0;
 }
 
+// One try of a bounded wait that suspends up to `ns` nanoseconds; 0 polls (the
+// suspend's limit is a hint, so a wait whose budget it may outlast polls).
+__device__ __forceinline__ bool mbar_arrived(uint64_t *bar, uint32_t parity, uint32_t ns) {
+    return ns == 0 ? mbar_test_wait(bar, parity) : mbar_try_wait_sleep(bar, parity, ns);
+}
+
 // ----------------------------------------------------------------- TMA
 
 __device__ __forceinline__ void tma_load_2d(void *smem_dst, const CUtensorMap *map, int x, int y,

@@ -168,3 +168,27 @@ def test_routing_follows_the_network(rsc, n, d, P, H):
     assert same.all()
     size = np.bincount(label[clear], minlength=P)
     assert (found.sum(axis=1)[clear] >= np.minimum(size[label[clear]], k)).all()
+
+
+@pytest.mark.parametrize("n,P,H", [(100, 9, 8), (20_001, 600, 256)])
+def test_routing_that_gave_up_is_recorded_and_the_next_call_recovers(rsc, n, P, H):
+    # a wait budget of a few hundred SM clocks makes the routing kernel's first
+    # waits give up (three weight blocks in all and one tile of rows, then many
+    # of both): the status word tells, and the next calls are those of a
+    # partitioner that never saw it
+    X = torch.from_numpy(synth.mixture(n, 50, n_comp=7, seed=n)).cuda()
+    part, other = (rsc.Partitioner(50, P, H, bf16_weights=True, seed=H) for _ in range(2))
+    ws = torch.zeros(part.workspace_size(n, 0, 10, n, 8), dtype=torch.uint8, device="cuda")
+    rsc.rsc_set_wait_budget(300)
+    try:
+        part.build_index(X, workspace=ws)
+        assert rsc.rsc_workspace_status(ws) == rsc.RSC_ERR_TIMEOUT
+    finally:
+        rsc.rsc_set_wait_budget(0)
+    for p in (part, other):
+        p.build_index(X, workspace=ws)
+        assert rsc.rsc_workspace_status(ws) == rsc.RSC_OK
+    got, want = (p.knn(X, k=10, n_probe=8, workspace=ws) for p in (part, other))
+    assert rsc.rsc_workspace_status(ws) == rsc.RSC_OK
+    for a, b in zip(got, want):
+        np.testing.assert_array_equal(a.cpu().numpy(), b.cpu().numpy())
