@@ -339,8 +339,11 @@ __global__ void top_logits_kernel(int64_t rows, int P, const float *__restrict__
 
 // ----------------------------------------------- counting sort by part
 
-// A network that produced NaN logits leaves no part id: such a row counts to part 0.
+// Logits that are NaN leave no part id (INT_MAX).  A database row without one
+// counts to part 0, and a query without any starts there; a further probe
+// without one is no probe (-1): part 0 searched again would list its rows twice.
 __device__ __forceinline__ int safe_part(int p, int P) { return (p >= 0 && p < P) ? p : 0; }
+__device__ __forceinline__ int probe_part(int p, int r, int P) { return (p >= 0 && p < P) ? p : r == 0 ? 0 : -1; }
 
 __global__ void histogram_kernel(int64_t count, int P, const int32_t *__restrict__ key, int32_t *__restrict__ hist) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -396,7 +399,7 @@ __global__ void scatter_kernel(int64_t count, int P, const int32_t *__restrict__
 }
 
 // Probe slots: the probes r0 .. r0 + M - 1 of every query (route [nq, R]),
-// grouped by part.  Blocks of kGroupEntries (query, probe) entries rank their
+// grouped by part (probes without a part take no slot).  Blocks of kGroupEntries (query, probe) entries rank their
 // entries per part in shared memory and take one range of each part's cursor,
 // so a part's counter sees one atomic per block and not one per entry.  4M
 // entries over 512 parts: 35 us for the counts and 197 us for the slots and
@@ -413,14 +416,16 @@ group_count_kernel(int64_t nq, int R, int r0, int M, int P, const int32_t *__res
     for (int p = threadIdx.x; p < P; p += kGroupThreads) hist[p] = 0;
     __syncthreads();
     const int64_t e0 = (int64_t)blockIdx.x * kGroupEntries, e1 = min(nq * M, e0 + kGroupEntries);
-    for (int64_t e = e0 + threadIdx.x; e < e1; e += kGroupThreads)
-        atomicAdd(&hist[safe_part(route[(e / M) * R + r0 + e % M], P)], 1);
+    for (int64_t e = e0 + threadIdx.x; e < e1; e += kGroupThreads) {
+        const int r = r0 + (int)(e % M), p = probe_part(route[(e / M) * R + r], r, P);
+        if (p >= 0) atomicAdd(&hist[p], 1);
+    }
     __syncthreads();
     for (int p = threadIdx.x; p < P; p += kGroupThreads)
         if (hist[p]) atomicAdd(&cnt[p], hist[p]);
 }
 
-// gpos[q * M + m] = slot of the entry; operand row of the slot = the query's
+// gpos[q * M + m] = slot of the entry (-1: none); operand row of the slot = the query's
 // row of Qb (rows[q], or q0 + q), read in query order and written as whole
 // 128-byte rows; slot_thr[slot] = thr[q] when given.
 __global__ void __launch_bounds__(kGroupThreads)
@@ -443,8 +448,14 @@ group_slots_kernel(int64_t nq, int R, int r0, int M, int P, const int32_t *__res
         rank[i] = 0;
         if (x < here) {
             const int64_t e = e0 + x;
-            part[i] = safe_part(route[(e / M) * R + r0 + e % M], P);
-            rank[i] = atomicAdd(&cnt[part[i]], 1);
+            const int r = r0 + (int)(e % M);
+            part[i] = probe_part(route[(e / M) * R + r], r, P);
+            if (part[i] >= 0) {
+                rank[i] = atomicAdd(&cnt[part[i]], 1);
+            } else {
+                slot[x] = -1;
+                gpos[e] = -1;
+            }
         }
     }
     __syncthreads();
@@ -465,6 +476,7 @@ group_slots_kernel(int64_t nq, int R, int r0, int M, int P, const int32_t *__res
     }
     __syncthreads();
     for (int x = threadIdx.x; x < here * 8; x += kGroupThreads) {
+        if (slot[x >> 3] < 0) continue;
         const int64_t q = (e0 + (x >> 3)) / M;
         const int64_t row = rows ? (int64_t)rows[q] : q0 + q;
         Qg[(int64_t)slot[x >> 3] * 8 + (x & 7)] = Qb[row * 8 + (x & 7)];
@@ -571,12 +583,13 @@ rerank_probe_kernel(const float *__restrict__ X, int d, const int32_t *__restric
     for (int t = lane; t < 64; t += 32) xq[t] = t < d ? X[row * d + t] : 0.f;
     int count = 0;
     for (int r = 0; r < R; ++r) {
-        const int32_t *c = r == 0 ? cand0 + (int64_t)gpos0[q] * kPerSlot
-                                  : cand1 + (int64_t)gpos1[q * (R - 1) + r - 1] * kPerSlot;
+        const int32_t at = r == 0 ? gpos0[q] : gpos1[q * (R - 1) + r - 1];
+        const bool probed = at >= 0;   // no branch: the probes' lists are fetched together
+        const int32_t *c = (r == 0 ? cand0 : cand1) + (int64_t)max(at, 0) * kPerSlot;
 #pragma unroll
         for (int h = 0; h < kPerSlot; h += 32) {
             const int32_t j = c[h + lane];
-            const bool ok = j >= 0 && (int64_t)j < n_db;   // empty, dropped, or ids of an aborted search
+            const bool ok = probed && j >= 0 && (int64_t)j < n_db;   // empty, dropped, or ids of an aborted search
             const unsigned m = __ballot_sync(0xffffffffu, ok);
             if (ok) ids[count + __popc(m & ((1u << lane) - 1u))] = j;
             count += __popc(m);

@@ -192,3 +192,37 @@ def test_routing_that_gave_up_is_recorded_and_the_next_call_recovers(rsc, n, P, 
     assert rsc.rsc_workspace_status(ws) == rsc.RSC_OK
     for a, b in zip(got, want):
         np.testing.assert_array_equal(a.cpu().numpy(), b.cpu().numpy())
+
+
+@pytest.mark.parametrize("H", [32, 300])
+def test_probes_without_a_part_are_left_out(rsc, H):
+    # eight parts, some of whose logits are made NaN, -inf or very small by
+    # their bias, through the fused routing kernel and (H = 300) the GEMMs.
+    # A part with a NaN logit is not probed and nothing is probed twice; one at
+    # -inf is probed last.
+    n, d, P, k = 5_000, 20, 8, 10
+    X = torch.from_numpy(synth.mixture(n, d, n_comp=12, seed=4)).cuda()
+    part = rsc.Partitioner(d, P, H, bf16_weights=True, seed=1)
+    part.build_index(X)
+    params = part.get_params()
+
+    def knn(bias, n_probe):
+        w = params.copy()
+        w[-P:] += np.asarray(bias, dtype=np.float32)
+        part.set_params(w)
+        return [t.cpu().numpy() for t in part.knn(X, k=k, n_probe=n_probe)]
+
+    def same(a, b):
+        np.testing.assert_array_equal(a[0], b[0])
+        np.testing.assert_array_equal(a[1], b[1])
+
+    zero, low = np.zeros(P), -1e6
+    last = lambda v: np.r_[np.zeros(P - 4), np.full(4, v)]   # noqa: E731
+    four = knn(last(low), 4)
+    same(knn(last(np.nan), 8), four)
+    for row in four[0]:
+        found = row[row >= 0]
+        assert len(set(found.tolist())) == len(found)
+    same(knn(last(-np.inf), 8), knn(zero, 8))
+    same(knn(np.r_[0, np.full(P - 1, -np.inf)], 2), knn(np.r_[0, -1e5, np.full(P - 2, -1e6)], 2))
+    same(knn(np.full(P, np.nan), 8), knn(np.r_[0, np.full(P - 1, low)], 1))
