@@ -187,7 +187,9 @@ __global__ void targets_kernel(int B, int k, const int32_t *__restrict__ pos, co
     const int64_t b = e / k;
     const int c = (int)(e - b * k);
     const int32_t j = nbr[(int64_t)pos[b] * k + c];
-    if (j >= 0) atomicAdd(&T[b * P + labels[j]], 1.f / (float)k);
+    if (j < 0) return;
+    const int p = labels[j];
+    if (p >= 0 && p < P) atomicAdd(&T[b * P + p], 1.f / (float)k);   // a row with a NaN has no part
 }
 
 // Copy 128-byte operand rows: dst[i] = src[map[i]].
@@ -260,14 +262,17 @@ nearest_centroids_kernel(const float *__restrict__ X, const int32_t *__restrict_
         for (int r = 0; r < R; ++r) out[i * R + r] = bi[r];
 }
 
+// A row with a NaN component is at no distance from any centroid: it has no
+// label in [0, P) and joins no cluster.
 __global__ void kmeans_accum_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, int64_t npts,
-                                    int d, const int32_t *__restrict__ lab, float *__restrict__ sums,
+                                    int d, int P, const int32_t *__restrict__ lab, float *__restrict__ sums,
                                     int32_t *__restrict__ counts) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= npts * d) return;
     const int64_t i = e / d;
     const int t = (int)(e - i * d);
     const int c = lab[i];
+    if (c < 0 || c >= P) return;
     atomicAdd(&sums[(int64_t)c * d + t], X[(int64_t)rows[i] * d + t]);
     if (t == 0) atomicAdd(&counts[c], 1);
 }
@@ -1251,7 +1256,7 @@ rsc_status rsc_partitioner_train(rsc_partitioner *p, const float *X, int64_t n, 
         RSC_CUDA_TRY(cudaMemsetAsync(L.ksum, 0, sizeof(float) * P * d, st));
         RSC_CUDA_TRY(cudaMemsetAsync(L.kcnt, 0, sizeof(int32_t) * P, st));
         part::kmeans_accum_kernel<<<(unsigned)ceil_div(n_train * d, 256), 256, 0, st>>>(X, train_rows, n_train, d,
-                                                                                      L.labels, L.ksum, L.kcnt);
+                                                                                      P, L.labels, L.ksum, L.kcnt);
         part::kmeans_finalize_kernel<<<(unsigned)ceil_div(P * d, 256), 256, 0, st>>>(P, d, L.ksum, L.kcnt,
                                                                                    p->centroids);
     }

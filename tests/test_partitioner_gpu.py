@@ -226,3 +226,23 @@ def test_probes_without_a_part_are_left_out(rsc, H):
     same(knn(last(-np.inf), 8), knn(zero, 8))
     same(knn(np.r_[0, np.full(P - 1, -np.inf)], 2), knn(np.r_[0, -1e5, np.full(P - 2, -1e6)], 2))
     same(knn(np.full(P, np.nan), 8), knn(np.r_[0, np.full(P - 1, low)], 1))
+
+
+def test_training_with_a_row_that_is_no_number(rsc):
+    # the row has no nearest centroid: it joins no cluster and is nobody's
+    # target, and the centroids of the others stay numbers (with a NaN centroid,
+    # or none, eight probes would not reach every part)
+    n, d, k = 2_000, 20, 10
+    X = synth.mixture(n, d, n_comp=12, seed=9)
+    bad = X.copy()
+    bad[100, 3] = np.nan
+    part = rsc.Partitioner(d, 8, 32, bf16_weights=True, seed=2)
+    train = torch.arange(n, dtype=torch.int32, device="cuda")
+    part.train(torch.from_numpy(bad).cuda(), train, k=k, kmeans_iters=4, epochs=1, batch=256)
+    part.set_params(rsc.Partitioner(d, 8, 32, bf16_weights=True, seed=2).get_params())
+    Xd = torch.from_numpy(X).cuda()
+    part.build_index(Xd)
+    gi, gd = part.knn(Xd, k=k, n_probe=8, routing="centroids")
+    oi, od, _ = oracle.knn(X, k)
+    np.testing.assert_allclose(gd.cpu().numpy(), od, rtol=1e-5, atol=1e-6)
+    assert (gi.cpu().numpy() >= 0).all()
