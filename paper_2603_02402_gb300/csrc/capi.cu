@@ -595,7 +595,8 @@ rsc_status rsc_knn(const float *X, int64_t n, int32_t d, int32_t k, int32_t metr
         const int width = d + (metric == RSC_COSINE ? 1 : 0);
         RSC_CUDA_TRY(launch_rerank_parts(R, rsr, n, d, metric, simt_flat_parts(L.prune_scratch, n, p.DP, k), width, k,
                                          idx, dist, st));
-        RSC_CUDA_TRY(launch_simt_flat_ties(n, d, p.DP, width, k, metric, L.prune_scratch, R, rsr, idx, dist, st));
+        RSC_CUDA_TRY(launch_simt_flat_ties(n, d, p.DP, width, k, metric, L.prune_scratch, R, rsr, idx, dist, L.status,
+                                           st));
         if (ev) RSC_CUDA_TRY(cudaEventRecord(ev[3], st));
         return RSC_OK;
     }
@@ -603,7 +604,7 @@ rsc_status rsc_knn(const float *X, int64_t n, int32_t d, int32_t k, int32_t metr
                                st));
     if (p.simt_prune)
         RSC_CUDA_TRY(launch_simt_ties(n, d, p.DP, d + (metric == RSC_COSINE ? 1 : 0), k, metric, L.prune_scratch, R,
-                                      rsr, idx, dist, st));
+                                      rsr, idx, dist, L.status, st));
     if (ev) RSC_CUDA_TRY(cudaEventRecord(ev[3], st));
     return RSC_OK;
 }

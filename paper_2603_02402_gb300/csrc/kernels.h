@@ -42,20 +42,22 @@ cudaError_t launch_knn_simt_pruned(const float *Y, const float *ny, int64_t n, i
                                    const int32_t *perm, const OrderLeaves &leaves, void *scratch, int32_t *cand,
                                    unsigned int *status, cudaStream_t st);
 cudaError_t launch_simt_ties(int64_t n, int d, int DP, int width, int k, int metric, void *scratch, const float *R,
-                             int64_t rs, int32_t *idx, float *dist, cudaStream_t st);
+                             int64_t rs, int32_t *idx, float *dist, unsigned int *status, cudaStream_t st);
 
 // The FP32 search of rows in their own order, k <= 32 (fewer than
 // kSimtPruneMinRows): every query's lists of simt_flat_segs parts of the
 // database, merged and re-ranked by launch_rerank_parts, ties as above.
 constexpr int kSimtFlatSegs = 16;
+constexpr int kTieItem = 128;   // rows the ties pass takes together
 struct SimtParts {
     const float *key;     // [n rounded up to 128][segs][list], each list ascending
     const int32_t *id;    // row ids, -1 pads
     const float *vv;      // |y|^2 of every row
     int segs, list;
-    int *tie_count;       // rows for the ties pass
-    int32_t *tie_rows;    // (row, place in the records)
-    float *tie_bound;
+    int *tie_count;       // items (128 rows) for the ties pass
+    int *tie_flag;        // [items] on the list already (zeroed)
+    int32_t *tie_items;
+    float *tie_bound;     // [row] its reach, -inf when the row is not for the pass
 };
 int simt_flat_segs(int64_t n, int DP);
 size_t simt_flat_scratch_bytes(int64_t n, int DP, int k);
@@ -63,7 +65,7 @@ SimtParts simt_flat_parts(void *scratch, int64_t n, int DP, int k);
 cudaError_t launch_knn_simt_flat(const float *Y, const float *ny, int64_t n, int DP, int width, int k, void *scratch,
                                  unsigned int *status, cudaStream_t st);
 cudaError_t launch_simt_flat_ties(int64_t n, int d, int DP, int width, int k, int metric, void *scratch, const float *R,
-                                  int64_t rs, int32_t *idx, float *dist, cudaStream_t st);
+                                  int64_t rs, int32_t *idx, float *dist, unsigned int *status, cudaStream_t st);
 
 // ---- knn_tc.cu ------------------------------------------------------------
 // BF16 tensor-core candidate search.  Qb/Db: [n, 64 * tc_kb(d, metric)] bf16

@@ -23,7 +23,8 @@
 // k nearest are always among the kept ones and the result is that of the full
 // scan.  Lists hold KC > k entries; a row whose list is full of entries within
 // its bound (many rows at nearly the same distance as the k-th) is finished by
-// ties_kernel, which scores every such row by the re-rank's own arithmetic.
+// a second search of its item (kTies), which scores every row within the bound
+// by the re-rank's own arithmetic.
 //
 // Tiles hold 64 consecutive rows, cut anew wherever two successive leaves of
 // the ordering lie apart (the tile before is padded): a tile across such a gap
@@ -53,6 +54,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -65,11 +67,14 @@ namespace rsc {
 namespace simtp {
 
 constexpr int kQ = 128;                   // query rows per item, threads per CTA
+static_assert(kQ == kTieItem && kQ <= 512, "ties items; 16 bits a hit");
 constexpr int kR = 64;                    // database rows per tile
 constexpr int kPitch = kR + 4;            // s rows on 16 bytes, conflict-free scans
 constexpr int kCap = 20;                  // top-k buffer entries per thread
 constexpr int kChunk = 256;               // tiles tested at a time
 constexpr int kWords = kChunk / 32;
+constexpr int kExactFirst = 2, kExactStep = 16;   // tiles between two looks at the bounds in the ties pass
+constexpr int kBatch = 1024;              // hits of the ties pass scored at a time
 constexpr int kSeeds = 8;                 // nearest tiles scanned first when the window's do not bound an item
 constexpr int kWin = 3;                   // tiles on each side of the query tile scanned first
 constexpr int kStages = 2;
@@ -192,10 +197,11 @@ __global__ void __launch_bounds__(256)
 pack_kernel(const float *__restrict__ Y, const float *__restrict__ ny, int DP, const int32_t *__restrict__ perm,
             int64_t tiles, const int32_t *__restrict__ tile_pos, int32_t *__restrict__ tile_rows,
             const int32_t *__restrict__ T, float *__restrict__ rec, int32_t *__restrict__ ids,
-            float *__restrict__ cenT, float *__restrict__ rad, float *__restrict__ nmax) {
+            float *__restrict__ cenT, float *__restrict__ rad, float *__restrict__ nmax, int32_t *__restrict__ id_min) {
     __shared__ float ys[64][kR + 1];
     __shared__ float cen[64];
     __shared__ float red[2][8];
+    __shared__ int first_id[8];
     const int64_t t = blockIdx.x;
     const int last = *T;
     if (t > last || (t == last && (last & 1) == 0)) return;   // an empty tile completes an odd count
@@ -217,7 +223,9 @@ pack_kernel(const float *__restrict__ Y, const float *__restrict__ ny, int DP, c
     }
     nn += __shfl_xor_sync(0xffffffffu, nn, 1);
     nn += __shfl_xor_sync(0xffffffffu, nn, 2);
-    if (l == 0) ids[t * kR + r] = r < rows ? (int32_t)o : INT_MAX;
+    const int own_id = r < rows ? (int32_t)o : INT_MAX, least = __reduce_min_sync(0xffffffffu, own_id);
+    if (l == 0) ids[t * kR + r] = own_id;
+    if ((tid & 31) == 0) first_id[tid >> 5] = least;
     __syncthreads();
     float *out = rec + t * record_floats(DP);
     for (int e = tid; e < DP * kR; e += 256) out[e] = ys[e >> 6][e & 63];
@@ -254,7 +262,9 @@ pack_kernel(const float *__restrict__ Y, const float *__restrict__ ny, int DP, c
         for (int w = 1; w < 8; ++w) {
             md = fmaxf(md, red[0][w]);
             mn = fmaxf(mn, red[1][w]);
+            first_id[0] = min(first_id[0], first_id[w]);
         }
+        id_min[t] = first_id[0];
         rad[t] = rows > 0 ? sqrtf(md) * (1.f + 0x1p-10f) + 1e-6f : -1.f;   // -1: an empty tile
         nmax[t] = mn;
     }
@@ -265,11 +275,15 @@ pack_kernel(const float *__restrict__ Y, const float *__restrict__ ny, int DP, c
 // The KC smallest s of one query in registers (RowTopK), fed through a
 // per-thread shared-memory buffer as BufferedTopK is, with the row's bound as
 // the filter.  Equal values beyond the list's end are dropped whatever their
-// ids: such a row is finished by ties_kernel.
+// ids: such a row is finished by the ties pass.  That is settled once a list is
+// full of entries within reach of its k-th, and from then on it takes in only
+// what lies below the k-th (rows that are all the same would otherwise buffer
+// every value they meet).
 template <int KC>
 struct List {
     RowTopK<KC> top;
-    float bound;          // values above it cannot be among the k nearest
+    float bound;          // values above it cannot be among the k nearest, or are left to the ties pass:
+    float floor;          // values from here on may have been left out
     float vv, v2;         // |y_i|^2 and |y_i|
     uint32_t sbase;
     int cnt, k, w;
@@ -279,6 +293,7 @@ struct List {
 #pragma unroll
         for (int c = 0; c < KC; ++c) top.key[c] = FLT_MAX;   // finite: infinite values are never accepted
         bound = FLT_MAX;
+        floor = INFINITY;
         vv = nn;
         v2 = sqrtf(nn);
         cnt = 0;
@@ -286,11 +301,18 @@ struct List {
         w = w_;
     }
     __device__ __forceinline__ float reach_of(float t) const { return rr::reach(t, vv, v2, w); }
-    __device__ __forceinline__ float reach() const {
+    __device__ __forceinline__ float kth() const {
         float t = top.key[0];
 #pragma unroll
         for (int c = 1; c < KC; ++c) t = fmaxf(t, c < k ? top.key[c] : -FLT_MAX);   // ascending: the k-th
-        return reach_of(t);
+        return t;
+    }
+    __device__ __forceinline__ float reach() const { return reach_of(kth()); }
+    // The list is final: its last key tells what was left out.  A last entry
+    // within the reach of the final k-th then means that the list is short of
+    // some row.
+    __device__ __forceinline__ void finish() {
+        if (floor <= reach()) top.key[KC - 1] = fminf(top.key[KC - 1], floor);
     }
     __device__ __forceinline__ void flush() {   // warp-synchronous
         const int rounds = __reduce_max_sync(0xffffffffu, cnt);
@@ -307,6 +329,18 @@ struct List {
         }
         cnt = 0;
         bound = fminf(bound, fminf(top.thr(), reach()));
+    }
+    // Between two scans: whether the row is one for the ties pass by now.
+    __device__ __forceinline__ void settle() {
+        const float t = kth();
+        if (top.id[KC - 1] >= 0 && top.thr() <= reach_of(t) && t < floor) {
+            floor = t;
+            bound = fminf(bound, below(t));
+        }
+    }
+    static __device__ __forceinline__ float below(float t) {   // the next smaller float
+        const int b = __float_as_int(t);
+        return __int_as_float(t > 0.f ? b - 1 : t < 0.f ? b + 1 : (int)0x80000001);
     }
     // An empty list whose first tile is known: the largest of its 16 minima
     // of four (k <= 16) or 32 minima of two bounds the k-th smallest, so what
@@ -364,16 +398,20 @@ struct Args {
     const float *rec;
     const int32_t *ids, *tile_pos, *tile_rows, *T;
     const float *cenT, *rad, *nmax;
+    const int32_t *id_min;  // smallest row id of a tile
     int64_t n, stride;      // rows; stride of cenT (tiles_max)
     int DP, width, k;
     float beta;
     int32_t *cand;          // [n, KC] positions, -1 for none
-    int32_t *tie_rows;      // rows for ties_kernel
-    float *tie_bound;       // (tie_rows: sorted position, then the row's place in the records)
+    int32_t *tie_items;     // items with rows for the ties pass
+    float *tie_bound;       // [item * kQ + row] their reach (-inf: not such a row), items on the list only
     int *tie_count, *counter;
+    int *tie_done;          // parts of a tie item that are done
+    int64_t tie_units;      // lists the parts of tie items may take (kQ rows each)
     uint32_t *bits;         // [CTAs][stride / 32] tiles an item keeps
     int32_t *big;           // [kBigItems][1 + kSeeds] items to be split, their seeds (-1 pads)
     int *big_count, *unit;  // their number (may exceed kBigItems), next part
+    int *tie_unit;          // next part of a tie item
     float *part_key;        // [query slots][part_segs][KC] lists of the parts; a slot is a query
     int32_t *part_id;       // tile pair's (split: position in `big`; flat: item) kQ rows
     int part_segs;
@@ -389,23 +427,106 @@ __device__ __forceinline__ int64_t seg_tiles(int64_t tiles) {
     return ceil_div(tiles, s);
 }
 
-// The candidates of an item's query row, and the row itself for ties_kernel if
-// more rows may lie within reach than the list holds.
+// The candidates of an item's rows (a thread each; lists finished), and the
+// item for the ties pass if more rows may lie within reach of one than its list
+// holds (cut: a part's list was short).
 template <int KC>
-__device__ __forceinline__ void emit(const Args &g, const List<KC> &tk, int64_t item, int tid) {
-    const int64_t q = g.tile_pos[2 * item + (tid >> 6)] + (tid & 63);
-    int32_t *out = g.cand + q * KC;
+__device__ __forceinline__ void emit(const Args &g, const List<KC> &tk, int64_t item, int tid, bool live, bool cut) {
     const float reach = tk.reach();
+    if (live) {
+        int32_t *out = g.cand + (g.tile_pos[2 * item + (tid >> 6)] + (tid & 63)) * (int64_t)KC;
 #pragma unroll
-    for (int c = 0; c < KC; ++c) {
-        out[c] = tk.top.key[c] <= reach ? tk.top.id[c] : -1;   // -1 also where empty
+        for (int c = 0; c < KC; ++c) {
+            out[c] = tk.top.key[c] <= reach ? tk.top.id[c] : -1;   // -1 also where empty
+        }
     }
-    if (tk.top.id[KC - 1] >= 0 && tk.top.key[KC - 1] <= reach) {
-        const int x = atomicAdd(g.tie_count, 1);
-        g.tie_rows[2 * x] = (int32_t)q;
-        g.tie_rows[2 * x + 1] = (int32_t)(item * kQ + tid);
-        g.tie_bound[x] = reach;
+    const bool tie = live && (cut || (tk.top.id[KC - 1] >= 0 && tk.top.key[KC - 1] <= reach));
+    if (__syncthreads_or(tie)) {
+        g.tie_bound[item * kQ + tid] = tie ? reach : -INFINITY;
+        if (tid == 0) g.tie_items[atomicAdd(g.tie_count, 1)] = (int32_t)item;
     }
+}
+
+// ---------------------------------------------------------------------- ties
+
+// The ties pass: the rows of the items on the tie list once more, against the
+// tiles that their bounds keep, in the tiled search's own way; a value within
+// a row's bound is a hit.  The block scores a tile's hits together, a thread each,
+// with the re-rank's arithmetic (one row may have all of them), and a thread takes
+// the scores of its own row into the k smallest (distance, id).  A row's list full of zeros
+// needs no larger id any more, scored or not, and a tile whose smallest id
+// is past those of all rows is left out: equal rows end after a few tiles.
+// What it costs, whole calls, k = 15 (in brackets a warp per row over all
+// tiles, hits scored one by one; then the full scan, which drops ties beyond its
+// lists): 100,000 equal rows 2.9 ms (about 1,500; 25.8), 20,000 of them 2.2 (58;
+// 1.4); 100,000 rows of one component 2.8 (41; 9.5); 100,000 clustered rows of 50,
+// 5 % of them in groups of 30 copies, 2.2 (18; 25.9); 50,000 rows of 50 zeros and
+// ones, which no sphere separates, 10.4 (31; 7.3).  The worst is a row as far from
+// most others: 99,990 copies of a row and ten others 33 ms (25.9).
+template <int KE>
+struct Exact {
+    static constexpr unsigned long long kNone = 0x7f8000007fffffffull;   // (+inf, INT_MAX)
+    unsigned long long best[KE];   // (bits of the squared distance, id), ascending
+    float bound;                   // -inf: nothing is wanted
+    float vv, v2, beta;            // |y_i|^2 and |y_i|; what s leaves out of a squared distance besides
+    int w;
+
+    __device__ __forceinline__ void start(float bound_, float nn, float beta_, int w_) {
+#pragma unroll
+        for (int c = 0; c < KE; ++c) best[c] = kNone;
+        bound = bound_;
+        vv = nn;
+        v2 = sqrtf(nn);
+        beta = beta_;
+        w = w_;
+    }
+    __device__ __forceinline__ void insert(unsigned long long v) {
+        if (!(v < best[KE - 1])) return;
+#pragma unroll
+        for (int c = KE - 1; c > 0; --c) best[c] = v < best[c - 1] ? best[c - 1] : v < best[c] ? v : best[c];
+        if (v < best[0]) best[0] = v;
+        // a row at a squared distance D has s within e of D - vv - beta
+        if (best[KE - 1] < kNone)
+            bound = fminf(bound, rr::reach(__uint_as_float((unsigned)(best[KE - 1] >> 32)) - vv - beta, vv, v2, w));
+    }
+    // nothing but zeros with smaller ids than this one
+    __device__ __forceinline__ bool full_before(int id) const { return best[KE - 1] <= (unsigned)id; }
+};
+
+// What the ties pass scores and where it puts it.
+struct TieArgs {
+    const float *R;   // the re-rank's rows, by position
+    int64_t rs;
+    int d;
+    bool cosine, vec;
+    int32_t *idx;
+    float *dist;
+
+    // (squared distance, id) of the rows at positions a and b, `id` the one of b
+    __device__ __forceinline__ unsigned long long score(int64_t a, int64_t b, int id) const {
+        const float *x = R + a * rs, *y = R + b * rs;
+        float key = rr::dist2_thread(x, y, d, cosine, vec);
+        if (cosine) {
+            const bool fx = x[d] != 0.f, fy = y[d] != 0.f;   // rows of zeros
+            if (fx || fy) key = (fx && fy) ? 0.f : 2.f;
+        }
+        return (unsigned long long)__float_as_uint(key) << 32 | (unsigned)id;
+    }
+};
+
+// Parts of a tie item: the count whose waves cost least, as far as the parts'
+// lists have room (one part needs none).
+__device__ __forceinline__ int tie_segs(const Args &g, int64_t count, int64_t tiles, int64_t slots) {
+    int best = 1;
+    int64_t cost = INT64_MAX;
+    for (int s = 1; s <= kSegs && (s == 1 || (count * s <= g.tie_units && tiles >= 8 * s)); ++s) {
+        const int64_t c = ceil_div(count * s, slots) * (ceil_div(tiles, (int64_t)s) + 3);
+        if (c < cost) {
+            cost = c;
+            best = s;
+        }
+    }
+    return best;
 }
 
 // kSplit = false: an item per query tile pair.  An item that keeps more than
@@ -416,10 +537,14 @@ __device__ __forceinline__ void emit(const Args &g, const List<KC> &tk, int64_t 
 // the item's own surroundings on, whose lists merge_kernel joins.
 // kFlat: rows in their own order, part_segs parts per item and no tests: the
 // search of fewer rows than an ordering pays for (see launch_knn_simt_flat).
-enum { kWhole, kSplitItems, kFlat };
+// kTies, kFlatTies: the ties pass after either search (KC: Exact's entries).
+enum { kWhole, kSplitItems, kFlat, kTies, kFlatTies };
 template <int KC, int kMode>
-__global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
-    constexpr bool kSplit = kMode == kSplitItems, kIsFlat = kMode == kFlat;
+__global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const TieArgs ta) {
+    constexpr bool kSplit = kMode == kSplitItems, kIsFlat = kMode == kFlat || kMode == kFlatTies;
+    constexpr bool kExact = kMode == kTies || kMode == kFlatTies;
+    const int64_t tie_items = kExact ? *g.tie_count : 0;
+    if (kExact && tie_items == 0) return;
     extern __shared__ __align__(128) uint8_t sm[];
     const int DP = g.DP;
     const Smem m = smem_layout(DP);
@@ -442,8 +567,8 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
         tc::fence_barrier_init();
     }
     __syncthreads();
-    List<KC> tk;
-    tk.sbase = (uint32_t)__cvta_generic_to_shared(reinterpret_cast<float *>(sm + m.buf) + tid);
+    typename std::conditional<kExact, Exact<KC>, List<KC>>::type tk;
+    if constexpr (!kExact) tk.sbase = (uint32_t)__cvta_generic_to_shared(reinterpret_cast<float *>(sm + m.buf) + tid);
     // bounded; a budget shorter than a few sleeps is polled
     const uint32_t sleep_ns = g.wait_budget < 8 * (long long)kSleepNs ? 0 : kSleepNs;
     auto wait = [&](uint64_t *bar, uint32_t parity, long long budget) -> bool {
@@ -457,10 +582,17 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
         return true;
     };
     const int64_t tiles = *g.T;   // an odd count is followed by an empty tile
-    const int64_t seg_len = kIsFlat ? ceil_div(tiles, (int64_t)g.part_segs) : seg_tiles(tiles);
-    const int segs = kIsFlat ? g.part_segs : (int)ceil_div(tiles, seg_len);
+    const int64_t seg_len = kExact    ? ceil_div(tiles, (int64_t)tie_segs(g, tie_items, tiles, gridDim.x))
+                            : kIsFlat ? ceil_div(tiles, (int64_t)g.part_segs)
+                                      : seg_tiles(tiles);
+    const int segs = kMode == kFlat ? g.part_segs : (int)ceil_div(tiles, seg_len);
     const int64_t pairs = ceil_div(tiles, (int64_t)2);
-    const int64_t units = kIsFlat ? pairs * segs : kSplit ? (int64_t)min(*g.big_count, kBigItems) * segs : pairs;
+    const int64_t units = kExact            ? tie_items * segs
+                          : kMode == kFlat ? pairs * segs
+                          : kSplit         ? (int64_t)min(*g.big_count, kBigItems) * segs
+                                           : pairs;
+    bool live = false;       // the thread has a query row
+    int64_t cur_item = 0;
     uint32_t tile_no = 0;     // tiles consumed by this CTA so far (stage tile_no % kStages)
     uint32_t items = 0;
     unsigned long long scanned = 0;
@@ -533,6 +665,60 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
             if (tid == 0 && i + 2 < nl) issue(tile_no + 2, list[i + 2]);
             const float *sr = S + tid * kPitch;
             const int tt = list[i], j0 = g.tile_pos[tt];
+            if constexpr (kExact) {
+                // this row's hits, and their places among the block's
+                unsigned hit[2] = {0u, 0u};
+                if (live && !tk.full_before(kIsFlat ? j0 : g.id_min[tt])) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll 8
+                        for (int c = 0; c < 32; c += 4) {
+                            const float4 v = *reinterpret_cast<const float4 *>(sr + 32 * h + c);
+                            hit[h] |= (v.x <= tk.bound ? 1u : 0u) << c | (v.y <= tk.bound ? 2u : 0u) << c |
+                                      (v.z <= tk.bound ? 4u : 0u) << c | (v.w <= tk.bound ? 8u : 0u) << c;
+                        }
+                }
+                int at = __popc(hit[0]) + __popc(hit[1]);
+                const int mine = at;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, at, o);
+                    if (lane >= o) at += y;
+                }
+                if (lane == 31) seeds[warp] = at;
+                __syncthreads();
+                int total = 0;
+                at -= mine;
+#pragma unroll
+                for (int w = 0; w < kQ / 32; ++w) {
+                    if (w < warp) at += seeds[w];
+                    total += seeds[w];
+                }
+                unsigned long long *keys = reinterpret_cast<unsigned long long *>(sm + m.buf);   // [kBatch]
+                uint16_t *pair = reinterpret_cast<uint16_t *>(keys + kBatch);                    // row, column
+                const int32_t *tile_ids = g.ids + (int64_t)tt * kR;
+                int end = at;   // hits of this row listed so far
+                for (int b0 = 0; b0 < total; b0 += kBatch) {
+                    const int from = end;
+                    for (; (hit[0] | hit[1]) != 0 && end < b0 + kBatch; ++end) {
+                        const int h = hit[0] != 0 ? 0 : 1, c = __ffs(h ? hit[1] : hit[0]) - 1;
+                        if (h) hit[1] &= hit[1] - 1;
+                        else hit[0] &= hit[0] - 1;
+                        pair[end - b0] = tk.full_before(tile_ids[32 * h + c]) ? 0xffffu : (uint16_t)(tid << 6 | 32 * h | c);
+                    }
+                    __syncthreads();
+                    for (int x = tid; x < min(kBatch, total - b0); x += kQ) {
+                        const int rc = pair[x], row = rc >> 6, c = rc & 63;
+                        keys[x] = rc == 0xffff ? Exact<KC>::kNone
+                                               : ta.score(g.tile_pos[2 * cur_item + (row >> 6)] + (row & 63), j0 + c, tile_ids[c]);
+                    }
+                    __syncthreads();
+                    for (int x = from; x < end; ++x) tk.insert(keys[x - b0]);
+                    __syncthreads();   // the lists and seeds may be rewritten
+                }
+                if (total == 0) __syncthreads();
+                continue;
+            } else {
             if (first && i == 0 && g.tile_rows[tt] == kR) tk.start_bound(sr);   // a full tile, empty lists
 #pragma unroll 1
             for (int h = 0; h < kR; h += 8) {
@@ -540,20 +726,24 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
                 const float v[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
                 tk.offer8(v, j0 + h);
             }
+            }
         }
         scanned += nl;
-        tk.flush();
+        if constexpr (!kExact) {
+            tk.flush();
+            if constexpr (kMode != kFlat) tk.settle();   // (a flat part is one scan, or a few)
+        }
         __syncthreads();   // the list may be rewritten
         return true;
     };
     for (;; ++items) {
         __syncthreads();
-        if (tid == 0) *item_s = atomicAdd(kSplit ? g.unit : g.counter, 1);
+        if (tid == 0) *item_s = atomicAdd(kExact ? g.tie_unit : kSplit ? g.unit : g.counter, 1);
         __syncthreads();
         const int64_t unit = *item_s;
         if (unit >= units) break;
         const int32_t *big = g.big + unit / segs * (1 + kSeeds);   // kSplit
-        const int64_t item = kSplit ? (int64_t)big[0] : kIsFlat ? unit / segs : unit;
+        const int64_t item = kExact ? (int64_t)g.tie_items[unit / segs] : kSplit ? (int64_t)big[0] : kIsFlat ? unit / segs : unit;
         if (tid == 0) {
             tc::mbar_arrive_expect_tx(xfull, 2 * x_bytes);
             tc::bulk_load(xs, g.rec + (2 * item) * rf, x_bytes, xfull);
@@ -569,11 +759,17 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
             if (tid == 0) wait(xfull, items & 1, kDrainBudget);
             return;
         }
-        const bool live = (tid & 63) < g.tile_rows[2 * item + (tid >> 6)];
+        live = (tid & 63) < g.tile_rows[2 * item + (tid >> 6)];
         float nn = 0.f;
         const float *xr = xs + (tid >> 6) * DP * kR + (tid & 63);
         for (int t = 0; t < g.width; ++t) nn = fmaf(xr[t * kR], xr[t * kR], nn);
-        tk.start(nn, g.k, g.width);
+        if constexpr (kExact) {
+            tk.start(live ? g.tie_bound[item * kQ + tid] : -INFINITY, nn, g.beta, g.width);
+            live = tk.bound > -INFINITY;
+            cur_item = item;
+        } else {
+            tk.start(nn, g.k, g.width);
+        }
         float rq[2] = {0.f, 0.f}, nq[2] = {0.f, 0.f};
         if (!kIsFlat) {
             rq[0] = g.rad[2 * item];
@@ -581,11 +777,12 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
             nq[0] = g.nmax[2 * item];
             nq[1] = g.nmax[2 * item + 1];
         }
-        const int wlo = (int)max((int64_t)0, 2 * item - kWin), whi = (int)min(tiles, 2 * item + 2 + kWin);
+        const int wlo = kExact ? 0 : (int)max((int64_t)0, 2 * item - kWin);
+        const int whi = kExact ? 0 : (int)min(tiles, 2 * item + 2 + kWin);
         // the range of tiles in chunks, from the chunk of the query tiles on
         const int64_t lo = kMode != kWhole ? min(tiles, (unit % segs) * seg_len) : 0;
         const int64_t hi = kMode != kWhole ? min(tiles, lo + seg_len) : tiles;
-        const int chunks = (int)ceil_div(hi - lo, (int64_t)kChunk), c0 = kSplit ? 0 : (int)((2 * item) / kChunk);
+        const int chunks = (int)ceil_div(hi - lo, (int64_t)kChunk), c0 = kMode != kWhole ? 0 : (int)((2 * item) / kChunk);
         const int64_t most = max((int64_t)64, tiles / 16);
         uint32_t *bits = g.bits + (int64_t)blockIdx.x * ceil_div(tiles, (int64_t)kChunk) * kWords;
         // The lists live in registers, so there is one scan call, and what it
@@ -598,25 +795,39 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
         //   kAgain   (no scan) the marks once more; still many: the item is split
         //   kChunks  the marked tiles, chunk by chunk, tested against the
         //            bounds as they are by then
-        // A part of a split item goes from kWindow over its seeds to kChunks.
+        // A part of a split item goes from kWindow over its seeds to kChunks; the
+        // ties pass, whose bounds are known, has kChunks only.
         enum { kWindow, kMark, kNearest, kAgain, kChunks };
-        int step = kWindow, ci = 0, n_seeds = 0;
+        int step = kExact ? kChunks : kWindow, ci = 0, n_seeds = 0;
         int64_t kept = 0;
         float near_d[2] = {INFINITY, INFINITY}, tq[2] = {INFINITY, INFINITY};
         int near_t[2] = {-1, -1};
-        bool fresh = true, deferred = false;   // fresh: tq must be taken anew
+        bool fresh = true, deferred = false, all_ties = false;   // fresh: tq must be taken anew
         if (kSplit) {
             if (tid < kSeeds) seeds[tid] = big[1 + tid];
             while (n_seeds < kSeeds && big[1 + n_seeds] >= 0) ++n_seeds;
         }
-        int64_t done = 0;   // flat: tiles of the part scanned so far
+        int64_t done = 0;   // flat, exact: tiles of the part seen so far
         bool first = true;
+        // exact: rows of ids from here on are wanted by no row (INT_MAX: some may be)
+        auto last_id = [&]() -> int {
+            unsigned v = 0;
+            if constexpr (kExact) v = !live ? 0u : tk.best[KC - 1] <= 0xffffffffull ? (unsigned)tk.best[KC - 1] : (unsigned)INT_MAX;
+            v = __reduce_max_sync(0xffffffffu, v);
+            if (lane == 0) seeds[warp] = (int)v;
+            __syncthreads();
+            const int most_id = max(max(seeds[0], seeds[1]), max(seeds[2], seeds[3]));
+            __syncthreads();
+            return most_id;
+        };
+        int id_end = INT_MAX;
         while (true) {
             int nl = 0;
             if (kIsFlat) {   // the part's tiles, from the query's own on when they are among them
-                const int64_t len = hi - lo, from = 2 * item >= lo && 2 * item < hi ? 2 * item - lo : 0;
-                nl = (int)min((int64_t)kChunk, len - done);
+                const int64_t len = hi - lo, from = !kExact && 2 * item >= lo && 2 * item < hi ? 2 * item - lo : 0;
+                nl = (int)min((int64_t)(!kExact ? kChunk : first ? kExactFirst : kExactStep), len - done);
                 if (nl <= 0) break;
+                if (kExact && (lo + done) * kR >= last_id()) break;   // uniform; ids ascend
                 for (int x = tid; x < nl; x += kQ) {
                     const int64_t at = from + done + x;
                     list[x] = (int)(lo + (at < len ? at : at - len));
@@ -630,7 +841,7 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
                 nl = n_seeds;
                 if (tid < nl) list[tid] = seeds[tid];
             } else {
-                if (ci == chunks) {
+                if (kExact ? lo + done >= hi : ci == chunks) {
                     if (step == kChunks) break;
                     ci = 0;
                     if (kept > most && step == kMark) {   // the nearest tile of every (warp, half)
@@ -664,6 +875,15 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
                         step = kNearest;
                         continue;
                     }
+                    if constexpr (kMode == kWhole) {
+                        // many tiles, and most rows are for the ties pass already:
+                        // all of them, with the bounds they have
+                        if (kept > most && step == kAgain &&
+                            2 * __syncthreads_count(live && tk.floor < INFINITY) >= __syncthreads_count(live)) {
+                            all_ties = true;
+                            break;
+                        }
+                    }
                     if (kept > most && step == kAgain) {
                         if (tid == 0) {
                             const int at = atomicAdd(g.big_count, 1);
@@ -681,10 +901,10 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
                     continue;
                 }
                 const int chunk = c0 + ci < chunks ? c0 + ci : c0 + ci - chunks;
-                const int64_t base = lo + (int64_t)chunk * kChunk;
+                const int64_t base = kExact ? lo + done : lo + (int64_t)chunk * kChunk;
                 uint32_t *word = bits + chunk * kWords;
                 ++ci;
-                const bool all = kSplit || step == kMark;
+                const bool all = kMode != kWhole || step == kMark;
                 if (!all) {
                     uint32_t any = 0;
 #pragma unroll
@@ -692,7 +912,7 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
                     if (any == 0) continue;
                 }
                 if (fresh) {   // the tiles' bounds (dead rows ask for nothing)
-                    float tau = live ? tk.bound + tk.vv : -INFINITY;
+                    float tau = live ? tk.bound + nn : -INFINITY;
                     if (live && !(tau < INFINITY)) tau = INFINITY;   // also NaN
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) tau = fmaxf(tau, __shfl_xor_sync(0xffffffffu, tau, o));
@@ -700,6 +920,7 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
                     __syncthreads();
                     tq[0] = fmaxf(redf[0], redf[1]);
                     tq[1] = fmaxf(redf[2], redf[3]);
+                    if (kExact) id_end = last_id();
                     fresh = false;
                 }
 #pragma unroll 1
@@ -727,6 +948,7 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
                                 near_t[h] = (int)t;
                             }
                         }
+                        if (kExact) keep &= g.id_min[t] < id_end;
                         if (step != kMark)
                             for (int y = 0; y < n_seeds; ++y) keep &= seeds[y] != (int)t;
                     }
@@ -741,6 +963,12 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
                         if (wd % 4 == warp && (b >> lane & 1u))
                             list[nl + __popc(b & ((1u << lane) - 1u))] = (int)base + wd * 32 + lane;
                         nl += __popc(b);
+                    }
+                    if (kExact) {   // few at a time, fewer at first: the bounds fall quickly
+                        const int few = first ? kExactFirst : kExactStep;
+                        __syncthreads();
+                        done += nl > few ? list[few - 1] + 1 - base : (int64_t)kChunk;
+                        nl = min(nl, few);
                     }
                 } else {
                     if (tid < kWords) word[tid] = masks[tid];
@@ -761,7 +989,44 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
                 kept = 0;
             }
         }
-        if (kMode != kWhole) {
+        if constexpr (kExact) {
+            // parts leave their lists to the one that is done last
+            const int64_t pos = unit / segs;
+            bool last = true;
+            if (segs > 1) {
+                unsigned long long *lists = reinterpret_cast<unsigned long long *>(g.part_key);
+                auto list_of = [&](int64_t u) { return lists + (u * kQ + tid) * KC; };
+                if (live)
+#pragma unroll
+                    for (int c = 0; c < KC; ++c) __stcg(list_of(unit) + c, tk.best[c]);
+                __threadfence();
+                __syncthreads();
+                if (tid == 0) *item_s = atomicAdd(g.tie_done + pos, 1) == segs - 1;
+                __syncthreads();
+                last = *item_s != 0;
+                if (last && live) {
+                    __threadfence();
+                    for (int64_t u = pos * segs; u < (pos + 1) * segs; ++u)
+                        for (int c = 0; u != unit && c < KC; ++c) {
+                            const unsigned long long v = __ldcg(list_of(u) + c);
+                            if (!(v < tk.best[KC - 1])) break;   // ascending
+                            tk.insert(v);
+                        }
+                }
+            }
+            if (last && live) {
+                const int64_t o = (int64_t)g.ids[item * kQ + tid] * g.k;
+#pragma unroll
+                for (int c = 0; c < KC; ++c)
+                    if (c < g.k) {
+                        const int id = (int)(unsigned)tk.best[c];
+                        const float d2 = __uint_as_float((unsigned)(tk.best[c] >> 32));
+                        ta.idx[o + c] = id != INT_MAX ? id : -1;
+                        ta.dist[o + c] = id != INT_MAX ? (ta.cosine ? 0.5f * d2 : sqrtf(d2)) : INFINITY;
+                    }
+            }
+        } else if constexpr (kMode != kWhole) {
+            if constexpr (kMode != kFlat) tk.finish();
             const int64_t slot = (kIsFlat ? item : unit / segs) * kQ + tid;
             if (live) {
                 float *pk = g.part_key + (slot * g.part_segs + unit % segs) * KC;
@@ -775,11 +1040,12 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g) {
                 }
                 if (kIsFlat && unit % segs == 0) g.vv[slot] = nn;
             }
-        } else if (live && !deferred) {
-            emit(g, tk, item, tid);
+        } else if (!deferred) {   // uniform
+            tk.finish();
+            emit(g, tk, item, tid, live, all_ties);
         }
     }
-    if (tid == 0 && scanned) atomicAdd(g.scanned, scanned);
+    if (!kExact && tid == 0 && scanned) atomicAdd(g.scanned, scanned);
 }
 
 // Joins the lists of a split item's parts (every part scanned the tiles around
@@ -791,14 +1057,15 @@ __global__ void __launch_bounds__(kQ) merge_kernel(const Args g) {
     const int b = blockIdx.x, tid = threadIdx.x;
     if (b >= min(*g.big_count, kBigItems)) return;
     const int64_t item = g.big[b * (1 + kSeeds)];
-    if ((tid & 63) >= g.tile_rows[2 * item + (tid >> 6)]) return;
+    const bool live = (tid & 63) < g.tile_rows[2 * item + (tid >> 6)];
     const float *xr = g.rec + (2 * item + (tid >> 6)) * record_floats(g.DP) + (tid & 63);
     float nn = 0.f;
     for (int t = 0; t < g.width; ++t) nn = fmaf(xr[t * kR], xr[t * kR], nn);
     List<KC> tk;
     tk.start(nn, g.k, g.width);
-    for (int s = 0; s < segs; ++s) {
-        const int64_t at = (((int64_t)b * kQ + tid) * g.part_segs + s) * KC;
+    const int64_t lists = ((int64_t)b * kQ + tid) * g.part_segs * KC;
+    for (int s = 0; live && s < segs; ++s) {
+        const int64_t at = lists + s * KC;
 #pragma unroll 1
         for (int c = 0; c < KC; ++c) {
             const float v = g.part_key[at + c];
@@ -810,80 +1077,31 @@ __global__ void __launch_bounds__(kQ) merge_kernel(const Args g) {
             if (!have) tk.top.insert(v, j);
         }
     }
-    emit(g, tk, item, tid);
-}
-
-// Rows whose list was too short for the rows within reach: a warp scans every
-// tile (lane per database row, the same FMA chain for s), scores the rows at
-// or below the bound with the re-rank's arithmetic and keeps the k <= 32
-// smallest (distance, id), one per lane.  Integer-like data with more equal
-// distances than a list holds come here; others hardly ever do.
-__global__ void __launch_bounds__(128)
-ties_kernel(const Args g, const float *__restrict__ R, int64_t rs, int d, bool cosine, bool vec,
-            int32_t *__restrict__ idx, float *__restrict__ dist) {
-    __shared__ float xs[4][64];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int count = *g.tie_count;
-    const int rf = record_floats(g.DP);
-    for (int64_t x = (int64_t)blockIdx.x * 4 + warp; x < count; x += (int64_t)gridDim.x * 4) {
-        const int64_t q = g.tie_rows[2 * x], slot = g.tie_rows[2 * x + 1];
-        const float bound = g.tie_bound[x];
-        const float *xr = g.rec + (slot / kR) * rf + slot % kR;
-        __syncwarp();
-        for (int t = lane; t < g.width; t += 32) xs[warp][t] = xr[(int64_t)t * kR];
-        __syncwarp();
-        float qv[8];
-        rr::load8(R + q * rs, lane & 7, d, cosine, vec, qv);
-        const bool fq = cosine && R[q * rs + d] != 0.f;
-        float bk = INFINITY;   // lane's entry of the sorted list
-        int bi = INT_MAX;
-        const int64_t slots = (int64_t)*g.T * kR;
-        for (int64_t j0 = 0; j0 < slots; j0 += 32) {
-            const float *yr = g.rec + (j0 / kR) * rf + (j0 % kR) + lane;
-            float acc = 0.f;
-            for (int t = 0; t < g.width; ++t) acc = fmaf(xs[warp][t], yr[t * kR], acc);
-            const float s = fmaf(-2.f, acc, yr[g.DP * kR]);
-            unsigned hits = __ballot_sync(0xffffffffu, s <= bound);
-            while (hits) {
-                const int64_t sj = j0 + __ffs(hits) - 1;   // place in the records
-                const int64_t j = g.tile_pos[sj / kR] + sj % kR;
-                hits &= hits - 1;
-                float yv[8];
-                rr::load8(R + j * rs, lane & 7, d, cosine, vec, yv);
-                float key = rr::dist2(qv, yv);
-                if (cosine) {
-                    const bool fy = R[j * rs + d] != 0.f;
-                    if (fq || fy) key = (fq && fy) ? 0.f : 2.f;
-                }
-                const int id = g.ids[sj];
-                const bool less = bk < key || (bk == key && bi < id);   // this lane's entry stays before it
-                const int at = __popc(__ballot_sync(0xffffffffu, less));
-                const float pk = __shfl_up_sync(0xffffffffu, bk, 1);
-                const int pi = __shfl_up_sync(0xffffffffu, bi, 1);
-                if (lane == at) {
-                    bk = key;
-                    bi = id;
-                } else if (lane > at) {
-                    bk = pk;
-                    bi = pi;
-                }
-            }
-        }
-        const int64_t o = g.ids[slot];
-        if (lane < g.k) {
-            idx[o * g.k + lane] = bi != INT_MAX ? bi : -1;
-            dist[o * g.k + lane] = bi != INT_MAX ? (cosine ? 0.5f * bk : sqrtf(bk)) : INFINITY;
-        }
+    // a part's full list whose last key is within reach is short of some rows
+    const float reach = tk.reach();
+    bool cut = false;
+    for (int s = 0; live && s < segs; ++s) {
+        const int64_t at = lists + s * KC + KC - 1;
+        cut |= g.part_id[at] >= 0 && g.part_key[at] <= reach;
     }
+    emit(g, tk, item, tid, live, cut);
 }
 
-constexpr int kCounters = 7;
+constexpr int kCounters = 8;
 constexpr int kMaxList = 40;
+
+// Parts' lists: the keys, then the ids (or Exact's entries in the whole of it).
+template <class L>
+void take_lists(Carve &cv, L &l, size_t entries) {
+    l.part_key = reinterpret_cast<float *>(cv.take<unsigned long long>(entries));
+    l.part_id = reinterpret_cast<int32_t *>(l.part_key + entries);
+}
 
 struct Layout {
     float *rec, *cenT, *rad, *nmax, *tie_bound;
-    int32_t *ids, *tile_pos, *tile_rows, *tie_rows;
-    int *counters;   // tie_count, counter, scanned (64 bits), tiles, big_count, unit
+    int32_t *ids, *tile_pos, *tile_rows, *tie_items, *id_min;
+    int *counters;   // tie_count, counter, scanned (64 bits), tiles, big_count, unit, tie_unit; tie_done follows
+    int64_t zeroed;  // ints
     int32_t *big, *part_id;
     uint32_t *bits;
     float *part_key;
@@ -900,14 +1118,14 @@ Layout layout(void *scratch, int64_t n, int DP) {
     L.nmax = cv.take<float>((size_t)tiles);
     L.tile_pos = cv.take<int32_t>((size_t)tiles);
     L.tile_rows = cv.take<int32_t>((size_t)tiles);
-    L.tie_rows = cv.take<int32_t>((size_t)2 * n);
-    L.tie_bound = cv.take<float>((size_t)n);
-    L.counters = cv.take<int>(kCounters);
+    L.id_min = cv.take<int32_t>((size_t)tiles);
+    L.tie_items = cv.take<int32_t>((size_t)tiles / 2);
+    L.tie_bound = cv.take<float>((size_t)tiles * kR);
+    L.zeroed = kCounters + tiles / 2;
+    L.counters = cv.take<int>((size_t)L.zeroed);
     L.big = cv.take<int32_t>(kBigItems * (1 + kSeeds));
     L.bits = cv.take<uint32_t>((size_t)kMaxCtas * ceil_div(tiles, (int64_t)kChunk) * kWords);
-    const size_t parts = (size_t)kBigItems * kSegs * kMaxList * kQ;
-    L.part_key = cv.take<float>(parts);
-    L.part_id = cv.take<int32_t>(parts);
+    take_lists(cv, L, (size_t)kBigItems * kSegs * kMaxList * kQ);
     L.bytes = cv.used;
     return L;
 }
@@ -929,9 +1147,13 @@ Args make_args(const Layout &L, int64_t n, int DP, int width, int k, int metric,
     g.k = k;
     g.beta = metric == RSC_COSINE ? 1.f : 0.f;
     g.cand = cand;
-    g.tie_rows = L.tie_rows;
+    g.id_min = L.id_min;
+    g.tie_items = L.tie_items;
     g.tie_bound = L.tie_bound;
     g.tie_count = L.counters;
+    g.tie_unit = L.counters + 7;
+    g.tie_done = L.counters + kCounters;
+    g.tie_units = kBigItems * kSegs;
     g.counter = L.counters + 1;
     g.scanned = reinterpret_cast<unsigned long long *>(L.counters + 2);
     g.bits = L.bits;
@@ -969,9 +1191,22 @@ cudaError_t launch_list(const Args &g, int64_t tiles, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(whole, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(split, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    whole<<<(unsigned)std::min<int64_t>(tiles / 2, std::min(kMaxCtas, 2 * sm_count())), kQ, smem, st>>>(g);
-    split<<<(unsigned)std::min<int64_t>(kBigItems * kSegs, 2 * sm_count()), kQ, smem, st>>>(g);
+    whole<<<(unsigned)std::min<int64_t>(tiles / 2, std::min(kMaxCtas, 2 * sm_count())), kQ, smem, st>>>(g, TieArgs{});
+    split<<<(unsigned)std::min<int64_t>(kBigItems * kSegs, 2 * sm_count()), kQ, smem, st>>>(g, TieArgs{});
     merge_kernel<KC><<<kBigItems, kQ, 0, st>>>(g);
+    return cudaGetLastError();
+}
+
+template <int kMode>
+cudaError_t launch_ties(const Args &g, int d, int metric, const float *R, int64_t rs, int32_t *idx, float *dist,
+                        cudaStream_t st) {
+    const bool vec = rs % 4 == 0 && reinterpret_cast<uintptr_t>(R) % 16 == 0;
+    const TieArgs ta{R, rs, d, metric == RSC_COSINE, vec, idx, dist};
+    const int smem = smem_layout(g.DP).total;
+    auto kern = g.k <= 16 ? simt_pruned_kernel<16, kMode> : simt_pruned_kernel<32, kMode>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)(2 * sm_count()), kQ, smem, st>>>(g, ta);
     return cudaGetLastError();
 }
 
@@ -985,24 +1220,20 @@ cudaError_t launch_knn_simt_pruned(const float *Y, const float *ny, int64_t n, i
     using namespace simtp;
     const Layout L = layout(scratch, n, DP);
     const int64_t tiles = tiles_max(n);
-    cudaError_t e = cudaMemsetAsync(L.counters, 0, kCounters * sizeof(int), st);
+    cudaError_t e = cudaMemsetAsync(L.counters, 0, L.zeroed * sizeof(int), st);
     if (e != cudaSuccess) return e;
     tile_table_kernel<<<1, 1024, 0, st>>>(leaves, n, DP, L.tile_pos, L.tile_rows, L.counters + 4);
     pack_kernel<<<(unsigned)tiles, 256, 0, st>>>(Y, ny, DP, perm, tiles, L.tile_pos, L.tile_rows, L.counters + 4, L.rec,
-                                                 L.ids, L.cenT, L.rad, L.nmax);
+                                                 L.ids, L.cenT, L.rad, L.nmax, L.id_min);
     const Args g = make_args(L, n, DP, width, k, metric, cand, status);
     return simt_pruned_list(k) == 24 ? launch_list<24>(g, tiles, st) : launch_list<kMaxList>(g, tiles, st);
 }
 
 cudaError_t launch_simt_ties(int64_t n, int d, int DP, int width, int k, int metric, void *scratch, const float *R,
-                             int64_t rs, int32_t *idx, float *dist, cudaStream_t st) {
+                             int64_t rs, int32_t *idx, float *dist, unsigned int *status, cudaStream_t st) {
     using namespace simtp;
-    const Layout L = layout(scratch, n, DP);
-    const Args g = make_args(L, n, DP, width, k, metric, nullptr, nullptr);
-    const bool vec = rs % 4 == 0 && reinterpret_cast<uintptr_t>(R) % 16 == 0;
-    ties_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n, (int64_t)4), 8 * sm_count()), 128, 0, st>>>(
-        g, R, rs, d, metric == RSC_COSINE, vec, idx, dist);
-    return cudaGetLastError();
+    const Args g = make_args(layout(scratch, n, DP), n, DP, width, k, metric, nullptr, status);
+    return launch_ties<kTies>(g, d, metric, R, rs, idx, dist, st);
 }
 
 // ------------------------------------------------------------- rows as they are
@@ -1039,10 +1270,13 @@ pack_flat_kernel(const float *__restrict__ Y, const float *__restrict__ ny, int6
     }
 }
 
+constexpr int kFlatCounters = 6;
+
 struct FlatLayout {
     float *rec, *part_key, *vv, *tie_bound;
-    int32_t *ids, *tile_pos, *tile_rows, *part_id, *tie_rows;
-    int *counters;   // tie_count, counter, scanned (64 bits), tiles
+    int32_t *ids, *tile_pos, *tile_rows, *part_id, *tie_items;
+    int *counters;   // tie_count, counter, scanned (64 bits), tiles, tie_unit; tie_done and tie_flag follow
+    int64_t zeroed;  // ints
     size_t bytes;
 };
 FlatLayout flat_layout(void *scratch, int64_t n, int DP, int k) {
@@ -1054,12 +1288,12 @@ FlatLayout flat_layout(void *scratch, int64_t n, int DP, int k) {
     L.ids = cv.take<int32_t>((size_t)items * kQ);
     L.tile_pos = cv.take<int32_t>((size_t)items * 2);
     L.tile_rows = cv.take<int32_t>((size_t)items * 2);
-    L.part_key = cv.take<float>(parts);
-    L.part_id = cv.take<int32_t>(parts);
+    take_lists(cv, L, parts);
     L.vv = cv.take<float>((size_t)items * kQ);
-    L.tie_rows = cv.take<int32_t>((size_t)2 * n);
-    L.tie_bound = cv.take<float>((size_t)n);
-    L.counters = cv.take<int>(5);
+    L.tie_items = cv.take<int32_t>((size_t)items);
+    L.tie_bound = cv.take<float>((size_t)items * kQ);
+    L.zeroed = kFlatCounters + 2 * items;
+    L.counters = cv.take<int>((size_t)L.zeroed);
     L.bytes = cv.used;
     return L;
 }
@@ -1082,8 +1316,12 @@ Args flat_args(const FlatLayout &L, int64_t n, int DP, int width, int k, unsigne
     g.part_id = L.part_id;
     g.part_segs = simt_flat_segs(n, DP);
     g.vv = L.vv;
-    g.tie_rows = L.tie_rows;
+    g.tie_items = L.tie_items;
     g.tie_bound = L.tie_bound;
+    g.tie_unit = L.counters + 5;
+    g.tie_done = L.counters + kFlatCounters;
+    // lists of 16 (k <= 16) or 32 entries in the room of part_segs lists an item
+    g.tie_units = ceil_div(n, (int64_t)kQ) * g.part_segs;
     g.status = status;
     g.wait_budget = tc_wait_budget();
     return g;
@@ -1118,7 +1356,8 @@ size_t simt_flat_scratch_bytes(int64_t n, int DP, int k) { return simtp::flat_la
 
 SimtParts simt_flat_parts(void *scratch, int64_t n, int DP, int k) {
     const simtp::FlatLayout L = simtp::flat_layout(scratch, n, DP, k);
-    return {L.part_key, L.part_id, L.vv, simt_flat_segs(n, DP), simt_pruned_list(k), L.counters, L.tie_rows, L.tie_bound};
+    return {L.part_key, L.part_id, L.vv, simt_flat_segs(n, DP), simt_pruned_list(k), L.counters,
+            L.counters + simtp::kFlatCounters + ceil_div(n, (int64_t)simtp::kQ), L.tie_items, L.tie_bound};
 }
 
 cudaError_t launch_knn_simt_flat(const float *Y, const float *ny, int64_t n, int DP, int width, int k, void *scratch,
@@ -1126,7 +1365,7 @@ cudaError_t launch_knn_simt_flat(const float *Y, const float *ny, int64_t n, int
     using namespace simtp;
     const FlatLayout L = flat_layout(scratch, n, DP, k);
     const Args g = flat_args(L, n, DP, width, k, status);
-    cudaError_t e = cudaMemsetAsync(L.counters, 0, 5 * sizeof(int), st);
+    cudaError_t e = cudaMemsetAsync(L.counters, 0, L.zeroed * sizeof(int), st);
     if (e != cudaSuccess) return e;
     const int64_t items = ceil_div(n, (int64_t)kQ);
     pack_flat_kernel<<<(unsigned)(2 * items), 256, 0, st>>>(Y, ny, n, DP, L.rec, L.ids, L.tile_pos, L.tile_rows,
@@ -1134,18 +1373,16 @@ cudaError_t launch_knn_simt_flat(const float *Y, const float *ny, int64_t n, int
     const int smem = smem_layout(DP).total;
     auto kern = simt_pruned_list(k) == 24 ? simt_pruned_kernel<24, kFlat> : simt_pruned_kernel<kMaxList, kFlat>;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-    kern<<<(unsigned)std::min<int64_t>(items * g.part_segs, 2 * sm_count()), kQ, smem, st>>>(g);
+    kern<<<(unsigned)std::min<int64_t>(items * g.part_segs, 2 * sm_count()), kQ, smem, st>>>(g, TieArgs{});
     return cudaGetLastError();
 }
 
 cudaError_t launch_simt_flat_ties(int64_t n, int d, int DP, int width, int k, int metric, void *scratch, const float *R,
-                                  int64_t rs, int32_t *idx, float *dist, cudaStream_t st) {
+                                  int64_t rs, int32_t *idx, float *dist, unsigned int *status, cudaStream_t st) {
     using namespace simtp;
-    const Args g = flat_args(flat_layout(scratch, n, DP, k), n, DP, width, k, nullptr);
-    const bool vec = rs % 4 == 0 && reinterpret_cast<uintptr_t>(R) % 16 == 0;
-    ties_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n, (int64_t)4), 8 * sm_count()), 128, 0, st>>>(
-        g, R, rs, d, metric == RSC_COSINE, vec, idx, dist);
-    return cudaGetLastError();
+    Args g = flat_args(flat_layout(scratch, n, DP, k), n, DP, width, k, status);
+    g.beta = metric == RSC_COSINE ? 1.f : 0.f;
+    return launch_ties<kFlatTies>(g, d, metric, R, rs, idx, dist, st);
 }
 
 }  // namespace rsc

@@ -231,15 +231,13 @@ rerank_parts_kernel(const float *__restrict__ R, int64_t rs, int64_t n, int d, i
     // a full list whose last entry is within reach may have left some out
     const bool cut = lane < P.segs && pi[lane * P.list + P.list - 1] >= 0 &&
                      order(pk[lane * P.list + P.list - 1]) <= within;
-    if (__any_sync(0xffffffffu, cut) || count > kMax) {
-        if (lane == 0) {
-            const int x = atomicAdd(P.tie_count, 1);
-            P.tie_rows[2 * x] = (int32_t)q;
-            P.tie_rows[2 * x + 1] = (int32_t)q;
-            P.tie_bound[x] = reach;
-        }
-        return;
+    const bool tie = __any_sync(0xffffffffu, cut) || count > kMax;
+    if (lane == 0) {
+        P.tie_bound[q] = tie ? reach : -INFINITY;
+        if (tie && atomicExch(P.tie_flag + q / kTieItem, 1) == 0)
+            P.tie_items[atomicAdd(P.tie_count, 1)] = (int32_t)(q / kTieItem);
     }
+    if (tie) return;
     __syncwarp();
     const bool cosine = metric == RSC_COSINE;
     float xv[8];

@@ -43,6 +43,26 @@ __device__ __forceinline__ float reach(float t, float vv, float v, int w) {
     return t + 2.f * e + 0x1p-22f * fabsf(t);
 }
 
+// The same distance by one thread alone: the eight partial sums one after the
+// other, added in the order in which the lanes' shuffles add them.
+__device__ __forceinline__ float dist2_thread(const float *x, const float *y, int d, bool cosine, bool vec) {
+    float part[8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+        part[s] = 0.f;
+        if (4 * s >= d) continue;   // uniform
+        float a[8], b[8];
+        load8(x, s, d, cosine, vec, a);
+        load8(y, s, d, cosine, vec, b);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float diff = a[i] - b[i];
+            part[s] = fmaf(diff, diff, part[s]);
+        }
+    }
+    return ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
+}
+
 // Sum of squared differences of the two rows (every lane of the eight gets it).
 __device__ __forceinline__ float dist2(const float (&x)[8], const float (&y)[8]) {
     float part = 0.f;

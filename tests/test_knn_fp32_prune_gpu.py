@@ -145,3 +145,57 @@ def test_search_that_gave_up_leaves_no_id_outside_the_rows(rsc, n):  # noqa: F81
     assert rsc.rsc_workspace_status(ws) == rsc.RSC_OK
     np.testing.assert_array_equal(gi.cpu().numpy(), fi)
     np.testing.assert_array_equal(gd.cpu().numpy(), fd)
+
+
+@pytest.mark.parametrize("case,n,k", [
+    ("binary", 17_000, 15), ("binary", 20_011, 32), ("binary", 9_001, 16), ("binary", 129, 32),
+    ("copies", 30_000, 15), ("copies", 20_000, 32), ("copies", 12_000, 17),
+    ("few", 20_000, 15), ("few", 16_400, 32), ("few", 5_000, 15),
+    ("line", 40_000, 15), ("line", 20_000, 32), ("line", 9_000, 15),
+])
+def test_ties_pass_finds_the_k_nearest(rsc, case, n, k):  # noqa: F811
+    # rows for the ties pass in most items or in few (their database in parts),
+    # with hits that one row has alone or all rows share, both list lengths,
+    # with and without the ordering.  Integer coordinates and copies have equal
+    # distances in FP32 and FP64 alike, so the ids must agree; the line's
+    # distances are those of FP64 to the rounding of two subtractions.
+    rng = np.random.Generator(np.random.PCG64(n + k))
+    if case == "binary":      # nothing separates these: all tiles are kept
+        X = rng.integers(0, 2, (n, 20)).astype(np.float32)
+    elif case == "copies":    # 100 groups of 60 copies among clusters
+        X = synth.mixture(n, 30, n_comp=20, seed=n)
+        X[:6000] = np.repeat(X[:100], 60, axis=0)
+        X = X[rng.permutation(n)]
+    elif case == "few":       # ten rows as far from all the others, which are one row
+        X = rng.standard_normal((n, 50)).astype(np.float32)
+        X[: n - 10] = X[0]
+        X = X[rng.permutation(n)]
+    else:                     # s of rows on a line loses what separates neighbours
+        X = rng.uniform(0, 1, (n, 1)).astype(np.float32)
+    gi, gd = run_knn(rsc, X, k, precision="fp32")
+    q = np.arange(n) if n < 500 else synth.query_sample(n, 300, seed=3)
+    if case in ("copies", "few"):   # some of the rows in question
+        q = np.unique(np.r_[q, np.argsort(gd.max(1), kind="stable")[[0, -1, -2, -3]]])
+    oi, od, _ = oracle.knn(X, k, queries=q)
+    np.testing.assert_allclose(gd[q], od, rtol=1e-5, atol=1e-7)
+    if case != "line":
+        same = gi[q] == oi
+        if case == "copies":   # neighbours of a mixture closer than FP32 tells may change places
+            same |= np.isclose(od, np.roll(od, 1, 1), rtol=1e-6) | np.isclose(od, np.roll(od, -1, 1), rtol=1e-6)
+            zero = od == 0
+            assert (gi[q] == oi)[zero].all()
+        assert same.all()
+
+
+@pytest.mark.parametrize("n", [17_000, 4_000])
+def test_ties_pass_of_cosine_rows(rsc, n):  # noqa: F811
+    # small whole numbers in three components: many rows along one direction
+    # and rows of zeros; distances to the rounding of normalised rows
+    rng = np.random.Generator(np.random.PCG64(n))
+    X = rng.integers(0, 4, (n, 3)).astype(np.float32)
+    gi, gd = run_knn(rsc, X, 15, metric="cosine", precision="fp32")
+    q = synth.query_sample(n, 300, seed=3)
+    _, od, _ = oracle.knn(X, 15, metric=oracle.COSINE, queries=q)
+    np.testing.assert_allclose(gd[q], od, rtol=0, atol=1e-6)
+    zeros = np.flatnonzero((X == 0).all(1))
+    assert (gi[zeros] == zeros[:15]).all()
