@@ -346,9 +346,9 @@ __global__ void top_logits_kernel(int64_t rows, int P, const float *__restrict__
 
 // Logits that are NaN leave no part id (INT_MAX).  A database row without one
 // counts to part 0, and a query without any starts there; a further probe
-// without one is no probe (-1): part 0 searched again would list its rows twice.
+// without one is none (P): part 0 searched again would list its rows twice.
 __device__ __forceinline__ int safe_part(int p, int P) { return (p >= 0 && p < P) ? p : 0; }
-__device__ __forceinline__ int probe_part(int p, int r, int P) { return (p >= 0 && p < P) ? p : r == 0 ? 0 : -1; }
+__device__ __forceinline__ int probe_part(int p, int r, int P) { return (p >= 0 && p < P) ? p : r == 0 ? 0 : P; }
 
 __global__ void histogram_kernel(int64_t count, int P, const int32_t *__restrict__ key, int32_t *__restrict__ hist) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -403,9 +403,15 @@ __global__ void scatter_kernel(int64_t count, int P, const int32_t *__restrict__
     perm[off[k] + atomicAdd(&cursor[k], 1)] = (int32_t)i;
 }
 
+constexpr int kSlotList = 16;     // ids per (slot, column part)
+constexpr int kSlotParts = 4;     // column parts per slot (k <= 16)
+constexpr int kPerSlot = kSlotList * kSlotParts;
+
 // Probe slots: the probes r0 .. r0 + M - 1 of every query (route [nq, R]),
-// grouped by part (probes without a part take no slot).  Blocks of kGroupEntries (query, probe) entries rank their
-// entries per part in shared memory and take one range of each part's cursor,
+// grouped by part; a probe without a part gets the slot after all others, whose
+// list is empty (so the re-rank has no case for it: testing the slot there cost
+// it 5 %).  Blocks of kGroupEntries (query, probe) entries rank their entries per
+// part in shared memory and take one range of each part's cursor,
 // so a part's counter sees one atomic per block and not one per entry.  4M
 // entries over 512 parts: 35 us for the counts and 197 us for the slots and
 // the operand rows (544 + 556 + 185 us with a global atomic per entry and the
@@ -417,31 +423,34 @@ constexpr int kMaxParts = 1024;
 __global__ void __launch_bounds__(kGroupThreads)
 group_count_kernel(int64_t nq, int R, int r0, int M, int P, const int32_t *__restrict__ route,
                    int32_t *__restrict__ cnt) {
-    __shared__ int hist[kMaxParts];
-    for (int p = threadIdx.x; p < P; p += kGroupThreads) hist[p] = 0;
+    __shared__ int hist[kMaxParts + 1];   // [P]: no part
+    for (int p = threadIdx.x; p <= P; p += kGroupThreads) hist[p] = 0;
     __syncthreads();
     const int64_t e0 = (int64_t)blockIdx.x * kGroupEntries, e1 = min(nq * M, e0 + kGroupEntries);
     for (int64_t e = e0 + threadIdx.x; e < e1; e += kGroupThreads) {
-        const int r = r0 + (int)(e % M), p = probe_part(route[(e / M) * R + r], r, P);
-        if (p >= 0) atomicAdd(&hist[p], 1);
+        const int r = r0 + (int)(e % M);
+        atomicAdd(&hist[probe_part(route[(e / M) * R + r], r, P)], 1);
     }
     __syncthreads();
     for (int p = threadIdx.x; p < P; p += kGroupThreads)
         if (hist[p]) atomicAdd(&cnt[p], hist[p]);
 }
 
-// gpos[q * M + m] = slot of the entry (-1: none); operand row of the slot = the query's
-// row of Qb (rows[q], or q0 + q), read in query order and written as whole
-// 128-byte rows; slot_thr[slot] = thr[q] when given.
+// gpos[q * M + m] = slot of the entry (nq * M: none, its list in cand made
+// empty); operand row of the slot = the query's row of Qb (rows[q], or q0 + q),
+// read in query order and written as whole 128-byte rows; slot_thr[slot] = thr[q] when given.
 __global__ void __launch_bounds__(kGroupThreads)
 group_slots_kernel(int64_t nq, int R, int r0, int M, int P, const int32_t *__restrict__ route,
                    const int64_t *__restrict__ off, int32_t *__restrict__ cursor, const int32_t *__restrict__ rows,
                    int64_t q0, const uint4 *__restrict__ Qb, const float *__restrict__ thr,
-                   int32_t *__restrict__ gpos, uint4 *__restrict__ Qg, float *__restrict__ slot_thr) {
+                   int32_t *__restrict__ gpos, uint4 *__restrict__ Qg, float *__restrict__ slot_thr,
+                   int32_t *__restrict__ cand) {
     constexpr int kPer = kGroupEntries / kGroupThreads;
-    __shared__ int cnt[kMaxParts];
+    __shared__ int cnt[kMaxParts + 1];
     __shared__ int32_t slot[kGroupEntries];
-    for (int p = threadIdx.x; p < P; p += kGroupThreads) cnt[p] = 0;
+    const int none = (int)(nq * M);
+    if (blockIdx.x == 0 && threadIdx.x < kPerSlot) cand[(int64_t)none * kPerSlot + threadIdx.x] = -1;
+    for (int p = threadIdx.x; p <= P; p += kGroupThreads) cnt[p] = 0;
     __syncthreads();
     const int64_t e0 = (int64_t)blockIdx.x * kGroupEntries, total = nq * M;
     const int here = (int)min((int64_t)kGroupEntries, total - e0);
@@ -455,12 +464,7 @@ group_slots_kernel(int64_t nq, int R, int r0, int M, int P, const int32_t *__res
             const int64_t e = e0 + x;
             const int r = r0 + (int)(e % M);
             part[i] = probe_part(route[(e / M) * R + r], r, P);
-            if (part[i] >= 0) {
-                rank[i] = atomicAdd(&cnt[part[i]], 1);
-            } else {
-                slot[x] = -1;
-                gpos[e] = -1;
-            }
+            rank[i] = atomicAdd(&cnt[part[i]], 1);
         }
     }
     __syncthreads();
@@ -473,18 +477,18 @@ group_slots_kernel(int64_t nq, int R, int r0, int M, int P, const int32_t *__res
     for (int i = 0; i < kPer; ++i) {
         if (part[i] >= 0) {
             const int x = threadIdx.x + i * kGroupThreads;
-            const int s = cnt[part[i]] + rank[i];
+            const int s = part[i] < P ? cnt[part[i]] + rank[i] : none;
             slot[x] = s;
             gpos[e0 + x] = s;
-            if (thr) slot_thr[s] = thr[(e0 + x) / M];
+            if (thr && s < none) slot_thr[s] = thr[(e0 + x) / M];
         }
     }
     __syncthreads();
     for (int x = threadIdx.x; x < here * 8; x += kGroupThreads) {
-        if (slot[x >> 3] < 0) continue;
         const int64_t q = (e0 + (x >> 3)) / M;
         const int64_t row = rows ? (int64_t)rows[q] : q0 + q;
-        Qg[(int64_t)slot[x >> 3] * 8 + (x & 7)] = Qb[row * 8 + (x & 7)];
+        const uint4 piece = Qb[row * 8 + (x & 7)];
+        if (slot[x >> 3] < none) Qg[(int64_t)slot[x >> 3] * 8 + (x & 7)] = piece;
     }
 }
 
@@ -501,10 +505,6 @@ __global__ void set_segment_kernel(int32_t *__restrict__ cnt, int32_t c0, int64_
 }
 
 // ------------------------------------------------ exact merge re-rank
-
-constexpr int kSlotList = 16;     // ids per (slot, column part)
-constexpr int kSlotParts = 4;     // column parts per slot (k <= 16)
-constexpr int kPerSlot = kSlotList * kSlotParts;
 
 // A query's first probe (the part the network ranks first) bounds what the
 // other probes can add.  Warp per query: T = the k-th smallest accumulator
@@ -588,13 +588,12 @@ rerank_probe_kernel(const float *__restrict__ X, int d, const int32_t *__restric
     for (int t = lane; t < 64; t += 32) xq[t] = t < d ? X[row * d + t] : 0.f;
     int count = 0;
     for (int r = 0; r < R; ++r) {
-        const int32_t at = r == 0 ? gpos0[q] : gpos1[q * (R - 1) + r - 1];
-        const bool probed = at >= 0;   // no branch: the probes' lists are fetched together
-        const int32_t *c = (r == 0 ? cand0 : cand1) + (int64_t)max(at, 0) * kPerSlot;
+        const int32_t *c = r == 0 ? cand0 + (int64_t)gpos0[q] * kPerSlot
+                                  : cand1 + (int64_t)gpos1[q * (R - 1) + r - 1] * kPerSlot;
 #pragma unroll
         for (int h = 0; h < kPerSlot; h += 32) {
             const int32_t j = c[h + lane];
-            const bool ok = probed && j >= 0 && (int64_t)j < n_db;   // empty, dropped, or ids of an aborted search
+            const bool ok = j >= 0 && (int64_t)j < n_db;   // empty, dropped, or ids of an aborted search
             const unsigned m = __ballot_sync(0xffffffffu, ok);
             if (ok) ids[count + __popc(m & ((1u << lane) - 1u))] = j;
             count += __popc(m);
@@ -1002,10 +1001,10 @@ struct PartLayout {
     int32_t *route;                 // [chunk, R]
     int32_t *gpos;                  // [chunk] slots of the first probes, then [chunk, R - 1] of the others
     void *Qg;                       // [slots of one pass, 64] bf16
-    int32_t *cand0;                 // [chunk, kPerSlot] candidates of the first probes
+    int32_t *cand0;                 // [chunk + 1, kPerSlot] candidates of the first probes (the last: none)
     float *key0;                    // [chunk, kPerSlot] their accumulator values
     float *thr;                     // [chunk] bound of every query
-    int32_t *cand1;                 // [chunk * (R - 1), kPerSlot] candidates of the other probes
+    int32_t *cand1;                 // [chunk * (R - 1) + 1, kPerSlot] candidates of the other probes (the last: none)
     float *slot_thr;                // [chunk * (R - 1)] bounds by slot
     float *Xq;                      // [kChunkRows, d] gathered network input
     void *packed;                   // the network's weights as the routing kernel reads them
@@ -1057,10 +1056,10 @@ PartLayout carve_part(void *ws, const rsc_partitioner *p, int64_t n, int64_t n_t
     L.route = cv.take<int32_t>((size_t)chunk * R);
     L.gpos = cv.take<int32_t>((size_t)(first + rest));
     L.Qg = cv.take<uint16_t>((size_t)std::max(first, rest) * 64);
-    L.cand0 = cv.take<int32_t>((size_t)first * kPerSlot);
+    L.cand0 = cv.take<int32_t>((size_t)(first + 1) * kPerSlot);
     L.key0 = cv.take<float>((size_t)chunk * kPerSlot);
     L.thr = cv.take<float>((size_t)chunk);
-    L.cand1 = cv.take<int32_t>((size_t)rest * kPerSlot);
+    L.cand1 = cv.take<int32_t>((size_t)(rest + 1) * kPerSlot);
     L.slot_thr = cv.take<float>((size_t)rest);
     L.Xq = cv.take<float>(fused ? 0 : (size_t)kChunkRows * p->d);
     L.packed = cv.take<uint8_t>(fused ? mlp_route_weight_bytes(p->H, p->P) : 0);
@@ -1090,14 +1089,14 @@ rsc_status probe_search(cudaStream_t st, const void *Dop, int64_t n_db, int64_t 
 // Groups probes r0 .. r0 + M - 1 of nq queries by part: counts, slot offsets
 // and work items, slots and operand rows (thr: bounds of the queries, nullable).
 void launch_group(cudaStream_t st, const rsc_partitioner *p, const PartLayout &L, int64_t nq, int R, int r0, int M,
-                  const int32_t *rows, int64_t q0, const float *thr, int32_t *gpos) {
+                  const int32_t *rows, int64_t q0, const float *thr, int32_t *gpos, int32_t *cand) {
     cudaMemsetAsync(L.gcnt, 0, sizeof(int32_t) * p->P * 2, st);
     const unsigned blocks = (unsigned)ceil_div(nq * M, part::kGroupEntries);
     part::group_count_kernel<<<blocks, part::kGroupThreads, 0, st>>>(nq, R, r0, M, p->P, L.route, L.gcnt);
     part::offsets_kernel<<<1, 1024, 0, st>>>(p->P, L.gcnt, L.goff, tck::BM, L.items);
     part::group_slots_kernel<<<blocks, part::kGroupThreads, 0, st>>>(
         nq, R, r0, M, p->P, L.route, L.goff, L.gcursor, rows, q0, static_cast<const uint4 *>(L.Qb), thr, gpos,
-        static_cast<uint4 *>(L.Qg), L.slot_thr);
+        static_cast<uint4 *>(L.Qg), L.slot_thr, cand);
 }
 
 // vector loads as wide as every row's start allows
@@ -1353,7 +1352,7 @@ rsc_status rsc_knn_partitioned(rsc_partitioner *p, const float *X, int64_t n, in
         }
         // 2. the first probe of every query: its part's gathered queries
         //    against that part's database rows, keys kept
-        launch_group(st, p, L, cq, R, 0, 1, rows, q0, nullptr, L.gpos);
+        launch_group(st, p, L, cq, R, 0, 1, rows, q0, nullptr, L.gpos, L.cand0);
         if ((s = probe_search<false>(st, p->Db_sorted, n, cq, p->P, L, p->doff, L.cand0, R > 1 ? L.key0 : nullptr)) !=
             RSC_OK)
             return s;
@@ -1362,7 +1361,7 @@ rsc_status rsc_knn_partitioned(rsc_partitioner *p, const float *X, int64_t n, in
         if (R > 1) {
             part::probe_bound_kernel<<<(unsigned)ceil_div(cq * 32, 256), 256, 0, st>>>(
                 cq, p->d, k, rows, q0, static_cast<const uint32_t *>(L.Qb), L.gpos, L.key0, L.cand0, L.thr);
-            launch_group(st, p, L, cq, R, 1, R - 1, rows, q0, L.thr, gpos1);
+            launch_group(st, p, L, cq, R, 1, R - 1, rows, q0, L.thr, gpos1, L.cand1);
             if ((s = probe_search<true>(st, p->Db_sorted, n, cq * (R - 1), p->P, L, p->doff, L.cand1, nullptr)) !=
                 RSC_OK)
                 return s;
