@@ -32,11 +32,12 @@
 // clusters, tiles cut every 64 rows whatever the leaves: 10.9 % of the pairs
 // scanned and a few items that scanned everything, 15.4 ms).
 //
-// One persistent CTA pair per SM; an item is two tiles of query rows, each
-// with its own sphere and tau (the database tile is scanned when either keeps
-// it).  The CTA scans the tiles around its own, then walks the database in
-// chunks of 256 tiles from its own chunk on: tests every tile's sphere against
-// its current taus, and scans the tiles that are left.  A tile's record (64 rows transposed, then
+// Persistent CTAs, two per SM (one with 64 components, whose tiles leave shared
+// memory for no more); an item is two tiles of query rows, each with its own
+// sphere and tau (the database tile is scanned when either keeps it).  The CTA
+// scans the tiles around its own, then walks the database in chunks of 256 tiles
+// from its own chunk on: tests every tile's sphere against its current taus, and
+// scans the tiles that are left.  A tile's record (64 rows transposed, then
 // |y|^2) is one contiguous block, brought in by a bulk copy two tiles ahead.
 // A thread accumulates an 8 x 8 block of (query, row) pairs by packed FP32
 // fused multiply-adds (fma.rn.f32x2: two pairs per instruction, each rounded
@@ -45,10 +46,15 @@
 //
 // What bounds it: the FMA pipe and, next to it, the insertions (a row takes in
 // about 70 values).  50 components, k = 15, one GB300, whole call (in brackets
-// the full scan): 100,003 rows, 60 clusters 1.6 ms (25.9), of which this kernel
-// 0.8 and the ordering 0.5; 1M rows, 100 clusters 31 ms (2054); rows without
-// any clusters, of which no tile is dropped, 1.9 ms (1.5) at 16,384 rows, 9.1
-// (7.3) at 50,000, 25.0 (25.9) at 100,003.
+// the full scan): 100,003 rows, 60 clusters 1.57 ms (25.9), of which this kernel
+// 0.8 and the ordering 0.5; 1M rows, 100 clusters 33 ms (2058).  Rows without any
+// clusters, of which no tile is dropped (in the second brackets with every item
+// run whole or, the first 192, in eight parts that each scanned the item's
+// surroundings again): 1.58 ms (1.47) (1.69) at 16,384 rows, 1.99 (2.13) (2.41) at
+// 20,000, 2.45 (2.72) (4.03) at 24,000, 3.74 (4.09) (4.93) at 32,000, 7.25 (7.30)
+// (8.99) at 50,000, 13.5 (15.5) (14.9) at 70,000, 25.3 (25.8) (28.4) at 100,003,
+// 193 (194) (198) at 300,000; 12 components 0.87 (1.10) at 16,384 and 2.94 (4.06)
+// at 50,000.
 #include <float.h>
 #include <limits.h>
 #include <math.h>
@@ -79,9 +85,10 @@ constexpr int kSeeds = 8;                 // nearest tiles scanned first when th
 constexpr int kWin = 3;                   // tiles on each side of the query tile scanned first
 constexpr int kStages = 2;
 constexpr int kMaxCtas = 320;             // persistent CTAs at most
-constexpr int kBigItems = 192;            // items that may be split
-constexpr int kSegs = 8;                  // parts of a split item at most
-constexpr int kSegTiles = 128;            // tiles per part at least
+constexpr int kBigItems = 640;            // items that may be split
+constexpr int kSegs = 16;                 // parts of a split item at most
+constexpr int kSegTiles = 16;             // tiles per part at least
+constexpr int kUnits = 1792;              // lists (of kQ rows) of split items and their parts
 constexpr uint32_t kSleepNs = 2000;                // suspend of a wait per try
 constexpr long long kDrainBudget = 2000000000LL;   // ~1 s of SM clocks, for copies in flight when a CTA leaves
 
@@ -407,12 +414,18 @@ struct Args {
     float *tie_bound;       // [item * kQ + row] their reach (-inf: not such a row), items on the list only
     int *tie_count, *counter;
     int *tie_done;          // parts of a tie item that are done
-    int64_t tie_units;      // lists the parts of tie items may take (kQ rows each)
     uint32_t *bits;         // [CTAs][stride / 32] tiles an item keeps
     int32_t *big;           // [kBigItems][1 + kSeeds] items to be split, their seeds (-1 pads)
-    int *big_count, *unit;  // their number (may exceed kBigItems), next part
+    int *big_count, *unit;  // their number (may exceed big_cap), next part
+    float *big_bound;       // [kBigItems * kQ] their rows' bounds
+    int *heavy, *light;     // items that kept many tiles (ties aside), and items done that kept few
+    int slots;              // CTAs that are resident at once
+    int64_t units;          // lists there is room for
+    int big_cap;            // entries of `big` at most: two lists each at least
     int *tie_unit;          // next part of a tie item
-    float *part_key;        // [query slots][part_segs][KC] lists of the parts; a slot is a query
+    // split: [units][kQ][KC], the lists of parts (position in `big`, part) from the
+    // front and the items' own, in that order, from the back
+    float *part_key;        // flat: [query slots][part_segs][KC] lists of the parts; a slot is a query
     int32_t *part_id;       // tile pair's (split: position in `big`; flat: item) kQ rows
     int part_segs;
     float *vv;              // [query slots] |y|^2 (flat)
@@ -421,10 +434,20 @@ struct Args {
     long long wait_budget;         // SM clocks a wait for a copy may take (tc_wait_budget)
 };
 
-// parts of a split item: segments of seg_tiles tiles
-__device__ __forceinline__ int64_t seg_tiles(int64_t tiles) {
-    const int64_t s = min((int64_t)kSegs, max((int64_t)1, tiles / kSegTiles));
-    return ceil_div(tiles, s);
+// Parts of each of `count` items over `tiles` tiles: as many as cost least, waves
+// of CTAs times a part's tiles (about three more for its start), while there is
+// room for them (own: lists an item takes besides its parts').
+__device__ __forceinline__ int part_count(const Args &g, int64_t count, int64_t tiles, int own) {
+    int best = 1;
+    int64_t cost = INT64_MAX;
+    for (int s = 1; s <= kSegs && (s == 1 || (count * (s + own) <= g.units && tiles >= (int64_t)s * kSegTiles)); ++s) {
+        const int64_t c = ceil_div(count * s, (int64_t)g.slots) * (ceil_div(tiles, (int64_t)s) + 3);
+        if (c < cost) {
+            cost = c;
+            best = s;
+        }
+    }
+    return best;
 }
 
 // The candidates of an item's rows (a thread each; lists finished), and the
@@ -514,27 +537,14 @@ struct TieArgs {
     }
 };
 
-// Parts of a tie item: the count whose waves cost least, as far as the parts'
-// lists have room (one part needs none).
-__device__ __forceinline__ int tie_segs(const Args &g, int64_t count, int64_t tiles, int64_t slots) {
-    int best = 1;
-    int64_t cost = INT64_MAX;
-    for (int s = 1; s <= kSegs && (s == 1 || (count * s <= g.tie_units && tiles >= 8 * s)); ++s) {
-        const int64_t c = ceil_div(count * s, slots) * (ceil_div(tiles, (int64_t)s) + 3);
-        if (c < cost) {
-            cost = c;
-            best = s;
-        }
-    }
-    return best;
-}
-
-// kSplit = false: an item per query tile pair.  An item that keeps more than
-// 1 / 16 of the tiles (a tile that holds a row far from its cluster, or spans
-// two) would outlast all others on its CTA (100k rows: 10 ms for one); such
-// items are put on a list instead, as long as it has room, and kSplit = true
-// runs them in up to kSegs parts, each over a segment of the database from
-// the item's own surroundings on, whose lists merge_kernel joins.
+// kWhole: an item per query tile pair.  An item that keeps more than 1 / 16 of
+// the tiles (a tile that holds a row far from its cluster, or spans two) would
+// outlast all others on its CTA (100k rows: 10 ms for one); such items are put on
+// a list with their rows' lists and bounds so far, as long as there is room, and
+// kSplitItems runs the rest of them in parts, segments of the database, whose
+// lists merge_kernel joins.  Where nearly all items are such (rows that no sphere
+// separates) they are run at once as long as they fill whole waves of CTAs, and
+// the last, partial wave is what is split.
 // kFlat: rows in their own order, part_segs parts per item and no tests: the
 // search of fewer rows than an ordering pays for (see launch_knn_simt_flat).
 // kTies, kFlatTies: the ties pass after either search (KC: Exact's entries).
@@ -582,17 +592,19 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const 
         return true;
     };
     const int64_t tiles = *g.T;   // an odd count is followed by an empty tile
-    const int64_t seg_len = kExact    ? ceil_div(tiles, (int64_t)tie_segs(g, tie_items, tiles, gridDim.x))
-                            : kIsFlat ? ceil_div(tiles, (int64_t)g.part_segs)
-                                      : seg_tiles(tiles);
+    const int64_t big_items = kSplit ? min(*g.big_count, g.big_cap) : 0;
+    if (kSplit && big_items == 0) return;
+    const int64_t seg_len = ceil_div(tiles, (int64_t)(kMode == kFlat ? g.part_segs
+                                                      : kExact       ? part_count(g, tie_items, tiles, 0)
+                                                      : kSplit       ? part_count(g, big_items, tiles, 1)
+                                                                     : 1));
     const int segs = kMode == kFlat ? g.part_segs : (int)ceil_div(tiles, seg_len);
     const int64_t pairs = ceil_div(tiles, (int64_t)2);
     const int64_t units = kExact            ? tie_items * segs
                           : kMode == kFlat ? pairs * segs
-                          : kSplit         ? (int64_t)min(*g.big_count, kBigItems) * segs
+                          : kSplit         ? big_items * segs
                                            : pairs;
-    bool live = false;       // the thread has a query row
-    int64_t cur_item = 0;
+    const int64_t whole_waves = pairs / g.slots * g.slots;
     uint32_t tile_no = 0;     // tiles consumed by this CTA so far (stage tile_no % kStages)
     uint32_t items = 0;
     unsigned long long scanned = 0;
@@ -668,7 +680,7 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const 
             if constexpr (kExact) {
                 // this row's hits, and their places among the block's
                 unsigned hit[2] = {0u, 0u};
-                if (live && !tk.full_before(kIsFlat ? j0 : g.id_min[tt])) {
+                if (!tk.full_before(kIsFlat ? j0 : g.id_min[tt])) {   // (a row that wants nothing has no hits)
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
 #pragma unroll 8
@@ -710,7 +722,7 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const 
                     for (int x = tid; x < min(kBatch, total - b0); x += kQ) {
                         const int rc = pair[x], row = rc >> 6, c = rc & 63;
                         keys[x] = rc == 0xffff ? Exact<KC>::kNone
-                                               : ta.score(g.tile_pos[2 * cur_item + (row >> 6)] + (row & 63), j0 + c, tile_ids[c]);
+                                               : ta.score(seeds[4 + (row >> 6)] + (row & 63), j0 + c, tile_ids[c]);
                     }
                     __syncthreads();
                     for (int x = from; x < end; ++x) tk.insert(keys[x - b0]);
@@ -759,14 +771,14 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const 
             if (tid == 0) wait(xfull, items & 1, kDrainBudget);
             return;
         }
-        live = (tid & 63) < g.tile_rows[2 * item + (tid >> 6)];
+        bool live = (tid & 63) < g.tile_rows[2 * item + (tid >> 6)];
         float nn = 0.f;
         const float *xr = xs + (tid >> 6) * DP * kR + (tid & 63);
         for (int t = 0; t < g.width; ++t) nn = fmaf(xr[t * kR], xr[t * kR], nn);
         if constexpr (kExact) {
             tk.start(live ? g.tie_bound[item * kQ + tid] : -INFINITY, nn, g.beta, g.width);
             live = tk.bound > -INFINITY;
-            cur_item = item;
+            if (tid < 2) seeds[4 + tid] = g.tile_pos[2 * item + tid];   // (read after the next barriers)
         } else {
             tk.start(nn, g.k, g.width);
         }
@@ -795,20 +807,22 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const 
         //   kAgain   (no scan) the marks once more; still many: the item is split
         //   kChunks  the marked tiles, chunk by chunk, tested against the
         //            bounds as they are by then
-        // A part of a split item goes from kWindow over its seeds to kChunks; the
-        // ties pass, whose bounds are known, has kChunks only.
+        // A part of a split item and an item of the ties pass, whose bounds are
+        // known, have kChunks only.
         enum { kWindow, kMark, kNearest, kAgain, kChunks };
-        int step = kExact ? kChunks : kWindow, ci = 0, n_seeds = 0;
+        int step = kMode == kWhole ? kWindow : kChunks, ci = 0, n_seeds = 0;
         int64_t kept = 0;
         float near_d[2] = {INFINITY, INFINITY}, tq[2] = {INFINITY, INFINITY};
         int near_t[2] = {-1, -1};
-        bool fresh = true, deferred = false, all_ties = false;   // fresh: tq must be taken anew
+        bool fresh = true, all_ties = false;   // fresh: tq must be taken anew
+        int deferred = -1;                     // place on the list of items to be split
         if (kSplit) {
             if (tid < kSeeds) seeds[tid] = big[1 + tid];
             while (n_seeds < kSeeds && big[1 + n_seeds] >= 0) ++n_seeds;
+            if constexpr (kSplit) tk.bound = live ? g.big_bound[unit / segs * kQ + tid] : -INFINITY;
         }
         int64_t done = 0;   // flat, exact: tiles of the part seen so far
-        bool first = true;
+        bool first = !kSplit;
         // exact: rows of ids from here on are wanted by no row (INT_MAX: some may be)
         auto last_id = [&]() -> int {
             unsigned v = 0;
@@ -879,23 +893,25 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const 
                         // many tiles, and most rows are for the ties pass already:
                         // all of them, with the bounds they have
                         if (kept > most && step == kAgain &&
-                            2 * __syncthreads_count(live && tk.floor < INFINITY) >= __syncthreads_count(live)) {
+                            16 * __syncthreads_count(live && tk.floor < INFINITY) >= __syncthreads_count(live)) {
                             all_ties = true;
                             break;
                         }
                     }
                     if (kept > most && step == kAgain) {
                         if (tid == 0) {
-                            const int at = atomicAdd(g.big_count, 1);
-                            *item_s = at < kBigItems;
-                            if (at < kBigItems) {
+                            const int h = atomicAdd(g.heavy, 1), l = *reinterpret_cast<volatile int *>(g.light);
+                            const bool now = unit < whole_waves && h >= 8 && h >= 4 * l;
+                            const int at = now ? g.big_cap : atomicAdd(g.big_count, 1);
+                            *item_s = at < g.big_cap ? at : -1;
+                            if (*item_s >= 0) {
                                 g.big[at * (1 + kSeeds)] = (int32_t)item;
                                 for (int x = 0; x < kSeeds; ++x) g.big[at * (1 + kSeeds) + 1 + x] = seeds[x];
                             }
                         }
                         __syncthreads();
-                        deferred = *item_s != 0;
-                        if (deferred) break;
+                        deferred = *item_s;
+                        if (deferred >= 0) break;
                     }
                     step = kChunks;
                     continue;
@@ -983,9 +999,9 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const 
                 first = false;
             }
             if (kIsFlat) continue;
-            if (step == kWindow) step = kSplit ? (n_seeds > 0 ? kNearest : kChunks) : kMark;
+            if (step == kWindow) step = kMark;
             else if (step == kNearest) {
-                step = kSplit ? kChunks : kAgain;
+                step = kAgain;
                 kept = 0;
             }
         }
@@ -1025,37 +1041,42 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const 
                         ta.dist[o + c] = id != INT_MAX ? (ta.cosine ? 0.5f * d2 : sqrtf(d2)) : INFINITY;
                     }
             }
-        } else if constexpr (kMode != kWhole) {
+        } else {
             if constexpr (kMode != kFlat) tk.finish();
-            const int64_t slot = (kIsFlat ? item : unit / segs) * kQ + tid;
-            if (live) {
-                float *pk = g.part_key + (slot * g.part_segs + unit % segs) * KC;
-                int32_t *pi = g.part_id + (slot * g.part_segs + unit % segs) * KC;
+            if (kMode != kWhole || deferred >= 0) {   // uniform
+                const int64_t at = kIsFlat  ? ((item * kQ + tid) * g.part_segs + unit % segs) * KC
+                                   : kSplit ? (unit * kQ + tid) * KC
+                                            : ((g.units - 1 - deferred) * kQ + tid) * KC;
+                if (live) {
+                    float *pk = g.part_key + at;
+                    int32_t *pi = g.part_id + at;
 #pragma unroll
-                for (int c = 0; c < KC; c += 4) {
-                    *reinterpret_cast<float4 *>(pk + c) =
-                        make_float4(tk.top.key[c], tk.top.key[c + 1], tk.top.key[c + 2], tk.top.key[c + 3]);
-                    *reinterpret_cast<int4 *>(pi + c) =
-                        make_int4(tk.top.id[c], tk.top.id[c + 1], tk.top.id[c + 2], tk.top.id[c + 3]);
+                    for (int c = 0; c < KC; c += 4) {
+                        *reinterpret_cast<float4 *>(pk + c) =
+                            make_float4(tk.top.key[c], tk.top.key[c + 1], tk.top.key[c + 2], tk.top.key[c + 3]);
+                        *reinterpret_cast<int4 *>(pi + c) =
+                            make_int4(tk.top.id[c], tk.top.id[c + 1], tk.top.id[c + 2], tk.top.id[c + 3]);
+                    }
+                    if (kIsFlat && unit % segs == 0) g.vv[item * kQ + tid] = nn;
+                    if (kMode == kWhole) g.big_bound[deferred * kQ + tid] = tk.bound;
                 }
-                if (kIsFlat && unit % segs == 0) g.vv[slot] = nn;
+            } else {
+                if (tid == 0 && kept <= most) atomicAdd(g.light, 1);
+                emit(g, tk, item, tid, live, all_ties);
             }
-        } else if (!deferred) {   // uniform
-            tk.finish();
-            emit(g, tk, item, tid, live, all_ties);
         }
     }
     if (!kExact && tid == 0 && scanned) atomicAdd(g.scanned, scanned);
 }
 
-// Joins the lists of a split item's parts (every part scanned the tiles around
-// the query tiles, so those entries come more than once).
+// Joins the lists of a split item and its parts.
 template <int KC>
 __global__ void __launch_bounds__(kQ) merge_kernel(const Args g) {
+    const int64_t b = blockIdx.x, count = min(*g.big_count, g.big_cap);
+    if (b >= count) return;
     const int64_t tiles = *g.T;
-    const int segs = (int)ceil_div(tiles, seg_tiles(tiles));
-    const int b = blockIdx.x, tid = threadIdx.x;
-    if (b >= min(*g.big_count, kBigItems)) return;
+    const int64_t segs = ceil_div(tiles, ceil_div(tiles, (int64_t)part_count(g, count, tiles, 1)));
+    const int tid = threadIdx.x;
     const int64_t item = g.big[b * (1 + kSeeds)];
     const bool live = (tid & 63) < g.tile_rows[2 * item + (tid >> 6)];
     const float *xr = g.rec + (2 * item + (tid >> 6)) * record_floats(g.DP) + (tid & 63);
@@ -1063,31 +1084,28 @@ __global__ void __launch_bounds__(kQ) merge_kernel(const Args g) {
     for (int t = 0; t < g.width; ++t) nn = fmaf(xr[t * kR], xr[t * kR], nn);
     List<KC> tk;
     tk.start(nn, g.k, g.width);
-    const int64_t lists = ((int64_t)b * kQ + tid) * g.part_segs * KC;
-    for (int s = 0; live && s < segs; ++s) {
-        const int64_t at = lists + s * KC;
+    auto list_at = [&](int64_t s) { return ((s < segs ? b * segs + s : g.units - 1 - b) * kQ + tid) * KC; };   // segs: the item's own
+    for (int64_t s = segs; live && s >= 0; --s) {
+        const int64_t at = list_at(s);
 #pragma unroll 1
         for (int c = 0; c < KC; ++c) {
             const float v = g.part_key[at + c];
             const int j = g.part_id[at + c];
             if (j < 0 || !(v < tk.top.thr())) break;   // ascending
-            bool have = false;
-#pragma unroll
-            for (int x = 0; x < KC; ++x) have |= tk.top.id[x] == j;
-            if (!have) tk.top.insert(v, j);
+            tk.top.insert(v, j);
         }
     }
     // a part's full list whose last key is within reach is short of some rows
     const float reach = tk.reach();
     bool cut = false;
-    for (int s = 0; live && s < segs; ++s) {
-        const int64_t at = lists + s * KC + KC - 1;
+    for (int64_t s = 0; live && s <= segs; ++s) {
+        const int64_t at = list_at(s) + KC - 1;
         cut |= g.part_id[at] >= 0 && g.part_key[at] <= reach;
     }
     emit(g, tk, item, tid, live, cut);
 }
 
-constexpr int kCounters = 8;
+constexpr int kCounters = 10;
 constexpr int kMaxList = 40;
 
 // Parts' lists: the keys, then the ids (or Exact's entries in the whole of it).
@@ -1100,11 +1118,12 @@ void take_lists(Carve &cv, L &l, size_t entries) {
 struct Layout {
     float *rec, *cenT, *rad, *nmax, *tie_bound;
     int32_t *ids, *tile_pos, *tile_rows, *tie_items, *id_min;
-    int *counters;   // tie_count, counter, scanned (64 bits), tiles, big_count, unit, tie_unit; tie_done follows
+    int *counters;   // tie_count, counter, scanned (64 bits), tiles, big_count, unit, tie_unit, heavy, light; tie_done follows
     int64_t zeroed;  // ints
     int32_t *big, *part_id;
     uint32_t *bits;
-    float *part_key;
+    float *part_key, *big_bound;
+    int64_t units;
     size_t bytes;
 };
 Layout layout(void *scratch, int64_t n, int DP) {
@@ -1124,11 +1143,17 @@ Layout layout(void *scratch, int64_t n, int DP) {
     L.zeroed = kCounters + tiles / 2;
     L.counters = cv.take<int>((size_t)L.zeroed);
     L.big = cv.take<int32_t>(kBigItems * (1 + kSeeds));
+    L.big_bound = cv.take<float>(kBigItems * kQ);
     L.bits = cv.take<uint32_t>((size_t)kMaxCtas * ceil_div(tiles, (int64_t)kChunk) * kWords);
-    take_lists(cv, L, (size_t)kBigItems * kSegs * kMaxList * kQ);
+    L.units = kUnits;
+    take_lists(cv, L, (size_t)L.units * kMaxList * kQ);
     L.bytes = cv.used;
     return L;
 }
+
+// CTAs of the search that the device holds at once: their shared memory lets two
+// share an SM up to DP = 56, one at 64.
+int resident_ctas(int DP) { return sm_count() * (DP <= 56 ? 2 : 1); }
 
 Args make_args(const Layout &L, int64_t n, int DP, int width, int k, int metric, int32_t *cand, unsigned int *status) {
     Args g;
@@ -1153,7 +1178,6 @@ Args make_args(const Layout &L, int64_t n, int DP, int width, int k, int metric,
     g.tie_count = L.counters;
     g.tie_unit = L.counters + 7;
     g.tie_done = L.counters + kCounters;
-    g.tie_units = kBigItems * kSegs;
     g.counter = L.counters + 1;
     g.scanned = reinterpret_cast<unsigned long long *>(L.counters + 2);
     g.bits = L.bits;
@@ -1162,7 +1186,13 @@ Args make_args(const Layout &L, int64_t n, int DP, int width, int k, int metric,
     g.unit = L.counters + 6;
     g.part_key = L.part_key;
     g.part_id = L.part_id;
-    g.part_segs = kSegs;
+    g.part_segs = 0;
+    g.heavy = L.counters + 8;
+    g.light = L.counters + 9;
+    g.big_bound = L.big_bound;
+    g.units = L.units;
+    g.big_cap = (int)std::min<int64_t>(kBigItems, L.units / 2);
+    g.slots = resident_ctas(DP);
     g.vv = nullptr;
     g.status = status;
     g.wait_budget = tc_wait_budget();
@@ -1192,7 +1222,7 @@ cudaError_t launch_list(const Args &g, int64_t tiles, cudaStream_t st) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(split, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     whole<<<(unsigned)std::min<int64_t>(tiles / 2, std::min(kMaxCtas, 2 * sm_count())), kQ, smem, st>>>(g, TieArgs{});
-    split<<<(unsigned)std::min<int64_t>(kBigItems * kSegs, 2 * sm_count()), kQ, smem, st>>>(g, TieArgs{});
+    split<<<(unsigned)(2 * sm_count()), kQ, smem, st>>>(g, TieArgs{});
     merge_kernel<KC><<<kBigItems, kQ, 0, st>>>(g);
     return cudaGetLastError();
 }
@@ -1321,7 +1351,8 @@ Args flat_args(const FlatLayout &L, int64_t n, int DP, int width, int k, unsigne
     g.tie_unit = L.counters + 5;
     g.tie_done = L.counters + kFlatCounters;
     // lists of 16 (k <= 16) or 32 entries in the room of part_segs lists an item
-    g.tie_units = ceil_div(n, (int64_t)kQ) * g.part_segs;
+    g.units = ceil_div(n, (int64_t)kQ) * g.part_segs;
+    g.slots = resident_ctas(DP);
     g.status = status;
     g.wait_budget = tc_wait_budget();
     return g;

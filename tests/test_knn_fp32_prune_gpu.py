@@ -199,3 +199,21 @@ def test_ties_pass_of_cosine_rows(rsc, n):  # noqa: F811
     np.testing.assert_allclose(gd[q], od, rtol=0, atol=1e-6)
     zeros = np.flatnonzero((X == 0).all(1))
     assert (gi[zeros] == zeros[:15]).all()
+
+
+@pytest.mark.parametrize("n,k,clustered", [
+    (20_000, 15, 0), (40_000, 15, 0), (40_000, 32, 0), (150_000, 15, 0), (180_000, 15, 90_000),
+])
+def test_rows_that_no_sphere_separates(rsc, n, k, clustered):  # noqa: F811
+    # every item keeps most tiles: fewer items than a wave of CTAs (all are
+    # split), a wave and a few more (these are), several waves, parts longer
+    # than a chunk of tiles; and beside as many clustered rows, where more
+    # items are put off than the list holds (640)
+    rng = np.random.Generator(np.random.PCG64(n + k))
+    X = rng.uniform(-1, 1, (n, 12)).astype(np.float32)
+    if clustered:
+        X[:clustered] = synth.mixture(clustered, 12, n_comp=60, seed=1)
+        X = X[rng.permutation(n)]
+    (pi, pd), (fi, fd) = _both(rsc, X, k)
+    np.testing.assert_array_equal(pi, fi)
+    np.testing.assert_array_equal(pd, fd)
