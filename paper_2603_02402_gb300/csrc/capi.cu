@@ -256,7 +256,7 @@ KnnLayout carve_knn(void *ws, int64_t n, const KnnPlan &p, size_t *bytes) {
     L.st_id = nullptr;
     L.prune_scratch = nullptr;
     if (p.simt_flat) L.prune_scratch = cv.take<uint8_t>(simt_flat_scratch_bytes(n, p.DP, p.k));
-    if (p.simt_prune) L.prune_scratch = cv.take<uint8_t>(simt_pruned_scratch_bytes(n, p.DP));
+    if (p.simt_prune) L.prune_scratch = cv.take<uint8_t>(simt_pruned_scratch_bytes(n, p.DP, p.k));
     if (p.prune) {
         L.st_key = cv.take<float>((size_t)n * p.parts * p.KC);
         L.st_id = cv.take<int32_t>((size_t)n * p.parts * p.KC);
@@ -627,7 +627,7 @@ rsc_status rsc_knn_scan_stats(int64_t n, int32_t d, int32_t k, int32_t metric, c
     if (p.simt_prune) {   // counted by 64-row tiles
         const KnnLayout L = carve_knn(workspace, n, p, nullptr);
         unsigned long long tiles = 0;
-        RSC_CUDA_TRY(cudaMemcpyAsync(&tiles, simt_pruned_scanned(L.prune_scratch, n, p.DP), sizeof(tiles),
+        RSC_CUDA_TRY(cudaMemcpyAsync(&tiles, simt_pruned_scanned(L.prune_scratch, n, p.DP, p.k), sizeof(tiles),
                                      cudaMemcpyDeviceToHost, st));
         RSC_CUDA_TRY(cudaStreamSynchronize(st));
         *pairs_scanned = std::min<int64_t>(*pairs_total, (int64_t)((tiles + 1) / 2));

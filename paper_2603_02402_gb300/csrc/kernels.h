@@ -35,9 +35,9 @@ struct OrderTarget;
 struct OrderLeaves;
 OrderTarget simt_pruned_target();   // the ordering this search wants
 int simt_pruned_list(int k);
-size_t simt_pruned_scratch_bytes(int64_t n, int DP);
+size_t simt_pruned_scratch_bytes(int64_t n, int DP, int k);
 // (tile of 64 rows, 128 query rows) pairs scanned by the last search, on the device
-const unsigned long long *simt_pruned_scanned(void *scratch, int64_t n, int DP);
+const unsigned long long *simt_pruned_scanned(void *scratch, int64_t n, int DP, int k);
 cudaError_t launch_knn_simt_pruned(const float *Y, const float *ny, int64_t n, int DP, int width, int k, int metric,
                                    const int32_t *perm, const OrderLeaves &leaves, void *scratch, int32_t *cand,
                                    unsigned int *status, cudaStream_t st);

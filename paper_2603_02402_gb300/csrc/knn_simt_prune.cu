@@ -1126,7 +1126,7 @@ struct Layout {
     int64_t units;
     size_t bytes;
 };
-Layout layout(void *scratch, int64_t n, int DP) {
+Layout layout(void *scratch, int64_t n, int DP, int k) {
     Carve cv(scratch);
     Layout L;
     const int64_t tiles = tiles_max(n);
@@ -1145,8 +1145,10 @@ Layout layout(void *scratch, int64_t n, int DP) {
     L.big = cv.take<int32_t>(kBigItems * (1 + kSeeds));
     L.big_bound = cv.take<float>(kBigItems * kQ);
     L.bits = cv.take<uint32_t>((size_t)kMaxCtas * ceil_div(tiles, (int64_t)kChunk) * kWords);
-    L.units = kUnits;
-    take_lists(cv, L, (size_t)L.units * kMaxList * kQ);
+    // room for eight parts of every item of a small input, of up to 1,792 lists in
+    // all: 30 MB at 16,384 rows, 44 MB from 25,000 on (k <= 16; 50 and 73 beyond)
+    L.units = std::min<int64_t>(kUnits, 9 * (ceil_div(n, (int64_t)kQ) + 8));
+    take_lists(cv, L, (size_t)L.units * simt_pruned_list(k) * kQ);
     L.bytes = cv.used;
     return L;
 }
@@ -1205,10 +1207,10 @@ Args make_args(const Layout &L, int64_t n, int DP, int width, int k, int metric,
 // fill the list.
 int simt_pruned_list(int k) { return k <= 16 ? 24 : k <= 32 ? 40 : 0; }
 
-size_t simt_pruned_scratch_bytes(int64_t n, int DP) { return simtp::layout(nullptr, n, DP).bytes; }
+size_t simt_pruned_scratch_bytes(int64_t n, int DP, int k) { return simtp::layout(nullptr, n, DP, k).bytes; }
 
-const unsigned long long *simt_pruned_scanned(void *scratch, int64_t n, int DP) {
-    return reinterpret_cast<unsigned long long *>(simtp::layout(scratch, n, DP).counters + 2);
+const unsigned long long *simt_pruned_scanned(void *scratch, int64_t n, int DP, int k) {
+    return reinterpret_cast<unsigned long long *>(simtp::layout(scratch, n, DP, k).counters + 2);
 }
 
 namespace simtp {
@@ -1248,7 +1250,7 @@ cudaError_t launch_knn_simt_pruned(const float *Y, const float *ny, int64_t n, i
                                    const int32_t *perm, const OrderLeaves &leaves, void *scratch, int32_t *cand,
                                    unsigned int *status, cudaStream_t st) {
     using namespace simtp;
-    const Layout L = layout(scratch, n, DP);
+    const Layout L = layout(scratch, n, DP, k);
     const int64_t tiles = tiles_max(n);
     cudaError_t e = cudaMemsetAsync(L.counters, 0, L.zeroed * sizeof(int), st);
     if (e != cudaSuccess) return e;
@@ -1262,7 +1264,7 @@ cudaError_t launch_knn_simt_pruned(const float *Y, const float *ny, int64_t n, i
 cudaError_t launch_simt_ties(int64_t n, int d, int DP, int width, int k, int metric, void *scratch, const float *R,
                              int64_t rs, int32_t *idx, float *dist, unsigned int *status, cudaStream_t st) {
     using namespace simtp;
-    const Args g = make_args(layout(scratch, n, DP), n, DP, width, k, metric, nullptr, status);
+    const Args g = make_args(layout(scratch, n, DP, k), n, DP, width, k, metric, nullptr, status);
     return launch_ties<kTies>(g, d, metric, R, rs, idx, dist, st);
 }
 

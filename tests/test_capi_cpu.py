@@ -311,3 +311,11 @@ def test_leiden_argument_errors(L):
             rsc.RSC_ERR_INVALID_ARG
     assert L.rsc_leiden(None, vp, vp, 10, 20, None, vp, None, None, ctypes.byref(o), vp, 1 << 30) == \
         rsc.RSC_ERR_INVALID_ARG
+
+
+def test_workspace_of_the_pruned_fp32_search_follows_its_lists(L):
+    # lists of 24 (k <= 16) and 40 entries of 8 bytes, 128 rows each; no more
+    # room for split items than a small input has items to split
+    short, long = (rsc.rsc_knn_workspace_size(16_384, 50, k, precision="fp32") for k in (16, 17))
+    assert short + (15 << 20) < long
+    assert short < 90 << 20
