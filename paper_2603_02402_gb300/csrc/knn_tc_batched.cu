@@ -237,8 +237,8 @@ size_t cross_smem(int w4) {
 // 32 candidates at a time, which lie in a row: eight lanes copy a candidate's
 // row to shared memory (a lane that reads a row of its own touches 32 lines an
 // instruction, and those lookups were what the kernel waited for), then a lane
-// sums a row in order.  The distances of 32 samples are kept, and a lane picks
-// its sample's best.  600k rows, 32 samples, d = 50: 11.66 -> 9.55 ms.
+// sums a row in order.  The distances of 16 samples (of four parts; 32 of two)
+// are kept, and a lane picks its sample's best.  600k rows, 32 samples, d = 50: 11.66 -> 9.55 ms.
 template <int E>
 __global__ void __launch_bounds__(kXWarps * 32)
 rerank_cross_kernel(const float *__restrict__ R, int64_t rs, int64_t N, int d, int metric, int w4,
@@ -323,7 +323,11 @@ rerank_cross_kernel(const float *__restrict__ R, int64_t rs, int64_t N, int d, i
                 }
                 __syncwarp();
             } else {
-                acc = row_dist2(xq, R + (int64_t)row * rs, d, 0);
+                const float *y = R + (int64_t)row * rs;   // rows that start anywhere, components in the same order
+                for (int c = 0; c < d; ++c) {
+                    const float u = xq[c] - __ldg(y + c);
+                    acc = fmaf(u, u, acc);
+                }
             }
             if (cosine) {
                 const bool fy = __ldg(R + (int64_t)row * rs + d) != 0.f;

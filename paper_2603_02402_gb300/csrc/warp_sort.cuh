@@ -82,37 +82,4 @@ __device__ __forceinline__ void warp_merge_best(float &bk, int &bi, float key, i
     }
 }
 
-// Squared distance sum_t (xq_t - y_t)^2 for t < d, accumulated in t order
-// (the same rounding whichever loader runs).  w4 > 0: the row is 16-byte
-// aligned and its first 4 * w4 floats (w4 <= 16) are read as independent
-// float4 loads up front; w4 == 0: scalar loads.
-__device__ __forceinline__ float row_dist2(const float *xq, const float *__restrict__ yr, int d, int w4) {
-    float acc = 0.f;
-    if (w4 > 0) {
-        float y[64];
-        const float4 *y4 = reinterpret_cast<const float4 *>(yr);
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-            const float4 v = (u < w4) ? __ldg(y4 + u) : make_float4(0.f, 0.f, 0.f, 0.f);
-            y[4 * u] = v.x;
-            y[4 * u + 1] = v.y;
-            y[4 * u + 2] = v.z;
-            y[4 * u + 3] = v.w;
-        }
-#pragma unroll
-        for (int t = 0; t < 64; ++t) {
-            if (t < d) {
-                const float diff = xq[t] - y[t];
-                acc = fmaf(diff, diff, acc);
-            }
-        }
-    } else {
-        for (int t = 0; t < d; ++t) {
-            const float diff = xq[t] - __ldg(yr + t);
-            acc = fmaf(diff, diff, acc);
-        }
-    }
-    return acc;
-}
-
 }  // namespace rsc
