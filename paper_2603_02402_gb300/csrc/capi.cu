@@ -190,7 +190,7 @@ rsc_status plan_knn(int64_t n, int32_t d, int32_t k, int32_t metric, const rsc_k
     }
     // database splits: enough CTAs to fill the GPU when there are few queries
     const int64_t qrows = tc ? 128 : 256;             // query rows per CTA work unit
-    const int64_t target = 152;                       // work units wanted (persistent CTAs)
+    const int64_t target = kPlanSMs;                  // work units wanted (persistent CTAs)
     const int64_t align = tc ? knn_tc_split_align() : 64;
     const int64_t qblocks = ceil_div(n, qrows);
     const int per_split = p->parts * p->KC;           // candidate ids per row and split
@@ -200,8 +200,8 @@ rsc_status plan_knn(int64_t n, int32_t d, int32_t k, int32_t metric, const rsc_k
         // (each split adds a candidate list per row), else the fullest
         double best = -1.0;
         for (int s = 1; s <= 8; ++s) {
-            const int64_t ctas = qblocks * s, waves = ceil_div(ctas, (int64_t)152);
-            const double fill = (double)ctas / (double)(152 * waves);
+            const int64_t ctas = qblocks * s, waves = ceil_div(ctas, (int64_t)kPlanSMs);
+            const double fill = (double)ctas / (double)(kPlanSMs * waves);
             if (fill >= 0.94) {
                 splits = s;
                 break;

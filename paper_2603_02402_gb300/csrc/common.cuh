@@ -54,6 +54,10 @@ constexpr size_t kStatusBytes = 256;
 __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 int sm_count();   // multiprocessors of the current device (cached per device)
+// Multiprocessors that sizes and layouts are planned for: workspace queries run
+// on hosts without a device, and a plan must not change between the query and
+// the call.
+constexpr int kPlanSMs = 152;
 
 // ------------------------------------------------------------- device side
 

@@ -1153,9 +1153,9 @@ Layout layout(void *scratch, int64_t n, int DP, int k) {
     return L;
 }
 
-// CTAs of the search that the device holds at once: their shared memory lets two
-// share an SM up to DP = 56, one at 64.
-int resident_ctas(int DP) { return sm_count() * (DP <= 56 ? 2 : 1); }
+// CTAs that an SM holds: their shared memory lets two share it up to DP = 56.
+int ctas_per_sm(int DP) { return DP <= 56 ? 2 : 1; }
+int resident_ctas(int DP) { return sm_count() * ctas_per_sm(DP); }
 
 Args make_args(const Layout &L, int64_t n, int DP, int width, int k, int metric, int32_t *cand, unsigned int *status) {
     Args g;
@@ -1372,7 +1372,7 @@ Args flat_args(const FlatLayout &L, int64_t n, int DP, int width, int k, unsigne
 // query tiles fetched).
 int simt_flat_segs(int64_t n, int DP) {
     const int64_t items = ceil_div(n, (int64_t)simtp::kQ), tiles = ceil_div(n, (int64_t)simtp::kR);
-    const int64_t slots = 152 * (DP <= 56 ? 2 : 1);   // CTAs an SM holds
+    const int64_t slots = kPlanSMs * simtp::ctas_per_sm(DP);
     int best = 1;
     int64_t cost = INT64_MAX;
     for (int s = 1; s <= kSimtFlatSegs && s <= tiles; ++s) {

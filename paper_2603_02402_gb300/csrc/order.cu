@@ -48,7 +48,7 @@ constexpr int kMaxSub = 1024;        // keys per warp slice at most
 // before the slices get longer.  68,579 keys: 5 us a scatter with slices of
 // 128, 16 us with slices of 1,024 on nine blocks.
 int sub_len(int64_t m) {
-    return (int)std::min<int64_t>(kMaxSub, std::max<int64_t>(128, ceil_div(m, (int64_t)kSortWarps * 152 * 32) * 32));
+    return (int)std::min<int64_t>(kMaxSub, std::max<int64_t>(128, ceil_div(m, (int64_t)kSortWarps * kPlanSMs * 32) * 32));
 }
 int64_t chunk_len(int64_t m) { return (int64_t)kSortWarps * sub_len(m); }
 
@@ -306,15 +306,15 @@ centroid_mean_kernel(const float *__restrict__ Y, int DP, const int32_t *__restr
 // Sub-cluster assignment: key i is row rows[i * step] (rows given) or
 // i * step; its coarse cluster c1 = lab1[row]; label = c1 * C2 + the nearest
 // of c1's C2 sub-centroids (|c|^2 - 2 x.c, ties to the lower index), written
-// at out[row] (by_row) or out[i].  kTwo: lab1b, a second coarse cluster of every row,
-// whose sub-centroids count too.  Thread per key; the C2
-// sub-centroids of a coarse cluster are read through L1 (neighbouring keys
-// share them).
+// at out[row] (by_row) or out[i].  kTwo: lab1b, a second coarse cluster of every
+// row, whose sub-centroids count too.  Thread per key; the C2 sub-centroids of a
+// coarse cluster are read through L1 (neighbouring keys share them).
 template <int DP, bool kTwo>
 __global__ void __launch_bounds__(kAssignThreads)
 assign_sub_kernel(const float *__restrict__ Y, int64_t m, int64_t step, const int32_t *__restrict__ rows,
                   const int32_t *__restrict__ lab1, const int32_t *__restrict__ lab1b,
-                  const float *__restrict__ cent2, const float *__restrict__ cnorm2, int C2, bool by_row, const int32_t *__restrict__ rank1, const int32_t *__restrict__ rank2,
+                  const float *__restrict__ cent2, const float *__restrict__ cnorm2, int C2, bool by_row,
+                  const int32_t *__restrict__ rank1, const int32_t *__restrict__ rank2,
                   int32_t *__restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
