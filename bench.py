@@ -61,6 +61,42 @@ NND_SOURCES = ("nndescent.cu",)
 ORDER_MIN_ROWS = 16384   # automatic locality ordering from this many rows
 
 
+def _cdiv(a, b):
+    return -(-a // b)
+
+
+def _second_scans(*counts):
+    """Scans that take a second launch: those of more than 65,536 counts (csrc/scan.cuh, launches)."""
+    return sum(c > 65536 for c in counts)
+
+
+def _sort_chunks(m):
+    """Count columns of a counting sort of m keys (csrc/order.cu, sub_len: 8 slices a chunk)."""
+    return _cdiv(m, 8 * min(1024, max(128, _cdiv(m, 8 * 152 * 32) * 32)))
+
+
+def order_scans(n, spread=False, groups=0):
+    """Second scan launches of the locality ordering (csrc/order.cu, order_shape: coarse clusters x
+    sub-clusters, sorts of a strided sample and of all rows at both levels, then of the groups)."""
+    if spread:
+        c1 = min(128, _cdiv(n, 128))
+        c2 = min(16, 2 + _cdiv(n, c1 * 128))
+    else:
+        c1, c2 = min(128, max(1, _cdiv(n, 16 * 512))), 16
+    sample = lambda m: n // (n // min(n, m))   # noqa: E731
+    m1, m2 = sample(c1 * 64), sample(c1 * c2 * 32)
+    sorts = [(m1, c1)] * 2 + [(n, c1)] + [(m2, c1 * c2)] * 2 + [(n, c1 * c2)] + ([(n, groups)] if groups else [])
+    return _second_scans(*(c * _sort_chunks(m) for m, c in sorts))
+
+
+def prune_scans(n):
+    """Second scan launches of the tile bounds (csrc/prune.cu, prune_shape)."""
+    qtiles, dtiles, chunk = _cdiv(n, 128), _cdiv(n, 256), 32
+    while chunk < 256 and _cdiv(qtiles, 128) * _cdiv(dtiles, chunk) > 1024:
+        chunk *= 2
+    return _second_scans(qtiles * _cdiv(dtiles, chunk))
+
+
 def launches_per_step(metric, precision, n):
     """Kernels this library launches per graph step.
 
@@ -71,17 +107,17 @@ def launches_per_step(metric, precision, n):
         tile and group spheres, tau, kept tiles, scan, fill, offsets, item order,
         list pass); below: operand prep and one scan;
       FP32 from ORDER_MIN_ROWS rows on: the ordering (33), tile table, records,
-        search, its split items, their merge, ties; below: records, search, ties.
-    Scans of more than 65,536 counts take a second launch, which is not counted.
+        search, its split items, their merge, ties; below: records, search, ties;
+    and the second launches of long scans (order_scans, prune_scans).
     rsc_connectivities: 8 (smooth, push, match, two scan launches, emit and the
     two queued-row passes).
     """
     ordered = n >= ORDER_MIN_ROWS
     knn = (3 if metric == "euclidean" else 1) + 1
     if precision == "fp32":
-        knn += 33 + 6 if ordered else 3
+        knn += 33 + 6 + order_scans(n, spread=True) if ordered else 3
     elif precision == "bf16":
-        knn += 1 + (33 + 10 if ordered else 1)
+        knn += 1 + (33 + 10 + order_scans(n) + prune_scans(n) if ordered else 1)
     else:
         knn += 1
     return knn + 8
@@ -618,9 +654,10 @@ def run_batched(args):
                          "note": "whole call (prep + pruned search + both re-ranks) timed; 2*d flops per "
                                  "(query, row) pair computed: 128*256 per scanned tile pair"},
             # prep, ordering, sample-preserving partition, operands, pruned search, gather, the two
-            # re-ranks; scans of more than 65,536 counts take a second launch, which is not counted;
-            # 7 without the ordering (fewer than ORDER_MIN_ROWS rows)
-            "gpu_launches": (52 if n >= ORDER_MIN_ROWS else 7) * args.steps, "clocks": sampler.summary(),
+            # re-ranks, and the second launches of long scans (the kept tiles are scanned by query
+            # tile and sample); 7 without the ordering (fewer than ORDER_MIN_ROWS rows)
+            "gpu_launches": (52 + order_scans(n, groups=64) + _second_scans(sum(_cdiv(int(s), 128) for s in sizes) * 64)
+                             if n >= ORDER_MIN_ROWS else 7) * args.steps, "clocks": sampler.summary(),
             "autotune": {"choice": tuned, "best_ms": tune_ms}}
     if rank == 0 and not args.no_cpu_baseline:
         line["cpu_baseline"] = batched_baseline(X, off, kw, kx, out)
