@@ -46,7 +46,7 @@
 //
 // What bounds it: the FMA pipe and, next to it, the insertions (a row takes in
 // about 70 values).  50 components, k = 15, one GB300, whole call (in brackets
-// the full scan): 100,003 rows, 60 clusters 1.57 ms (25.9), of which this kernel
+// the full scan): 100,003 rows, 60 clusters 1.58 ms (25.9), of which this kernel
 // 0.8 and the ordering 0.5; 1M rows, 100 clusters 33 ms (2058).  Rows without any
 // clusters, of which no tile is dropped (in the second brackets with every item
 // run whole or, the first 192, in eight parts that each scanned the item's
