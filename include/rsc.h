@@ -360,8 +360,9 @@ rsc_status rsc_partitioner_build_index(rsc_partitioner *p, const float *X, int64
  * k nearest neighbours (Euclidean, ids of X, self included when probed,
  * ordered by (distance, id)) of query_rows (device int32 [n_queries]; NULL =
  * every row, n_queries ignored) among the rows of the indexed X, probing
- * n_probe in {1, 2, 4, 8} parts per query.  routing: 0 = the network's
- * top parts, 1 = nearest centroids.  idx/dist [n_queries, k].
+ * n_probe in {1, 2, 4, 8} parts per query (fewer where fewer have a logit or a
+ * distance that is a number).  routing: 0 = the network's top parts, 1 =
+ * nearest centroids.  idx/dist [n_queries, k].
  */
 rsc_status rsc_knn_partitioned(rsc_partitioner *p, const float *X, int64_t n, int32_t k,
                                int32_t n_probe, int32_t routing, const int32_t *query_rows,

@@ -305,10 +305,10 @@ route_kernel(const float *__restrict__ X, const int32_t *__restrict__ rows, int6
     const int kb = k_blocks(H), nc = chunks(P), nb = weight_blocks(H, P);
     const int64_t tiles = ceil_div(count, (int64_t)kTM);
 
-    // bounded; after the first try a budget shorter than a few sleeps is polled
+    // bounded; a budget shorter than a few sleeps is polled
     const uint32_t sleep_ns = wait_budget < 8 * (long long)kSleepNs ? 0 : kSleepNs;
     auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {
-        if (tc::mbar_try_wait(bar, parity)) return true;
+        if (sleep_ns == 0 ? tc::mbar_test_wait(bar, parity) : tc::mbar_try_wait(bar, parity)) return true;
         const long long t0 = clock64();
         while (!tc::mbar_arrived(bar, parity, sleep_ns)) {
             if (*abort_flag) return false;
