@@ -1190,9 +1190,10 @@ rsc_status rsc_partitioner_workspace_size(const rsc_partitioner *p, int64_t n, i
     return RSC_OK;
 }
 
-rsc_status rsc_partitioner_build_index(rsc_partitioner *p, const float *X, int64_t n, void *workspace,
-                                       size_t workspace_bytes, void *stream) {
-    RSC_TRACE("rsc_partitioner_build_index");
+// The index of X's rows; `fresh`: a call of its own, whose status word starts
+// clear (training has recorded in it already).
+static rsc_status build_index(rsc_partitioner *p, const float *X, int64_t n, void *workspace, size_t workspace_bytes,
+                              void *stream, bool fresh) {
     rsc_status s = check_handle(p);
     if (s != RSC_OK) return s;
     if (!X || n < 1 || n >= (int64_t(1) << 31)) return fail(RSC_ERR_INVALID_ARG, "X / n");
@@ -1201,6 +1202,7 @@ rsc_status rsc_partitioner_build_index(rsc_partitioner *p, const float *X, int64
     if (!workspace || workspace_bytes < need) return fail(RSC_ERR_WORKSPACE, "workspace needs %zu bytes", need);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     PartLayout L = carve_part(workspace, p, n, 0, 1, 1, 1, nullptr);
+    if (fresh) RSC_CUDA_TRY(cudaMemsetAsync(L.status, 0, sizeof(unsigned int), st));
     if (p->n_db != n) {   // (re)allocate the index arrays owned by the handle
         RSC_CUDA_TRY(cudaStreamSynchronize(st));
         cudaFree(p->perm);
@@ -1226,6 +1228,12 @@ rsc_status rsc_partitioner_build_index(rsc_partitioner *p, const float *X, int64
         static_cast<const uint4 *>(L.Db), p->perm, n, static_cast<uint4 *>(p->Db_sorted));
     RSC_CUDA_TRY(cudaGetLastError());
     return RSC_OK;
+}
+
+rsc_status rsc_partitioner_build_index(rsc_partitioner *p, const float *X, int64_t n, void *workspace,
+                                       size_t workspace_bytes, void *stream) {
+    RSC_TRACE("rsc_partitioner_build_index");
+    return build_index(p, X, n, workspace, workspace_bytes, stream, true);
 }
 
 rsc_status rsc_partitioner_train(rsc_partitioner *p, const float *X, int64_t n, const int32_t *train_rows,
@@ -1313,7 +1321,7 @@ rsc_status rsc_partitioner_train(rsc_partitioner *p, const float *X, int64_t n, 
     if (ks != RSC_OK) return ks;
     if (final_loss) *final_loss = epoch_loss;
     // 4. index the database by the trained network
-    return rsc_partitioner_build_index(p, X, n, workspace, workspace_bytes, stream);
+    return build_index(p, X, n, workspace, workspace_bytes, stream, false);
 }
 
 rsc_status rsc_knn_partitioned(rsc_partitioner *p, const float *X, int64_t n, int32_t k, int32_t n_probe,

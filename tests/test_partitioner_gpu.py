@@ -246,3 +246,20 @@ def test_training_with_a_row_that_is_no_number(rsc):
     oi, od, _ = oracle.knn(X, k)
     np.testing.assert_allclose(gd.cpu().numpy(), od, rtol=1e-5, atol=1e-6)
     assert (gi.cpu().numpy() >= 0).all()
+
+
+def test_build_index_starts_with_a_clear_status_word(rsc):
+    # whatever the workspace held before: a word left there would read as a
+    # failure, and a failure would not be recorded over it
+    X = torch.from_numpy(synth.mixture(2_000, 20, n_comp=5, seed=1)).cuda()
+    part = rsc.Partitioner(20, 16, 32, bf16_weights=True, seed=1)
+    ws = torch.full((part.workspace_size(2_000, 0, 10, 2_000, 8),), 7, dtype=torch.uint8, device="cuda")
+    part.build_index(X, workspace=ws)
+    assert rsc.rsc_workspace_status(ws) == rsc.RSC_OK
+    ws.fill_(7)
+    rsc.rsc_set_wait_budget(300)
+    try:
+        part.build_index(X, workspace=ws)
+        assert rsc.rsc_workspace_status(ws) == rsc.RSC_ERR_TIMEOUT
+    finally:
+        rsc.rsc_set_wait_budget(0)
