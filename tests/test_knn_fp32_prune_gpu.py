@@ -217,3 +217,15 @@ def test_rows_that_no_sphere_separates(rsc, n, k, clustered):  # noqa: F811
     (pi, pd), (fi, fd) = _both(rsc, X, k)
     np.testing.assert_array_equal(pi, fi)
     np.testing.assert_array_equal(pd, fd)
+
+
+@pytest.mark.parametrize("n,strays", [(30_000, 60), (30_000, 900), (100_003, 2_500)])
+def test_rows_far_from_every_cluster(rsc, n, strays):  # noqa: F811
+    # strays get small leaves of their own: tiles of few rows where these are
+    # few, small leaves in common tiles where they would be many
+    X = synth.mixture(n, 50, n_comp=30, seed=n)
+    rng = np.random.Generator(np.random.PCG64(strays))
+    X[rng.permutation(n)[:strays]] = 20 * rng.standard_normal((strays, 50)).astype(np.float32)
+    (pi, pd), (fi, fd) = _both(rsc, X, 15)
+    np.testing.assert_array_equal(pi, fi)
+    np.testing.assert_array_equal(pd, fd)
