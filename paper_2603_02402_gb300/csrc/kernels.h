@@ -59,7 +59,7 @@ struct SimtParts {
     int32_t *tie_items;
     float *tie_bound;     // [row] its reach, -inf when the row is not for the pass
 };
-int simt_flat_segs(int64_t n, int DP);
+int simt_flat_segs(int64_t n);
 size_t simt_flat_scratch_bytes(int64_t n, int DP, int k);
 SimtParts simt_flat_parts(void *scratch, int64_t n, int DP, int k);
 cudaError_t launch_knn_simt_flat(const float *Y, const float *ny, int64_t n, int DP, int width, int k, void *scratch,

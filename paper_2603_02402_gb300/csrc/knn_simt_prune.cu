@@ -32,8 +32,7 @@
 // clusters, tiles cut every 64 rows whatever the leaves: 10.9 % of the pairs
 // scanned and a few items that scanned everything, 15.4 ms).
 //
-// Persistent CTAs, two per SM (one with 64 components, whose tiles leave shared
-// memory for no more); an item is two tiles of query rows, each with its own
+// Persistent CTAs, two per SM; an item is two tiles of query rows, each with its own
 // sphere and tau (the database tile is scanned when either keeps it).  The CTA
 // scans the tiles around its own, then walks the database in chunks of 256 tiles
 // from its own chunk on: tests every tile's sphere against its current taus, and
@@ -76,7 +75,12 @@ constexpr int kQ = 128;                   // query rows per item, threads per CT
 static_assert(kQ == kTieItem && kQ <= 512, "ties items; 16 bits a hit");
 constexpr int kR = 64;                    // database rows per tile
 constexpr int kPitch = kR + 4;            // s rows on 16 bytes, conflict-free scans
-constexpr int kCap = 20;                  // top-k buffer entries per thread
+// top-k buffer entries per thread: with 12 two CTAs share an SM at DP = 64 too
+// (cap_of).  64 components, k = 15, one CTA with 20 entries and two with 12: rows
+// without clusters 10.7 and 8.5 ms at 50,000 rows (full scan 8.7), 36.7 and 30.0 at
+// 100,003 (31.7), 2.0 and 1.8 at 16,384 (1.6); clustered rows 2.09 and 1.74 at
+// 100,003, 0.69 and 0.52 at 10,000, 0.88 and 0.92 at 16,384.
+constexpr int kCapNarrow = 20, kCapWide = 12;
 constexpr int kChunk = 256;               // tiles tested at a time
 constexpr int kWords = kChunk / 32;
 constexpr int kExactFirst = 2, kExactStep = 16;   // tiles between two looks at the bounds in the ties pass
@@ -98,6 +102,10 @@ __host__ __device__ inline int64_t tiles_max(int64_t n) { return (ceil_div(n, (i
 // record of a tile: DP x 64 components, then 64 |y|^2
 __host__ __device__ inline int record_floats(int DP) { return (DP + 1) * kR; }
 
+static_assert(kBatch * (sizeof(unsigned long long) + sizeof(uint16_t)) <= 2 * kCapWide * kQ * sizeof(float),
+              "the ties pass keeps its batch where the buffers lie");
+__host__ __device__ inline int cap_of(int DP) { return DP <= 56 ? kCapNarrow : kCapWide; }
+
 struct Smem {
     int xs, ys, s, buf, list, cen, bars, total;   // byte offsets
 };
@@ -107,7 +115,7 @@ __host__ __device__ inline Smem smem_layout(int DP) {
     m.ys = m.xs + 2 * DP * kR * 4;
     m.s = m.ys + kStages * record_floats(DP) * 4;
     m.buf = m.s + kQ * kPitch * 4;
-    m.list = m.buf + 2 * kCap * kQ * 4;
+    m.list = m.buf + 2 * cap_of(DP) * kQ * 4;
     m.cen = m.list + kChunk * 4;
     m.bars = m.cen + 2 * 64 * 4;
     m.total = m.bars + 256;
@@ -302,7 +310,7 @@ pack_kernel(const float *__restrict__ Y, const float *__restrict__ ny, int DP, c
 // full of entries within reach of its k-th, and from then on it takes in only
 // what lies below the k-th (rows that are all the same would otherwise buffer
 // every value they meet).
-template <int KC>
+template <int KC, int kCap>
 struct List {
     RowTopK<KC> top;
     float bound;          // values above it cannot be among the k nearest, or are left to the ties pass:
@@ -469,8 +477,8 @@ __device__ __forceinline__ int part_count(const Args &g, int64_t count, int64_t 
 // The candidates of an item's rows (a thread each; lists finished), and the
 // item for the ties pass if more rows may lie within reach of one than its list
 // holds (cut: a part's list was short).
-template <int KC>
-__device__ __forceinline__ void emit(const Args &g, const List<KC> &tk, int64_t item, int tid, bool live, bool cut) {
+template <int KC, int kCap>
+__device__ __forceinline__ void emit(const Args &g, const List<KC, kCap> &tk, int64_t item, int tid, bool live, bool cut) {
     const float reach = tk.reach();
     if (live) {
         int32_t *out = g.cand + (g.tile_pos[2 * item + (tid >> 6)] + (tid & 63)) * (int64_t)KC;
@@ -565,7 +573,7 @@ struct TieArgs {
 // search of fewer rows than an ordering pays for (see launch_knn_simt_flat).
 // kTies, kFlatTies: the ties pass after either search (KC: Exact's entries).
 enum { kWhole, kSplitItems, kFlat, kTies, kFlatTies };
-template <int KC, int kMode>
+template <int KC, int kMode, int kCap>
 __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const TieArgs ta) {
     constexpr bool kSplit = kMode == kSplitItems, kIsFlat = kMode == kFlat || kMode == kFlatTies;
     constexpr bool kExact = kMode == kTies || kMode == kFlatTies;
@@ -593,7 +601,7 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const 
         tc::fence_barrier_init();
     }
     __syncthreads();
-    typename std::conditional<kExact, Exact<KC>, List<KC>>::type tk;
+    typename std::conditional<kExact, Exact<KC>, List<KC, kCap>>::type tk;
     if constexpr (!kExact) tk.sbase = (uint32_t)__cvta_generic_to_shared(reinterpret_cast<float *>(sm + m.buf) + tid);
     // bounded; a budget shorter than a few sleeps is polled
     const uint32_t sleep_ns = g.wait_budget < 8 * (long long)kSleepNs ? 0 : kSleepNs;
@@ -1098,7 +1106,7 @@ __global__ void __launch_bounds__(kQ) merge_kernel(const Args g) {
     const float *xr = g.rec + (2 * item + (tid >> 6)) * record_floats(g.DP) + (tid & 63);
     float nn = 0.f;
     for (int t = 0; t < g.width; ++t) nn = fmaf(xr[t * kR], xr[t * kR], nn);
-    List<KC> tk;
+    List<KC, kCapWide> tk;   // (no buffer is used)
     tk.start(nn, g.k, g.width);
     auto list_at = [&](int64_t s) { return ((s < segs ? b * segs + s : g.units - 1 - b) * kQ + tid) * KC; };   // segs: the item's own
     for (int64_t s = segs; live && s >= 0; --s) {
@@ -1169,9 +1177,7 @@ Layout layout(void *scratch, int64_t n, int DP, int k) {
     return L;
 }
 
-// CTAs that an SM holds: their shared memory lets two share it up to DP = 56.
-int ctas_per_sm(int DP) { return DP <= 56 ? 2 : 1; }
-int resident_ctas(int DP) { return sm_count() * ctas_per_sm(DP); }
+constexpr int kCtasPerSm = 2;   // resident
 
 Args make_args(const Layout &L, int64_t n, int DP, int width, int k, int metric, int32_t *cand, unsigned int *status) {
     Args g;
@@ -1210,7 +1216,7 @@ Args make_args(const Layout &L, int64_t n, int DP, int width, int k, int metric,
     g.big_bound = L.big_bound;
     g.units = L.units;
     g.big_cap = (int)std::min<int64_t>(kBigItems, L.units / 2);
-    g.slots = resident_ctas(DP);
+    g.slots = kCtasPerSm * sm_count();
     g.vv = nullptr;
     g.status = status;
     g.wait_budget = tc_wait_budget();
@@ -1234,13 +1240,14 @@ namespace simtp {
 template <int KC>
 cudaError_t launch_list(const Args &g, int64_t tiles, cudaStream_t st) {
     const int smem = smem_layout(g.DP).total;
-    auto whole = simt_pruned_kernel<KC, kWhole>;
-    auto split = simt_pruned_kernel<KC, kSplitItems>;
+    const bool wide = cap_of(g.DP) == kCapWide;
+    auto whole = wide ? simt_pruned_kernel<KC, kWhole, kCapWide> : simt_pruned_kernel<KC, kWhole, kCapNarrow>;
+    auto split = wide ? simt_pruned_kernel<KC, kSplitItems, kCapWide> : simt_pruned_kernel<KC, kSplitItems, kCapNarrow>;
     cudaError_t e = cudaFuncSetAttribute(whole, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(split, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    whole<<<(unsigned)std::min<int64_t>(tiles / 2, std::min(kMaxCtas, 2 * sm_count())), kQ, smem, st>>>(g, TieArgs{});
-    split<<<(unsigned)(2 * sm_count()), kQ, smem, st>>>(g, TieArgs{});
+    whole<<<(unsigned)std::min<int64_t>(tiles / 2, std::min(kMaxCtas, kCtasPerSm * sm_count())), kQ, smem, st>>>(g, TieArgs{});
+    split<<<(unsigned)(kCtasPerSm * sm_count()), kQ, smem, st>>>(g, TieArgs{});
     merge_kernel<KC><<<kBigItems, kQ, 0, st>>>(g);
     return cudaGetLastError();
 }
@@ -1251,10 +1258,10 @@ cudaError_t launch_ties(const Args &g, int d, int metric, const float *R, int64_
     const bool vec = rs % 4 == 0 && reinterpret_cast<uintptr_t>(R) % 16 == 0;
     const TieArgs ta{R, rs, d, metric == RSC_COSINE, vec, idx, dist};
     const int smem = smem_layout(g.DP).total;
-    auto kern = g.k <= 16 ? simt_pruned_kernel<16, kMode> : simt_pruned_kernel<32, kMode>;
+    auto kern = g.k <= 16 ? simt_pruned_kernel<16, kMode, kCapWide> : simt_pruned_kernel<32, kMode, kCapWide>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)(2 * sm_count()), kQ, smem, st>>>(g, ta);
+    kern<<<(unsigned)(kCtasPerSm * sm_count()), kQ, smem, st>>>(g, ta);
     return cudaGetLastError();
 }
 
@@ -1331,7 +1338,7 @@ FlatLayout flat_layout(void *scratch, int64_t n, int DP, int k) {
     Carve cv(scratch);
     FlatLayout L;
     const int64_t items = ceil_div(n, (int64_t)kQ);
-    const size_t parts = (size_t)items * kQ * simt_flat_segs(n, DP) * simt_pruned_list(k);
+    const size_t parts = (size_t)items * kQ * simt_flat_segs(n) * simt_pruned_list(k);
     L.rec = cv.take<float>((size_t)items * 2 * record_floats(DP));
     L.ids = cv.take<int32_t>((size_t)items * kQ);
     L.tile_pos = cv.take<int32_t>((size_t)items * 2);
@@ -1362,7 +1369,7 @@ Args flat_args(const FlatLayout &L, int64_t n, int DP, int width, int k, unsigne
     g.k = k;
     g.part_key = L.part_key;
     g.part_id = L.part_id;
-    g.part_segs = simt_flat_segs(n, DP);
+    g.part_segs = simt_flat_segs(n);
     g.vv = L.vv;
     g.tie_items = L.tie_items;
     g.tie_bound = L.tie_bound;
@@ -1370,7 +1377,7 @@ Args flat_args(const FlatLayout &L, int64_t n, int DP, int width, int k, unsigne
     g.tie_done = L.counters + kFlatCounters;
     // lists of 16 (k <= 16) or 32 entries in the room of part_segs lists an item
     g.units = ceil_div(n, (int64_t)kQ) * g.part_segs;
-    g.slots = resident_ctas(DP);
+    g.slots = kCtasPerSm * sm_count();
     g.status = status;
     g.wait_budget = tc_wait_budget();
     return g;
@@ -1386,9 +1393,9 @@ Args flat_args(const FlatLayout &L, int64_t n, int DP, int width, int k, unsigne
 // Parts per query tile pair: the count whose waves of persistent CTAs cost
 // least, a part costing its tiles plus about three (lists built anew, the
 // query tiles fetched).
-int simt_flat_segs(int64_t n, int DP) {
+int simt_flat_segs(int64_t n) {
     const int64_t items = ceil_div(n, (int64_t)simtp::kQ), tiles = ceil_div(n, (int64_t)simtp::kR);
-    const int64_t slots = kPlanSMs * simtp::ctas_per_sm(DP);
+    const int64_t slots = kPlanSMs * simtp::kCtasPerSm;
     int best = 1;
     int64_t cost = INT64_MAX;
     for (int s = 1; s <= kSimtFlatSegs && s <= tiles; ++s) {
@@ -1405,7 +1412,7 @@ size_t simt_flat_scratch_bytes(int64_t n, int DP, int k) { return simtp::flat_la
 
 SimtParts simt_flat_parts(void *scratch, int64_t n, int DP, int k) {
     const simtp::FlatLayout L = simtp::flat_layout(scratch, n, DP, k);
-    return {L.part_key, L.part_id, L.vv, simt_flat_segs(n, DP), simt_pruned_list(k), L.counters,
+    return {L.part_key, L.part_id, L.vv, simt_flat_segs(n), simt_pruned_list(k), L.counters,
             L.counters + simtp::kFlatCounters + ceil_div(n, (int64_t)simtp::kQ), L.tie_items, L.tie_bound};
 }
 
@@ -1420,9 +1427,12 @@ cudaError_t launch_knn_simt_flat(const float *Y, const float *ny, int64_t n, int
     pack_flat_kernel<<<(unsigned)(2 * items), 256, 0, st>>>(Y, ny, n, DP, L.rec, L.ids, L.tile_pos, L.tile_rows,
                                                            L.counters + 4);
     const int smem = smem_layout(DP).total;
-    auto kern = simt_pruned_list(k) == 24 ? simt_pruned_kernel<24, kFlat> : simt_pruned_kernel<kMaxList, kFlat>;
+    const bool wide = cap_of(DP) == kCapWide;
+    auto kern = simt_pruned_list(k) == 24
+                    ? (wide ? simt_pruned_kernel<24, kFlat, kCapWide> : simt_pruned_kernel<24, kFlat, kCapNarrow>)
+                    : (wide ? simt_pruned_kernel<kMaxList, kFlat, kCapWide> : simt_pruned_kernel<kMaxList, kFlat, kCapNarrow>);
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-    kern<<<(unsigned)std::min<int64_t>(items * g.part_segs, 2 * sm_count()), kQ, smem, st>>>(g, TieArgs{});
+    kern<<<(unsigned)std::min<int64_t>(items * g.part_segs, kCtasPerSm * sm_count()), kQ, smem, st>>>(g, TieArgs{});
     return cudaGetLastError();
 }
 
