@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(kQ, 2) simt_pruned_kernel(const Args g, const 
     // bounded; a budget shorter than a few sleeps is polled
     const uint32_t sleep_ns = g.wait_budget < 8 * (long long)kSleepNs ? 0 : kSleepNs;
     auto wait = [&](uint64_t *bar, uint32_t parity, long long budget) -> bool {
-        if (tc::mbar_arrived(bar, parity, sleep_ns)) return true;
+        if (sleep_ns == 0 ? tc::mbar_test_wait(bar, parity) : tc::mbar_try_wait(bar, parity)) return true;
         const long long t0 = clock64();
         while (!tc::mbar_arrived(bar, parity, sleep_ns))
             if (clock64() - t0 > budget) {
